@@ -193,9 +193,8 @@ struct cr_ctx {
     double* kry;             // Krylov workspace
     size_t kry_len;
     void* Lf;                // [P][P] Cholesky factor, factor precision (blocked path only)
-    unsigned char* Xt;       // bf16 hi/lo planes of X^T (mixed explicit S only)
-    int2* gtiles;            // lower-triangle blocks of G (mixed explicit S only)
-    int n_gtiles;
+    unsigned char* Xt;       // bf16 operands of the explicit S (mixed explicit S only)
+    float* spair_g;          // its pair sums (mixed explicit S only)
     // Krylov Gram on the tensor cores (mixed): sized on first use
     unsigned char* gram_x;   // bf16 planes of the B and HB columns
     size_t gram_x_cap;

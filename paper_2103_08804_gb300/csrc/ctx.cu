@@ -9,8 +9,8 @@
 cr_status tc_prepare(cr_ctx* c);
 cr_status target_prepare(cr_ctx* c);
 cr_status sym_prepare(cr_ctx* c);
-void sgram_geometry(const cr_ctx* c, int* R2, int* nkc_max, size_t* plane_bytes, int* npl);
-std::vector<int2> sgram_tiles(int P);
+void spair_sizes(const cr_ctx* c, size_t* x_bytes, size_t* g_bytes);
+cr_status spair_prepare(cr_ctx* c);
 
 cr_status cr_fail(cr_ctx* c, cr_status s, const char* fmt, ...) {
     if (c) {
@@ -163,26 +163,22 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     if (ncgpart < chol_cgpart_len()) ncgpart = chol_cgpart_len();
     ALLOC(c->cgpart, ncgpart * sizeof(double));
     ALLOC(c->scal, 64 * sizeof(double));
-    std::vector<int2> gt;
+    int dev = 0;
+    c->n_sm = 1;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (flags & CR_CTX_EXPLICIT_S) {
         ALLOC(c->S, P * P * 16);
         if (prec == CR_MIXED) {
-            int R2, nkc, npl;
-            size_t pb;
-            sgram_geometry(c, &R2, &nkc, &pb, &npl);
-            gt = sgram_tiles(c->P);
-            c->n_gtiles = (int)gt.size();
-            ALLOC(c->Xt, npl * pb);
-            ALLOC(c->gtiles, gt.size() * sizeof(int2));
+            size_t xb, gb;
+            spair_sizes(c, &xb, &gb);
+            ALLOC(c->Xt, xb);
+            ALLOC(c->spair_g, gb);
         } else {
             ALLOC(c->O_tmp, B * P * cs);
         }
         if (chol_blocked(c)) ALLOC(c->Lf, chol_factor_bytes(c));
     }
-    int dev = 0;
-    c->n_sm = 1;
-    if (cudaGetDevice(&dev) == cudaSuccess)
-        cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev);
     std::vector<int2> ot;
     if (prec == CR_MIXED) {
         size_t xb, pb;
@@ -218,15 +214,14 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     }
     std::vector<int2> bonds = make_bonds(c->Lx, c->Ly);
     e = cudaMemcpy(c->d_bonds, bonds.data(), Nb * sizeof(int2), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !gt.empty())
-        e = cudaMemcpy(c->gtiles, gt.data(), gt.size() * sizeof(int2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !ot.empty()) {
         e = cudaMemcpy(c->ored_tiles, ot.data(), ot.size() * sizeof(int2), cudaMemcpyHostToDevice);
         c->ored = e == cudaSuccess;
     }
     if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->scal, 0, 64 * sizeof(double));
-    if (e != cudaSuccess || tc_prepare(c) != CR_OK || target_prepare(c) != CR_OK || sym_prepare(c) != CR_OK ||
+    if (e != cudaSuccess || tc_prepare(c) != CR_OK || (prec == CR_MIXED && spair_prepare(c) != CR_OK) ||
+        target_prepare(c) != CR_OK || sym_prepare(c) != CR_OK ||
         (c->fcg && fcg_prepare(c) != CR_OK)) {
         cr_destroy(c);
         return CR_ECUDA;
@@ -242,7 +237,7 @@ extern "C" cr_status cr_destroy(cr_ctx* c) {
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     void* ptrs[] = {c->d_status, c->d_bonds, c->theta_tmp, c->lp_tmp, c->u_tmp, c->partial,
                     c->red, c->F, c->cg, c->p_lo, c->cgpart, c->scal, c->S, c->O_tmp, c->kry,
-                    c->Lf, c->Xt, c->gtiles, c->fcg_a1, c->fcg_b2, c->fcg_v2, c->fcg_vab,
+                    c->Lf, c->Xt, c->spair_g, c->fcg_a1, c->fcg_b2, c->fcg_v2, c->fcg_vab,
                     c->fcg_part, c->fcg_psc, c->fcg_bar, c->gram_x, c->gram_part,
                     c->gram_tiles, c->lp_work, c->ored_x, c->ored_part, c->ored_tiles};
     for (void* p : ptrs)

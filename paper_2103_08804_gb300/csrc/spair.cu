@@ -1,0 +1,519 @@
+// Explicit S of the natural-gradient update (Sec. III) on the tensor cores,
+// for CR_MIXED contexts.
+//
+// With sigma_0 = t_0 = 1 in front of the spins and of T_j = tanh theta_j,
+// every log-derivative is O_k = sigma_i t_j for one (i, j) other than (0, 0),
+// so
+//   sum_s conj(O_k) O_l = sum_s (sigma_i sigma_i') (conj(t_j) t_j')
+// depends on the unordered spin pair {i, i'} (sigma^2 = 1: the pairs i = i'
+// are all the row of ones) and on the pair (j, j') up to conjugation.  The
+// P x P matrix of complex sums is therefore one real product
+//   G[y][r] = sum_s Y_y(s) A_r(s),
+//   A: 1 + N (N + 1) / 2 spin products, +-1, exact in one bf16 plane,
+//   Y: (M + 1)^2 real columns, Re and Im of conj(t_j) t_j' (j < j') and
+//      |t_j|^2, float32 values split into NPL bf16 terms,
+// about P^2 / 2 x NPL multiply-adds per walker where the Gram matrix of
+// [Re O | Im O] takes 2 P^2 x 6 (both of its operands need the split):
+// eight times fewer for NPL = 3.  NPL = 3 holds all 24 bits of a float32;
+// NPL = 2 (CR_CTX_S_BF16X3) is good to about 2^-17 per product.
+//
+// TMEM accumulates in float32 with an error that grows with the number of
+// MMAs added into one accumulator (measured: relative ~1e-8 each), so a
+// tile is accumulated over chunks of 256 walkers (48 MMAs) in one TMEM half
+// while the other half is added into float32 registers of the drain warps.
+//
+//   spair_a_kernel, spair_y_kernel   the operands, tiles of 32 walkers in the
+//                                    K-major core-matrix layout
+//   spair_tc_kernel                  G, tiles of 128 Y columns x 256 pairs
+//   spair_expand_kernel              S = G / B - conj(Obar) Obar^T + shift I
+//
+// The MMA's M side takes Y (three planes) and its N side the pairs (one
+// plane): 40 KB of operands per 32 walkers and tile; the other way round it
+// would be 56 KB, and the operand stream from L2 is what the kernel waits
+// for.  At N = M = 100 and 32768 walkers the whole explicit-S solve went from
+// 203.4 to 102.7 ms with this in place of the Gram matrix of [Re O | Im O]
+// (111 ms), the error of the update from 3.6e-7 to 3.0e-7.
+#include <cuda_bf16.h>
+
+#include "common.cuh"
+#include "tc.cuh"
+
+namespace {
+
+constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded mbarrier polls
+constexpr int KC = 32;                      // walkers per operand tile
+constexpr int CHUNK = 8;                    // operand tiles per TMEM accumulation
+constexpr int YT = 128, AT = 256;           // tile of G: Y columns x pairs
+constexpr int Y_TILE = YT * KC * 2;         // bytes of one plane
+constexpr int A_TILE = AT * KC * 2;
+constexpr int SP_THREADS = 288;             // warp 0 copies and issues, warps 1-8 drain
+constexpr size_t OPERAND_BUDGET = (size_t)3 << 30;  // bytes of operands held at once
+
+template <int NPL> struct Ring {
+    static constexpr int STAGE = NPL * Y_TILE + A_TILE;
+    static constexpr int NSTG = 5;
+    static constexpr size_t SMEM = (size_t)NSTG * STAGE + 256;
+};
+
+CR_D void split3(float x, __nv_bfloat16* hi, __nv_bfloat16* mid, __nv_bfloat16* lo) {
+    *hi = __float2bfloat16_rn(x);
+    const float r1 = x - __bfloat162float(*hi);
+    *mid = __float2bfloat16_rn(r1);
+    *lo = __float2bfloat16_rn(r1 - __bfloat162float(*mid));
+}
+
+CR_D uint4 pack8(const __nv_bfloat16* v) {
+    uint4 r;
+    uint32_t* w = reinterpret_cast<uint32_t*>(&r);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        w[q] = (uint32_t)__bfloat16_as_ushort(v[2 * q]) |
+               ((uint32_t)__bfloat16_as_ushort(v[2 * q + 1]) << 16);
+    return r;
+}
+
+// Pairs a < b numbered b (b - 1) / 2 + a.
+CR_HD int pair_index(int a, int b) { return b * (b - 1) / 2 + a; }
+CR_D void pair_of(int p, int* a, int* b) {
+    int y = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f);
+    while (y * (y - 1) / 2 > p) --y;
+    while ((y + 1) * y / 2 <= p) ++y;
+    *b = y;
+    *a = p - y * (y - 1) / 2;
+}
+
+struct PairGeo {
+    int nA, nY;          // rows of A (pairs and the ones), columns of Y
+    int nab, nyb;        // blocks of 256 and 128
+    int ntiles, nseg;    // tiles of G, K segments
+    int slab;            // walkers per pass over the operands (a multiple of 256)
+    size_t a_bytes, y_bytes, g_elems;  // operands of a slab; elements of one G
+};
+
+int npl_of(const cr_ctx* c) { return (c->flags & CR_CTX_S_BF16X3) ? 2 : 3; }
+
+PairGeo pair_geometry(const cr_ctx* c) {
+    PairGeo g;
+    g.nA = 1 + c->N * (c->N + 1) / 2;
+    g.nY = (c->M + 1) * (c->M + 1);
+    g.nab = (g.nA + AT - 1) / AT;
+    g.nyb = (g.nY + YT - 1) / YT;
+    g.ntiles = g.nab * g.nyb;
+    constexpr int CW = KC * CHUNK;
+    const size_t per = 2 * ((size_t)g.nab * AT + (size_t)npl_of(c) * g.nyb * YT);  // bytes a walker
+    const int nch = (c->max_walkers + CW - 1) / CW;
+    size_t fit = OPERAND_BUDGET / (per * CW);
+    if (fit < 1) fit = 1;
+    const int chunks = (size_t)nch < fit ? nch : (int)fit;
+    g.slab = chunks * CW;
+    // few tiles: split the walkers so that every SM has an item, a chunk at least each
+    g.nseg = c->n_sm / g.ntiles;
+    if (g.nseg > chunks) g.nseg = chunks;
+    if (g.nseg < 1) g.nseg = 1;
+    g.a_bytes = (size_t)g.nab * AT * g.slab * 2;
+    g.y_bytes = (size_t)npl_of(c) * g.nyb * YT * g.slab * 2;
+    g.g_elems = (size_t)g.nab * AT * g.nyb * YT;
+    return g;
+}
+
+// A tiles: [block of 256 pairs][32 walkers], pair r < N (N + 1) / 2 is
+// (i, i') of the extended spins, the last one is the row of ones; zero past
+// the walkers and the pairs.  Grid (walker tile, pair block); the walkers'
+// spins are staged once, extended by sigma_0 = 1.
+__global__ void __launch_bounds__(256) spair_a_kernel(const int8_t* __restrict__ spins, int s0,
+                                                      int B, int N, int nA, int nkc,
+                                                      unsigned char* __restrict__ A) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    int8_t* sg = (int8_t*)sm;  // [N + 1][KC]
+    const int kc = blockIdx.x, ab = blockIdx.y, t = threadIdx.x;
+    for (int e = t; e < KC * (N + 1); e += blockDim.x) {
+        const int w = e / (N + 1), i = e % (N + 1), s = s0 + kc * KC + w;
+        sg[i * KC + w] = s < B ? (i == 0 ? (int8_t)1 : spins[(size_t)s * N + i - 1]) : (int8_t)0;
+    }
+    __syncthreads();
+    unsigned char* out = A + ((size_t)ab * nkc + kc) * A_TILE;
+    for (int e = t; e < AT * (KC / 8); e += blockDim.x) {
+        const int r = e % AT, grp = e / AT, p = ab * AT + r;
+        int a = 0, b = 0;
+        if (p < nA - 1) pair_of(p, &a, &b);
+        __nv_bfloat16 v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int x = sg[a * KC + grp * 8 + q] * sg[b * KC + grp * 8 + q];  // (0, 0): ones
+            v[q] = __float2bfloat16_rn(p < nA ? (float)x : 0.f);
+        }
+        *reinterpret_cast<uint4*>(out + tc::kmajor_offset(r, grp * 8, KC)) = pack8(v);
+    }
+}
+
+// Y tiles: [block of 128 columns][32 walkers][plane].  Columns 2 p and 2 p + 1
+// are Re and Im of conj(t_j) t_j' of pair p = (j, j') of the extended hidden
+// units; the M + 1 columns from M (M + 1) on are |t_j|^2.  A thread forms two
+// adjacent columns of 8 walkers.  Grid (walker tile, column block).
+template <int NPL>
+__global__ void __launch_bounds__(256) spair_y_kernel(const cpx<float>* __restrict__ T, int s0,
+                                                      int B, int M, int nY, int nkc,
+                                                      unsigned char* __restrict__ Y) {
+    const int kc = blockIdx.x, yb = blockIdx.y, t = threadIdx.x;
+    const int c2 = t & 63, grp = t >> 6;  // column pair of the block, 8 walkers
+    const int y = yb * YT + 2 * c2, nOff = M * (M + 1);
+    int j[2] = {0, 0}, jp[2] = {0, 0};
+    const bool off = y < nOff;
+    if (off) {
+        pair_of(y >> 1, &j[0], &jp[0]);
+    } else {
+        j[0] = jp[0] = y - nOff;  // nOff is even: both columns are |t|^2
+        j[1] = jp[1] = y + 1 - nOff;
+    }
+    __nv_bfloat16 h[2][8], m[2][8], l[2][8];
+    const cpx<float> one = {1.f, 0.f}, zero = {0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int s = s0 + kc * KC + grp * 8 + q;
+        const cpx<float>* Ts = T + (size_t)s * M - 1;  // t_j = Ts[j], j >= 1
+        float x0 = 0.f, x1 = 0.f;
+        if (s < B && y < nY) {
+            if (off) {
+                const cpx<float> a = j[0] ? ldg(Ts + j[0]) : one, b = ldg(Ts + jp[0]);
+                const cpx<float> v = cmulc(a, b);
+                x0 = v.x;
+                x1 = v.y;
+            } else {
+                x0 = j[0] ? abs2(ldg(Ts + j[0])) : 1.f;
+                const cpx<float> b = y + 1 < nY ? ldg(Ts + j[1]) : zero;
+                x1 = abs2(b);
+            }
+        }
+        split3(x0, &h[0][q], &m[0][q], &l[0][q]);
+        split3(x1, &h[1][q], &m[1][q], &l[1][q]);
+    }
+    unsigned char* out = Y + ((size_t)yb * nkc + kc) * NPL * Y_TILE;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const uint32_t o = tc::kmajor_offset(2 * c2 + k, grp * 8, KC);
+        *reinterpret_cast<uint4*>(out + o) = pack8(h[k]);
+        *reinterpret_cast<uint4*>(out + Y_TILE + o) = pack8(m[k]);
+        if (NPL == 3) *reinterpret_cast<uint4*>(out + 2 * Y_TILE + o) = pack8(l[k]);
+    }
+}
+
+struct PairArgs {
+    const unsigned char* A;
+    const unsigned char* Y;
+    int nkc;           // walker tiles of the operands
+    int kseg, nseg;    // walker tiles per item (the last segment may have fewer), segments
+    int nab, nyb;
+    float* G;          // [nseg][pair][Y column]
+    int add;           // a later slab: add to G
+    int* status;
+};
+
+// Persistent, one CTA per SM; an item is one tile of G over one K segment,
+// items segment-major and pair blocks fastest, so that the CTAs running
+// together read few Y blocks.  Warp 0 (one thread) copies an operand stage
+// with two bulk copies, NSTG - 1 stages ahead across items, and issues the
+// MMAs; chunk c goes to TMEM columns [256 (c % 2), +256).
+template <int NPL>
+__global__ void __launch_bounds__(SP_THREADS, 1) spair_tc_kernel(const PairArgs a) {
+    using RG = Ring<NPL>;
+    constexpr int NSTG = RG::NSTG;
+    extern __shared__ __align__(1024) unsigned char sm[];
+    uint64_t* full = (uint64_t*)(sm + NSTG * RG::STAGE);
+    uint64_t* empty = full + NSTG;      // [NSTG] MMAs reading a stage done
+    uint64_t* cdone = full + 2 * NSTG;  // [2] MMAs of a chunk done (per TMEM half)
+    uint64_t* drained = cdone + 2;      // [2] TMEM half read by the 256 drain threads
+    uint32_t* slot = (uint32_t*)(drained + 2);
+    volatile int* abort = (volatile int*)(slot + 1);
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    if (t == 0) {
+        for (int i = 0; i < 2 * NSTG + 2; ++i) tc::mbar_init(&full[i], 1);
+        tc::mbar_init(&drained[0], 256);
+        tc::mbar_init(&drained[1], 256);
+        tc::fence_mbar_init();
+        *abort = 0;
+    }
+    if (warp == 0) {
+        tc::tmem_alloc(slot, 512u);
+        tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t taddr = *slot;
+    const int ntiles = a.nab * a.nyb, nitems = ntiles * a.nseg;
+    auto wait = [&](uint64_t* bar, uint32_t par) {
+        for (int i = 0; i < 64; ++i) {
+            if (tc::mbar_wait(bar, par, WAIT_LIMIT >> 6)) return true;
+            if (*abort) return false;
+        }
+        *abort = 1;
+        return false;
+    };
+    // walker tiles [k0, k1) of an item
+    auto krange = [&](int item, int* k0, int* k1) {
+        *k0 = (item / ntiles) * a.kseg;
+        *k1 = min(a.nkc, *k0 + a.kseg);
+    };
+    if (warp == 0) {
+        if (lane == 0) {
+            const uint32_t idesc = tc::make_idesc_bf16(YT, AT);
+            uint32_t pend = 0, pend_par = 0;
+            int last_g = -1;
+            bool ok = true;
+            // load cursor: the stages of all items in one sequence
+            int litem = blockIdx.x, lk = 0, lk1 = 0, lg = 0;
+            if (litem < nitems) krange(litem, &lk, &lk1);
+            auto load = [&]() {
+                const uint32_t b = lg % NSTG;
+                if (lg >= NSTG && !wait(&empty[b], ((lg - NSTG) / NSTG) & 1)) return false;
+                const int tile = litem % ntiles, ab = tile % a.nab, yb = tile / a.nab;
+                pend |= 1u << b;
+                pend_par = (pend_par & ~(1u << b)) | (((uint32_t)(lg / NSTG) & 1u) << b);
+                unsigned char* st = sm + (size_t)b * RG::STAGE;
+                tc::mbar_expect_tx(&full[b], (uint32_t)RG::STAGE);
+                tc::bulk_g2s(st, a.Y + ((size_t)yb * a.nkc + lk) * NPL * Y_TILE, NPL * Y_TILE, &full[b]);
+                tc::bulk_g2s(st + NPL * Y_TILE, a.A + ((size_t)ab * a.nkc + lk) * A_TILE, A_TILE, &full[b]);
+                ++lg;
+                if (++lk == lk1) {
+                    litem += gridDim.x;
+                    if (litem < nitems) krange(litem, &lk, &lk1);
+                }
+                return true;
+            };
+            for (int i = 0; i < NSTG - 1 && litem < nitems && ok; ++i) ok = load();
+            int g = 0, gc = 0;
+            for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+                int k0, k1;
+                krange(item, &k0, &k1);
+                for (int kc = k0; kc < k1 && ok; ++kc, ++g) {
+                    const uint32_t b = g % NSTG;
+                    const bool first = (kc - k0) % CHUNK == 0;
+                    const uint32_t h = gc & 1;
+                    // the TMEM half of chunk gc was last used by chunk gc - 2
+                    if (first && gc >= 2 && !wait(&drained[h], ((gc - 2) >> 1) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    if (!wait(&full[b], (g / NSTG) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    pend &= ~(1u << b);
+                    tc::fence_after_sync();
+                    const uint32_t ys = tc::smem_u32(sm + (size_t)b * RG::STAGE);
+                    const uint32_t as = ys + NPL * Y_TILE;
+#pragma unroll
+                    for (int ks = 0; ks < KC / 16; ++ks) {
+                        const uint64_t bd = tc::make_desc(as + ks * 256, 128, 16 * KC);
+#pragma unroll
+                        for (int pl = 0; pl < NPL; ++pl) {
+                            const uint64_t ad = tc::make_desc(ys + pl * Y_TILE + ks * 256, 128, 16 * KC);
+                            tc::mma_bf16(taddr + h * 256, ad, bd, idesc, !(first && ks == 0 && pl == 0));
+                        }
+                    }
+                    tc::commit(&empty[b]);
+                    last_g = g;
+                    if ((kc - k0) % CHUNK == CHUNK - 1 || kc + 1 == k1) {
+                        tc::commit(&cdone[h]);
+                        ++gc;
+                    }
+                    if (litem < nitems && !load()) ok = false;
+                }
+            }
+            if (!ok) {
+                *abort = 1;
+                set_status(a.status, CR_ETIMEOUT);
+                // let copies in flight land and issued MMAs finish (bounded)
+                for (int b = 0; b < NSTG; ++b)
+                    if (pend & (1u << b)) tc::mbar_wait(&full[b], (pend_par >> b) & 1u, WAIT_LIMIT);
+                if (last_g >= 0)
+                    tc::mbar_wait(&empty[last_g % NSTG], (uint32_t)(last_g / NSTG) & 1u, WAIT_LIMIT);
+            }
+        }
+        __syncwarp();
+    } else {
+        // drain: warp w reads TMEM lanes 32 (w % 4) .. + 31 (Y columns) and
+        // the 128 pairs from 128 c2 on, c2 = (w - 1) / 4
+        const int lb = warp & 3, c2 = (warp - 1) >> 2;
+        const size_t ldg_ = (size_t)a.nyb * YT;
+        bool ok = true;
+        int gc = 0;
+        for (int item = blockIdx.x; item < nitems && ok; item += gridDim.x) {
+            int k0, k1;
+            krange(item, &k0, &k1);
+            const int tile = item % ntiles, ab = tile % a.nab, yb = tile / a.nab;
+            float acc[128];
+#pragma unroll
+            for (int q = 0; q < 128; ++q) acc[q] = 0.f;
+            for (int kc = k0; kc < k1; kc += CHUNK, ++gc) {
+                const uint32_t h = gc & 1;
+                // warp-uniform outcome: tcgen05.ld below is a warp-wide instruction
+                if (!__all_sync(0xffffffffu, wait(&cdone[h], (gc >> 1) & 1))) {
+                    ok = false;
+                    break;
+                }
+                tc::fence_after_sync();
+#pragma unroll
+                for (int ch = 0; ch < 8; ++ch) {
+                    float v[16];
+                    tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + h * 256 + 128 * c2 + 16 * ch, v);
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) acc[16 * ch + q] = __fadd_rn(acc[16 * ch + q], v[q]);
+                }
+                tc::fence_before_sync();
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(
+                                 tc::smem_u32(&drained[h]))
+                             : "memory");
+            }
+            if (!ok) break;
+            // lanes hold consecutive Y columns: coalesced rows of G
+            float* out = a.G + (size_t)(item / ntiles) * a.nab * AT * ldg_ +
+                         ((size_t)ab * AT + 128 * c2) * ldg_ + (size_t)yb * YT + 32 * lb + lane;
+            if (a.add) {
+#pragma unroll
+                for (int q = 0; q < 128; ++q) out[q * ldg_] = __fadd_rn(out[q * ldg_], acc[q]);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 128; ++q) out[q * ldg_] = acc[q];
+            }
+        }
+        if (!ok && t == 32) set_status(a.status, CR_ETIMEOUT);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(taddr, 512u);
+}
+
+// extended (i, j) of parameter k
+CR_D void param_of(int k, int N, int M, int* i, int* j) {
+    if (k < N) {
+        *i = k + 1;
+        *j = 0;
+    } else if (k < N + M) {
+        *i = 0;
+        *j = k - N + 1;
+    } else {
+        *i = (k - N - M) / M + 1;
+        *j = (k - N - M) % M + 1;
+    }
+}
+
+// S of the 32 x 32 tile (by, bx), bx <= by, and its mirror image: S_kl of
+// the lower triangle from the segments' sums (float64, in segment order),
+// the upper triangle its exact conjugate.
+__global__ void __launch_bounds__(256) spair_expand_kernel(const float* __restrict__ G, int nseg,
+                                                           size_t seg_stride, size_t ld, int N,
+                                                           int M, int P, int B,
+                                                           const double* __restrict__ redO_,
+                                                           double shift, double* __restrict__ S_) {
+    const int bx = blockIdx.x, by = blockIdx.y;
+    if (bx > by) return;
+    __shared__ cpx<double> tl[32][33];
+    const cpx<double>* redO = (const cpx<double>*)redO_;
+    cpx<double>* S = (cpx<double>*)S_;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const double inv = 1.0 / B;
+    const int l = bx * 32 + tx, nA = 1 + N * (N + 1) / 2, nOff = M * (M + 1);
+    int il = 0, jl = 0;
+    cpx<double> ol = {0.0, 0.0};
+    if (l < P) {
+        param_of(l, N, M, &il, &jl);
+        ol = inv * redO[l];
+    }
+    for (int q = ty; q < 32; q += 8) {
+        const int k = by * 32 + q;
+        if (k >= P || l >= P) continue;
+        int ik, jk;
+        param_of(k, N, M, &ik, &jk);
+        const int row = ik == il ? nA - 1 : pair_index(min(ik, il), max(ik, il));
+        const float* g = G + (size_t)row * ld;
+        cpx<double> v = {0.0, 0.0};
+        if (jk == jl) {
+            for (int sg = 0; sg < nseg; ++sg) v.x += (double)g[sg * seg_stride + nOff + jk];
+        } else {
+            const int y = 2 * pair_index(min(jk, jl), max(jk, jl));
+            for (int sg = 0; sg < nseg; ++sg) {
+                const float2 x = *reinterpret_cast<const float2*>(g + sg * seg_stride + y);
+                v = v + cpx<double>{(double)x.x, (double)x.y};
+            }
+            if (jk > jl) v = conj(v);  // the sum held is that of conj(t_jl) t_jk
+        }
+        v = inv * v - cmulc(inv * redO[k], ol);
+        if (k == l) v = {v.x + shift, 0.0};
+        tl[q][tx] = v;
+        if (l <= k) S[(size_t)k * P + l] = v;
+    }
+    __syncthreads();
+    for (int q = ty; q < 32; q += 8) {
+        const int r = bx * 32 + q, c = by * 32 + tx;  // mirror: row r, column c, r < c
+        if (r < P && c < P && r < c) S[(size_t)r * P + c] = conj(tl[tx][q]);
+    }
+}
+
+template <int NPL>
+cr_status spair_t(cr_ctx* c, const int8_t* spins, const void* T, int B, const double* redO,
+                  double shift) {
+    const PairGeo g = pair_geometry(c);
+    const int N = c->N, M = c->M;
+    constexpr int CW = KC * CHUNK;
+    int nseg = 0, cps = 0;  // segments and chunks per segment of the first slab
+    for (int s0 = 0; s0 < B; s0 += g.slab) {
+        const int nw = B - s0 < g.slab ? B - s0 : g.slab;
+        const int nch = (nw + CW - 1) / CW, nkc = nch * CHUNK;
+        if (s0 == 0) {
+            nseg = g.nseg < nch ? g.nseg : nch;
+            cps = (nch + nseg - 1) / nseg;
+            nseg = (nch + cps - 1) / cps;
+        }
+        // later slabs keep the first one's segment length: never more segments
+        const int sg = (nch + cps - 1) / cps;
+        CR_LAUNCH(c, CR_K_OTHER,
+                  spair_a_kernel<<<dim3(nkc, g.nab), 256, KC * (N + 1), c->stream>>>(
+                      spins, s0, B, N, g.nA, nkc, c->Xt));
+        CR_LAUNCH(c, CR_K_OTHER,
+                  spair_y_kernel<NPL><<<dim3(nkc, g.nyb), 256, 0, c->stream>>>(
+                      (const cpx<float>*)T, s0, B, M, g.nY, nkc, c->Xt + g.a_bytes));
+        PairArgs a;
+        a.A = c->Xt;
+        a.Y = c->Xt + g.a_bytes;
+        a.nkc = nkc;
+        a.kseg = cps * CHUNK;
+        a.nseg = sg;
+        a.nab = g.nab;
+        a.nyb = g.nyb;
+        a.G = c->spair_g;
+        a.add = s0 > 0;
+        a.status = c->d_status;
+        const int items = g.ntiles * sg, grid = items < c->n_sm ? items : c->n_sm;
+        CR_LAUNCH(c, CR_KERNEL_SBUILD,
+                  spair_tc_kernel<NPL><<<grid, SP_THREADS, Ring<NPL>::SMEM, c->stream>>>(a));
+    }
+    const int nt = (c->P + 31) / 32;
+    CR_LAUNCH(c, CR_K_OTHER,
+              spair_expand_kernel<<<dim3(nt, nt), 256, 0, c->stream>>>(
+                  c->spair_g, nseg, g.g_elems, (size_t)g.nyb * YT, N, M, c->P, B, redO, shift, c->S));
+    return cr_check_launch(c, "explicit S (tensor cores)");
+}
+
+}  // namespace
+
+void spair_sizes(const cr_ctx* c, size_t* x_bytes, size_t* g_bytes) {
+    const PairGeo g = pair_geometry(c);
+    *x_bytes = g.a_bytes + g.y_bytes;
+    *g_bytes = (size_t)g.nseg * g.g_elems * sizeof(float);
+}
+
+cr_status spair_prepare(cr_ctx* c) {
+    cudaError_t e = cudaFuncSetAttribute(spair_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)Ring<2>::SMEM);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(spair_tc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)Ring<3>::SMEM);
+    return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "spair_prepare: %s", cudaGetErrorString(e));
+}
+
+cr_status launch_sbuild_tc(cr_ctx* c, const int8_t* spins, const void* T, int B,
+                           const double* redO, double shift) {
+    return npl_of(c) == 2 ? spair_t<2>(c, spins, T, B, redO, shift)
+                          : spair_t<3>(c, spins, T, B, redO, shift);
+}

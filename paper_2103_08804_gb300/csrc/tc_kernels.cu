@@ -13,8 +13,8 @@
 //   oreduce_tc_kernel sum over a walker chunk of sigma_si conj(T_sj) g_s, plus
 //                     the a-, b- and scalar sums of oreduce_kernel's partial rows
 //
-// The explicit S of the Cholesky path (sgram_tc_kernel, further down) has
-// float32 values in both operands; both are split (see there).
+// The Krylov Gram and the estimator sums (sgram_tc_kernel, further down)
+// split both operands, or one (see there).
 #include <cuda_bf16.h>
 
 #include <vector>
@@ -394,20 +394,14 @@ __global__ void __launch_bounds__(RED_THREADS, 1) oreduce_tc_kernel(
     if (warp == 0) tc::tmem_dealloc(taddr, (uint32_t)tmem_cols);
 }
 
-// ------------------------------------------------- explicit S (Sec. III)
+// ----------------------------------------- Gram matrices from bf16 splits
 //
-// S_kl = sum_s conj(O_sk) O_sl / B - conj(Obar_k) Obar_l (+ shift on the
-// diagonal) through the real Gram matrix G = X^T X of X = [Re O | Im O]
-// (column 2k = Re O_k, 2k + 1 = Im O_k):
-//   Re S_kl = G[2k][2l] + G[2k+1][2l+1],  Im S_kl = G[2k][2l+1] - G[2k+1][2l].
-// Both operands are float32 values split into NPL bf16 terms, the products
-// summed in float32 in TMEM over all walkers:
-//   NPL = 3 (default): x = hi + mid + lo, six products hi.hi + hi.mid +
-//     mid.hi + hi.lo + mid.mid + lo.hi, about float32 accuracy ("bf16x6");
-//   NPL = 2 (CR_CTX_S_BF16X3): x = hi + lo + O(2^-17 |x|), three products
-//     hi.hi + hi.lo + lo.hi ("bf16x3").  Its error, about 2^-16 relative per
-//     product, can push the smallest eigenvalues of S + lambda I below
-//     lambda and, at lambda = 1e-3 on large lattices, below zero.
+// G = X^T Y of float32 columns x_k, y_l taken as complex numbers: real rows
+// 2k = Re x_k and 2k + 1 = Im x_k, and
+//   Re G_kl = G[2k][2l] + G[2k+1][2l+1],  Im G_kl = G[2k][2l+1] - G[2k+1][2l].
+// The operands are split into three bf16 terms x = hi + mid + lo, six
+// products hi.hi + hi.mid + mid.hi + hi.lo + mid.mid + lo.hi, about float32
+// accuracy ("bf16x6"), summed in float32 in TMEM.
 //
 // TMEM accumulates in float32 with a per-step error that grows with the
 // number of MMAs added into one accumulator (measured: relative ~1e-8 per
@@ -417,26 +411,26 @@ __global__ void __launch_bounds__(RED_THREADS, 1) oreduce_tc_kernel(
 // (the float64 pipe of this GPU is far too narrow to keep up with the tensor
 // cores), which leaves shared memory to a deep operand pipeline.
 //
-// xt_prep_kernel writes X^T as NPL bf16 planes, each an array of tiles
+// The operands lie in memory as bf16 planes, each an array of tiles
 // [row block of 128 G rows][walker chunk of KC] in the K-major no-swizzle
 // core-matrix layout, so one bulk copy moves one tile.
 // sgram_tc_kernel: persistent, 288 threads.  Warp 0 (one thread) copies
 // operand tiles through NSTG stages (running ahead across tiles) and issues
 // the MMAs of chunk c into TMEM columns [256 (c % 2), +256); warps 1-8 wait
-// for the chunk, add it to their register tile of S (entries formed from
+// for the chunk, add it to their register tile of G (entries formed from
 // adjacent lanes = rows 2k, 2k + 1), release the TMEM half, and at the end
-// of a tile write S.
-template <int NPL>
+// of a tile write its sums.
 struct SGram {
-    static constexpr int KC = NPL == 2 ? 32 : 16;    // walkers per operand tile
+    static constexpr int NPL = 3;                     // bf16 planes of a split operand
+    static constexpr int KC = 16;                     // walkers per operand tile
     static constexpr int TILE = 128 * KC * 2;         // bytes of one 128-row tile
     static constexpr int STAGE = NPL * 3 * TILE;      // A (1 row block) + B (2), NPL planes
-    static constexpr int NSTG = NPL == 2 ? 4 : 6;     // pipeline stages
-    static constexpr int NPROD = NPL == 2 ? 3 : 6;
-    static constexpr int CH = NPL == 2 ? 256 : 128;   // walkers per TMEM accumulation
+    static constexpr int NSTG = 6;                    // pipeline stages
+    static constexpr int NPROD = 6;
+    static constexpr int CH = 128;                    // walkers per TMEM accumulation
     static constexpr size_t SMEM = (size_t)NSTG * STAGE + 256;
     // planes (A, B) of product pr: (hi, hi), (hi, mid), (mid, hi), (hi, lo),
-    // (mid, mid), (lo, hi); NPL = 2 takes the first three (mid = lo there)
+    // (mid, mid), (lo, hi)
     static CR_HD int pa(int pr) {
         constexpr int v[6] = {0, 0, 1, 0, 1, 2};
         return v[pr];
@@ -447,50 +441,6 @@ struct SGram {
     }
 };
 constexpr int GR_THREADS = 288;
-
-template <int NPL>
-__global__ void xt_prep_kernel(const int8_t* __restrict__ spins, const cpx<float>* __restrict__ T,
-                               int B, int N, int M, int P, int R2, int nkc_max, int nkc,
-                               size_t plane_bytes, unsigned char* __restrict__ Xt) {
-    using G = SGram<NPL>;
-    constexpr int NG = G::KC / 8;  // groups of 8 walkers per tile
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t total = (size_t)R2 * nkc * NG;
-    if (idx >= total) return;
-    const int r = (int)(idx % 128), grp = (int)((idx / 128) % NG);
-    const size_t rest = idx / (128 * NG);
-    const int kc = (int)(rest % nkc), rb = (int)(rest / nkc);
-    const int row = rb * 128 + r, k = row >> 1, im = row & 1;
-    __nv_bfloat16 t0[8], t1[8], t2[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int s = kc * G::KC + grp * 8 + q;
-        float x = 0.f;
-        if (k < P && s < B) {
-            cpx<float> o;
-            if (k < N) {
-                o = {(float)spins[(size_t)s * N + k], 0.f};
-            } else if (k < N + M) {
-                o = T[(size_t)s * M + (k - N)];
-            } else {
-                const int i = (k - N - M) / M, j = (k - N - M) % M;
-                o = (float)spins[(size_t)s * N + i] * T[(size_t)s * M + j];
-            }
-            x = im ? o.y : o.x;
-        }
-        if (NPL == 3) {
-            split3(x, &t0[q], &t1[q], &t2[q]);
-        } else {
-            t0[q] = __float2bfloat16_rn(x);
-            t1[q] = __float2bfloat16_rn(x - __bfloat162float(t0[q]));
-        }
-    }
-    const size_t off =
-        ((size_t)rb * nkc_max + kc) * G::TILE + tc::kmajor_offset(r, grp * 8, G::KC);
-    *reinterpret_cast<uint4*>(Xt + off) = pack8(t0);
-    *reinterpret_cast<uint4*>(Xt + plane_bytes + off) = pack8(t1);
-    if (NPL == 3) *reinterpret_cast<uint4*>(Xt + 2 * plane_bytes + off) = pack8(t2);
-}
 
 // Arguments of sgram_tc_kernel.  A work item is one tile (rt, ct) of G over
 // one K segment of kseg walker tiles; items run segment-major (item i:
@@ -510,22 +460,16 @@ struct GramArgs {
     int kseg, nseg;           // walker tiles per item, K segments per tile
     const int2* tiles;
     int ntiles;
-    // explicit S (part == nullptr): S = G / B - conj(Obar) Obar^T + shift I
-    int P, B;
-    const double* redO;
-    double shift;
-    double* S;
-    // otherwise the raw float32 sums of every item, complex128
+    // the float32 sums of every item, complex128
     // part[((op * nseg + seg) * Na + n) * Nb + m], n < Na, m < Nb
     double* part;
     int Na, Nb;
     int* status;
 };
 
-template <int NPL>
 __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs a) {
-    using G = SGram<NPL>;
-    constexpr int NSTG = G::NSTG, TILE = G::TILE, KPC = G::CH / G::KC;  // tiles per chunk
+    using G = SGram;
+    constexpr int NPL = G::NPL, NSTG = G::NSTG, TILE = G::TILE, KPC = G::CH / G::KC;  // tiles per chunk
     const size_t plane_bytes = a.plane_bytes;
     const int nkc_max = a.nkc_max, kseg = a.kseg, ntiles = a.ntiles;
     const int2* __restrict__ tiles = a.tiles;
@@ -672,10 +616,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs 
         // own error).
         const int lb = warp & 3, c2 = (warp - 1) >> 2, odd = lane & 1;
         const int row = 32 * lb + lane;
-        const cpx<double>* redO = (const cpx<double>*)a.redO;
-        cpx<double>* S = (cpx<double>*)a.S;
-        const int P = a.P;
-        const double inv = 1.0 / a.B;
         bool ok = true;
         for (int ti = 0; ti < nmine && ok; ++ti) {
             const int item = blockIdx.x + ti * gridDim.x;
@@ -719,38 +659,18 @@ __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs 
                              : "memory");
             }
             if (!ok) break;
-            if (a.part) {
-                // raw sums of this item: n = row pair, m = column
-                const int n = 64 * rt + (row >> 1), Na = a.Na, Nb = a.Nb;
-                cpx<double>* out = (cpx<double>*)a.part +
-                                   (size_t)((tl.y >> 16) * a.nseg + item / ntiles) * Na * Nb;
-                if (n < Na) {
-#pragma unroll
-                    for (int ch = 0; ch < 8; ++ch)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int m = 128 * ct + 64 * c2 + 8 * ch + 4 * odd + q;
-                            if (m < Nb)
-                                out[(size_t)n * Nb + m] = {(double)acc[ch][q][0], (double)acc[ch][q][1]};
-                        }
-                }
-                continue;
-            }
-            // tile done: S = acc / B - conj(Obar_k) Obar_l (+ shift)
-            const int k = 64 * rt + (row >> 1);
-            if (k < P) {
-                const cpx<double> obk = conj(inv * redO[k]);
+            // the item's sums: n = row pair, m = column
+            const int n = 64 * rt + (row >> 1), Na = a.Na, Nb = a.Nb;
+            cpx<double>* out = (cpx<double>*)a.part +
+                               (size_t)((tl.y >> 16) * a.nseg + item / ntiles) * Na * Nb;
+            if (n < Na) {
 #pragma unroll
                 for (int ch = 0; ch < 8; ++ch)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const int l = 128 * ct + 64 * c2 + 8 * ch + 4 * odd + q;
-                        if (l < P) {
-                            const cpx<double> g = {(double)acc[ch][q][0], (double)acc[ch][q][1]};
-                            cpx<double> val = inv * g - obk * (inv * redO[l]);
-                            if (k == l) val.x += a.shift;
-                            S[(size_t)k * P + l] = val;
-                        }
+                        const int m = 128 * ct + 64 * c2 + 8 * ch + 4 * odd + q;
+                        if (m < Nb)
+                            out[(size_t)n * Nb + m] = {(double)acc[ch][q][0], (double)acc[ch][q][1]};
                     }
             }
         }
@@ -784,17 +704,16 @@ __global__ void smirror_kernel(double* __restrict__ S_, int P) {
 // G = B^dag B / B_s and H = B^dag HB / B_s of cheb_gram on the tensor cores:
 // the complex columns B_n (and HB_n) become rows 2n (real part) and 2n + 1
 // (imaginary part) of a real matrix X (Y), split into three bf16 planes as
-// for the explicit S, and sgram_tc_kernel forms X^T X and X^T Y over K
+// above, and sgram_tc_kernel forms X^T X and X^T Y over K
 // segments of the samples.  gram_reduce_kernel adds the segments in float64
 // in a fixed order, scales by 1/B_s, and writes G (Hermitian by construction:
 // upper triangle mirrored, real diagonal) and (H + H^dag)/2.
 
 // Planes of X from the columns Bm[n * ld + s] (complex64): row 2n + im,
 // walkers s; rows past 2 Nm and walkers past B are zero.
-template <int NPL>
 __global__ void gram_prep_kernel(const cpx<float>* __restrict__ Bm, int Nm, int B, int ld, int nrb,
                                  int nkc, size_t plane_bytes, unsigned char* __restrict__ X) {
-    using G = SGram<NPL>;
+    using G = SGram;
     constexpr int NG = G::KC / 8;
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (size_t)nrb * nkc * NG * 128) return;
@@ -811,17 +730,12 @@ __global__ void gram_prep_kernel(const cpx<float>* __restrict__ Bm, int Nm, int 
             const cpx<float> v = Bm[(size_t)n * ld + s];
             x = im ? v.y : v.x;
         }
-        if (NPL == 3) {
-            split3(x, &t0[q], &t1[q], &t2[q]);
-        } else {
-            t0[q] = __float2bfloat16_rn(x);
-            t1[q] = __float2bfloat16_rn(x - __bfloat162float(t0[q]));
-        }
+        split3(x, &t0[q], &t1[q], &t2[q]);
     }
     const size_t off = ((size_t)rb * nkc + kc) * G::TILE + tc::kmajor_offset(r, grp * 8, G::KC);
     *reinterpret_cast<uint4*>(X + off) = pack8(t0);
     *reinterpret_cast<uint4*>(X + plane_bytes + off) = pack8(t1);
-    if (NPL == 3) *reinterpret_cast<uint4*>(X + 2 * plane_bytes + off) = pack8(t2);
+    *reinterpret_cast<uint4*>(X + 2 * plane_bytes + off) = pack8(t2);
 }
 
 __global__ void gram_reduce_kernel(const double* __restrict__ part_, int nseg, int Nm, int B,
@@ -922,73 +836,6 @@ cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const
     return cr_check_launch(c, "oreduce_tc_kernel");
 }
 
-static int sgram_npl(const cr_ctx* c) { return (c->flags & CR_CTX_S_BF16X3) ? 2 : 3; }
-
-template <int NPL> size_t sgram_smem_t() { return SGram<NPL>::SMEM; }
-
-// Operand planes of the explicit-S Gram kernel: rows of G padded to a
-// multiple of 512, walkers to a multiple of the tile's walker count.
-void sgram_geometry(const cr_ctx* c, int* R2, int* nkc_max, size_t* plane_bytes, int* npl) {
-    *npl = sgram_npl(c);
-    const int kc = *npl == 2 ? SGram<2>::KC : SGram<3>::KC;
-    *R2 = ((2 * c->P + 511) / 512) * 512;
-    *nkc_max = (c->max_walkers + kc - 1) / kc;
-    *plane_bytes = (size_t)(*R2 / 128) * (size_t)(*nkc_max) * (size_t)(128 * kc * 2);
-}
-
-// Lower-triangle blocks of G (128-row block rt, 256-column block ct with
-// 256 ct <= 128 rt + 127), column-block major so that concurrently running
-// CTAs share the column operand in L2.
-std::vector<int2> sgram_tiles(int P) {
-    const int R2 = ((2 * P + 511) / 512) * 512;
-    std::vector<int2> v;
-    for (int ct = 0; ct < R2 / 256; ++ct)
-        for (int rt = 0; rt * 128 < 2 * P; ++rt)
-            if (256 * ct <= 128 * rt + 127) v.push_back(make_int2(rt, ct));
-    return v;
-}
-
-void launch_smirror(cr_ctx* c);
-
-template <int NPL>
-static cr_status sbuild_tc_t(cr_ctx* c, const int8_t* spins, const void* T, int B,
-                             const double* redO, double shift) {
-    int R2, nkc_max, npl;
-    size_t pb;
-    sgram_geometry(c, &R2, &nkc_max, &pb, &npl);
-    constexpr int KC = SGram<NPL>::KC;
-    const int nkc = (B + KC - 1) / KC;
-    const size_t n = (size_t)R2 * nkc * (KC / 8);
-    CR_LAUNCH(c, CR_K_OTHER,
-              xt_prep_kernel<NPL><<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(
-                  spins, (const cpx<float>*)T, B, c->N, c->M, c->P, R2, nkc_max, nkc, pb, c->Xt));
-    const int grid = c->n_gtiles < c->n_sm ? c->n_gtiles : c->n_sm;
-    GramArgs a{};
-    a.xa = a.xb0 = a.xb1 = c->Xt;
-    a.plane_bytes = pb;
-    a.nkc_max = nkc_max;
-    a.kseg = nkc;
-    a.nseg = 1;
-    a.tiles = c->gtiles;
-    a.ntiles = c->n_gtiles;
-    a.P = c->P;
-    a.B = B;
-    a.redO = redO;
-    a.shift = shift;
-    a.S = c->S;
-    a.status = c->d_status;
-    CR_LAUNCH(c, CR_KERNEL_SBUILD,
-              sgram_tc_kernel<NPL><<<grid, GR_THREADS, sgram_smem_t<NPL>(), c->stream>>>(a));
-    launch_smirror(c);
-    return cr_check_launch(c, "explicit S (tensor cores)");
-}
-
-cr_status launch_sbuild_tc(cr_ctx* c, const int8_t* spins, const void* T, int B,
-                           const double* redO, double shift) {
-    return sgram_npl(c) == 2 ? sbuild_tc_t<2>(c, spins, T, B, redO, shift)
-                             : sbuild_tc_t<3>(c, spins, T, B, redO, shift);
-}
-
 void launch_smirror(cr_ctx* c) {
     const int nt = (c->P + 31) / 32;
     CR_LAUNCH(c, CR_K_OTHER, smirror_kernel<<<dim3(nt, nt), dim3(32, 8), 0, c->stream>>>(c->S, c->P));
@@ -1005,7 +852,7 @@ struct GramGeo {
 };
 
 static GramGeo gram_geometry(const cr_ctx* c, int Nm, int B, bool withH) {
-    using G = SGram<3>;
+    using G = SGram;
     constexpr int KPC = G::CH / G::KC;
     GramGeo g;
     const int R2 = ((2 * Nm + 255) / 256) * 256;
@@ -1049,15 +896,15 @@ cr_status launch_gram_tc(cr_ctx* c, const void* Bm, const void* HBm, int Nm, int
             return cr_fail(c, CR_ECUDA, "cheb_gram: tile list copy");
         c->gram_key = key;
     }
-    constexpr int NG = SGram<3>::KC / 8;
+    constexpr int NG = SGram::KC / 8;
     const size_t n = (size_t)g.nrb * g.nkc * NG * 128;
     const unsigned nb = (unsigned)((n + 255) / 256);
     unsigned char* X = c->gram_x;
     unsigned char* Y = HBm ? X + 3 * g.plane_bytes : X;
-    CR_LAUNCH(c, CR_K_OTHER, gram_prep_kernel<3><<<nb, 256, 0, c->stream>>>(
+    CR_LAUNCH(c, CR_K_OTHER, gram_prep_kernel<<<nb, 256, 0, c->stream>>>(
                                  (const cpx<float>*)Bm, Nm, B, ld, g.nrb, g.nkc, g.plane_bytes, X));
     if (HBm)
-        CR_LAUNCH(c, CR_K_OTHER, gram_prep_kernel<3><<<nb, 256, 0, c->stream>>>(
+        CR_LAUNCH(c, CR_K_OTHER, gram_prep_kernel<<<nb, 256, 0, c->stream>>>(
                                      (const cpx<float>*)HBm, Nm, B, ld, g.nrb, g.nkc, g.plane_bytes, Y));
     GramArgs a{};
     a.xa = a.xb0 = X;
@@ -1068,14 +915,13 @@ cr_status launch_gram_tc(cr_ctx* c, const void* Bm, const void* HBm, int Nm, int
     a.nseg = g.nseg;
     a.tiles = c->gram_tiles;
     a.ntiles = (int)g.tiles.size();
-    a.B = B;
     a.part = c->gram_part;
     a.Na = a.Nb = Nm;
     a.status = c->d_status;
     const int items = a.ntiles * a.nseg;
     const int grid = items < c->n_sm ? items : c->n_sm;
     CR_LAUNCH(c, CR_KERNEL_GRAM,
-              sgram_tc_kernel<3><<<grid, GR_THREADS, sgram_smem_t<3>(), c->stream>>>(a));
+              sgram_tc_kernel<<<grid, GR_THREADS, SGram::SMEM, c->stream>>>(a));
     CR_LAUNCH(c, CR_K_OTHER, gram_reduce_kernel<<<(Nm * Nm + 255) / 256, 256, 0, c->stream>>>(
                                  c->gram_part, g.nseg, Nm, B, G, H));
     return cr_check_launch(c, "cheb_gram (tensor cores)");
@@ -1099,7 +945,7 @@ struct OredGeo {
 };
 
 static OredGeo ored_geometry(const cr_ctx* c) {
-    using G = SGram<3>;
+    using G = SGram;
     constexpr int KPC = G::CH / G::KC;
     OredGeo g;
     g.Na = c->N + 1;
@@ -1137,7 +983,7 @@ __global__ void ored_prep_kernel(const int8_t* __restrict__ spins, const cpx<flo
                                  const cpx<float>* __restrict__ g, int B, int N, int M, int nrb,
                                  int nkc, int nkc_cap, size_t plane_bytes,
                                  unsigned char* __restrict__ X) {
-    using G = SGram<3>;
+    using G = SGram;
     constexpr int NG = G::KC / 8;
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (size_t)nrb * nkc * NG * 128) return;
@@ -1214,7 +1060,7 @@ __global__ void ored_reduce_kernel(const double* __restrict__ part_, int nseg, i
 
 cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const void* g, int B,
                             double* redR, double* redO) {
-    using G = SGram<3>;
+    using G = SGram;
     constexpr int KPC = G::CH / G::KC, NG = G::KC / 8;
     OredGeo geo = ored_geometry(c);
     const int nch = (B + G::CH - 1) / G::CH;
@@ -1235,7 +1081,6 @@ cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const
     a.nseg = nseg;
     a.tiles = c->ored_tiles;
     a.ntiles = (int)geo.tiles.size();
-    a.B = B;
     a.part = c->ored_part;
     a.Na = geo.Na;
     a.Nb = geo.Nb;
@@ -1243,7 +1088,7 @@ cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const
     const int items = a.ntiles * nseg;
     const int grid = items < c->n_sm ? items : c->n_sm;
     CR_LAUNCH(c, CR_KERNEL_REDUCE,
-              sgram_tc_kernel<3><<<grid, GR_THREADS, sgram_smem_t<3>(), c->stream>>>(a));
+              sgram_tc_kernel<<<grid, GR_THREADS, SGram::SMEM, c->stream>>>(a));
     const int len = c->P + 2 + c->M;
     CR_LAUNCH(c, CR_K_OTHER, ored_reduce_kernel<<<(len + 255) / 256, 256, 0, c->stream>>>(
                                  c->ored_part, nseg, c->N, c->M, c->P, geo.Na, geo.Nb, redR, redO));
@@ -1254,14 +1099,9 @@ cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const
 // per context (not from a hot call, so that hot calls stay capturable).
 cr_status tc_prepare(cr_ctx* c) {
     if (c->prec == CR_MIXED) {
-        // explicit S (either split) and the Krylov Gram (three planes)
-        cudaError_t e = cudaFuncSetAttribute(sgram_tc_kernel<2>,
+        cudaError_t e = cudaFuncSetAttribute(sgram_tc_kernel,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)sgram_smem_t<2>());
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(sgram_tc_kernel<3>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)sgram_smem_t<3>());
+                                             (int)SGram::SMEM);
         if (e != cudaSuccess) return cr_fail(c, CR_ECUDA, "tc_prepare: %s", cudaGetErrorString(e));
     }
     if (!tc_supported(c)) return CR_OK;
