@@ -1,278 +1,583 @@
 // Direct shifted solve (S + lambda I) x = F of the natural-gradient update
-// (Sec. III) for large P: blocked right-looking Cholesky S = L L^dag on many
-// CTAs, then iterative refinement in float64.
+// (Sec. III): blocked right-looking Cholesky S = L L^dag on many CTAs, then
+// iterative refinement in float64.
 //
 // S (float64, full Hermitian, shift on its diagonal) stays untouched; its
-// lower triangle is copied into the factor buffer L in the factor precision
-// (float64 for float64 contexts, float32 otherwise) and factored in place in
-// 64 x 64 blocks.  Per block column J:
-//   potrf_kernel   L_JJ = chol(A_JJ)                   (one CTA, in shared memory)
-//   trsm_kernel    L_IJ = A_IJ L_JJ^{-dag}, I > J      (one warp per row)
-//   syrk_kernel    A_IK -= L_IJ L_KJ^dag, J < K <= I   (one CTA per 64 x 64 block)
+// lower triangle is copied into the factor buffer and factored in place.
+// Float64 contexts factor in float64 (chol64.cu).  The others factor in
+// float32, in 64-column panels.  Per panel J:
+//   potrf_inv_kernel  L_JJ = chol(A_JJ) and X_JJ = L_JJ^-1   (one CTA, registers)
+//   trsm_kernel       L_IJ = A_IJ X_JJ^dag, I > J             (64 x 64 tiles)
+//   syrk_tc_kernel    A_IK -= L_IJ L_KJ^dag, J < K <= I       (mixed: tcgen05)
+//   syrk_kernel       the same on the FMA pipes               (float32)
+// The inverses X_JJ turn the panel's triangular solve into a product, and,
+// merged pairwise into the inverses of 512 x 512 diagonal blocks, the
+// triangular solves of the refinement into two products per 512 rows.
+//
 // The solve with a float32 factor (and float32 arithmetic in the triangular
 // solves) is accurate to about kappa * 2^-24, so it is refined in float64
 // (Wilkinson's iterative refinement; the residual is formed in float64):
 //   x = 0, r = F;  repeat { d = L^{-dag} L^{-1} r;  x += d;  r = F - S x }
 // until |r| <= REFINE_TOL |F|, the residual stops shrinking (by 2x), or
-// REFINE_MAXIT steps.  A float64 factor needs one step.  The triangular
-// solves run one 64-row block column per launch; every later launch of a
-// refinement step returns at once when the done flag is set, so the launch
-// sequence is fixed (graph-capturable).
+// REFINE_MAXIT steps.  Float64 contexts up to CHOL_SMALL_P parameters take
+// the float64 solve without refinement.  Every later launch of a refinement
+// step returns at once when the done flag is set, so the launch sequence is
+// fixed (graph-capturable).
+#include <cuda_bf16.h>
+
 #include "common.cuh"
+#include "tc.cuh"
 
 namespace {
 
+using cf = cpx<float>;
+
 constexpr int NB = 64;
-constexpr int NTRI = NB * (NB + 1) / 2;
+constexpr int SB = 512;                     // rows of a merged diagonal inverse
 constexpr int REFINE_MAXIT = 10;
 constexpr double REFINE_TOL = 1e-12;
-constexpr int RES_GRID = 304;  // CTAs of the residual kernel (fixed: deterministic sums)
+constexpr int RES_ROWS = 2;    // rows of S a warp of the residual kernel reads at once
 
-CR_HD int tri(int i, int j) { return i * (i + 1) / 2 + j; }
+// L is held as [lrows(P)][lcols(P)], rows and columns past P zero, so that
+// the tensor-core update needs no masks and every row starts on 128 bytes.
+CR_HD int lcols(int P) { return (P + NB - 1) / NB * NB; }
+CR_HD int lrows(int P) { return lcols(P) + 256; }  // a 256-row tile may start at any 64
 
-template <typename R> CR_D cpx<R> shfl(cpx<R> v, int src) {
-    return {__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src)};
+// L <- S in float32 (only the lower triangle is used).
+__global__ void chol_copy_kernel(const double* __restrict__ S_, int P, cf* __restrict__ L) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y, ld = lcols(P);
+    if (k >= ld) return;
+    L[(size_t)i * ld + k] = i < P && k < P ? ccast<float>(((const cpx<double>*)S_)[(size_t)i * P + k])
+                                           : cf{0.f, 0.f};
 }
 
-// L <- S in the factor precision (whole matrix; only the lower triangle is used).
-template <typename R>
-__global__ void chol_copy_kernel(const double* __restrict__ S_, int P, cpx<R>* __restrict__ L) {
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < (size_t)P * P) L[idx] = ccast<R>(((const cpx<double>*)S_)[idx]);
+// Merged inverses: X holds one [SB][SB] block per SB rows of L.
+CR_D cf* xblock(cf* X, int row) {
+    return X + (size_t)(row / SB) * SB * SB + (size_t)(row % SB) * SB + row % SB;
 }
 
-// Factor the diagonal block J in shared memory (packed lower triangle, in
-// the factor precision: float64 is a narrow pipe on this GPU and the
-// float64 refinement corrects the float32 factor anyway); zero its strict
-// upper part.  A non-positive pivot sets CR_ESINGULAR and is replaced by 1
-// so the factorisation runs to the end.
-template <typename R>
-__global__ void __launch_bounds__(256) potrf_kernel(cpx<R>* __restrict__ L, int P, int J,
-                                                    int* __restrict__ status) {
-    __shared__ cpx<R> a[NTRI];
-    __shared__ R piv;
-    __shared__ int bad;
-    const int base = J * NB, n = min(NB, P - base), t = threadIdx.x;
-    if (t == 0) bad = 0;
-    for (int e = t; e < n * n; e += blockDim.x) {
-        const int i = e / n, j = e % n;
-        if (j <= i) a[tri(i, j)] = L[(size_t)(base + i) * P + base + j];
-    }
-    for (int j = 0; j < n; ++j) {
-        __syncthreads();
-        if (t == 0) {
-            R d = a[tri(j, j)].x;
-            if (!(d > R(0))) {
-                bad = 1;
-                d = R(1);
+// Factor the diagonal block J and invert the factor, 16 x 16 threads with 4
+// x 4 entries each (rows ty + 16 a, columns tx + 16 b) in registers.  At
+// column j the entries of columns k > j belong to the block still to be
+// factored and those of columns k <= j to the inverse that grows in their
+// place (column j of L itself is stored when it is formed), so one 64 x 64
+// array and one rank-1 update per column serve both.  Row and column j go
+// through shared memory, double-buffered: one barrier per column.  A
+// non-positive pivot sets CR_ESINGULAR and is replaced by 1 so the
+// factorisation runs to the end.  Bound by the 64 dependent column steps
+// (barrier, square root, divide, update).
+__global__ void __launch_bounds__(256) potrf_inv_kernel(cf* __restrict__ L, int P, int J,
+                                                        cf* __restrict__ X, int* __restrict__ status) {
+    __shared__ cf col[2][NB], xrow[2][NB];
+    const int base = J * NB, n = min(NB, P - base), ld = lcols(P);
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    cf a[4][4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = ty + 16 * p, k = tx + 16 * q;
+            a[p][q] = (i < n && k <= i) ? L[(size_t)(base + i) * ld + base + k]
+                                        : cf{i == k ? 1.f : 0.f, 0.f};
+        }
+    bool bad = false;
+#pragma unroll
+    for (int jb = 0; jb < 4; ++jb)
+        for (int jj = 0; jj < 16; ++jj) {
+            const int j = 16 * jb + jj, buf = j & 1;
+            if (tx == jj)
+#pragma unroll
+                for (int p = 0; p < 4; ++p) col[buf][ty + 16 * p] = a[p][jb];
+            if (ty == jj)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) xrow[buf][tx + 16 * q] = a[jb][q];
+            __syncthreads();
+            float d = col[buf][j].x;
+            if (!(d > 0.f)) {
+                bad = true;
+                d = 1.f;
             }
-            piv = m_sqrt(d);
-            a[tri(j, j)] = {piv, R(0)};
+            const float piv = m_sqrt(d), ip = 1.f / piv;
+            // row factors: conj(l_k) of the block to the right of column j, the
+            // inverse's row j (scaled) to the left of it
+            cf rk[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = tx + 16 * q;
+                rk[q] = k > j ? conj(ip * col[buf][k]) : ip * xrow[buf][k];
+                if (k == j) rk[q] = {ip, 0.f};
+            }
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                const int i = ty + 16 * p;
+                if (i > j) {
+                    const cf li = ip * col[buf][i];
+                    if (tx == jj) {
+                        if (i < n) L[(size_t)(base + i) * ld + base + j] = li;
+                        a[p][jb] = {0.f, 0.f};  // the unit matrix's entry, updated below
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) a[p][q] = a[p][q] - li * rk[q];
+                } else if (i == j) {
+                    if (tx == jj && j < n) L[(size_t)(base + j) * ld + base + j] = {piv, 0.f};
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (tx + 16 * q <= j) a[p][q] = rk[q];
+                }
+            }
         }
-        __syncthreads();
-        const R ip = R(1) / piv;
-        for (int i = j + 1 + t; i < n; i += blockDim.x) a[tri(i, j)] = ip * a[tri(i, j)];
-        __syncthreads();
-        const int m = n - j - 1;
-        for (int e = t; e < m * m; e += blockDim.x) {
-            const int i = j + 1 + e / m, l = j + 1 + e % m;
-            if (l <= i) a[tri(i, l)] = a[tri(i, l)] - a[tri(i, j)] * conj(a[tri(l, j)]);
+    cf* Xb = xblock(X, base);
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = ty + 16 * p, k = tx + 16 * q;
+            Xb[(size_t)i * SB + k] = k <= i ? a[p][q] : cf{0.f, 0.f};
         }
-    }
-    __syncthreads();
-    for (int e = t; e < n * n; e += blockDim.x) {
-        const int i = e / n, j = e % n;
-        L[(size_t)(base + i) * P + base + j] = j <= i ? a[tri(i, j)] : cpx<R>{R(0), R(0)};
-    }
     if (t == 0 && bad) set_status(status, CR_ESINGULAR);
 }
 
-// Rows below block J (block J is full here: it is not the last block):
-// x L_JJ^dag = a solved column by column, lanes holding columns lane and
-// lane + 32 of one row.
-template <typename R>
-__global__ void __launch_bounds__(256) trsm_kernel(cpx<R>* __restrict__ L, int P, int J) {
-    __shared__ cpx<R> d[NTRI];
-    const int base = J * NB, t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    for (int e = t; e < NB * NB; e += blockDim.x) {
-        const int i = e / NB, j = e % NB;
-        if (j <= i) d[tri(i, j)] = L[(size_t)(base + i) * P + base + j];
-    }
-    __syncthreads();
-    for (int row = base + NB + blockIdx.x * 8 + warp; row < P; row += gridDim.x * 8) {
-        cpx<R>* Lr = L + (size_t)row * P + base;
-        cpx<R> v0 = Lr[lane], v1 = Lr[lane + 32];
-        for (int c = 0; c < NB; ++c) {
-            cpx<R> xc = shfl(c < 32 ? v0 : v1, c & 31);
-            xc = (R(1) / d[tri(c, c)].x) * xc;
-            if (lane == (c & 31)) {
-                if (c < 32) v0 = xc;
-                else v1 = xc;
-            }
-            if (lane > c) v0 = v0 - xc * conj(d[tri(lane, c)]);
-            if (lane + 32 > c) v1 = v1 - xc * conj(d[tri(lane + 32, c)]);
+// One 32-deep step of a 64 x 64 tile product, 16 x 16 threads, 4 x 4 outputs
+// each (rows ty + 16 q, columns 4 tx + q).
+constexpr int KT = 32;
+constexpr int BP = NB + 2;  // rows of Bs start on 16 bytes
+CR_D void tile_step(const cf (*As)[NB + 1], const cf (*Bs)[BP], int tx, int ty, cf (&acc)[4][4]) {
+#pragma unroll
+    for (int c = 0; c < KT; ++c) {
+        cf av[4], bv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) av[q] = As[c][ty + 16 * q];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const float4 v = *reinterpret_cast<const float4*>(&Bs[c][4 * tx + 2 * q]);
+            bv[2 * q] = {v.x, v.y};
+            bv[2 * q + 1] = {v.z, v.w};
         }
-        Lr[lane] = v0;
-        Lr[lane + 32] = v1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int q2 = 0; q2 < 4; ++q2) acc[q][q2] = acc[q][q2] + av[q] * bv[q2];
     }
 }
 
+// ------------------------------------------- trailing update, tensor cores
+//
+// A_IK -= L_IJ L_KJ^dag with the panel's float32 values split into three
+// bf16 terms (six products, all 24 bits, float32 accumulation).  With K real
+// index 2 c + part,
+//   rows   N side, row i:                [Re L_ic, Im L_ic]
+//   cols   M side, row 2k: [Re, Im] of L_kc; row 2k + 1: [-Im, Re]
+// so that D[2k + part][i] = (Re, Im)(L_i . conj(L_k)): lanes (D rows) hold
+// consecutive floats of a row of A, and a tile's 256 rows x 64 columns are
+// read and written coalesced.  A panel is 128 real deep: 48 MMAs into one
+// float32 accumulator, then one float32 subtraction, as long a run as the
+// explicit S takes.
+constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded mbarrier polls
+constexpr int TC_ROWS = 256, TC_COLS = 64;  // tile of A
+constexpr int TC_KC = 32, TC_NKC = 2 * NB / TC_KC;
+constexpr int N_TILE = TC_ROWS * TC_KC * 2, M_TILE = 2 * TC_COLS * TC_KC * 2;  // bytes, one plane
+constexpr int TC_STAGE = 3 * (N_TILE + M_TILE);
+constexpr int TC_NSTG = 3;
+constexpr size_t TC_SMEM = (size_t)TC_NSTG * TC_STAGE + 256;
+constexpr int TC_THREADS = 288;
+
+CR_D void split3(float x, __nv_bfloat16* hi, __nv_bfloat16* mid, __nv_bfloat16* lo) {
+    *hi = __float2bfloat16_rn(x);
+    const float r1 = x - __bfloat162float(*hi);
+    *mid = __float2bfloat16_rn(r1);
+    *lo = __float2bfloat16_rn(r1 - __bfloat162float(*mid));
+}
+
+CR_D uint4 pack8(const __nv_bfloat16* v) {
+    uint4 r;
+    uint32_t* w = reinterpret_cast<uint32_t*>(&r);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        w[q] = (uint32_t)__bfloat16_as_ushort(v[2 * q]) |
+               ((uint32_t)__bfloat16_as_ushort(v[2 * q + 1]) << 16);
+    return r;
+}
+
+// the three terms of 8 consecutive K values of one operand row
+CR_D void put_row(unsigned char* tile, int plane, int row, int kk, const float* x) {
+    __nv_bfloat16 h[8], m[8], l[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) split3(x[q], &h[q], &m[q], &l[q]);
+    const uint32_t o = tc::kmajor_offset(row, kk, TC_KC);
+    *reinterpret_cast<uint4*>(tile + o) = pack8(h);
+    *reinterpret_cast<uint4*>(tile + plane + o) = pack8(m);
+    *reinterpret_cast<uint4*>(tile + 2 * plane + o) = pack8(l);
+}
+
+// L_IJ = A_IJ X_JJ^dag for one 64-row block below block J (full here: it is
+// not the last block).  planes: also the bf16 operands of the trailing
+// update (rows past P are zero there); a thread's outputs are 4 adjacent
+// columns, so it forms 16-byte operand groups from its own registers.
+__global__ void __launch_bounds__(256) trsm_kernel(cf* __restrict__ L, int P, int J, cf* __restrict__ X,
+                                                   unsigned char* __restrict__ planes, size_t m_off) {
+    __shared__ __align__(16) cf As[KT][NB + 1];
+    __shared__ __align__(16) cf Bs[KT][BP];
+    const int base = J * NB, r0 = base + NB, i0 = r0 + blockIdx.x * NB, ld = lcols(P);
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    const cf* Xb = xblock(X, base);
+    cf acc[4][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) acc[q][q2] = {0.f, 0.f};
+    for (int cc = 0; cc < NB; cc += KT) {
+#pragma unroll
+        for (int e = t; e < NB * KT; e += 256) {
+            const int r = e / KT, c = e % KT;
+            As[c][r] = i0 + r < P ? L[(size_t)(i0 + r) * ld + base + cc + c] : cf{0.f, 0.f};
+            Bs[c][r] = conj(Xb[(size_t)r * SB + cc + c]);
+        }
+        __syncthreads();
+        tile_step(As, Bs, tx, ty, acc);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int r = ty + 16 * q;
+        float re[8], im[8];
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) {
+            re[2 * q2] = acc[q][q2].x;
+            re[2 * q2 + 1] = acc[q][q2].y;
+            im[2 * q2] = -acc[q][q2].y;
+            im[2 * q2 + 1] = acc[q][q2].x;
+        }
+        if (i0 + r < P) {
+            float4* out = reinterpret_cast<float4*>(L + (size_t)(i0 + r) * ld + base + 4 * tx);
+            out[0] = make_float4(re[0], re[1], re[2], re[3]);
+            out[1] = make_float4(re[4], re[5], re[6], re[7]);
+        }
+        if (!planes) continue;
+        const int row = i0 - r0 + r, k = 8 * tx, kc = k / TC_KC, kk = k % TC_KC;
+        put_row(planes + ((size_t)(row / TC_ROWS) * TC_NKC + kc) * 3 * N_TILE, N_TILE, row % TC_ROWS, kk, re);
+        unsigned char* mt = planes + m_off + ((size_t)(row / TC_COLS) * TC_NKC + kc) * 3 * M_TILE;
+        put_row(mt, M_TILE, 2 * (row % TC_COLS), kk, re);
+        put_row(mt, M_TILE, 2 * (row % TC_COLS) + 1, kk, im);
+    }
+}
+
+// Tiles of the trailing matrix (from row r0): row block rb takes the column
+// blocks cb <= 4 rb + 3 that exist; tile index 2 rb (rb + 1) + cb.
+// Persistent, 288 threads: warp 0 (one thread) copies operand stages and
+// issues the MMAs, tile t into TMEM columns [256 (t % 2), +256); warps 1-8
+// fetch their part of the tile of A while the MMAs run, subtract and store.
+__global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restrict__ Lf, int P, int r0,
+                                                                int ntiles,
+                                                                const unsigned char* __restrict__ planes,
+                                                                size_t m_off, int* __restrict__ status) {
+    extern __shared__ __align__(1024) unsigned char sm[];
+    uint64_t* full = (uint64_t*)(sm + TC_NSTG * TC_STAGE);
+    uint64_t* empty = full + TC_NSTG;
+    uint64_t* dfull = empty + TC_NSTG;  // [2] MMAs of a tile done
+    uint64_t* dempty = dfull + 2;       // [2] TMEM half read by the 256 drain threads
+    uint32_t* slot = (uint32_t*)(dempty + 2);
+    volatile int* abort = (volatile int*)(slot + 1);
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    if (t == 0) {
+        for (int i = 0; i < 2 * TC_NSTG + 2; ++i) tc::mbar_init(&full[i], 1);
+        tc::mbar_init(&dempty[0], 256);
+        tc::mbar_init(&dempty[1], 256);
+        tc::fence_mbar_init();
+        *abort = 0;
+    }
+    if (warp == 0) {
+        tc::tmem_alloc(slot, 512u);
+        tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t taddr = *slot;
+    auto wait = [&](uint64_t* bar, uint32_t par) {
+        for (int i = 0; i < 64; ++i) {
+            if (tc::mbar_wait(bar, par, WAIT_LIMIT >> 6)) return true;
+            if (*abort) return false;
+        }
+        *abort = 1;
+        return false;
+    };
+    auto tile_of = [&](int idx, int* rb, int* cb) {
+        int r = (int)((sqrtf(1.0f + 2.0f * (float)idx) - 1.0f) * 0.5f);
+        while (2 * r * (r + 1) > idx) --r;
+        while (2 * (r + 1) * (r + 2) <= idx) ++r;
+        *rb = r;
+        *cb = idx - 2 * r * (r + 1);
+    };
+    const int nmine = ntiles > (int)blockIdx.x ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    if (warp == 0) {
+        if (lane == 0) {
+            constexpr int PA[6] = {0, 0, 1, 0, 1, 2}, PB[6] = {0, 1, 0, 2, 1, 0};
+            const uint32_t idesc = tc::make_idesc_bf16(2 * TC_COLS, TC_ROWS);
+            const int total = nmine * TC_NKC;
+            uint32_t pend = 0, pend_par = 0;
+            int last_g = -1;
+            bool ok = true;
+            auto load = [&](int g) {
+                const uint32_t b = g % TC_NSTG;
+                if (g >= TC_NSTG && !wait(&empty[b], ((g - TC_NSTG) / TC_NSTG) & 1)) return false;
+                int rb, cb;
+                tile_of(blockIdx.x + (g / TC_NKC) * gridDim.x, &rb, &cb);
+                const int kc = g % TC_NKC;
+                pend |= 1u << b;
+                pend_par = (pend_par & ~(1u << b)) | (((uint32_t)(g / TC_NSTG) & 1u) << b);
+                unsigned char* st = sm + (size_t)b * TC_STAGE;
+                tc::mbar_expect_tx(&full[b], (uint32_t)TC_STAGE);
+                tc::bulk_g2s(st, planes + ((size_t)rb * TC_NKC + kc) * 3 * N_TILE, 3 * N_TILE, &full[b]);
+                tc::bulk_g2s(st + 3 * N_TILE, planes + m_off + ((size_t)cb * TC_NKC + kc) * 3 * M_TILE,
+                             3 * M_TILE, &full[b]);
+                return true;
+            };
+            for (int g = 0; g < TC_NSTG - 1 && g < total && ok; ++g) ok = load(g);
+            for (int g = 0; g < total && ok; ++g) {
+                const int ti = g / TC_NKC, kc = g % TC_NKC, b = g % TC_NSTG;
+                const uint32_t h = ti & 1;
+                if (kc == 0 && ti >= 2 && !wait(&dempty[h], ((ti - 2) >> 1) & 1)) {
+                    ok = false;
+                    break;
+                }
+                if (!wait(&full[b], (g / TC_NSTG) & 1)) {
+                    ok = false;
+                    break;
+                }
+                pend &= ~(1u << b);
+                tc::fence_after_sync();
+                const uint32_t ns = tc::smem_u32(sm + (size_t)b * TC_STAGE), ms = ns + 3 * N_TILE;
+#pragma unroll
+                for (int ks = 0; ks < TC_KC / 16; ++ks)
+#pragma unroll
+                    for (int pr = 0; pr < 6; ++pr)
+                        tc::mma_bf16(taddr + h * 256,
+                                     tc::make_desc(ms + PA[pr] * M_TILE + ks * 256, 128, 16 * TC_KC),
+                                     tc::make_desc(ns + PB[pr] * N_TILE + ks * 256, 128, 16 * TC_KC),
+                                     idesc, !(kc == 0 && ks == 0 && pr == 0));
+                tc::commit(&empty[b]);
+                last_g = g;
+                if (kc == TC_NKC - 1) tc::commit(&dfull[h]);
+                if (g + TC_NSTG - 1 < total && !load(g + TC_NSTG - 1)) ok = false;
+            }
+            if (!ok) {
+                *abort = 1;
+                set_status(status, CR_ETIMEOUT);
+                // let copies in flight land and issued MMAs finish (bounded)
+                for (int b = 0; b < TC_NSTG; ++b)
+                    if (pend & (1u << b)) tc::mbar_wait(&full[b], (pend_par >> b) & 1u, WAIT_LIMIT);
+                if (last_g >= 0)
+                    tc::mbar_wait(&empty[last_g % TC_NSTG], (uint32_t)(last_g / TC_NSTG) & 1u, WAIT_LIMIT);
+            }
+        }
+        __syncwarp();
+    } else {
+        const int lb = warp & 3, c2 = (warp - 1) >> 2;
+        bool ok = true;
+        for (int ti = 0; ti < nmine && ok; ++ti) {
+            int rb, cb;
+            tile_of(blockIdx.x + ti * gridDim.x, &rb, &cb);
+            const size_t ld = 2 * (size_t)lcols(P);
+            float* Af = Lf + ((size_t)r0 + rb * TC_ROWS + 128 * c2) * ld + 2 * (r0 + cb * TC_COLS) +
+                        32 * lb + lane;
+            // 16 rows at a time, fetched two groups ahead of their use
+            float c[3][16];
+            auto fetch = [&](int ch, float (&v)[16]) {
+#pragma unroll
+                for (int q = 0; q < 16; ++q) v[q] = Af[(16 * ch + q) * ld];
+            };
+            fetch(0, c[0]);
+            fetch(1, c[1]);
+            const uint32_t h = ti & 1;
+            if (!__all_sync(0xffffffffu, wait(&dfull[h], (ti >> 1) & 1))) {
+                ok = false;
+                break;
+            }
+            tc::fence_after_sync();
+#pragma unroll
+            for (int ch = 0; ch < 8; ++ch) {
+                if (ch + 2 < 8) fetch(ch + 2, c[(ch + 2) % 3]);
+                float v[16];
+                tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + h * 256 + 128 * c2 + 16 * ch, v);
+#pragma unroll
+                for (int q = 0; q < 16; ++q) Af[(16 * ch + q) * ld] = __fsub_rn(c[ch % 3][q], v[q]);
+            }
+            tc::fence_before_sync();
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(&dempty[h]))
+                         : "memory");
+        }
+        if (!ok && t == 32) set_status(status, CR_ETIMEOUT);
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(taddr, 512u);
+}
+
 // Trailing update of the lower block pairs (I, K), J < K <= I, one CTA per
-// pair (linear index -> row a = I - J - 1, column b = K - J - 1 with b <= a);
-// 16 x 16 threads, 4 x 4 outputs each (rows ty + 16 q, columns tx + 16 q).
-template <typename R>
-__global__ void __launch_bounds__(256) syrk_kernel(cpx<R>* __restrict__ L, int P, int J) {
-    constexpr int KC = 16;
-    __shared__ cpx<R> As[KC][NB + 1], Bs[KC][NB + 1];
+// pair (linear index -> row a = I - J - 1, column b = K - J - 1 with b <= a).
+__global__ void __launch_bounds__(256) syrk_kernel(cf* __restrict__ L, int P, int J) {
+    __shared__ __align__(16) cf As[KT][NB + 1];
+    __shared__ __align__(16) cf Bs[KT][BP];
     const long long idx = blockIdx.x;
     int a = (int)((sqrt(8.0 * (double)idx + 1.0) - 1.0) * 0.5);
     while ((long long)a * (a + 1) / 2 > idx) --a;
     while ((long long)(a + 1) * (a + 2) / 2 <= idx) ++a;
     const int b = (int)(idx - (long long)a * (a + 1) / 2);
-    const int i0 = (J + 1 + a) * NB, k0 = (J + 1 + b) * NB, c0 = J * NB;
+    const int i0 = (J + 1 + a) * NB, k0 = (J + 1 + b) * NB, c0 = J * NB, ld = lcols(P);
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    cpx<R> acc[4][4];
+    cf acc[4][4];
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int q2 = 0; q2 < 4; ++q2) acc[q][q2] = {R(0), R(0)};
-    for (int cc = 0; cc < NB; cc += KC) {
-        for (int e = threadIdx.x; e < NB * KC; e += blockDim.x) {
-            const int r = e / KC, c = e % KC, gi = i0 + r, gk = k0 + r;
-            As[c][r] = gi < P ? L[(size_t)gi * P + c0 + cc + c] : cpx<R>{R(0), R(0)};
-            Bs[c][r] = gk < P ? L[(size_t)gk * P + c0 + cc + c] : cpx<R>{R(0), R(0)};
+        for (int q2 = 0; q2 < 4; ++q2) acc[q][q2] = {0.f, 0.f};
+    for (int cc = 0; cc < NB; cc += KT) {
+        for (int e = threadIdx.x; e < NB * KT; e += 256) {
+            const int r = e / KT, c = e % KT, gi = i0 + r, gk = k0 + r;
+            As[c][r] = gi < P ? L[(size_t)gi * ld + c0 + cc + c] : cf{0.f, 0.f};
+            Bs[c][r] = gk < P ? conj(L[(size_t)gk * ld + c0 + cc + c]) : cf{0.f, 0.f};
         }
         __syncthreads();
-#pragma unroll
-        for (int c = 0; c < KC; ++c) {
-            cpx<R> av[4], bv[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                av[q] = As[c][ty + 16 * q];
-                bv[q] = conj(Bs[c][tx + 16 * q]);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-#pragma unroll
-                for (int q2 = 0; q2 < 4; ++q2) acc[q][q2] = acc[q][q2] + av[q] * bv[q2];
-        }
+        tile_step(As, Bs, tx, ty, acc);
         __syncthreads();
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int q2 = 0; q2 < 4; ++q2) {
-            const int i = i0 + ty + 16 * q, k = k0 + tx + 16 * q2;
+            const int i = i0 + ty + 16 * q, k = k0 + 4 * tx + q2;
             if (i < P && k < P) {
-                cpx<R>* p = L + (size_t)i * P + k;
+                cf* p = L + (size_t)i * ld + k;
                 *p = *p - acc[q][q2];
             }
         }
 }
 
-// Block column J of L y = r: every CTA stages L_JJ in shared memory and
-// solves y_J = L_JJ^{-1} r_J (warp 0), CTA 0 stores it; rows below get
-// r_i -= L_iJ y_J (one warp per row).  r is scratch (overwritten below
-// block J), y the result.
-template <typename R>
-__global__ void __launch_bounds__(256) trsv_fwd_kernel(const cpx<R>* __restrict__ L, int P, int J,
+// Inverse of a lower-triangular [[L11, 0], [L21, L22]] from X11 and X22 of
+// size s: X21 = -X22 (L21 X11), one 64 x 64 tile per CTA.  Pass 0 writes W =
+// L21 X11 into the unused upper block (rows of X11, columns of X22), pass 1
+// writes X21.  Grid (s / 64, s / 64, pairs of all SB blocks); pairs whose
+// lower part lies past P do not exist.
+__global__ void __launch_bounds__(256) xmerge_kernel(const cf* __restrict__ L, int P, int s, int pass,
+                                                     cf* __restrict__ X) {
+    __shared__ __align__(16) cf As[KT][NB + 1];
+    __shared__ __align__(16) cf Bs[KT][BP];
+    const int ppb = SB / (2 * s), sb = blockIdx.z / ppb, pr = blockIdx.z % ppb;
+    const int o1 = pr * 2 * s, o2 = o1 + s, base = sb * SB, ld = lcols(P);
+    if (base + o2 >= P) return;
+    const int ib = blockIdx.y, jb = blockIdx.x;  // 64-blocks of the s x s result
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4;
+    cf* Xs = X + (size_t)sb * SB * SB;
+    cf acc[4][4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) acc[q][q2] = {0.f, 0.f};
+    // X11 is lower triangular (rows k >= column j), so is X22 (k <= i)
+    const int kb = pass == 0 ? jb * NB : 0, ke = pass == 0 ? s : (ib + 1) * NB;
+    for (int cc = kb; cc < ke; cc += KT) {
+        for (int e = t; e < NB * KT; e += 256) {
+            const int r = e / KT, c = e % KT, i = ib * NB + r, gi = base + o2 + i;
+            As[c][r] = pass == 0 ? (gi < P ? L[(size_t)gi * ld + base + o1 + cc + c] : cf{0.f, 0.f})
+                                 : Xs[(size_t)(o2 + i) * SB + o2 + cc + c];
+            const int k = e / NB, j = e % NB;
+            Bs[k][j] = pass == 0 ? Xs[(size_t)(o1 + cc + k) * SB + o1 + jb * NB + j]
+                                 : Xs[(size_t)(o1 + cc + k) * SB + o2 + jb * NB + j];
+        }
+        __syncthreads();
+        tile_step(As, Bs, tx, ty, acc);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) {
+            const int i = ib * NB + ty + 16 * q, j = jb * NB + 4 * tx + q2;
+            if (pass == 0) Xs[(size_t)(o1 + i) * SB + o2 + j] = acc[q][q2];
+            else Xs[(size_t)(o2 + i) * SB + o1 + j] = -acc[q][q2];
+        }
+}
+
+// Triangular solves by 512-row blocks b.  Forward, L y = r:
+//   y_b = X_b r_b (diag), then r_i -= L_ib y_b below (rest; r is scratch);
+// one warp per row.  Backward, L^dag x = y:
+//   x_b = X_b^dag y_b (diag), then y_i -= sum_c conj(L_ci) x_c above (rest; y
+// is scratch); a CTA takes 32 rows i (lanes), its warps share the c.  The
+// products run in float32, the vectors are float64.  Bound by
+// reading L once per direction.
+__global__ void __launch_bounds__(256) trsv_fwd_kernel(const cf* __restrict__ L, int P, int b,
+                                                       const cf* __restrict__ X, int rest,
                                                        double* __restrict__ r_,
                                                        double* __restrict__ y_,
                                                        const double* __restrict__ skip) {
-    if (*skip != 0.0) return;
-    __shared__ cpx<R> d[NTRI];
-    __shared__ cpx<R> ys[NB];
+    if (skip && *skip != 0.0) return;
+    __shared__ cf v[SB];
     cpx<double>* r = (cpx<double>*)r_;
     cpx<double>* y = (cpx<double>*)y_;
-    const int base = J * NB, n = min(NB, P - base), t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    for (int e = t; e < n * n; e += blockDim.x) {
-        const int i = e / n, j = e % n;
-        if (j <= i) d[tri(i, j)] = L[(size_t)(base + i) * P + base + j];
-    }
+    const int base = b * SB, n = min(SB, P - base), t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const cpx<double>* src = (rest ? y : r) + base;
+    for (int e = t; e < SB; e += 256) v[e] = e < n ? ccast<float>(src[e]) : cf{0.f, 0.f};
     __syncthreads();
-    if (warp == 0) {
-        const cpx<R> z = {R(0), R(0)};
-        cpx<R> v0 = lane < n ? ccast<R>(r[base + lane]) : z;
-        cpx<R> v1 = lane + 32 < n ? ccast<R>(r[base + lane + 32]) : z;
-        for (int c = 0; c < n; ++c) {
-            cpx<R> yc = shfl(c < 32 ? v0 : v1, c & 31);
-            yc = (R(1) / d[tri(c, c)].x) * yc;
-            if (lane == (c & 31)) {
-                if (c < 32) v0 = yc;
-                else v1 = yc;
-            }
-            if (lane > c && lane < n) v0 = v0 - d[tri(lane, c)] * yc;
-            if (lane + 32 > c && lane + 32 < n) v1 = v1 - d[tri(lane + 32, c)] * yc;
-        }
-        if (lane < n) ys[lane] = v0;
-        if (lane + 32 < n) ys[lane + 32] = v1;
-    }
-    __syncthreads();
-    if (blockIdx.x == 0)
-        for (int e = t; e < n; e += blockDim.x) y[base + e] = ccast<double>(ys[e]);
-    for (int row = base + n + blockIdx.x * 8 + warp; row < P; row += gridDim.x * 8) {
-        const cpx<R>* Lr = L + (size_t)row * P + base;
-        cpx<R> s = Lr[lane] * ys[lane];
-        s = s + Lr[lane + 32] * ys[lane + 32];
+    const int i = blockIdx.x * 8 + warp;  // row of the block, or below it
+    if (rest) {
+        const int row = base + n + i;
+        if (row >= P) return;
+        const cf* Lr = L + (size_t)row * lcols(P) + base;  // n = SB: not the last block
+        cf s = {0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < SB; c += 32) s = s + Lr[c + lane] * v[c + lane];
         s = warp_sum(s);
         if (lane == 0) r[row] = r[row] - ccast<double>(s);
+    } else if (i < n) {
+        const cf* Xr = X + (size_t)b * SB * SB + (size_t)i * SB;
+        cf s = {0.f, 0.f};
+        for (int c = 0; c <= i; c += 32)
+            if (c + lane <= i) s = s + Xr[c + lane] * v[c + lane];
+        s = warp_sum(s);
+        if (lane == 0) y[base + i] = ccast<double>(s);
     }
 }
 
-// Block column J of L^dag x = y (J descending): every CTA stages L_JJ in
-// shared memory and solves x_J = L_JJ^{-dag} y_J (warp 0), CTA 0 stores it;
-// the 32 rows i above the block that a CTA owns get
-// y_i -= sum_c conj(L_{base + c, i}) x_c (lanes along i, warps along c).
-template <typename R>
-__global__ void __launch_bounds__(256) trsv_bwd_kernel(const cpx<R>* __restrict__ L, int P, int J,
+__global__ void __launch_bounds__(256) trsv_bwd_kernel(const cf* __restrict__ L, int P, int b,
+                                                       const cf* __restrict__ X, int rest,
                                                        double* __restrict__ y_,
                                                        double* __restrict__ x_,
                                                        const double* __restrict__ skip) {
-    if (*skip != 0.0) return;
-    __shared__ cpx<R> d[NTRI];
-    __shared__ cpx<R> xs[NB];
+    if (skip && *skip != 0.0) return;
+    __shared__ cf v[SB];
+    __shared__ cf part[8][32];
     cpx<double>* y = (cpx<double>*)y_;
     cpx<double>* x = (cpx<double>*)x_;
-    const int base = J * NB, n = min(NB, P - base), t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    for (int e = t; e < n * n; e += blockDim.x) {
-        const int i = e / n, j = e % n;
-        if (j <= i) d[tri(i, j)] = L[(size_t)(base + i) * P + base + j];
-    }
+    const int base = b * SB, n = min(SB, P - base), t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const cpx<double>* src = (rest ? x : y) + base;
+    for (int e = t; e < SB; e += 256) v[e] = e < n ? ccast<float>(src[e]) : cf{0.f, 0.f};
     __syncthreads();
-    if (warp == 0) {
-        const cpx<R> z = {R(0), R(0)};
-        cpx<R> v0 = lane < n ? ccast<R>(y[base + lane]) : z;
-        cpx<R> v1 = lane + 32 < n ? ccast<R>(y[base + lane + 32]) : z;
-        for (int c = n - 1; c >= 0; --c) {
-            cpx<R> xc = shfl(c < 32 ? v0 : v1, c & 31);
-            xc = (R(1) / d[tri(c, c)].x) * xc;
-            if (lane == (c & 31)) {
-                if (c < 32) v0 = xc;
-                else v1 = xc;
+    const int i = blockIdx.x * 32 + lane, lim = rest ? base : n;
+    const size_t ld = rest ? (size_t)lcols(P) : (size_t)SB;
+    const cf* A = rest ? L + (size_t)base * ld : X + (size_t)b * SB * SB;
+    cf s = {0.f, 0.f};
+    if (i < lim) {
+        // warp w takes the columns c in [64 w, 64 w + 64), sixteen loads in flight;
+        // in the diagonal block, entries above the diagonal of a 64-block are
+        // zero and the 64-blocks above it are left out
+        const int c1 = min(n, 64 * warp + 64);
+        int c = 64 * warp;
+        if (rest || c + 63 >= blockIdx.x * 32)
+            for (; c < c1; c += 16) {
+                cf a[16];
+#pragma unroll
+                for (int q = 0; q < 16; ++q)
+                    a[q] = c + q < c1 ? A[(size_t)(c + q) * ld + i] : cf{0.f, 0.f};
+#pragma unroll
+                for (int q = 0; q < 16; ++q) s = s + conj(a[q]) * v[c + q];
             }
-            if (lane < c) v0 = v0 - conj(d[tri(c, lane)]) * xc;
-            if (lane + 32 < c) v1 = v1 - conj(d[tri(c, lane + 32)]) * xc;
-        }
-        if (lane < n) xs[lane] = v0;
-        if (lane + 32 < n) xs[lane + 32] = v1;
     }
-    __syncthreads();
-    if (blockIdx.x == 0)
-        for (int e = t; e < n; e += blockDim.x) x[base + e] = ccast<double>(xs[e]);
-    // rows i in [32 blockIdx.x, +32): warp w sums the columns c in [8 w, 8 w + 8)
-    // (coalesced along i), then warp 0 adds the eight partial sums
-    __shared__ cpx<R> part[8][32];
-    const int i = blockIdx.x * 32 + lane;
-    cpx<R> s = {R(0), R(0)};
-    if (i < base)
-        for (int c = 8 * warp; c < 8 * warp + 8 && c < n; ++c)
-            s = s + conj(L[(size_t)(base + c) * P + i]) * xs[c];
     part[warp][lane] = s;
     __syncthreads();
-    if (warp == 0 && i < base) {
-        cpx<R> tot = part[0][lane];
+    if (warp == 0 && i < lim) {
+        cf tot = part[0][lane];
         for (int w = 1; w < 8; ++w) tot = tot + part[w][lane];
-        y[i] = y[i] - ccast<double>(tot);
+        if (rest) y[i] = y[i] - ccast<double>(tot);
+        else x[base + i] = ccast<double>(tot);
     }
 }
 
@@ -305,7 +610,8 @@ __global__ void __launch_bounds__(1024) refine_init_kernel(const double* __restr
     }
 }
 
-// r = F - S (x + d), one warp per row; per-CTA partial sums of |r|^2.
+// r = F - S (x + d), RES_ROWS rows of S per warp (they share the reads of x
+// and d); per-CTA partial sums of |r|^2.
 __global__ void __launch_bounds__(256) refine_resid_kernel(const double* __restrict__ S_, int P,
                                                            const double* __restrict__ F_,
                                                            const double* __restrict__ x_,
@@ -320,15 +626,29 @@ __global__ void __launch_bounds__(256) refine_resid_kernel(const double* __restr
     const cpx<double>* d = (const cpx<double>*)d_;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double acc = 0.0;
-    for (int row = blockIdx.x * 8 + warp; row < P; row += gridDim.x * 8) {
-        const cpx<double>* Sr = S + (size_t)row * P;
-        cpx<double> s = {0.0, 0.0};
-        for (int l = lane; l < P; l += 32) s = s + Sr[l] * (x[l] + d[l]);
-        s = warp_sum(s);
-        if (lane == 0) {
-            const cpx<double> rv = ((const cpx<double>*)F_)[row] - s;
-            ((cpx<double>*)r_)[row] = rv;
-            acc += abs2(rv);
+    const int row = (blockIdx.x * 8 + warp) * RES_ROWS;
+    if (row < P) {
+        cpx<double> s[RES_ROWS];
+        const cpx<double>* Sr[RES_ROWS];
+#pragma unroll
+        for (int q = 0; q < RES_ROWS; ++q) {
+            s[q] = {0.0, 0.0};
+            Sr[q] = S + (size_t)min(row + q, P - 1) * P;
+        }
+#pragma unroll 4
+        for (int l = lane; l < P; l += 32) {
+            const cpx<double> v = x[l] + d[l];
+#pragma unroll
+            for (int q = 0; q < RES_ROWS; ++q) s[q] = s[q] + Sr[q][l] * v;
+        }
+#pragma unroll
+        for (int q = 0; q < RES_ROWS; ++q) {
+            s[q] = warp_sum(s[q]);
+            if (lane == 0 && row + q < P) {
+                const cpx<double> rv = ((const cpx<double>*)F_)[row + q] - s[q];
+                ((cpx<double>*)r_)[row + q] = rv;
+                acc += abs2(rv);
+            }
         }
     }
     if (lane == 0) red[warp] = acc;
@@ -351,9 +671,11 @@ __global__ void __launch_bounds__(1024) refine_check_kernel(int P, double* __res
     cpx<double>* x = (cpx<double>*)x_;
     const cpx<double>* d = (const cpx<double>*)d_;
     for (int k = threadIdx.x; k < P; k += blockDim.x) x[k] = x[k] + d[k];
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
         double rr = 0.0;
-        for (int b = 0; b < npart; ++b) rr += part[b];
+        for (int b = threadIdx.x; b < npart; b += 32) rr += part[b];
+        rr = warp_sum(rr);
+        if (threadIdx.x != 0) return;
         const double prev = scal[8];
         scal[3] += 1.0;
         scal[4] = rr;
@@ -362,30 +684,113 @@ __global__ void __launch_bounds__(1024) refine_check_kernel(int P, double* __res
     }
 }
 
-template <typename R>
-cr_status factor_t(cr_ctx* c) {
+// Bytes of the trailing update's operands: the N side (rows in blocks of
+// 256), then the M side (two real rows per column).
+size_t n_plane_bytes(int P) { return (size_t)((P + TC_ROWS - 1) / TC_ROWS) * TC_NKC * 3 * N_TILE; }
+size_t m_plane_bytes(int P) {
+    return (size_t)((P + TC_ROWS - 1) / TC_ROWS) * (TC_ROWS / TC_COLS) * TC_NKC * 3 * M_TILE;
+}
+
+cr_status factor32(cr_ctx* c) {
     const int P = c->P, nb = (P + NB - 1) / NB;
-    cpx<R>* L = (cpx<R>*)c->Lf;
-    const size_t n = (size_t)P * P;
+    cf* L = (cf*)c->Lf;
+    cf* X = (cf*)c->chol_x;
+    const bool tcu = c->prec == CR_MIXED;
+    const size_t m_off = n_plane_bytes(P);
     CR_LAUNCH(c, CR_K_OTHER,
-              chol_copy_kernel<R><<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(c->S, P, L));
+              chol_copy_kernel<<<dim3((lcols(P) + 255) / 256, lrows(P)), 256, 0, c->stream>>>(c->S, P, L));
     for (int J = 0; J < nb; ++J) {
-        CR_LAUNCH(c, CR_KERNEL_CHOL, potrf_kernel<R><<<1, 256, 0, c->stream>>>(L, P, J, c->d_status));
+        CR_LAUNCH(c, CR_KERNEL_CHOL, potrf_inv_kernel<<<1, 256, 0, c->stream>>>(L, P, J, X, c->d_status));
         const int rows = P - (J + 1) * NB;
         if (rows <= 0) break;
-        const int g = min((rows + 7) / 8, 4 * c->n_sm);
-        CR_LAUNCH(c, CR_KERNEL_CHOL, trsm_kernel<R><<<g, 256, 0, c->stream>>>(L, P, J));
-        const int T = nb - J - 1;
+        const int nrb = (rows + TC_ROWS - 1) / TC_ROWS, ncb = (rows + NB - 1) / NB;
+        // the tensor-core update takes rows in blocks of 256, zero past P
         CR_LAUNCH(c, CR_KERNEL_CHOL,
-                  syrk_kernel<R><<<(unsigned)((long long)T * (T + 1) / 2), 256, 0, c->stream>>>(L, P, J));
+                  trsm_kernel<<<tcu ? 4 * nrb : ncb, 256, 0, c->stream>>>(
+                      L, P, J, X, tcu ? c->chol_pl : nullptr, m_off));
+        if (tcu) {
+            const int nt = 2 * (nrb - 1) * nrb + ncb;
+            CR_LAUNCH(c, CR_KERNEL_CHOL,
+                      syrk_tc_kernel<<<nt < c->n_sm ? nt : c->n_sm, TC_THREADS, TC_SMEM, c->stream>>>(
+                          (float*)c->Lf, P, (J + 1) * NB, nt, c->chol_pl, m_off, c->d_status));
+        } else {
+            const long long T = nb - J - 1;
+            CR_LAUNCH(c, CR_KERNEL_CHOL,
+                      syrk_kernel<<<(unsigned)(T * (T + 1) / 2), 256, 0, c->stream>>>(L, P, J));
+        }
     }
+    // merge the 64-row inverses up to SB rows (or all of a smaller matrix)
+    const int nsb = (P + SB - 1) / SB;
+    for (int s = NB; s < SB && s < P; s *= 2)
+        for (int pass = 0; pass < 2; ++pass)
+            CR_LAUNCH(c, CR_KERNEL_CHOL,
+                      xmerge_kernel<<<dim3(s / NB, s / NB, nsb * (SB / (2 * s))), 256, 0, c->stream>>>(
+                          L, P, s, pass, X));
     return cr_check_launch(c, "blocked Cholesky");
 }
 
-template <typename R>
-cr_status refine_t(cr_ctx* c, const double* F, int maxit) {
-    const int P = c->P, nb = (P + NB - 1) / NB;
-    const cpx<R>* L = (const cpx<R>*)c->Lf;
+// d = L^{-dag} L^{-1} r (r and y are scratch)
+void solve32(cr_ctx* c, double* r, double* y, double* d, const double* done) {
+    const int P = c->P, nsb = (P + SB - 1) / SB;
+    const cf* L = (const cf*)c->Lf;
+    const cf* X = (const cf*)c->chol_x;
+    for (int b = 0; b < nsb; ++b) {
+        const int n = P - b * SB < SB ? P - b * SB : SB, rows = P - b * SB - n;
+        CR_LAUNCH(c, CR_KERNEL_TRSV,
+                  trsv_fwd_kernel<<<(n + 7) / 8, 256, 0, c->stream>>>(L, P, b, X, 0, r, y, done));
+        if (rows > 0)
+            CR_LAUNCH(c, CR_KERNEL_TRSV,
+                      trsv_fwd_kernel<<<(rows + 7) / 8, 256, 0, c->stream>>>(L, P, b, X, 1, r, y, done));
+    }
+    for (int b = nsb - 1; b >= 0; --b) {
+        const int n = P - b * SB < SB ? P - b * SB : SB, rows = b * SB;
+        CR_LAUNCH(c, CR_KERNEL_TRSV,
+                  trsv_bwd_kernel<<<(n + 31) / 32, 256, 0, c->stream>>>(L, P, b, X, 0, y, d, done));
+        if (rows > 0)
+            CR_LAUNCH(c, CR_KERNEL_TRSV,
+                      trsv_bwd_kernel<<<(rows + 31) / 32, 256, 0, c->stream>>>(L, P, b, X, 1, y, d, done));
+    }
+}
+
+int resid_grid(int P) { return (P + 8 * RES_ROWS - 1) / (8 * RES_ROWS); }
+
+}  // namespace
+
+bool chol_refined(const cr_ctx* c) {
+    return (c->flags & CR_CTX_EXPLICIT_S) && (c->prec != CR_FP64 || c->P > CHOL_SMALL_P);
+}
+
+void chol_sizes(const cr_ctx* c, size_t* factor, size_t* inverses, size_t* planes) {
+    const size_t P = c->P;
+    if (c->prec == CR_FP64) {
+        *factor = P * P * 16;
+        *inverses = chol64_diag_bytes(c->P);
+        *planes = 0;
+        return;
+    }
+    *factor = (size_t)lrows(c->P) * lcols(c->P) * sizeof(cf);
+    *inverses = ((P + SB - 1) / SB) * (size_t)SB * SB * sizeof(cf);
+    *planes = c->prec == CR_MIXED ? n_plane_bytes(c->P) + m_plane_bytes(c->P) : 0;
+}
+
+size_t chol_cgpart_len(const cr_ctx* c) { return resid_grid(c->P); }
+
+cr_status chol_prepare(cr_ctx* c) {
+    if (c->prec == CR_FP64) return chol64_prepare(c);
+    cudaError_t e = cudaFuncSetAttribute(syrk_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)TC_SMEM);
+    return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "chol_prepare: %s", cudaGetErrorString(e));
+}
+
+cr_status chol_factor(cr_ctx* c) {
+    return c->prec == CR_FP64 ? chol64_factor(c, (double*)c->Lf, (double*)c->chol_x) : factor32(c);
+}
+
+// The iterates above into cg[0 .. P); scal[3] steps, scal[4] |r|^2.
+cr_status chol_refine_solve(cr_ctx* c, const double* F, int maxit) {
+    if (maxit > REFINE_MAXIT) maxit = REFINE_MAXIT;
+    if (maxit < 1) maxit = 1;
+    const int P = c->P, grid = resid_grid(P);
     double* x = c->cg;
     double* r = c->cg + 2 * (size_t)P;
     double* y = c->cg + 4 * (size_t)P;
@@ -393,42 +798,23 @@ cr_status refine_t(cr_ctx* c, const double* F, int maxit) {
     const double* done = c->scal + 2;
     CR_LAUNCH(c, CR_K_OTHER, refine_init_kernel<<<1, 1024, 0, c->stream>>>(F, P, x, r, c->scal));
     for (int it = 0; it < maxit; ++it) {
-        for (int J = 0; J < nb; ++J) {
-            const int rows = P - (J + 1) * NB;
-            const int g = rows > 0 ? (rows + 31) / 32 : 1;
-            CR_LAUNCH(c, CR_KERNEL_TRSV,
-                      trsv_fwd_kernel<R><<<g, 256, 0, c->stream>>>(L, P, J, r, y, done));
-        }
-        for (int J = nb - 1; J >= 0; --J) {
-            const int rows = J * NB;
-            const int g = rows > 0 ? (rows + 31) / 32 : 1;
-            CR_LAUNCH(c, CR_KERNEL_TRSV,
-                      trsv_bwd_kernel<R><<<g, 256, 0, c->stream>>>(L, P, J, y, d, done));
-        }
-        CR_LAUNCH(c, CR_K_OTHER, refine_resid_kernel<<<RES_GRID, 256, 0, c->stream>>>(
+        if (c->prec == CR_FP64) chol64_solve(c, (double*)c->Lf, (double*)c->chol_x, r, y, d, done);
+        else solve32(c, r, y, d, done);
+        CR_LAUNCH(c, CR_K_OTHER, refine_resid_kernel<<<grid, 256, 0, c->stream>>>(
                                      c->S, P, F, x, d, r, c->cgpart, done));
         CR_LAUNCH(c, CR_K_OTHER, refine_check_kernel<<<1, 1024, 0, c->stream>>>(
-                                     P, x, d, c->cgpart, RES_GRID, REFINE_TOL, c->scal));
+                                     P, x, d, c->cgpart, grid, REFINE_TOL, c->scal));
     }
     return cr_check_launch(c, "refined solve");
 }
 
-}  // namespace
-
-bool chol_blocked(const cr_ctx* c) {
-    return (c->flags & CR_CTX_EXPLICIT_S) && (c->prec != CR_FP64 || c->P > CHOL_SMALL_P);
-}
-
-size_t chol_factor_bytes(const cr_ctx* c) { return (size_t)c->P * c->P * 2 * rsize(c); }
-
-size_t chol_cgpart_len() { return RES_GRID; }
-
-cr_status chol_factor(cr_ctx* c) {
-    return c->prec == CR_FP64 ? factor_t<double>(c) : factor_t<float>(c);
-}
-
-cr_status chol_refine_solve(cr_ctx* c, const double* F, int maxit) {
-    if (maxit > REFINE_MAXIT) maxit = REFINE_MAXIT;
-    if (maxit < 1) maxit = 1;
-    return c->prec == CR_FP64 ? refine_t<double>(c, F, maxit) : refine_t<float>(c, F, maxit);
+// x = (L L^dag)^-1 F in float64, no refinement (small float64 contexts):
+// scal[1] = F.F on the way.
+cr_status chol_plain_solve(cr_ctx* c, const double* F) {
+    const size_t P = c->P;
+    double* x = c->cg;
+    double* r = c->cg + 2 * P;
+    CR_LAUNCH(c, CR_K_OTHER, refine_init_kernel<<<1, 1024, 0, c->stream>>>(F, c->P, x, r, c->scal));
+    chol64_solve(c, (double*)c->Lf, (double*)c->chol_x, r, c->cg + 4 * P, x, nullptr);
+    return cr_check_launch(c, "direct solve");
 }

@@ -189,12 +189,13 @@ struct cr_ctx {
                              // r.r and r.z [2][ceil(P/256)]
     double* scal;            // scalars [64]
     double* S;               // [P][P] complex128 (explicit S only)
-    void* O_tmp;             // [maxB][P] context precision (explicit S only)
     double* kry;             // Krylov workspace
     size_t kry_len;
-    void* Lf;                // [P][P] Cholesky factor, factor precision (blocked path only)
+    void* Lf;                // Cholesky factor, factor precision, padded (explicit S only)
+    void* chol_x;            // inverses of its 512 x 512 diagonal blocks
+    unsigned char* chol_pl;  // bf16 operands of the trailing update (mixed only)
     unsigned char* Xt;       // bf16 operands of the explicit S (mixed explicit S only)
-    float* spair_g;          // its pair sums (mixed explicit S only)
+    float* spair_g;          // its pair sums (float32 in mixed contexts, else float64)
     // Krylov Gram on the tensor cores (mixed): sized on first use
     unsigned char* gram_x;   // bf16 planes of the B and HB columns
     size_t gram_x_cap;
@@ -244,15 +245,22 @@ void cr_kt_end(cr_ctx* c);
 #define CR_K_OTHER (-2)
 cr_status cr_check_launch(cr_ctx* c, const char* what);
 
-// Explicit S and the direct solve (chol.cu, tc_kernels.cu).  Float64
-// contexts up to CHOL_SMALL_P parameters keep the single-CTA float64
-// Cholesky; every other explicit-S context takes the blocked path.
+// Explicit S and the direct solve (spair.cu, chol.cu).  Float64 contexts up
+// to CHOL_SMALL_P parameters solve once in float64; every other explicit-S
+// context refines the solution.
 #define CHOL_SMALL_P 2048
-bool chol_blocked(const cr_ctx* c);
-size_t chol_factor_bytes(const cr_ctx* c);
-size_t chol_cgpart_len();
+bool chol_refined(const cr_ctx* c);
+void chol_sizes(const cr_ctx* c, size_t* factor, size_t* inverses, size_t* planes);
+size_t chol_cgpart_len(const cr_ctx* c);
+cr_status chol_prepare(cr_ctx* c);
 cr_status chol_factor(cr_ctx* c);
 cr_status chol_refine_solve(cr_ctx* c, const double* F, int maxit);
+cr_status chol_plain_solve(cr_ctx* c, const double* F);
+size_t chol64_diag_bytes(int P);
+cr_status chol64_prepare(cr_ctx* c);
+cr_status chol64_factor(cr_ctx* c, double* A, double* D);
+void chol64_solve(cr_ctx* c, const double* A, const double* D, double* r, double* y, double* d,
+                  const double* skip);
 // Device scratch that grows on demand (once-per-sequence calls only): frees
 // and reallocates *p when cap < need; CR_ENOMEM with the caller's name.
 cr_status cr_grow(cr_ctx* c, void** p, size_t* cap, size_t need, const char* who);
@@ -261,9 +269,8 @@ cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const
                             double* redR, double* redO);
 cr_status launch_gram_tc(cr_ctx* c, const void* Bm, const void* HBm, int Nm, int B, int ld,
                          double* G, double* H);
-cr_status launch_sbuild_tc(cr_ctx* c, const int8_t* spins, const void* T, int B,
-                           const double* redO, double shift);
-void launch_smirror(cr_ctx* c);  // S[k][l] = conj(S[l][k]) for k < l
+cr_status launch_sbuild(cr_ctx* c, const int8_t* spins, const void* T, int B, const double* redO,
+                        double shift);
 
 // Fused CG solve (cg_fused.cu).
 bool fcg_supported(const cr_ctx* c);

@@ -160,7 +160,7 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     ALLOC(c->cg, 5 * P * 16);
     ALLOC(c->p_lo, P * cs);
     size_t ncgpart = (P + 31) / 32 + 2 * ((P + 255) / 256);
-    if (ncgpart < chol_cgpart_len()) ncgpart = chol_cgpart_len();
+    if (ncgpart < chol_cgpart_len(c)) ncgpart = chol_cgpart_len(c);
     ALLOC(c->cgpart, ncgpart * sizeof(double));
     ALLOC(c->scal, 64 * sizeof(double));
     int dev = 0;
@@ -169,15 +169,15 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
         cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (flags & CR_CTX_EXPLICIT_S) {
         ALLOC(c->S, P * P * 16);
-        if (prec == CR_MIXED) {
-            size_t xb, gb;
-            spair_sizes(c, &xb, &gb);
-            ALLOC(c->Xt, xb);
-            ALLOC(c->spair_g, gb);
-        } else {
-            ALLOC(c->O_tmp, B * P * cs);
-        }
-        if (chol_blocked(c)) ALLOC(c->Lf, chol_factor_bytes(c));
+        size_t xb, gb;
+        spair_sizes(c, &xb, &gb);
+        ALLOC(c->Xt, xb);
+        ALLOC(c->spair_g, gb);
+        size_t lf, lx, lp;
+        chol_sizes(c, &lf, &lx, &lp);
+        ALLOC(c->Lf, lf);
+        ALLOC(c->chol_x, lx);
+        ALLOC(c->chol_pl, lp);
     }
     std::vector<int2> ot;
     if (prec == CR_MIXED) {
@@ -220,7 +220,7 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     }
     if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->scal, 0, 64 * sizeof(double));
-    if (e != cudaSuccess || tc_prepare(c) != CR_OK || (prec == CR_MIXED && spair_prepare(c) != CR_OK) ||
+    if (e != cudaSuccess || tc_prepare(c) != CR_OK || (prec == CR_MIXED && spair_prepare(c) != CR_OK) || chol_prepare(c) != CR_OK ||
         target_prepare(c) != CR_OK || sym_prepare(c) != CR_OK ||
         (c->fcg && fcg_prepare(c) != CR_OK)) {
         cr_destroy(c);
@@ -236,8 +236,8 @@ extern "C" cr_status cr_destroy(cr_ctx* c) {
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
     void* ptrs[] = {c->d_status, c->d_bonds, c->theta_tmp, c->lp_tmp, c->u_tmp, c->partial,
-                    c->red, c->F, c->cg, c->p_lo, c->cgpart, c->scal, c->S, c->O_tmp, c->kry,
-                    c->Lf, c->Xt, c->spair_g, c->fcg_a1, c->fcg_b2, c->fcg_v2, c->fcg_vab,
+                    c->red, c->F, c->cg, c->p_lo, c->cgpart, c->scal, c->S, c->kry,
+                    c->Lf, c->chol_x, c->chol_pl, c->Xt, c->spair_g, c->fcg_a1, c->fcg_b2, c->fcg_v2, c->fcg_vab,
                     c->fcg_part, c->fcg_psc, c->fcg_bar, c->gram_x, c->gram_part,
                     c->gram_tiles, c->lp_work, c->ored_x, c->ored_part, c->ored_tiles};
     for (void* p : ptrs)

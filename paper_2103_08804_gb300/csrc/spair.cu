@@ -1,5 +1,4 @@
-// Explicit S of the natural-gradient update (Sec. III) on the tensor cores,
-// for CR_MIXED contexts.
+// Explicit S of the natural-gradient update (Sec. III).
 //
 // With sigma_0 = t_0 = 1 in front of the spins and of T_j = tanh theta_j,
 // every log-derivative is O_k = sigma_i t_j for one (i, j) other than (0, 0),
@@ -15,7 +14,12 @@
 // about P^2 / 2 x NPL multiply-adds per walker where the Gram matrix of
 // [Re O | Im O] takes 2 P^2 x 6 (both of its operands need the split):
 // eight times fewer for NPL = 3.  NPL = 3 holds all 24 bits of a float32;
-// NPL = 2 (CR_CTX_S_BF16X3) is good to about 2^-17 per product.
+// NPL = 2 (CR_CTX_S_BF16X3) is good to about 2^-17 per product.  That is the
+// form of CR_MIXED contexts; the others form the same sums on the FMA pipes
+// (spair_fma_kernel), an eighth of the additions of the P x P sums: float64
+// in CR_FP64, compensated float32 in CR_FP32 (products rounded to float32 as
+// before, the sum and its compensation together good to about 2^-46; the
+// float64 pipe does 1/64 of the float32 rate here).
 //
 // TMEM accumulates in float32 with an error that grows with the number of
 // MMAs added into one accumulator (measured: relative ~1e-8 each), so a
@@ -25,6 +29,7 @@
 //   spair_a_kernel, spair_y_kernel   the operands, tiles of 32 walkers in the
 //                                    K-major core-matrix layout
 //   spair_tc_kernel                  G, tiles of 128 Y columns x 256 pairs
+//   spair_mean_kernel                Obar = (sum_s O) / B
 //   spair_expand_kernel              S = G / B - conj(Obar) Obar^T + shift I
 //
 // The MMA's M side takes Y (three planes) and its N side the pairs (one
@@ -123,7 +128,7 @@ PairGeo pair_geometry(const cr_ctx* c) {
 __global__ void __launch_bounds__(256) spair_a_kernel(const int8_t* __restrict__ spins, int s0,
                                                       int B, int N, int nA, int nkc,
                                                       unsigned char* __restrict__ A) {
-    extern __shared__ __align__(16) unsigned char sm[];
+    extern __shared__ __align__(1024) unsigned char sm[];
     int8_t* sg = (int8_t*)sm;  // [N + 1][KC]
     const int kc = blockIdx.x, ab = blockIdx.y, t = threadIdx.x;
     for (int e = t; e < KC * (N + 1); e += blockDim.x) {
@@ -398,18 +403,26 @@ CR_D void param_of(int k, int N, int M, int* i, int* j) {
     }
 }
 
+// Obar in float64, formed once: the float64 pipe is what the expansion waits
+// for.
+__global__ void spair_mean_kernel(const double* __restrict__ redO, int P, int B, double* __restrict__ ob) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < P) ((cpx<double>*)ob)[k] = (1.0 / B) * ((const cpx<double>*)redO)[k];
+}
+
 // S of the 32 x 32 tile (by, bx), bx <= by, and its mirror image: S_kl of
 // the lower triangle from the segments' sums (float64, in segment order),
 // the upper triangle its exact conjugate.
-__global__ void __launch_bounds__(256) spair_expand_kernel(const float* __restrict__ G, int nseg,
+template <typename T>
+__global__ void __launch_bounds__(256) spair_expand_kernel(const T* __restrict__ G, int nseg,
                                                            size_t seg_stride, size_t ld, int N,
                                                            int M, int P, int B,
-                                                           const double* __restrict__ redO_,
+                                                           const double* __restrict__ ob_,
                                                            double shift, double* __restrict__ S_) {
     const int bx = blockIdx.x, by = blockIdx.y;
     if (bx > by) return;
     __shared__ cpx<double> tl[32][33];
-    const cpx<double>* redO = (const cpx<double>*)redO_;
+    const cpx<double>* ob = (const cpx<double>*)ob_;
     cpx<double>* S = (cpx<double>*)S_;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const double inv = 1.0 / B;
@@ -418,7 +431,7 @@ __global__ void __launch_bounds__(256) spair_expand_kernel(const float* __restri
     cpx<double> ol = {0.0, 0.0};
     if (l < P) {
         param_of(l, N, M, &il, &jl);
-        ol = inv * redO[l];
+        ol = ob[l];
     }
     for (int q = ty; q < 32; q += 8) {
         const int k = by * 32 + q;
@@ -426,19 +439,20 @@ __global__ void __launch_bounds__(256) spair_expand_kernel(const float* __restri
         int ik, jk;
         param_of(k, N, M, &ik, &jk);
         const int row = ik == il ? nA - 1 : pair_index(min(ik, il), max(ik, il));
-        const float* g = G + (size_t)row * ld;
+        const T* g = G + (size_t)row * ld;
         cpx<double> v = {0.0, 0.0};
         if (jk == jl) {
-            for (int sg = 0; sg < nseg; ++sg) v.x += (double)g[sg * seg_stride + nOff + jk];
+            v.x = (double)g[nOff + jk];
+            for (int sg = 1; sg < nseg; ++sg) v.x += (double)g[sg * seg_stride + nOff + jk];
         } else {
             const int y = 2 * pair_index(min(jk, jl), max(jk, jl));
-            for (int sg = 0; sg < nseg; ++sg) {
-                const float2 x = *reinterpret_cast<const float2*>(g + sg * seg_stride + y);
-                v = v + cpx<double>{(double)x.x, (double)x.y};
-            }
+            v = ccast<double>(*reinterpret_cast<const cpx<T>*>(g + y));
+            for (int sg = 1; sg < nseg; ++sg)
+                v = v + ccast<double>(*reinterpret_cast<const cpx<T>*>(g + sg * seg_stride + y));
             if (jk > jl) v = conj(v);  // the sum held is that of conj(t_jl) t_jk
         }
-        v = inv * v - cmulc(inv * redO[k], ol);
+        const cpx<double> m = cmulc(ob[k], ol);
+        v = {fma(inv, v.x, -m.x), fma(inv, v.y, -m.y)};
         if (k == l) v = {v.x + shift, 0.0};
         tl[q][tx] = v;
         if (l <= k) S[(size_t)k * P + l] = v;
@@ -448,6 +462,153 @@ __global__ void __launch_bounds__(256) spair_expand_kernel(const float* __restri
         const int r = bx * 32 + q, c = by * 32 + tx;  // mirror: row r, column c, r < c
         if (r < P && c < P && r < c) S[(size_t)r * P + c] = conj(tl[tx][q]);
     }
+}
+
+// The pair sums on the FMA pipes: a tile of 8 Q pairs x 16 Q columns of Y per
+// CTA and K segment, 8 x 16 threads with Q x Q sums each.  32 walkers at a
+// time, their spin products and tanh products formed in shared memory.
+// Float32: products rounded to float32, Kahan sums (s - c carries them);
+// float64: plain sums, Q = 2, so that small systems still spread over the SMs.
+template <typename R> struct FmaTile { static constexpr int Q = sizeof(R) == 4 ? 4 : 2; };
+constexpr int FMA_W = 32;
+
+template <typename R>
+__global__ void __launch_bounds__(128) spair_fma_kernel(const int8_t* __restrict__ spins,
+                                                        const cpx<R>* __restrict__ T, int B, int N,
+                                                        int M, int nA, int nY, int seg_walkers,
+                                                        double* __restrict__ G, size_t seg_stride) {
+    constexpr int Q = FmaTile<R>::Q, TI = 8 * Q, TJ = 16 * Q;
+    __shared__ R as[FMA_W][TI];
+    __shared__ __align__(16) R ys[FMA_W][TJ];
+    __shared__ int2 pa[TI], py[TJ / 2];
+    const int y0 = blockIdx.x * TJ, a0 = blockIdx.y * TI, seg = blockIdx.z;
+    const int s0 = seg * seg_walkers, s1 = min(B, s0 + seg_walkers);
+    const int t = threadIdx.x, tx = t & 15, ty = t >> 4, nOff = M * (M + 1);
+    if (t < TI) {
+        int a = 0, b = 0;
+        if (a0 + t < nA - 1) pair_of(a0 + t, &a, &b);
+        pa[t] = make_int2(a, b);
+    }
+    for (int e = t; e < TJ / 2; e += 128) {
+        const int y = y0 + 2 * e;
+        int a, b;
+        if (y < nOff) pair_of(y >> 1, &a, &b);
+        else { a = y - nOff; b = a + 1; }  // two squares |t_a|^2, |t_b|^2
+        py[e] = make_int2(a, b);
+    }
+    R acc[Q][Q], cmp[Q][Q];
+#pragma unroll
+    for (int p = 0; p < Q; ++p)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) acc[p][q] = cmp[p][q] = R(0);
+    const cpx<R> one = {R(1), R(0)}, zero = {R(0), R(0)};
+    for (int sb = s0; sb < s1; sb += FMA_W) {
+        __syncthreads();
+        for (int e = t; e < FMA_W * TI; e += 128) {
+            const int w = e / TI, r = e % TI, s = sb + w;
+            R v = R(0);
+            if (s < s1 && a0 + r < nA) {
+                const int2 p = pa[r];
+                const int8_t* sp = spins + (size_t)s * N - 1;
+                v = R((p.x ? sp[p.x] : 1) * (p.y ? sp[p.y] : 1));
+            }
+            as[w][r] = v;
+        }
+        for (int e = t; e < FMA_W * TJ / 2; e += 128) {
+            const int w = e / (TJ / 2), c = e % (TJ / 2), s = sb + w, y = y0 + 2 * c;
+            cpx<R> v = zero;
+            if (s < s1 && y < nY) {
+                const int2 p = py[c];
+                const cpx<R>* ts = T + (size_t)s * M - 1;
+                const cpx<R> a = p.x ? ldg(ts + p.x) : one;
+                const cpx<R> b = y < nOff || y + 1 < nY ? ldg(ts + p.y) : zero;
+                v = y < nOff ? cmulc(a, b) : cpx<R>{abs2(a), abs2(b)};
+            }
+            ys[w][2 * c] = v.x;
+            ys[w][2 * c + 1] = v.y;
+        }
+        __syncthreads();
+        const int nw = min(FMA_W, s1 - sb);
+#pragma unroll 4
+        for (int w = 0; w < nw; ++w) {
+            R av[Q], yv[Q];
+#pragma unroll
+            for (int p = 0; p < Q; ++p) av[p] = as[w][ty + 8 * p];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) yv[q] = ys[w][Q * tx + q];
+#pragma unroll
+            for (int p = 0; p < Q; ++p)
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    if constexpr (sizeof(R) == 8) {
+                        acc[p][q] = fma(av[p], yv[q], acc[p][q]);
+                    } else {
+                        // Kahan: av = +-1, so the product is exact
+                        const R x = __fmaf_rn(av[p], yv[q], -cmp[p][q]);
+                        const R u = __fadd_rn(acc[p][q], x);
+                        cmp[p][q] = __fsub_rn(__fsub_rn(u, acc[p][q]), x);
+                        acc[p][q] = u;
+                    }
+                }
+        }
+    }
+    double* out = G + seg * seg_stride;
+#pragma unroll
+    for (int p = 0; p < Q; ++p)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int r = a0 + ty + 8 * p, y = y0 + Q * tx + q;
+            if (r < nA && y < nY) out[(size_t)r * (nY + (nY & 1)) + y] = (double)acc[p][q] - (double)cmp[p][q];
+        }
+}
+
+// Grid of the FMA form: segments of whole 32-walker stages, about four CTAs
+// per SM, their sums held at once.
+struct FmaGeo {
+    int nA, nY, ga, gy, nseg, seg_walkers;
+    size_t ld, seg_stride;
+};
+
+FmaGeo fma_geometry(const cr_ctx* c) {
+    FmaGeo g;
+    const int Q = c->prec == CR_FP64 ? FmaTile<double>::Q : FmaTile<float>::Q;
+    g.nA = 1 + c->N * (c->N + 1) / 2;
+    g.nY = (c->M + 1) * (c->M + 1);
+    g.ga = (g.nA + 8 * Q - 1) / (8 * Q);
+    g.gy = (g.nY + 16 * Q - 1) / (16 * Q);
+    const long long tiles = (long long)g.ga * g.gy;
+    const int stages = (c->max_walkers + FMA_W - 1) / FMA_W;
+    long long ns = (4LL * c->n_sm + tiles - 1) / tiles;
+    if (ns > stages) ns = stages;
+    const int per = (int)((stages + ns - 1) / ns);
+    g.nseg = (stages + per - 1) / per;
+    g.seg_walkers = per * FMA_W;
+    g.ld = g.nY + (g.nY & 1);
+    g.seg_stride = (size_t)g.nA * g.ld;
+    return g;
+}
+
+template <typename T>
+cr_status expand(cr_ctx* c, const T* G, int nseg, size_t seg_stride, size_t ld, int B,
+                 const double* redO, double shift) {
+    const int P = c->P, nt = (P + 31) / 32;
+    double* ob = c->cg;  // the solution vectors are not in use yet
+    CR_LAUNCH(c, CR_K_OTHER, spair_mean_kernel<<<(P + 255) / 256, 256, 0, c->stream>>>(redO, P, B, ob));
+    CR_LAUNCH(c, CR_K_OTHER, spair_expand_kernel<T><<<dim3(nt, nt), 256, 0, c->stream>>>(
+                                 G, nseg, seg_stride, ld, c->N, c->M, P, B, ob, shift, c->S));
+    return cr_check_launch(c, "explicit S");
+}
+
+template <typename R>
+cr_status spair_fma_t(cr_ctx* c, const int8_t* spins, const void* T, int B, const double* redO,
+                      double shift) {
+    const FmaGeo g = fma_geometry(c);
+    const int nseg = (B + g.seg_walkers - 1) / g.seg_walkers;
+    double* G = (double*)c->spair_g;
+    CR_LAUNCH(c, CR_KERNEL_SBUILD, spair_fma_kernel<R><<<dim3(g.gy, g.ga, nseg), 128, 0, c->stream>>>(
+                                       spins, (const cpx<R>*)T, B, c->N, c->M, g.nA, g.nY,
+                                       g.seg_walkers, G, g.seg_stride));
+    return expand<double>(c, G, nseg, g.seg_stride, g.ld, B, redO, shift);
 }
 
 template <int NPL>
@@ -488,16 +649,18 @@ cr_status spair_t(cr_ctx* c, const int8_t* spins, const void* T, int B, const do
         CR_LAUNCH(c, CR_KERNEL_SBUILD,
                   spair_tc_kernel<NPL><<<grid, SP_THREADS, Ring<NPL>::SMEM, c->stream>>>(a));
     }
-    const int nt = (c->P + 31) / 32;
-    CR_LAUNCH(c, CR_K_OTHER,
-              spair_expand_kernel<<<dim3(nt, nt), 256, 0, c->stream>>>(
-                  c->spair_g, nseg, g.g_elems, (size_t)g.nyb * YT, N, M, c->P, B, redO, shift, c->S));
-    return cr_check_launch(c, "explicit S (tensor cores)");
+    return expand<float>(c, c->spair_g, nseg, g.g_elems, (size_t)g.nyb * YT, B, redO, shift);
 }
 
 }  // namespace
 
 void spair_sizes(const cr_ctx* c, size_t* x_bytes, size_t* g_bytes) {
+    if (c->prec != CR_MIXED) {
+        const FmaGeo g = fma_geometry(c);
+        *x_bytes = 0;
+        *g_bytes = (size_t)g.nseg * g.seg_stride * sizeof(double);
+        return;
+    }
     const PairGeo g = pair_geometry(c);
     *x_bytes = g.a_bytes + g.y_bytes;
     *g_bytes = (size_t)g.nseg * g.g_elems * sizeof(float);
@@ -512,8 +675,11 @@ cr_status spair_prepare(cr_ctx* c) {
     return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "spair_prepare: %s", cudaGetErrorString(e));
 }
 
-cr_status launch_sbuild_tc(cr_ctx* c, const int8_t* spins, const void* T, int B,
-                           const double* redO, double shift) {
+// S + shift I into c->S (full Hermitian, float64).
+cr_status launch_sbuild(cr_ctx* c, const int8_t* spins, const void* T, int B, const double* redO,
+                        double shift) {
+    if (c->prec == CR_FP64) return spair_fma_t<double>(c, spins, T, B, redO, shift);
+    if (c->prec == CR_FP32) return spair_fma_t<float>(c, spins, T, B, redO, shift);
     return npl_of(c) == 2 ? spair_t<2>(c, spins, T, B, redO, shift)
                           : spair_t<3>(c, spins, T, B, redO, shift);
 }

@@ -414,116 +414,6 @@ __global__ void force_kernel(const double* __restrict__ redR_, const double* __r
     }
 }
 
-// ------------------------------------------------------ explicit S (small P)
-
-template <typename R>
-__global__ void o_from_tanh_kernel(const int8_t* __restrict__ spins, const cpx<R>* __restrict__ T,
-                                   int B, int N, int M, int P, cpx<R>* __restrict__ O) {
-    size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)B * P) return;
-    int s = (int)(idx / P), k = (int)(idx % P);
-    cpx<R> v;
-    if (k < N) v = {R(spins[(size_t)s * N + k]), R(0)};
-    else if (k < N + M) v = T[(size_t)s * M + (k - N)];
-    else {
-        int i = (k - N - M) / M, j = (k - N - M) % M;
-        v = R(spins[(size_t)s * N + i]) * T[(size_t)s * M + j];
-    }
-    O[idx] = v;
-}
-
-// S[k][l] = sum_s conj(O_sk) O_sl / B - conj(Obar_k) Obar_l + shift delta_kl, float64.
-template <typename R>
-__global__ void sbuild_kernel(const cpx<R>* __restrict__ O, int B, int P,
-                              const double* __restrict__ redO_, double shift,
-                              double* __restrict__ S_) {
-    __shared__ cpx<R> tk[16][17], tl[16][17];
-    const int k = blockIdx.y * 16 + threadIdx.y, l = blockIdx.x * 16 + threadIdx.x;
-    cpx<double> acc = {0.0, 0.0};
-    for (int s0 = 0; s0 < B; s0 += 16) {
-        int s = s0 + threadIdx.x;
-        int kk = blockIdx.y * 16 + threadIdx.y;
-        tk[threadIdx.y][threadIdx.x] = (s < B && kk < P) ? O[(size_t)s * P + kk] : cpx<R>{R(0), R(0)};
-        s = s0 + threadIdx.y;
-        tl[threadIdx.y][threadIdx.x] = (s < B && l < P) ? O[(size_t)s * P + l] : cpx<R>{R(0), R(0)};
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-            acc = acc + ccast<double>(cmulc(tk[threadIdx.y][q], tl[q][threadIdx.x]));
-        __syncthreads();
-    }
-    if (k < P && l < P) {
-        const cpx<double>* redO = (const cpx<double>*)redO_;
-        const double inv = 1.0 / B;
-        cpx<double> v = inv * acc - cmulc(inv * redO[k], inv * redO[l]);
-        if (k == l) v.x += shift;
-        ((cpx<double>*)S_)[(size_t)k * P + l] = v;
-    }
-}
-
-// In-place Cholesky S = L L^dag (lower triangle), one CTA, then
-// L y = F, L^dag x = y; x written to out.  Column-oriented so each step is
-// one parallel update and one barrier.
-__global__ void __launch_bounds__(1024) chol_solve_kernel(double* __restrict__ S_, int P,
-                                                          const double* __restrict__ F_,
-                                                          double* __restrict__ x_,
-                                                          int* __restrict__ status) {
-    cpx<double>* S = (cpx<double>*)S_;
-    cpx<double>* x = (cpx<double>*)x_;
-    const cpx<double>* F = (const cpx<double>*)F_;
-    __shared__ double piv;
-    __shared__ int bad;
-    if (threadIdx.x == 0) bad = 0;
-    // right-looking factorisation
-    for (int j = 0; j < P; ++j) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double d = S[(size_t)j * P + j].x;
-            if (!(d > 0.0)) {
-                bad = 1;
-                d = 1.0;
-            }
-            piv = sqrt(d);
-            S[(size_t)j * P + j] = {piv, 0.0};
-        }
-        __syncthreads();
-        const double ip = 1.0 / piv;
-        for (int i = j + 1 + threadIdx.x; i < P; i += blockDim.x)
-            S[(size_t)i * P + j] = ip * S[(size_t)i * P + j];
-        __syncthreads();
-        // trailing update of the lower triangle: S_il -= L_ij conj(L_lj), l <= i
-        const int n = P - j - 1;
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-            int i = j + 1 + e / n, l = j + 1 + e % n;
-            if (l <= i) S[(size_t)i * P + l] = S[(size_t)i * P + l] -
-                                               S[(size_t)i * P + j] * conj(S[(size_t)l * P + j]);
-        }
-    }
-    __syncthreads();
-    if (bad) {
-        if (threadIdx.x == 0) set_status(status, CR_ESINGULAR);
-    }
-    for (int i = threadIdx.x; i < P; i += blockDim.x) x[i] = F[i];
-    // forward: L y = F
-    for (int k = 0; k < P; ++k) {
-        __syncthreads();
-        cpx<double> yk = (1.0 / S[(size_t)k * P + k].x) * x[k];
-        __syncthreads();
-        if (threadIdx.x == 0) x[k] = yk;
-        for (int i = k + 1 + threadIdx.x; i < P; i += blockDim.x)
-            x[i] = x[i] - S[(size_t)i * P + k] * yk;
-    }
-    // backward: L^dag x = y
-    for (int k = P - 1; k >= 0; --k) {
-        __syncthreads();
-        cpx<double> xk = (1.0 / S[(size_t)k * P + k].x) * x[k];
-        __syncthreads();
-        if (threadIdx.x == 0) x[k] = xk;
-        for (int i = threadIdx.x; i < k; i += blockDim.x)
-            x[i] = x[i] - conj(S[(size_t)k * P + i]) * xk;
-    }
-}
-
 // ------------------------------------------------------------------- CG
 //
 // Matrix-free S v = (O^dag (O v) - conj(Obar) sum_s (O v)_s) / B, using
@@ -732,36 +622,6 @@ __global__ void apply_update_kernel(cpx<R>* __restrict__ prm, const double* __re
     }
 }
 
-__global__ void fnorm_kernel(const double* __restrict__ F_, int P, double* __restrict__ scal) {
-    __shared__ double red[32];
-    const cpx<double>* F = (const cpx<double>*)F_;
-    double s = 0.0;
-    for (int k = threadIdx.x; k < P; k += blockDim.x) s += abs2(F[k]);
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) scal[1] = s;
-}
-
-// S + shift I into c->S (full Hermitian, float64; the upper triangle a
-// mirror of the lower): tensor cores (bf16x3) for mixed contexts; otherwise
-// O materialised in the context precision and its Gram matrix accumulated
-// in float64.
-template <typename R>
-static cr_status build_s(cr_ctx* c, const int8_t* spins, const void* T, int B,
-                         const double* redO, double shift) {
-    if (c->prec == CR_MIXED) return launch_sbuild_tc(c, spins, T, B, redO, shift);
-    const int P = c->P;
-    const size_t n = (size_t)B * P;
-    CR_LAUNCH(c, CR_K_OTHER,
-              o_from_tanh_kernel<R><<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(
-                  spins, (const cpx<R>*)T, B, c->N, c->M, P, (cpx<R>*)c->O_tmp));
-    dim3 g((P + 15) / 16, (P + 15) / 16);
-    CR_LAUNCH(c, CR_KERNEL_SBUILD,
-              sbuild_kernel<R><<<g, dim3(16, 16), 0, c->stream>>>((const cpx<R>*)c->O_tmp, B, P,
-                                                                  redO, shift, c->S));
-    launch_smirror(c);  // exactly Hermitian off the diagonal
-    return cr_check_launch(c, "explicit S");
-}
-
 template <typename R>
 static cr_status sr_step_t(cr_ctx* c, void* params, const int8_t* spins, const void* T,
                            const void* Rv, int B, const cr_sr_opts* o, double* stats) {
@@ -784,17 +644,12 @@ static cr_status sr_step_t(cr_ctx* c, void* params, const int8_t* spins, const v
                                  redR, redO, P, B, o->dgamma, o->mode, c->F, stats, c->d_status));
     if ((s = cr_check_launch(c, "force_kernel")) != CR_OK) return s;
     double* x = c->cg;
-    const bool blocked = o->solver == CR_SOLVE_CHOLESKY && chol_blocked(c);
+    const bool refined = o->solver == CR_SOLVE_CHOLESKY && chol_refined(c);
     if (o->solver == CR_SOLVE_CHOLESKY) {
-        if ((s = build_s<R>(c, spins, T, B, redO, o->shift)) != CR_OK) return s;
-        if (blocked) {
-            if ((s = chol_factor(c)) != CR_OK) return s;
-            if ((s = chol_refine_solve(c, c->F, o->cg_maxit)) != CR_OK) return s;
-        } else {
-            CR_LAUNCH(c, CR_K_OTHER, chol_solve_kernel<<<1, 1024, 0, c->stream>>>(c->S, P, c->F, x, c->d_status));
-            CR_LAUNCH(c, CR_K_OTHER, fnorm_kernel<<<1, 1024, 0, c->stream>>>(c->F, P, c->scal));
-            if ((s = cr_check_launch(c, "cholesky path")) != CR_OK) return s;
-        }
+        if ((s = launch_sbuild(c, spins, T, B, redO, o->shift)) != CR_OK) return s;
+        if ((s = chol_factor(c)) != CR_OK) return s;
+        s = refined ? chol_refine_solve(c, c->F, o->cg_maxit) : chol_plain_solve(c, c->F);
+        if (s != CR_OK) return s;
     } else if (c->fcg) {
         // mixed precision: the whole CG in one persistent tensor-core kernel
         s = launch_cg_fused(c, spins, T, B, redO, o->shift, o->cg_tol, o->cg_maxit, o->cg_precond,
@@ -833,7 +688,7 @@ static cr_status sr_step_t(cr_ctx* c, void* params, const int8_t* spins, const v
         }
     }
     CR_LAUNCH(c, CR_K_OTHER, apply_update_kernel<R><<<(P + 255) / 256, 256, 0, c->stream>>>(
-        (cpx<R>*)params, x, P, c->scal, stats, c->F, c->d_status, o->solver == CR_SOLVE_CG || blocked,
+        (cpx<R>*)params, x, P, c->scal, stats, c->F, c->d_status, o->solver == CR_SOLVE_CG || refined,
         o->solver == CR_SOLVE_CG && o->cg_strict));
     return cr_check_launch(c, "apply_update");
 }
@@ -926,13 +781,12 @@ extern "C" cr_status sr_sv(cr_ctx* ctx, const int8_t* spins, const void* tanh_th
                                 : sv_t<float>(ctx, spins, tanh_theta, B, v, shift, u_out, out);
 }
 
-template <typename R>
-static cr_status smatrix_t(cr_ctx* c, const int8_t* spins, const void* T, int B, double shift,
+static cr_status smatrix(cr_ctx* c, const int8_t* spins, const void* T, int B, double shift,
                            double* S_out) {
     double* redO = c->red + 2 * (c->P + 2 + c->M);
     cr_status s = oreduce(c, false, spins, T, nullptr, B, redO, nullptr);
     if (s != CR_OK) return s;
-    if ((s = build_s<R>(c, spins, T, B, redO, shift)) != CR_OK) return s;
+    if ((s = launch_sbuild(c, spins, T, B, redO, shift)) != CR_OK) return s;
     cudaError_t e = cudaMemcpyAsync(S_out, c->S, (size_t)c->P * c->P * 16,
                                     cudaMemcpyDeviceToDevice, c->stream);
     return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "sr_smatrix copy: %s", cudaGetErrorString(e));
@@ -947,8 +801,7 @@ extern "C" cr_status sr_smatrix(cr_ctx* ctx, const int8_t* spins, const void* ta
                  ctx->max_walkers);
     CR_CHECK_ARG(spins && tanh_theta && S_out, "sr_smatrix: null array");
     CR_CHECK_ARG(shift >= 0.0, "sr_smatrix: shift must be >= 0");
-    return ctx->prec == CR_FP64 ? smatrix_t<double>(ctx, spins, tanh_theta, B, shift, S_out)
-                                : smatrix_t<float>(ctx, spins, tanh_theta, B, shift, S_out);
+    return smatrix(ctx, spins, tanh_theta, B, shift, S_out);
 }
 
 // ------------------------------------------------------ backward of log psi

@@ -681,24 +681,6 @@ __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs 
     if (warp == 0) tc::tmem_dealloc(taddr, 512u);
 }
 
-// S[k][l] = conj(S[l][k]) for k < l (32 x 32 tiles through shared memory).
-__global__ void smirror_kernel(double* __restrict__ S_, int P) {
-    __shared__ cpx<double> tl[32][33];
-    const int bx = blockIdx.x, by = blockIdx.y;  // tile column, tile row
-    if (bx < by) return;                         // tiles on or above the diagonal only
-    cpx<double>* S = (cpx<double>*)S_;
-    const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-    for (int j = ty; j < 32; j += 8) {
-        const int r = bx * 32 + j, c = by * 32 + tx;  // source: lower block (row bx, col by)
-        if (r < P && c < P) tl[j][tx] = S[(size_t)r * P + c];
-    }
-    __syncthreads();
-    for (int j = ty; j < 32; j += 8) {
-        const int r = by * 32 + j, c = bx * 32 + tx;  // destination (row by, col bx)
-        if (r < P && c < P && r < c) S[(size_t)r * P + c] = conj(tl[tx][j]);
-    }
-}
-
 // ---------------------------------------------- Krylov Gram (Sec. IV)
 //
 // G = B^dag B / B_s and H = B^dag HB / B_s of cheb_gram on the tensor cores:
@@ -834,11 +816,6 @@ cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const
                   NCp, NT, cols, c->partial, skip, c->d_status));
     *nch_out = nch;
     return cr_check_launch(c, "oreduce_tc_kernel");
-}
-
-void launch_smirror(cr_ctx* c) {
-    const int nt = (c->P + 31) / 32;
-    CR_LAUNCH(c, CR_K_OTHER, smirror_kernel<<<dim3(nt, nt), dim3(32, 8), 0, c->stream>>>(c->S, c->P));
 }
 
 // Geometry of the Krylov Gram on the tensor cores (three-plane split): rows
