@@ -177,6 +177,8 @@ struct cr_ctx {
     int* d_status;           // device status word
     int2* d_bonds;           // [Nb]
     cr_tables tab[2];        // 0: sampler / moment state, 1: target state
+    void* xtab;              // exchange table (float32 contexts)
+    void* xout;              // xsum_out [maxB] (float32 contexts)
     void* theta_tmp;         // [maxB][M]
     void* lp_tmp;            // [2][maxB]
     void* u_tmp;             // [maxB]
@@ -225,6 +227,16 @@ struct cr_ctx {
     unsigned* fcg_bar;       // grid-barrier counter and abort flag
     int fcg_ctas;            // CTAs of the fused CG (0: one per SM)
     cudaEvent_t ev_fork, ev_join;  // batched runs: fork from / join into the caller's stream
+};
+
+// What xsum_kernel (exchange.cu) leaves per configuration: with
+// lam = base + ex ln 2, the exchanged amplitudes of the antiparallel bonds sum to
+// e^lam (off + slow), and weighted with s_i d_b of the probe to
+// e^lam (offd + slow_d).  float4: (re hi, re lo, im hi, im lo).
+struct alignas(16) xsum_out {
+    float4 off, offd, base;
+    int nanti, ex, pad[2];
+    cpx<double> slow, slow_d;
 };
 
 static inline int rsize(const cr_ctx* c) { return c->prec == CR_FP64 ? 8 : 4; }
@@ -279,6 +291,12 @@ cr_status fcg_prepare(cr_ctx* c);
 cr_status launch_cg_fused(cr_ctx* c, const int8_t* spins, const void* T, int B, const double* redO,
                           double shift, double tol, int maxit, int precond, int apply_only,
                           const double* v_in, void* u_out);
+
+// Sums over exchanged amplitudes in float32 (exchange.cu).
+size_t xsum_table_bytes(const cr_ctx* c);
+cr_status xsum_prepare(cr_ctx* c);
+cr_status launch_xsum(cr_ctx* c, const void* params, const int8_t* spins, const void* theta, int n,
+                      int probe, double qx, double qy, xsum_out* out);
 
 // Tables for a state (rbm.cu).
 cr_status build_tables(cr_ctx* c, const void* params, int slot);

@@ -143,7 +143,11 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     if (e == cudaSuccess) e = alloc((void**)&(ptr), (bytes))
     ALLOC(c->d_status, sizeof(int));
     ALLOC(c->d_bonds, Nb * sizeof(int2));
-    for (int s = 0; s < 2; ++s) {
+    if (prec != CR_FP64) {
+        ALLOC(c->xtab, xsum_table_bytes(c));
+        ALLOC(c->xout, B * sizeof(xsum_out));
+    }
+    for (int s = 0; s < (prec == CR_FP64 ? 2 : 1); ++s) {  // slot 1: the float64 local target
         ALLOC(c->tab[s].D, Nb * Mp * cs);
         ALLOC(c->tab[s].Ch, Nb * Mp * cs);
         ALLOC(c->tab[s].Sh, Nb * Mp * cs);
@@ -221,7 +225,7 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->scal, 0, 64 * sizeof(double));
     if (e != cudaSuccess || tc_prepare(c) != CR_OK || (prec == CR_MIXED && spair_prepare(c) != CR_OK) || chol_prepare(c) != CR_OK ||
-        target_prepare(c) != CR_OK || sym_prepare(c) != CR_OK ||
+        (prec != CR_FP64 && xsum_prepare(c) != CR_OK) || target_prepare(c) != CR_OK || sym_prepare(c) != CR_OK ||
         (c->fcg && fcg_prepare(c) != CR_OK)) {
         cr_destroy(c);
         return CR_ECUDA;
@@ -235,7 +239,7 @@ extern "C" cr_status cr_destroy(cr_ctx* c) {
     kt_free(c);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
-    void* ptrs[] = {c->d_status, c->d_bonds, c->theta_tmp, c->lp_tmp, c->u_tmp, c->partial,
+    void* ptrs[] = {c->d_status, c->d_bonds, c->xtab, c->xout, c->theta_tmp, c->lp_tmp, c->u_tmp, c->partial,
                     c->red, c->F, c->cg, c->p_lo, c->cgpart, c->scal, c->S, c->kry,
                     c->Lf, c->chol_x, c->chol_pl, c->Xt, c->spair_g, c->fcg_a1, c->fcg_b2, c->fcg_v2, c->fcg_vab,
                     c->fcg_part, c->fcg_psc, c->fcg_bar, c->gram_x, c->gram_part,

@@ -22,9 +22,10 @@
 // is the same rotation average and Fourier sum taken over
 // (H' t_n)(s') / psi(s) at each transformed configuration.  That value is
 // formed without dividing by t_n(s'): the transformed configurations are not
-// samples of |t_n|^2 and can sit next to a node of t_n (cosh theta_m ~ 0),
-// where the ratio tables of the target kernel (tanh theta) lose all
-// precision in float32.
+// samples of |t_n|^2 and can sit next to a node of t_n (cosh theta_m ~ 0).
+// Float32 contexts take the sums over exchanged amplitudes from xsum_kernel
+// (exchange.cu) and finish a configuration per thread; float64 contexts run
+// sym_hprime_kernel.
 #include "common.cuh"
 
 namespace {
@@ -216,6 +217,23 @@ __global__ void __launch_bounds__(128) sym_hprime_kernel(
     }
 }
 
+// The same value from the float32 sums of xsum_kernel, one thread per
+// configuration.
+__global__ void sym_hfinish_kernel(const xsum_out* __restrict__ xo, const cpx<float>* __restrict__ lp,
+                                   const cpx<float>* __restrict__ lp_ref, int nc, int B, int Nb, double J,
+                                   double E0, double a, double Wp, cpx<float>* __restrict__ hb) {
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= nc) return;
+    const xsum_out o = xo[w];
+    const cpx<double> ref = ccast<double>(lp_ref[w % B]);
+    const cpx<double> lam = {(double)o.base.x + (double)o.base.y + o.ex * 0.6931471805599453 - ref.x,
+                             (double)o.base.z + (double)o.base.w - ref.y};
+    const cpx<double> off = cpx<double>{(double)o.off.x + (double)o.off.y,
+                                        (double)o.off.z + (double)o.off.w} + o.slow;
+    const double ia = 1.0 / a, ed = 0.25 * J * (Nb - 2 * o.nanti);
+    const cpx<double> v = cexp_(ccast<double>(lp[w]) - ref);
+    hb[w] = ccast<float>((ia * ed - (E0 * ia + Wp)) * v + (0.5 * J * ia) * (cexp_(lam) * off));
+}
 
 // Bt[(k Nm + n) B + s] = L^-1 sum_m e^{-i 2 pi (k1 m1 + k2 m2) / L} A[m][s]
 template <typename R>
@@ -246,7 +264,7 @@ __global__ void sym_dft_kernel(const cpx<R>* __restrict__ A, int L, int B, int n
 // values (H' t_n)(s') / psi(s) [4N B] and HA [N][B].  Every part 256-byte
 // aligned.
 struct sym_ws {
-    size_t lp, A, theta, hb, HA, total;
+    size_t lp, A, theta, hb, HA, xo, total;
 };
 
 sym_ws ws_layout(const cr_ctx* c, int B, bool with_h) {
@@ -261,6 +279,10 @@ sym_ws ws_layout(const cr_ctx* c, int B, bool with_h) {
         o.hb = o.theta + up(nc * c->M * cs);
         o.HA = o.hb + up(nc * cs);
         o.total = o.HA + N * B * cs;
+        if (c->prec != CR_FP64) {  // the exchange sums of the float32 form
+            o.xo = up(o.total);
+            o.total = o.xo + nc * sizeof(xsum_out);
+        }
     }
     return o;
 }
@@ -274,31 +296,37 @@ template <typename R> size_t sym_hprime_smem(const cr_ctx* c) {
 // Opt sym_hprime_kernel into the shared memory of this context where it
 // exceeds the default (called once per context, outside any capture).
 cr_status sym_prepare_impl(cr_ctx* c) {
-    const size_t s4 = sym_hprime_smem<float>(c), s8 = sym_hprime_smem<double>(c);
-    cudaError_t e = cudaSuccess;
-    if (s4 > 48 * 1024)
-        e = cudaFuncSetAttribute(sym_hprime_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)s4);
-    if (e == cudaSuccess && s8 > 48 * 1024)
-        e = cudaFuncSetAttribute(sym_hprime_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)s8);
+    const size_t s8 = sym_hprime_smem<double>(c);
+    if (c->prec != CR_FP64 || s8 <= 48 * 1024) return CR_OK;
+    cudaError_t e = cudaFuncSetAttribute(sym_hprime_kernel<double>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s8);
     return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "sym_prepare: %s", cudaGetErrorString(e));
 }
 
-template <typename R>
 cr_status launch_sym_hprime(cr_ctx* c, const void* params, const int8_t* sp, int nc, int B,
-                            const cpx<R>* th, const cpx<R>* lp, const void* lp_ref,
-                            const double* hp, cpx<R>* hb) {
+                            const cpx<double>* th, const cpx<double>* lp, const void* lp_ref,
+                            const double* hp, cpx<double>* hb, xsum_out*) {
     cr_status s = build_tables(c, params, 1);
     if (s != CR_OK) return s;
     const cr_tables& t = c->tab[1];
-    const size_t sm = sym_hprime_smem<R>(c);
+    const size_t sm = sym_hprime_smem<double>(c);
     CR_LAUNCH(c, CR_KERNEL_TARGET,
-              sym_hprime_kernel<R><<<(unsigned)((nc + 127) / 128), 128, sm, c->stream>>>(
-                  sp, th, lp, (const cpx<R>*)lp_ref, (const cpx<R>*)params, (const cpx<R>*)t.ChT,
-                  (const cpx<R>*)t.ShT, (const cpx<R>*)t.ea, c->d_bonds, nc, B, c->N, c->M, c->Mp,
-                  c->Nb, c->J, hp[0], hp[1], hp[2], hb));
+              sym_hprime_kernel<double><<<(unsigned)((nc + 127) / 128), 128, sm, c->stream>>>(
+                  sp, th, lp, (const cpx<double>*)lp_ref, (const cpx<double>*)params,
+                  (const cpx<double>*)t.ChT, (const cpx<double>*)t.ShT, (const cpx<double>*)t.ea,
+                  c->d_bonds, nc, B, c->N, c->M, c->Mp, c->Nb, c->J, hp[0], hp[1], hp[2], hb));
     return cr_check_launch(c, "sym_hprime_kernel");
+}
+
+cr_status launch_sym_hprime(cr_ctx* c, const void* params, const int8_t* sp, int nc, int B,
+                            const cpx<float>* th, const cpx<float>* lp, const void* lp_ref,
+                            const double* hp, cpx<float>* hb, xsum_out* xo) {
+    cr_status s = launch_xsum(c, params, sp, th, nc, 0, 0.0, 0.0, xo);
+    if (s != CR_OK) return s;
+    CR_LAUNCH(c, CR_K_OTHER, sym_hfinish_kernel<<<(unsigned)((nc + 127) / 128), 128, 0, c->stream>>>(
+                                 xo, lp, (const cpx<float>*)lp_ref, nc, B, c->Nb, c->J, hp[0], hp[1],
+                                 hp[2], hb));
+    return cr_check_launch(c, "sym_hfinish_kernel");
 }
 
 template <typename R>
@@ -323,7 +351,8 @@ cr_status btilde_t(cr_ctx* c, const cr_state* states, int Nm, const int8_t* spin
         cr_status s = launch_logpsi(c, states[n].params, sp, nc, th, lp);
         if (s != CR_OK) return s;
         if (h) {
-            s = launch_sym_hprime<R>(c, states[n].params, sp, nc, B, th, lp, lp_ref, hp, hb);
+            s = launch_sym_hprime(c, states[n].params, sp, nc, B, th, lp, lp_ref, hp, hb,
+                                  (xsum_out*)(ws + o.xo));
             if (s != CR_OK) return s;
         }
         CR_LAUNCH(c, CR_K_OTHER, sym_rot_kernel<R><<<gb, 256, 0, c->stream>>>(

@@ -4,10 +4,17 @@
 // Both apply H' = (H - E0)/a - W' to a state v at a sample s, relative to a
 // reference amplitude psi_ref(s):
 //   (H v)(s) = sum_b [(J/4) s_i s_j v(s) + (J/2)[s_i != s_j] v(s^{ij})]   (Sec. V)
-// One warp per sample.  Lanes take the antiparallel bonds of the sample
-// (compacted with a ballot) and run over the hidden units sequentially,
-// forming the exchanged amplitude relative to the reference amplitude with
-// no division:
+// Float32 and mixed contexts: the sums over exchanged amplitudes come from
+// xsum_kernel (exchange.cu); hfinish_kernel, one thread per sample, adds the
+// diagonal part, the probe factors and the recursion's second state, in
+// float64 (its few exponentials cost a warp the same for one sample as for
+// 32: in the lanes of one warp per sample they took a millisecond of the
+// 16 x 16 lattice's target at 65536 samples).
+//
+// Float64 contexts, hprime_kernel: one warp per sample; lanes take the
+// antiparallel bonds of the sample (compacted with a ballot) and run over the
+// hidden units sequentially, forming the exchanged amplitude relative to the
+// reference amplitude with no division:
 //   v(s^{ij}) / psi_ref(s) = exp(a.s - 2 s_i (a_i - a_i') + X + M ln 2 - log psi_ref(s))
 //                            prod_m (C_m cosh D_m - s_i S_m sinh D_m),
 // C_m, S_m = cosh, sinh theta_m times e^{-|Re theta_m|} and X = sum_m |Re theta_m|,
@@ -225,6 +232,66 @@ __global__ void __launch_bounds__(128) hprime_kernel(hp_args<R> A) {
     }
 }
 
+// The float32 form's second half: out1, out2 and mu_terms of hprime_kernel,
+// from the sums in xo.  f_q(s) is summed in order with its rounding errors
+// carried along.
+__global__ void __launch_bounds__(128) hfinish_kernel(hp_args<float> A, double E0, double a, double Wp,
+                                                      const xsum_out* __restrict__ xo) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cpx<float>* ph = (cpx<float>*)smem_raw;  // [3][N] e^{-iq.r} of the probes in use
+    const probe_desc pd[3] = {A.pr, A.pr2, A.prm};
+    for (int k = 0; k < 3; ++k)
+        if (pd[k].on)
+            for (int r = threadIdx.x; r < A.N; r += blockDim.x)
+                ph[k * A.N + r] = phase<float>(r, A.Lx, pd[k].qx, pd[k].qy);
+    __syncthreads();
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= A.B) return;
+    const double isn = rsqrt((double)A.N);
+    cpx<double> f[3];
+    for (int k = 0; k < 3; ++k) {
+        f[k] = {1.0, 0.0};
+        if (!pd[k].on) continue;
+        const int8_t* sg = A.spins + (size_t)w * A.N;
+        const cpx<float>* pk = ph + k * A.N;
+        float sx = 0.f, sy = 0.f, cx = 0.f, cy = 0.f;
+        for (int r = 0; r < A.N; ++r) {
+            const float s = (float)sg[r];
+            const float ux = __fmaf_rn(s, pk[r].x, -cx), uy = __fmaf_rn(s, pk[r].y, -cy);
+            const float tx = __fadd_rn(sx, ux), ty = __fadd_rn(sy, uy);
+            cx = __fsub_rn(__fsub_rn(tx, sx), ux);
+            cy = __fsub_rn(__fsub_rn(ty, sy), uy);
+            sx = tx;
+            sy = ty;
+        }
+        f[k] = (0.5 * isn) * cpx<double>{(double)sx - (double)cx, (double)sy - (double)cy};
+    }
+    const cpx<double> ref = ccast<double>(A.L_ref[w]);
+    const cpx<double> V = f[0] * cexp_(ccast<double>(A.L_prev[w]) - ref);
+    cpx<double> E = {0.0, 0.0};
+    if (A.want_E) {
+        const xsum_out o = xo[w];
+        const cpx<double> lam = {(double)o.base.x + (double)o.base.y + o.ex * 0.6931471805599453 - ref.x,
+                                 (double)o.base.z + (double)o.base.w - ref.y};
+        cpx<double> off = f[0] * (cpx<double>{(double)o.off.x + (double)o.off.y,
+                                              (double)o.off.z + (double)o.off.w} + o.slow);
+        if (A.pr.on)
+            off = off + isn * (cpx<double>{(double)o.offd.x + (double)o.offd.y,
+                                           (double)o.offd.z + (double)o.offd.w} + o.slow_d);
+        const double ia = 1.0 / a, ed = 0.25 * (double)A.J * (A.Nb - 2 * o.nanti);
+        E = (ia * ed - (E0 * ia + Wp)) * V + (0.5 * (double)A.J * ia) * (cexp_(lam) * off);
+    }
+    const cpx<double> ba = {A.beta_a[0], A.beta_a[1]};
+    cpx<double> o1 = (A.ka * ba) * E;
+    if (A.L_prev2)
+        o1 = o1 - cpx<double>{A.beta_b[0], A.beta_b[1]} *
+                      (f[1] * cexp_(ccast<double>(A.L_prev2[w]) - ref));
+    const cpx<double> o2 = ba * V;
+    if (A.out1) A.out1[w] = ccast<float>(o1);
+    if (A.out2) A.out2[w] = ccast<float>(o2);
+    if (A.mu_terms) A.mu_terms[w] = ccast<float>(cmulc(f[2], o2));
+}
+
 // mu = sum_s terms[s] / B, summed in float64 by one CTA in a fixed order.
 template <typename R>
 __global__ void mean_kernel(const cpx<R>* __restrict__ terms, int B, double* __restrict__ out) {
@@ -261,22 +328,16 @@ static size_t hprime_smem(const cr_ctx* c) {
 }
 
 cr_status target_prepare(cr_ctx* c) {
-    const size_t sm = c->prec == CR_FP64 ? hprime_smem<double>(c) : hprime_smem<float>(c);
+    if (c->prec != CR_FP64) return CR_OK;
+    const size_t sm = hprime_smem<double>(c);
     if (sm <= 48 * 1024) return CR_OK;
-    cudaError_t e = c->prec == CR_FP64
-                        ? cudaFuncSetAttribute(hprime_kernel<double>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)
-                        : cudaFuncSetAttribute(hprime_kernel<float>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    cudaError_t e = cudaFuncSetAttribute(hprime_kernel<double>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "target_prepare: %s", cudaGetErrorString(e));
 }
 
 template <typename R>
-static cr_status launch_hprime(cr_ctx* c, hp_args<R>& A) {
-    const cr_tables& t = c->tab[1];
-    A.ChT = (const cpx<R>*)t.ChT;
-    A.ShT = (const cpx<R>*)t.ShT;
-    A.ea = (const cpx<R>*)t.ea;
+static void fill_hp(const cr_ctx* c, hp_args<R>& A) {
     A.bonds = c->d_bonds;
     A.N = c->N;
     A.Lx = c->Lx;
@@ -284,9 +345,37 @@ static cr_status launch_hprime(cr_ctx* c, hp_args<R>& A) {
     A.Mp = c->Mp;
     A.Nb = c->Nb;
     A.J = (R)c->J;
-    const size_t sm = hprime_smem<R>(c);
-    CR_LAUNCH(c, CR_KERNEL_TARGET, hprime_kernel<R><<<(A.B + 3) / 4, 128, sm, c->stream>>>(A));
+}
+
+// params: the state H' is applied to; E0, a, Wp of H'
+static cr_status launch_hprime(cr_ctx* c, hp_args<double>& A, const void* params, double E0, double a,
+                               double Wp) {
+    cr_status s = A.want_E ? build_tables(c, params, 1) : CR_OK;
+    if (s != CR_OK) return s;
+    const cr_tables& t = c->tab[1];
+    A.ChT = (const cpx<double>*)t.ChT;
+    A.ShT = (const cpx<double>*)t.ShT;
+    A.ea = (const cpx<double>*)t.ea;
+    fill_hp(c, A);
+    A.E0 = E0;
+    A.a = a;
+    A.Wp = Wp;
+    const size_t sm = hprime_smem<double>(c);
+    CR_LAUNCH(c, CR_KERNEL_TARGET, hprime_kernel<double><<<(A.B + 3) / 4, 128, sm, c->stream>>>(A));
     return cr_check_launch(c, "hprime_kernel");
+}
+
+static cr_status launch_hprime(cr_ctx* c, hp_args<float>& A, const void* params, double E0, double a,
+                               double Wp) {
+    fill_hp(c, A);
+    xsum_out* xo = (xsum_out*)c->xout;
+    if (A.want_E) {
+        cr_status s = launch_xsum(c, params, A.spins, A.th_prev, A.B, A.pr.on, A.pr.qx, A.pr.qy, xo);
+        if (s != CR_OK) return s;
+    }
+    CR_LAUNCH(c, CR_K_OTHER, hfinish_kernel<<<(A.B + 127) / 128, 128, 3 * A.N * sizeof(cpx<float>), c->stream>>>(
+                                 A, E0, a, Wp, xo));
+    return cr_check_launch(c, "hfinish_kernel");
 }
 
 static probe_desc pd(const cr_state* s) { return probe_desc{s->probe != 0, s->qx, s->qy}; }
@@ -294,10 +383,8 @@ static probe_desc pd(const cr_state* s) { return probe_desc{s->probe != 0, s->qx
 template <typename R>
 static cr_status target_t(cr_ctx* c, const cr_target* tg, const int8_t* spins, const void* lpn,
                           int B, void* R_out, double* mean_out) {
-    cr_status s = build_tables(c, tg->prev.params, 1);
-    if (s != CR_OK) return s;
     cpx<R>* lp = (cpx<R>*)c->lp_tmp;
-    s = launch_logpsi(c, tg->prev.params, spins, B, c->theta_tmp, lp);
+    cr_status s = launch_logpsi(c, tg->prev.params, spins, B, c->theta_tmp, lp);
     if (s != CR_OK) return s;
     if (tg->n >= 2) {
         s = launch_logpsi(c, tg->prev2.params, spins, B, nullptr, lp + c->max_walkers);
@@ -316,12 +403,9 @@ static cr_status target_t(cr_ctx* c, const cr_target* tg, const int8_t* spins, c
     A.ka = tg->n == 1 ? 1.0 : 2.0;
     A.beta_a = tg->beta_prev;
     A.beta_b = tg->n >= 2 ? tg->beta_prev2 : nullptr;
-    A.E0 = (R)tg->E0;
-    A.a = (R)tg->a;
-    A.Wp = (R)tg->Wp;
     A.B = B;
     A.out1 = (cpx<R>*)R_out;
-    s = launch_hprime<R>(c, A);
+    s = launch_hprime(c, A, tg->prev.params, tg->E0, tg->a, tg->Wp);
     if (s != CR_OK || !mean_out) return s;
     CR_LAUNCH(c, CR_K_OTHER, mean_kernel<R><<<1, 1024, 0, c->stream>>>((const cpx<R>*)R_out, B, mean_out));
     return cr_check_launch(c, "mean_kernel");
@@ -348,13 +432,8 @@ template <typename R>
 static cr_status moment_t(cr_ctx* c, const cr_state* st, const double* beta, double qx, double qy,
                           const int8_t* spins, const void* lpref, int B, const double* hp,
                           void* Bcol, void* HBcol, double* mu_out) {
-    cr_status s;
-    if (HBcol) {
-        s = build_tables(c, st->params, 1);
-        if (s != CR_OK) return s;
-    }
     cpx<R>* lp = (cpx<R>*)c->lp_tmp;
-    s = launch_logpsi(c, st->params, spins, B, HBcol ? c->theta_tmp : nullptr, lp);
+    cr_status s = launch_logpsi(c, st->params, spins, B, HBcol ? c->theta_tmp : nullptr, lp);
     if (s != CR_OK) return s;
     hp_args<R> A = {};
     A.spins = spins;
@@ -368,18 +447,11 @@ static cr_status moment_t(cr_ctx* c, const cr_state* st, const double* beta, dou
     A.ka = 1.0;
     A.beta_a = beta;
     A.beta_b = nullptr;
-    if (hp) {
-        A.E0 = (R)hp[0];
-        A.a = (R)hp[1];
-        A.Wp = (R)hp[2];
-    } else {
-        A.a = R(1);
-    }
     A.B = B;
     A.out1 = (cpx<R>*)HBcol;
     A.out2 = (cpx<R>*)Bcol;
     A.mu_terms = mu_out ? lp + c->max_walkers : nullptr;
-    s = launch_hprime<R>(c, A);
+    s = launch_hprime(c, A, st->params, hp ? hp[0] : 0.0, hp ? hp[1] : 1.0, hp ? hp[2] : 0.0);
     if (s != CR_OK || !mu_out) return s;
     CR_LAUNCH(c, CR_K_OTHER, mean_kernel<R><<<1, 1024, 0, c->stream>>>(lp + c->max_walkers, B, mu_out));
     return cr_check_launch(c, "mean_kernel");
