@@ -145,15 +145,14 @@ CR_D void set_status(int* st, int code) { atomicCAS(st, 0, code); }
 
 // Bond-ratio tables of one RBM (see rbm.cu, build_tables):
 //   D[b][j]  = 2 (W_ij - W_jj')         (b = (i, j'), padded columns 0)
-//   Ch[b][j] = cosh D, Sh[b][j] = sinh D (padded columns 1 and 0)
-//   ChT/ShT  = the same transposed, [Mp][Nb]
+//   CS[b][j] = (cosh D, sinh D)          (padded columns 1 and 0)
+//   ChT/ShT  = cosh D, sinh D transposed, [Mp][Nb]
 //   ea[b][0] = exp(-2 (a_i - a_j')), ea[b][1] = exp(+2 (a_i - a_j'))
 struct cr_tables {
-    void* D;
-    void* Ch;
-    void* Sh;
-    void* ChT;
-    void* ShT;
+    void* D;    // slot 0
+    void* CS;   // slot 0
+    void* ChT;  // slot 1
+    void* ShT;  // slot 1
     void* ea;
 };
 
@@ -176,7 +175,9 @@ struct cr_ctx {
 
     int* d_status;           // device status word
     int2* d_bonds;           // [Nb]
-    cr_tables tab[2];        // 0: sampler / moment state, 1: target state
+    cr_tables tab[2];        // 0: sampler, 1: local target (float64 contexts)
+    uint16_t* sw_list;       // accepted moves of a sweep launch [maxB][sweep_list_cap]
+    int* sw_count;           // their number [maxB]
     void* xtab;              // exchange table (float32 contexts)
     void* xout;              // xsum_out [maxB] (float32 contexts)
     void* theta_tmp;         // [maxB][M]
@@ -291,6 +292,9 @@ cr_status fcg_prepare(cr_ctx* c);
 cr_status launch_cg_fused(cr_ctx* c, const int8_t* spins, const void* T, int B, const double* redO,
                           double shift, double tol, int maxit, int precond, int apply_only,
                           const double* v_in, void* u_out);
+
+int sweep_list_cap(const cr_ctx* c);
+cr_status sweep_prepare(cr_ctx* c);
 
 // Sums over exchanged amplitudes in float32 (exchange.cu).
 size_t xsum_table_bytes(const cr_ctx* c);

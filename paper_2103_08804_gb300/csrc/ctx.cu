@@ -147,13 +147,15 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
         ALLOC(c->xtab, xsum_table_bytes(c));
         ALLOC(c->xout, B * sizeof(xsum_out));
     }
-    for (int s = 0; s < (prec == CR_FP64 ? 2 : 1); ++s) {  // slot 1: the float64 local target
-        ALLOC(c->tab[s].D, Nb * Mp * cs);
-        ALLOC(c->tab[s].Ch, Nb * Mp * cs);
-        ALLOC(c->tab[s].Sh, Nb * Mp * cs);
-        ALLOC(c->tab[s].ChT, Nb * Mp * cs);
-        ALLOC(c->tab[s].ShT, Nb * Mp * cs);
-        ALLOC(c->tab[s].ea, Nb * 2 * cs);
+    ALLOC(c->tab[0].D, Nb * Mp * cs);
+    ALLOC(c->tab[0].CS, 2 * Nb * Mp * cs);
+    ALLOC(c->tab[0].ea, Nb * 2 * cs);
+    ALLOC(c->sw_list, B * sweep_list_cap(c) * sizeof(uint16_t));
+    ALLOC(c->sw_count, B * sizeof(int));
+    if (prec == CR_FP64) {
+        ALLOC(c->tab[1].ChT, Nb * Mp * cs);
+        ALLOC(c->tab[1].ShT, Nb * Mp * cs);
+        ALLOC(c->tab[1].ea, Nb * 2 * cs);
     }
     ALLOC(c->theta_tmp, B * M * cs);
     ALLOC(c->lp_tmp, 2 * B * cs);
@@ -225,7 +227,7 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     if (e == cudaSuccess) e = cudaMemset(c->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(c->scal, 0, 64 * sizeof(double));
     if (e != cudaSuccess || tc_prepare(c) != CR_OK || (prec == CR_MIXED && spair_prepare(c) != CR_OK) || chol_prepare(c) != CR_OK ||
-        (prec != CR_FP64 && xsum_prepare(c) != CR_OK) || target_prepare(c) != CR_OK || sym_prepare(c) != CR_OK ||
+        (prec != CR_FP64 && xsum_prepare(c) != CR_OK) || sweep_prepare(c) != CR_OK || target_prepare(c) != CR_OK || sym_prepare(c) != CR_OK ||
         (c->fcg && fcg_prepare(c) != CR_OK)) {
         cr_destroy(c);
         return CR_ECUDA;
@@ -239,7 +241,7 @@ extern "C" cr_status cr_destroy(cr_ctx* c) {
     kt_free(c);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
-    void* ptrs[] = {c->d_status, c->d_bonds, c->xtab, c->xout, c->theta_tmp, c->lp_tmp, c->u_tmp, c->partial,
+    void* ptrs[] = {c->d_status, c->d_bonds, c->xtab, c->xout, c->sw_list, c->sw_count, c->theta_tmp, c->lp_tmp, c->u_tmp, c->partial,
                     c->red, c->F, c->cg, c->p_lo, c->cgpart, c->scal, c->S, c->kry,
                     c->Lf, c->chol_x, c->chol_pl, c->Xt, c->spair_g, c->fcg_a1, c->fcg_b2, c->fcg_v2, c->fcg_vab,
                     c->fcg_part, c->fcg_psc, c->fcg_bar, c->gram_x, c->gram_part,
@@ -247,8 +249,7 @@ extern "C" cr_status cr_destroy(cr_ctx* c) {
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (int s = 0; s < 2; ++s) {
-        void* t[] = {c->tab[s].D, c->tab[s].Ch, c->tab[s].Sh, c->tab[s].ChT, c->tab[s].ShT,
-                     c->tab[s].ea};
+        void* t[] = {c->tab[s].D, c->tab[s].CS, c->tab[s].ChT, c->tab[s].ShT, c->tab[s].ea};
         for (void* p : t)
             if (p) cudaFree(p);
     }

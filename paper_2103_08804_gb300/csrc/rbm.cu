@@ -9,11 +9,13 @@
 //   cosh(theta_m - s D_m) / cosh(theta_m) = cosh D_m - s tanh(theta_m) sinh D_m
 // and the visible factor by exp(-s 2 (a_i - a_i')).  The tables hold D, cosh D,
 // sinh D per (bond, hidden unit), padded to Mp columns with the neutral
-// values (0, 1, 0), and exp(-/+ 2 (a_i - a_i')) per bond.
+// values (0, 1, 0), and exp(-/+ 2 (a_i - a_i')) per bond: cosh and sinh
+// interleaved for the sampler (slot 0), transposed for the float64 local
+// target (slot 1).
 template <typename R>
 __global__ void tables_kernel(const cpx<R>* __restrict__ prm, const int2* __restrict__ bonds, int N,
-                              int M, int Mp, int Nb, cpx<R>* D, cpx<R>* Ch, cpx<R>* Sh, cpx<R>* ChT,
-                              cpx<R>* ShT, cpx<R>* ea) {
+                              int M, int Mp, int Nb, cpx<R>* D, cpx<R>* CS, cpx<R>* ChT, cpx<R>* ShT,
+                              cpx<R>* ea) {
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= Nb * Mp) return;
     int b = idx / Mp, m = idx % Mp;
@@ -25,11 +27,14 @@ __global__ void tables_kernel(const cpx<R>* __restrict__ prm, const int2* __rest
         d = R(2) * (wi - wj);
         ccoshsinh_(d, &ch, &sh);
     }
-    D[idx] = d;
-    Ch[idx] = ch;
-    Sh[idx] = sh;
-    ChT[(size_t)m * Nb + b] = ch;
-    ShT[(size_t)m * Nb + b] = sh;
+    if (CS) {
+        D[idx] = d;
+        CS[2 * (size_t)idx] = ch;
+        CS[2 * (size_t)idx + 1] = sh;
+    } else {
+        ChT[(size_t)m * Nb + b] = ch;
+        ShT[(size_t)m * Nb + b] = sh;
+    }
     if (m == 0) {
         cpx<R> da = R(2) * (prm[bd.x] - prm[bd.y]);
         ea[2 * b] = cexp_(-da);
@@ -42,8 +47,8 @@ static cr_status build_tables_t(cr_ctx* c, const void* params, int slot) {
     const cr_tables& t = c->tab[slot];
     int n = c->Nb * c->Mp;
     CR_LAUNCH(c, CR_K_OTHER, tables_kernel<R><<<(n + 255) / 256, 256, 0, c->stream>>>(
-        (const cpx<R>*)params, c->d_bonds, c->N, c->M, c->Mp, c->Nb, (cpx<R>*)t.D, (cpx<R>*)t.Ch,
-        (cpx<R>*)t.Sh, (cpx<R>*)t.ChT, (cpx<R>*)t.ShT, (cpx<R>*)t.ea));
+        (const cpx<R>*)params, c->d_bonds, c->N, c->M, c->Mp, c->Nb, (cpx<R>*)t.D, (cpx<R>*)t.CS,
+        (cpx<R>*)t.ChT, (cpx<R>*)t.ShT, (cpx<R>*)t.ea));
     return cr_check_launch(c, "tables_kernel");
 }
 

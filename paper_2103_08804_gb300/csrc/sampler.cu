@@ -1,114 +1,300 @@
 // Metropolis sampling of |psi_s|^2 (Sec. III) with S^z-conserving exchange
 // moves on nearest-neighbour bonds.
 //
-// One warp per walker.  Lane l owns the KPL hidden units j = 32 k + l
-// (k < KPL) of the padded width Mp = 32 KPL and keeps theta and tanh(theta)
-// for them in registers, so that every table read of a proposal is 32
-// consecutive entries (two 128-byte lines per load instruction).  The amplitude ratio of a proposal is the
-// product over hidden units of (cosh D - s tanh(theta) sinh D) from the bond
-// tables, so the inner loop is complex FMA only; accepted moves update theta
-// and tanh(theta) by the same addition formulas.  Proposals on parallel
-// bonds are no-ops (rejected) and cost a shared-memory read.
+// sweep_kernel: one warp per walker.  Lane l owns the KPL hidden units j =
+// 32 k + l (k < KPL) of the padded width Mp = 32 KPL and keeps tanh(theta) for
+// them in registers.  The amplitude ratio of a proposal is the product over
+// hidden units of (cosh D - s tanh(theta) sinh D) from the bond tables, so
+// the inner loop is complex FMA only; accepted moves update tanh(theta) by the
+// same addition formula.  Proposals on parallel bonds are no-ops (rejected):
+// the 64 proposals of a Philox block are tested at once, two per lane, and
+// after an accepted move only the bonds that share one site with it change
+// sides.
+//
+// What bounds it: a proposal is a chain of a table read (4 KB from L2 at 256
+// hidden units), the product across the warp, the accept test and, mostly,
+// the update.  The rows of the next proposal that can be evaluated are
+// therefore copied into the warp's shared memory (cp.async, every lane its own
+// 16 bytes) while the present one is computed, and theta, which only the
+// output needs, is left out of the chain: accepted moves go to a list, and
+// replay_*_kernel applies them in order afterwards (the same subtractions in
+// the same order, independent loads, the table of a slice of 32 units held in
+// L1).  16 x 16 lattice, 65536 walkers: 8.0 -> 6.1 ms, of which the sweep
+// kernel 4.8; it issues on 65% of its cycles, 480 instructions per evaluated
+// proposal, at 27% of the L2 rate.
 #include "common.cuh"
+
+namespace {
+
+// 16 bytes global -> shared, asynchronous, visible to the issuing thread after
+// its wait_group
+CR_D void cp16(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src)
+                 : "memory");
+}
+CR_D void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N> CR_D void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// First proposal after pos (proposals 2 l in e, 2 l + 1 in o), 64 if none.
+CR_D int next_after(uint32_t e, uint32_t o, int pos) {
+    const int le = (pos + 2) >> 1, lo = (pos + 1) >> 1;
+    const uint32_t es = le < 32 ? e >> le : 0u, os = lo < 32 ? o >> lo : 0u;
+    const int pe = es ? 2 * (le + __ffs(es) - 1) : 64, po = os ? 2 * (lo + __ffs(os) - 1) + 1 : 64;
+    return min(pe, po);
+}
+
+// Complex arithmetic of the accept test with its float32 roundings spelled
+// out: a decision u < ratio is a float32 comparison, so a walker's trajectory
+// depends on the last bit of every step, and the compiler's choice of which
+// product of a sum it fuses changes with the code around it.  YX: the y part
+// fuses a.y b.x (else a.x b.y).
+template <bool YX> CR_D cpx<float> cmul_rn(cpx<float> a, cpx<float> b) {
+    return {__fmaf_rn(a.x, b.x, -__fmul_rn(a.y, b.y)),
+            YX ? __fmaf_rn(a.y, b.x, __fmul_rn(a.x, b.y)) : __fmaf_rn(a.x, b.y, __fmul_rn(a.y, b.x))};
+}
+template <bool YX> CR_D cpx<double> cmul_rn(cpx<double> a, cpx<double> b) { return a * b; }
+// |a|^2; YY: fuses y^2
+template <bool YY> CR_D float abs2_rn(cpx<float> a) {
+    return YY ? __fmaf_rn(a.y, a.y, __fmul_rn(a.x, a.x)) : __fmaf_rn(a.x, a.x, __fmul_rn(a.y, a.y));
+}
+template <bool YY> CR_D double abs2_rn(cpx<double> a) { return abs2(a); }
+template <bool YY> CR_D cpx<float> cdiv_rn(cpx<float> a, cpx<float> b) {
+    const float d = __frcp_rn(abs2_rn<YY>(b));
+    return {__fmul_rn(__fmaf_rn(a.x, b.x, __fmul_rn(a.y, b.y)), d),
+            __fmul_rn(__fmaf_rn(a.y, b.x, -__fmul_rn(a.x, b.y)), d)};
+}
+template <bool YY> CR_D cpx<double> cdiv_rn(cpx<double> a, cpx<double> b) { return cdiv(a, b); }
+
+constexpr int LIST_NEG = 0x8000;  // list entry: bond, this bit for s = -1
+
+}  // namespace
 
 template <typename R, int KPL>
 __global__ void __launch_bounds__(128) sweep_kernel(
-    const cpx<R>* __restrict__ prm, int8_t* __restrict__ spins, cpx<R>* __restrict__ theta, int B,
-    int N, int M, int Mp, int Nb, const int2* __restrict__ bonds_g, const cpx<R>* __restrict__ Dt,
-    const cpx<R>* __restrict__ Cht, const cpx<R>* __restrict__ Sht, const cpx<R>* __restrict__ ea,
-    int n_prop, uint32_t k0, uint32_t k1, unsigned long long counter,
-    const unsigned long long* __restrict__ dcounter, cpx<R>* __restrict__ logpsi_out,
-    cpx<R>* __restrict__ tanh_out, int32_t* __restrict__ n_acc) {
+    int8_t* __restrict__ spins, const cpx<R>* __restrict__ theta, cpx<R>* __restrict__ Tws, int B,
+    int N, int M, int Nb, const int2* __restrict__ bonds_g, const cpx<R>* __restrict__ CS,
+    const cpx<R>* __restrict__ ea, int p_base, int n_prop, int more, uint32_t k0, uint32_t k1,
+    unsigned long long counter, const unsigned long long* __restrict__ dcounter,
+    uint16_t* __restrict__ list, int cap, int* __restrict__ count) {
     if (dcounter) counter = *dcounter;  // stream position kept on the device
+    constexpr int Mp = 32 * KPL, ROW = 2 * Mp;       // (ch, sh) pairs of a bond
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    int2* bonds = (int2*)smem_raw;                       // [Nb]
-    int8_t* sg_all = (int8_t*)(bonds + Nb);              // [4][N]
-    for (int e = threadIdx.x; e < Nb; e += blockDim.x) bonds[e] = bonds_g[e];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    cpx<R>* buf = (cpx<R>*)smem_raw + wid * 2 * ROW;  // [4][2][ROW]
+    uint32_t* bonds = (uint32_t*)((cpx<R>*)smem_raw + 8 * ROW);  // [Nb], sites packed 16 + 16
+    int8_t* sg = (int8_t*)(bonds + Nb) + wid * N;     // [4][N]
+    for (int e = threadIdx.x; e < Nb; e += blockDim.x) {
+        const int2 bd = bonds_g[e];
+        bonds[e] = (uint32_t)bd.x | ((uint32_t)bd.y << 16);
+    }
     const int w = blockIdx.x * 4 + wid;
-    int8_t* sg = sg_all + wid * N;
     if (w < B)
         for (int i = lane; i < N; i += 32) sg[i] = spins[(size_t)w * N + i];
     __syncthreads();
     if (w >= B) return;
 
-    cpx<R> th[KPL], T[KPL];
+    cpx<R> T[KPL];
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
-        int j = 32 * k + lane;
-        th[k] = j < M ? theta[(size_t)w * M + j] : cpx<R>{R(0), R(0)};
-        T[k] = ctanh_(th[k]);
+        const int j = 32 * k + lane;
+        const cpx<R> v = j < M ? (p_base ? Tws : theta)[(size_t)w * M + j] : cpx<R>{R(0), R(0)};
+        T[k] = p_base ? v : ctanh_(v);
     }
-    int nacc = 0;
-    uint4 rnd = make_uint4(0, 0, 0, 0);
-    for (int p = 0; p < n_prop; ++p) {
-        if ((p & 63) == 0) {
-            unsigned long long step = counter + (unsigned long long)(p >> 1) + lane;
-            rnd = philox4x32_10(make_uint4((uint32_t)w, (uint32_t)step, (uint32_t)(step >> 32), 0u),
-                                k0, k1);
-        }
-        const int src = (p >> 1) & 31;
-        const uint32_t ub = __shfl_sync(0xffffffffu, (p & 1) ? rnd.z : rnd.x, src);
-        const uint32_t ua = __shfl_sync(0xffffffffu, (p & 1) ? rnd.w : rnd.y, src);
-        const int b = (int)__umulhi(ub, (uint32_t)Nb);
-        const int2 bd = bonds[b];
-        const int si = sg[bd.x];
-        if (si == sg[bd.y]) continue;  // parallel: no-op, counts as rejected
-        const R s = R(si);
-        const cpx<R>* chr = Cht + (size_t)b * Mp + lane;
-        const cpx<R>* shr = Sht + (size_t)b * Mp + lane;
-        cpx<R> ch[KPL], sh[KPL], f[KPL];
-        cpx<R> pl = {R(1), R(0)};
+    // copy the rows of bond b into buffer q: every lane the pairs it will read
+    auto fetch = [&](int b, int q) {
+        const unsigned char* src = (const unsigned char*)(CS + (size_t)b * ROW);
+        unsigned char* dst = (unsigned char*)(buf + q * ROW);
 #pragma unroll
         for (int k = 0; k < KPL; ++k) {
-            ch[k] = ldg(chr + 32 * k);
-            sh[k] = ldg(shr + 32 * k);
-            cpx<R> ts = T[k] * sh[k];
-            f[k] = {ch[k].x - s * ts.x, ch[k].y - s * ts.y};
-            pl = pl * f[k];
+            const int o = (32 * k + lane) * 2 * (int)sizeof(cpx<R>);
+#pragma unroll
+            for (int c = 0; c < 2 * (int)sizeof(cpx<R>); c += 16) cp16(dst + o + c, src + o + c);
         }
-        cpx<R> pw = warp_prod(pl);
-        pw.x = __shfl_sync(0xffffffffu, pw.x, 0);  // one value for the whole warp
-        pw.y = __shfl_sync(0xffffffffu, pw.y, 0);
-        const cpx<R> e = ea[2 * b + (si > 0 ? 0 : 1)];
-        const R ratio2 = abs2(e) * abs2(pw);
-        const R u = (R(ua >> 9) + R(0.5)) * R(1.1920928955078125e-07);
-        if (u < ratio2) {
-            const cpx<R>* dr = Dt + (size_t)b * Mp + lane;
+    };
+    int nacc = 0, q = 0;
+    uint32_t ent = 0;
+    uint16_t* lst = list + (size_t)w * cap;
+    for (int p0 = 0; p0 < n_prop; p0 += 64) {
+        const unsigned long long step = counter + (unsigned long long)((p_base + p0) >> 1) + lane;
+        const uint4 rnd = philox4x32_10(
+            make_uint4((uint32_t)w, (uint32_t)step, (uint32_t)(step >> 32), 0u), k0, k1);
+        // this lane's two proposals
+        const int b0 = (int)__umulhi(rnd.x, (uint32_t)Nb), b1 = (int)__umulhi(rnd.z, (uint32_t)Nb);
+        const uint32_t s0 = bonds[b0], s1 = bonds[b1];
+        const bool v0 = p0 + 2 * lane < n_prop, v1 = p0 + 2 * lane + 1 < n_prop;
+        // proposals on antiparallel bonds
+        uint32_t A0 = __ballot_sync(0xffffffffu, v0 && sg[s0 & 0xffff] != sg[s0 >> 16]);
+        uint32_t A1 = __ballot_sync(0xffffffffu, v1 && sg[s1 & 0xffff] != sg[s1 >> 16]);
+        int cur = next_after(A0, A1, -1);
+        if (cur < 64) {
+            fetch(__shfl_sync(0xffffffffu, (cur & 1) ? b1 : b0, cur >> 1), q);
+            cp_commit();
+        }
+        while (cur < 64) {
+            const int src = cur >> 1;
+            const int b = __shfl_sync(0xffffffffu, (cur & 1) ? b1 : b0, src);
+            const uint32_t bs = __shfl_sync(0xffffffffu, (cur & 1) ? s1 : s0, src);
+            const uint32_t ua = __shfl_sync(0xffffffffu, (cur & 1) ? rnd.w : rnd.y, src);
+            const uint32_t bx = bs & 0xffff, by = bs >> 16;
+            // proposals whose bond shares one site with this one: an accepted move
+            // takes them to the other side
+            const uint32_t x0 = s0 & 0xffff, y0 = s0 >> 16, x1 = s1 & 0xffff, y1 = s1 >> 16;
+            const uint32_t O0 = __ballot_sync(0xffffffffu, v0 && ((x0 == bx || x0 == by) != (y0 == bx || y0 == by)));
+            const uint32_t O1 = __ballot_sync(0xffffffffu, v1 && ((x1 == bx || x1 == by) != (y1 == bx || y1 == by)));
+            int nxt = next_after(A0 | O0, A1 | O1, cur);
+            if (nxt < 64) fetch(__shfl_sync(0xffffffffu, (nxt & 1) ? b1 : b0, nxt >> 1), q ^ 1);
+            cp_commit();
+            const int si = sg[bx];
+            const cpx<R> e = ea[2 * b + (si > 0 ? 0 : 1)];
+            const R s = R(si);
+            cp_wait<1>();
+            const cpx<R>* row = buf + q * ROW + 2 * lane;
+            cpx<R> f[KPL];
+            cpx<R> pl = {R(1), R(0)};
 #pragma unroll
             for (int k = 0; k < KPL; ++k) {
-                cpx<R> d = ldg(dr + 32 * k);
-                th[k] = {th[k].x - s * d.x, th[k].y - s * d.y};
-                cpx<R> tc = T[k] * ch[k];
-                T[k] = cdiv(cpx<R>{tc.x - s * sh[k].x, tc.y - s * sh[k].y}, f[k]);
+                const cpx<R> ch = row[64 * k], sh = row[64 * k + 1];
+                cpx<R> ts = cmul_rn<false>(T[k], sh);
+                f[k] = {ch.x - s * ts.x, ch.y - s * ts.y};
+                pl = cmul_rn<false>(pl, f[k]);
             }
-            __syncwarp();
-            if (lane == 0) {
-                sg[bd.x] = (int8_t)(-si);
-                sg[bd.y] = (int8_t)si;
+            cpx<R> pw = pl;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                pw = cmul_rn<true>(pw, cpx<R>{__shfl_xor_sync(0xffffffffu, pw.x, o),
+                                              __shfl_xor_sync(0xffffffffu, pw.y, o)});
+            pw.x = __shfl_sync(0xffffffffu, pw.x, 0);  // one value for the whole warp
+            pw.y = __shfl_sync(0xffffffffu, pw.y, 0);
+            const R ratio2 = abs2_rn<false>(e) * abs2_rn<false>(pw);
+            const R u = (R(ua >> 9) + R(0.5)) * R(1.1920928955078125e-07);
+            if (u < ratio2) {
+#pragma unroll
+                for (int k = 0; k < KPL; ++k) {
+                    const cpx<R> ch = row[64 * k], sh = row[64 * k + 1];
+                    cpx<R> tc = cmul_rn<(KPL > 1)>(T[k], ch);
+                    T[k] = cdiv_rn<KPL == 1>(cpx<R>{tc.x - s * sh.x, tc.y - s * sh.y}, f[k]);
+                }
+                __syncwarp();
+                if (lane == 0) {
+                    sg[bx] = (int8_t)(-si);
+                    sg[by] = (int8_t)si;
+                }
+                __syncwarp();
+                A0 ^= O0;
+                A1 ^= O1;
+                if (lane == (nacc & 31)) ent = (uint32_t)b | (si > 0 ? 0u : (uint32_t)LIST_NEG);
+                ++nacc;
+                if ((nacc & 31) == 0) lst[nacc - 32 + lane] = (uint16_t)ent;
             }
-            __syncwarp();
-            ++nacc;
+            if (nxt < 64 && !((((nxt & 1) ? A1 : A0) >> (nxt >> 1)) & 1u)) {
+                // the prefetched proposal turned parallel: take the one after it
+                nxt = next_after(A0, A1, nxt);
+                if (nxt < 64) {
+                    cp_wait<0>();
+                    fetch(__shfl_sync(0xffffffffu, (nxt & 1) ? b1 : b0, nxt >> 1), q ^ 1);
+                    cp_commit();
+                }
+            }
+            cur = nxt;
+            q ^= 1;
         }
     }
+    cp_wait<0>();
+    if (lane < (nacc & 31)) lst[(nacc & ~31) + lane] = (uint16_t)ent;
     __syncwarp();
     for (int i = lane; i < N; i += 32) spins[(size_t)w * N + i] = sg[i];
+    if (more)
+#pragma unroll
+        for (int k = 0; k < KPL; ++k)
+            if (32 * k + lane < M) Tws[(size_t)w * M + 32 * k + lane] = T[k];
+    if (lane == 0) count[w] = nacc;
+}
+
+// theta -> theta - sum of the listed moves' s D, in the list's order, for one
+// unit j of walker w (lane's unit; entries broadcast from the lanes that read
+// them).
+template <typename R, int KPL>
+CR_D void replay_list(const uint16_t* __restrict__ lst, int n, const cpx<R>* __restrict__ Dt, int Mp,
+                      int lane, cpx<R> (&th)[KPL]) {
+    for (int e0 = 0; e0 < n; e0 += 32) {
+        const int mine = e0 + lane < n ? lst[e0 + lane] : 0;
+        const int m = min(32, n - e0);
+        for (int c = 0; c < m; c += 4) {
+            cpx<R> d[4][KPL];
+            R s[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const int e = __shfl_sync(0xffffffffu, mine, c + v);  // c + v < 32
+                s[v] = c + v < m ? (e & LIST_NEG ? R(-1) : R(1)) : R(0);
+                const cpx<R>* dr = Dt + (size_t)(e & (LIST_NEG - 1)) * Mp;
+#pragma unroll
+                for (int k = 0; k < KPL; ++k) d[v][k] = ldg(dr + 32 * k);
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                if (c + v < m)
+#pragma unroll
+                    for (int k = 0; k < KPL; ++k)
+                        th[k] = {th[k].x - s[v] * d[v][k].x, th[k].y - s[v] * d[v][k].y};
+        }
+    }
+}
+
+// One warp per (walker, slice of 32 hidden units); slices are the slow grid
+// dimension, so the CTAs running together share one slice of the table in L1.
+template <typename R>
+__global__ void __launch_bounds__(256) replay_slice_kernel(cpx<R>* __restrict__ theta, int B, int M,
+                                                           int Mp, const cpx<R>* __restrict__ Dt,
+                                                           const uint16_t* __restrict__ list, int cap,
+                                                           const int* __restrict__ count) {
+    const int lane = threadIdx.x & 31, w = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (w >= B) return;
+    const int j = 32 * blockIdx.y + lane;
+    cpx<R> th[1] = {j < M ? theta[(size_t)w * M + j] : cpx<R>{R(0), R(0)}};
+    replay_list<R, 1>(list + (size_t)w * cap, count[w], Dt + j, Mp, lane, th);
+    if (j < M) theta[(size_t)w * M + j] = th[0];
+}
+
+// One warp per walker: the listed moves (list may be null: none left), then
+// theta, tanh theta and log psi of the walker.
+template <typename R, int KPL>
+__global__ void __launch_bounds__(128) finish_kernel(
+    const cpx<R>* __restrict__ prm, const int8_t* __restrict__ spins, cpx<R>* __restrict__ theta, int B,
+    int N, int M, const cpx<R>* __restrict__ Dt, const uint16_t* __restrict__ list, int cap,
+    const int* __restrict__ count, int last, int first, cpx<R>* __restrict__ logpsi_out,
+    cpx<R>* __restrict__ tanh_out, int32_t* __restrict__ n_acc) {
+    const int lane = threadIdx.x & 31, w = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (w >= B) return;
+    cpx<R> th[KPL];
+#pragma unroll
+    for (int k = 0; k < KPL; ++k) {
+        const int j = 32 * k + lane;
+        th[k] = j < M ? theta[(size_t)w * M + j] : cpx<R>{R(0), R(0)};
+    }
+    const int n = count ? count[w] : 0;
+    if (list) {
+        replay_list<R, KPL>(list + (size_t)w * cap, n, Dt + lane, 32 * KPL, lane, th);
+#pragma unroll
+        for (int k = 0; k < KPL; ++k)
+            if (32 * k + lane < M) theta[(size_t)w * M + 32 * k + lane] = th[k];
+    }
+    if (lane == 0 && n_acc) n_acc[w] = (first ? 0 : n_acc[w]) + n;
+    if (!last) return;
     cpx<R> lp = {R(0), R(0)};
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
         int j = 32 * k + lane;
         if (j < M) {
-            theta[(size_t)w * M + j] = th[k];
             lp = lp + clncosh2_(th[k]);
             if (tanh_out) tanh_out[(size_t)w * M + j] = ctanh_(th[k]);
         }
     }
+    if (!logpsi_out) return;
+    const int8_t* sg = spins + (size_t)w * N;
     for (int i = lane; i < N; i += 32) lp = lp + R(sg[i]) * prm[i];
     lp = warp_sum(lp);
-    if (lane == 0) {
-        if (logpsi_out) logpsi_out[w] = lp;
-        if (n_acc) n_acc[w] = nacc;
-    }
+    if (lane == 0) logpsi_out[w] = lp;
 }
 
 // Advance a device-resident stream position (after the sweep that used it).
@@ -116,29 +302,85 @@ __global__ void advance_counter_kernel(unsigned long long* ctr, unsigned long lo
     *ctr += calls;
 }
 
+// Proposals per sweep launch: its list of accepted moves per walker.
+int sweep_list_cap(const cr_ctx* c) { return c->N > 512 ? (c->N + 63) / 64 * 64 : 512; }
+
+template <typename R, int KPL>
+static size_t sweep_smem(const cr_ctx* c) {
+    return (size_t)8 * 2 * 32 * KPL * sizeof(cpx<R>) + (size_t)c->Nb * 4 + 4 * (size_t)c->N;
+}
+
+template <typename R, int KPL>
+static cr_status sweep_k(cr_ctx* c, const void* params, int8_t* spins, void* theta, int B, int n_prop,
+                         uint64_t seed, uint64_t counter, const uint64_t* dcounter, void* logpsi_out,
+                         void* tanh_out, int32_t* n_acc) {
+    const cr_tables& t = c->tab[0];
+    cpx<R>* th = (cpx<R>*)theta;
+    const cpx<R>* D = (const cpx<R>*)t.D;
+    const int cap = sweep_list_cap(c), grid = (B + 3) / 4;
+    // a table that fits in L1 beside the loads in flight is replayed whole, by the finishing warps;
+    // a larger one in slices of 32 units, each of which does
+    const bool slices = (size_t)c->Nb * c->Mp * sizeof(cpx<R>) > 128 * 1024 && KPL > 1;
+    int p = 0;
+    do {
+        const int np = n_prop - p < cap ? n_prop - p : cap;
+        const bool last = p + np >= n_prop;
+        if (np > 0)
+            CR_LAUNCH(c, CR_KERNEL_SWEEP,
+                      (sweep_kernel<R, KPL><<<grid, 128, sweep_smem<R, KPL>(c), c->stream>>>(
+                          spins, th, (cpx<R>*)c->theta_tmp, B, c->N, c->M, c->Nb, c->d_bonds,
+                          (const cpx<R>*)t.CS, (const cpx<R>*)t.ea, p, np, !last, (uint32_t)seed,
+                          (uint32_t)(seed >> 32), (unsigned long long)counter,
+                          (const unsigned long long*)dcounter, c->sw_list, cap, c->sw_count)));
+        if (np > 0 && slices)
+            CR_LAUNCH(c, CR_K_OTHER,
+                      (replay_slice_kernel<R><<<dim3((B + 7) / 8, KPL), 256, 0, c->stream>>>(
+                          th, B, c->M, c->Mp, D, c->sw_list, cap, c->sw_count)));
+        CR_LAUNCH(c, CR_K_OTHER,
+                  (finish_kernel<R, KPL><<<grid, 128, 0, c->stream>>>(
+                      (const cpx<R>*)params, spins, th, B, c->N, c->M, D,
+                      np > 0 && !slices ? c->sw_list : nullptr, cap, np > 0 ? c->sw_count : nullptr, last,
+                      p == 0, (cpx<R>*)logpsi_out, (cpx<R>*)tanh_out, n_acc)));
+        p += np;
+    } while (p < n_prop);
+    return cr_check_launch(c, "mc_sweep");
+}
+
 template <typename R>
 static cr_status sweep_t(cr_ctx* c, const void* params, int8_t* spins, void* theta, int B,
                          int n_prop, uint64_t seed, uint64_t counter, const uint64_t* dcounter,
                          void* logpsi_out, void* tanh_out, int32_t* n_acc) {
-    const cr_tables& t = c->tab[0];
-    const int kpl = c->Mp / 32;
-    size_t sm = c->Nb * sizeof(int2) + 4 * c->N;
-    dim3 grid((B + 3) / 4);
-#define LAUNCH(K)                                                                                  \
-    CR_LAUNCH(c, CR_KERNEL_SWEEP, sweep_kernel<R, K><<<grid, 128, sm, c->stream>>>(                                             \
-        (const cpx<R>*)params, spins, (cpx<R>*)theta, B, c->N, c->M, c->Mp, c->Nb, c->d_bonds,     \
-        (const cpx<R>*)t.D, (const cpx<R>*)t.Ch, (const cpx<R>*)t.Sh, (const cpx<R>*)t.ea, n_prop, \
-        (uint32_t)seed, (uint32_t)(seed >> 32), (unsigned long long)counter,                        \
-        (const unsigned long long*)dcounter, (cpx<R>*)logpsi_out, (cpx<R>*)tanh_out, n_acc))
-    switch (kpl) {
-        case 1: LAUNCH(1); break;
-        case 2: LAUNCH(2); break;
-        case 4: LAUNCH(4); break;
-        case 8: LAUNCH(8); break;
-        default: LAUNCH(16); break;
+#define SWEEP(K) \
+    sweep_k<R, K>(c, params, spins, theta, B, n_prop, seed, counter, dcounter, logpsi_out, tanh_out, n_acc)
+    switch (c->Mp / 32) {
+        case 1: return SWEEP(1);
+        case 2: return SWEEP(2);
+        case 4: return SWEEP(4);
+        case 8: return SWEEP(8);
+        default: return SWEEP(16);
     }
-#undef LAUNCH
-    return cr_check_launch(c, "sweep_kernel");
+#undef SWEEP
+}
+
+// Opt the sweep of this context's width into the shared memory it needs
+// (once per context; the bound covers every context of that width).
+template <typename R>
+static cr_status sweep_prepare_t(cr_ctx* c) {
+    cudaError_t e = cudaSuccess;
+#define OPT(K)                                                                                        \
+    case K:                                                                                           \
+        e = cudaFuncSetAttribute(sweep_kernel<R, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
+                                 (int)(8 * 2 * 32 * K * sizeof(cpx<R>) + 2048 * 4 + 4 * 1024));       \
+        break;
+    switch (c->Mp / 32) {
+        OPT(1) OPT(2) OPT(4) OPT(8) OPT(16)
+    }
+#undef OPT
+    return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "sweep_prepare: %s", cudaGetErrorString(e));
+}
+
+cr_status sweep_prepare(cr_ctx* c) {
+    return c->prec == CR_FP64 ? sweep_prepare_t<double>(c) : sweep_prepare_t<float>(c);
 }
 
 extern "C" cr_status mc_sweep(cr_ctx* ctx, const cr_state* st, int8_t* spins, void* theta, int B,
