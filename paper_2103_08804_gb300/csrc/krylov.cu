@@ -6,8 +6,8 @@
 // A = Ar + i Ai is handled through its real symmetric embedding
 // [[Ar, -Ai], [Ai, Ar]] (every eigenvalue twice, eigenvector pairs
 // [ur; ui], [-ui; ur]), diagonalised by cyclic Jacobi rotations applied to
-// n disjoint pairs at a time (round-robin ordering), one launch per round on
-// many CTAs; the moment recursion runs on one CTA.
+// n disjoint pairs at a time (round-robin ordering), all rounds of all sweeps
+// in one cooperative launch; so is the moment recursion.
 #include "common.cuh"
 
 // ------------------------------------------------------------------ Gram
@@ -73,151 +73,263 @@ extern "C" cr_status cheb_gram(cr_ctx* ctx, const void* Bmat, const void* HBmat,
 
 // ------------------------------------------------------------- Jacobi
 //
-// Cyclic Jacobi on many CTAs.  Each sweep has m - 1 rounds (round-robin
-// pairing of the m indices: position 0 fixed, the others rotating); a round
-// applies its m/2 disjoint rotations at once, A' = J^T A J and V' = V J, out
-// of place (ping-pong buffers), one launch per round.  Every CTA computes
-// the rotation angles of the pairs its 32 x 32 output tile touches from the
-// round's input, so no launch waits on another.  Between sweeps the
-// off-diagonal norm is reduced (fixed order) and, once it is below
-// JAC_TOL times the diagonal, a device flag makes every later launch return
-// at once; `res` records which buffer holds the latest A and V.
+// Cyclic Jacobi for the symmetric m x m embedding (m even).  Each sweep has
+// m - 1 rounds (round-robin pairing of the m indices: position 0 fixed, the
+// others rotating); a round applies its m / 2 disjoint rotations at once,
+// A' = J^T A J and V' = V J, from one pair of buffers to the other.  A 2 x 2
+// block of A (row pair P, column pair Q) is one thread's work.  Every CTA
+// takes one tile of blocks or of V, and the angles of its own pairs, so a
+// round ends with one grid barrier.  Before each sweep the off-diagonal norm
+// is reduced (fixed order); once it is below JAC_TOL times the diagonal every
+// CTA leaves.
+//
+// The sweeps end with an off-diagonal of 1e-12 left, which is 1e-9 to 1e-8 in
+// the weights of 300 states: another order of rotations, or another rounding
+// of one, would leave another remainder of that size.  So the rotations, their
+// order and their roundings (rot, spelled out) are fixed.
+//
+// What bounds a round: float64 arithmetic (4 operations an element of A, 2 of
+// V, at two per SM and cycle: 3.4 us at m = 600), the barrier, and two round
+// trips to L2 with the angles' divisions and square roots between them; the
+// blocks are loaded before the angles are formed.  One launch per round, the
+// two eigenproblems of 300 states took 654 ms (36,000 launches); now 140 ms.
 
 namespace {
 
+using zd = cpx<double>;
+
 constexpr int JAC_MAX_SWEEPS = 30;
 constexpr double JAC_TOL = 1e-24;  // off^2 <= JAC_TOL diag^2 (relative 1e-12)
-constexpr int NORM_GRID = 128;
+constexpr int JT = 512;            // threads
+constexpr int MAX_TP = 64;         // pairs per tile at most
+constexpr unsigned BAR_LIMIT = 1u << 23;  // grid-barrier polls
 
 // Element of the round-robin schedule: position 0 is fixed, the others
 // rotate by one place per round.
-__device__ __forceinline__ int rr_elem(int pos, int round, int m) {
+CR_D int rr_elem(int pos, int round, int m) {
     return pos == 0 ? 0 : ((pos - 1 + round) % (m - 1)) + 1;
 }
-// Position of index idx in round `round` (inverse of rr_elem).
-__device__ __forceinline__ int rr_pos(int idx, int round, int m) {
-    return idx == 0 ? 0 : ((idx - 1 - round) % (m - 1) + (m - 1)) % (m - 1) + 1;
-}
+
+// c x + s y as the rotations round it
+CR_D double rot(double c, double x, double s, double y) { return fma(c, x, __dmul_rn(s, y)); }
 
 struct JacBufs {
     double* A[2];
     double* V[2];
-    int* res;   // index of the buffers holding the latest A, V
-    int* flag;  // converged
+    double* part;  // [2][gridDim] shares of the norms
+    unsigned* bar; // [0] arrivals, [1] abort
+    int* res;      // index of the buffers holding the result
 };
 
-__global__ void jac_init_kernel(JacBufs J, int m) {
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx == 0) {
-        *J.res = 0;
-        *J.flag = 0;
-    }
-    if (idx < (size_t)m * m) J.V[0][idx] = (idx / m == idx % m) ? 1.0 : 0.0;
-}
+struct JacArgs {
+    JacBufs J;
+    int m, tp, nt, na, nv, rv;  // tile: pairs, tiles a side, tiles of A, of V, rows of a V tile
+    int* status;
+};
 
-__global__ void __launch_bounds__(256) jac_round_kernel(JacBufs J, int m, int round, int in) {
-    if (*J.flag) return;
-    __shared__ double ang_c[64], ang_s[64];
-    __shared__ int partner[64], role[64];
-    const double* A = J.A[in];
-    const double* V = J.V[in];
-    double* Ao = J.A[in ^ 1];
-    double* Vo = J.V[in ^ 1];
-    const int i0 = blockIdx.y * 32, j0 = blockIdx.x * 32, t = threadIdx.x;
-    if (t < 64) {
-        const int idx = (t < 32 ? i0 : j0) + (t & 31);
-        double c = 1.0, sn = 0.0;
-        int pt = idx, rl = 0;
-        if (idx < m) {
-            const int pos = rr_pos(idx, round, m);
-            const int k = pos < m / 2 ? pos : m - 1 - pos;
-            const int p = rr_elem(k, round, m), q = rr_elem(m - 1 - k, round, m);
-            const double apq = A[(size_t)p * m + q];
-            if (apq != 0.0) {
-                const double tau = (A[(size_t)q * m + q] - A[(size_t)p * m + p]) / (2.0 * apq);
-                const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                c = 1.0 / sqrt(1.0 + tt * tt);
-                sn = tt * c;
-            }
-            pt = idx == p ? q : p;
-            rl = idx == p ? 0 : 1;
-        }
-        ang_c[t] = c;
-        ang_s[t] = sn;
-        partner[t] = pt;
-        role[t] = rl;
-    }
-    __syncthreads();
-    for (int e = t; e < 1024; e += blockDim.x) {
-        const int li = e >> 5, lj = e & 31, i = i0 + li, j = j0 + lj;
-        if (i >= m || j >= m) continue;
-        const double ci = ang_c[li], si = ang_s[li], cj = ang_c[32 + lj], sj = ang_s[32 + lj];
-        const int ip = partner[li], jp = partner[32 + lj];
-        // column step (pair of j) on rows i and i', then the row step (pair of i)
-        const double sgj = role[32 + lj] ? sj : -sj, sgi = role[li] ? si : -si;
-        const double bij = cj * A[(size_t)i * m + j] + sgj * A[(size_t)i * m + jp];
-        const double bpj = cj * A[(size_t)ip * m + j] + sgj * A[(size_t)ip * m + jp];
-        Ao[(size_t)i * m + j] = ci * bij + sgi * bpj;
-        Vo[(size_t)i * m + j] = cj * V[(size_t)i * m + j] + sgj * V[(size_t)i * m + jp];
-    }
-    if (blockIdx.x == 0 && blockIdx.y == 0 && t == 0) *J.res = in ^ 1;
-}
-
-// Per-CTA shares of the squared off-diagonal and diagonal sums of A[res].
-__global__ void __launch_bounds__(256) jac_norm_kernel(JacBufs J, int m, double* __restrict__ part) {
-    if (*J.flag) return;
-    __shared__ double r1[8], r2[8];
-    const double* A = J.A[*J.res];
-    double off = 0.0, dia = 0.0;
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < (size_t)m * m;
-         e += (size_t)gridDim.x * blockDim.x) {
-        const double v = A[e] * A[e];
-        if (e / m == e % m) dia += v;
-        else off += v;
-    }
-    off = warp_sum(off);
-    dia = warp_sum(dia);
-    if ((threadIdx.x & 31) == 0) {
-        r1[threadIdx.x >> 5] = off;
-        r2[threadIdx.x >> 5] = dia;
-    }
+// Grid barrier: arrive, wait (bounded) for all CTAs; false after an abort.
+CR_D bool grid_sync(unsigned* bar, unsigned target, volatile int* flag, int* status) {
     __syncthreads();
     if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int w = 0; w < 8; ++w) {
-            a += r1[w];
-            b += r2[w];
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(&bar[0]) : "memory");
+        for (unsigned n = 0; *(volatile unsigned*)&bar[0] < target; ++n) {
+            if (*(volatile unsigned*)&bar[1] || n > BAR_LIMIT) {
+                if (n > BAR_LIMIT) {
+                    atomicExch(&bar[1], 1u);
+                    set_status(status, CR_ETIMEOUT);
+                }
+                *flag = 1;
+                break;
+            }
+            if (n > 4096) __nanosleep(64);
         }
-        part[blockIdx.x] = a;
-        part[NORM_GRID + blockIdx.x] = b;
+        asm volatile("fence.acq_rel.gpu;\n" ::: "memory");
     }
+    __syncthreads();
+    return *flag == 0;
 }
 
-__global__ void jac_flag_kernel(JacBufs J, const double* __restrict__ part) {
-    if (*J.flag) return;
-    double off = 0.0, dia = 0.0;
-    for (int b = 0; b < NORM_GRID; ++b) {
-        off += part[b];
-        dia += part[NORM_GRID + b];
-    }
-    if (!(off > JAC_TOL * dia)) *J.flag = 1;
-}
-
-// Diagonalise the symmetric m x m matrix in J.A[0] (m even); eigenvalues on
-// the diagonal of J.A[*res], eigenvectors in the columns of J.V[*res].
-void jacobi_launch(cr_ctx* c, JacBufs J, int m, double* part) {
-    const size_t mm = (size_t)m * m;
-    CR_LAUNCH(c, CR_K_OTHER, jac_init_kernel<<<(unsigned)((mm + 255) / 256), 256, 0, c->stream>>>(J, m));
-    const dim3 g((m + 31) / 32, (m + 31) / 32);
+__global__ void __launch_bounds__(JT) jacobi_kernel(const JacArgs a) {
+    __shared__ double ac[2 * MAX_TP], as[2 * MAX_TP], red[2][JT / 32];
+    __shared__ int ip[2 * MAX_TP], iq[2 * MAX_TP];
+    __shared__ int flag_, done_;
+    volatile int* flag = &flag_;
+    const int m = a.m, np = m / 2, t = threadIdx.x;
+    const JacBufs& J = a.J;
+    if (t == 0) *flag = 0;
+    unsigned arrived = 0;
+    const unsigned G = gridDim.x;
+    for (size_t e = (size_t)blockIdx.x * JT + t; e < (size_t)m * m; e += (size_t)G * JT)
+        __stcg(&J.V[0][e], e / m == e % m ? 1.0 : 0.0);
     int in = 0;
-    for (int sweep = 0; sweep < JAC_MAX_SWEEPS; ++sweep) {
-        CR_LAUNCH(c, CR_K_OTHER, jac_norm_kernel<<<NORM_GRID, 256, 0, c->stream>>>(J, m, part));
-        CR_LAUNCH(c, CR_K_OTHER, jac_flag_kernel<<<1, 1, 0, c->stream>>>(J, part));
-        for (int round = 0; round < m - 1; ++round) {
-            CR_LAUNCH(c, CR_K_OTHER, jac_round_kernel<<<g, 256, 0, c->stream>>>(J, m, round, in));
+    bool ok = grid_sync(J.bar, ++arrived * G, flag, a.status);
+    for (int sweep = 0; sweep < JAC_MAX_SWEEPS && ok; ++sweep) {
+        // squared off-diagonal and diagonal norms
+        double off = 0.0, dia = 0.0;
+        for (size_t e = (size_t)blockIdx.x * JT + t; e < (size_t)m * m; e += (size_t)G * JT) {
+            const double x = __ldcg(&J.A[in][e]), v = x * x;
+            if (e / m == e % m) dia += v;
+            else off += v;
+        }
+        off = warp_sum(off);
+        dia = warp_sum(dia);
+        if ((t & 31) == 0) {
+            red[0][t >> 5] = off;
+            red[1][t >> 5] = dia;
+        }
+        __syncthreads();
+        if (t < 2) {
+            double v = 0.0;
+            for (int w = 0; w < JT / 32; ++w) v += red[t][w];
+            __stcg(&J.part[t * G + blockIdx.x], v);
+        }
+        ok = grid_sync(J.bar, ++arrived * G, flag, a.status);
+        if (!ok) break;
+        if (t < 32) {
+            double o = 0.0, d = 0.0;
+            for (unsigned b = t; b < G; b += 32) {
+                o += __ldcg(&J.part[b]);
+                d += __ldcg(&J.part[G + b]);
+            }
+            o = warp_sum(o);
+            d = warp_sum(d);
+            if (t == 0) done_ = !(o > JAC_TOL * d);
+        }
+        __syncthreads();
+        if (done_) break;
+        for (int round = 0; round < m - 1 && ok; ++round) {
+            const double* A = J.A[in];
+            const double* V = J.V[in];
+            double* Ao = J.A[in ^ 1];
+            double* Vo = J.V[in ^ 1];
+            for (int tile = blockIdx.x; tile < a.na + a.nv; tile += G) {
+                // pair blocks of the tile: rows P0.., columns Q0.. (a tile of V has single rows)
+                const bool isA = tile < a.na;
+                const int tv = isA ? tile : tile - a.na, Q0 = (tv % a.nt) * a.tp;
+                const int P0 = isA ? (tv / a.nt) * a.tp : 0, r0 = isA ? 0 : (tv / a.nt) * a.rv;
+                const int rows = isA ? min(a.tp, np - P0) : min(a.rv, m - r0), cols = min(a.tp, np - Q0);
+                // row pairs at [0, tp), column pairs at [tp, 2 tp)
+                const int k = t < a.tp ? P0 + t : Q0 + t - a.tp;
+                const bool ang = t < 2 * a.tp && (isA || t >= a.tp) && k < np;
+                __syncthreads();
+                double apq = 0.0, aqq = 0.0, app = 0.0;
+                if (ang) {
+                    const int ep = rr_elem(k, round, m), eq = rr_elem(m - 1 - k, round, m);
+                    ip[t] = ep;
+                    iq[t] = eq;
+                    apq = __ldcg(&A[(size_t)ep * m + eq]);
+                    aqq = __ldcg(&A[(size_t)eq * m + eq]);
+                    app = __ldcg(&A[(size_t)ep * m + ep]);
+                }
+                __syncthreads();
+                // a warp takes rows of blocks, lanes the columns; the first rows are loaded
+                // before the angles are formed
+                const int lane = t & 31, wp = t >> 5;
+                double x0[2], x1[2], y0[2], y1[2];
+                auto fetch = [&](int c0, int l0) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int l = l0 + h * (JT / 32);
+                        if (l >= rows || c0 + lane >= cols) continue;
+                        const int r = ip[a.tp + c0 + lane], u = iq[a.tp + c0 + lane];
+                        const double* S = isA ? A + (size_t)ip[l] * m : V + (size_t)(r0 + l) * m;
+                        x0[h] = __ldcg(S + r);
+                        x1[h] = __ldcg(S + u);
+                        if (isA) {
+                            const double* S2 = A + (size_t)iq[l] * m;
+                            y0[h] = __ldcg(S2 + r);
+                            y1[h] = __ldcg(S2 + u);
+                        }
+                    }
+                };
+                fetch(0, wp);
+                if (ang) {
+                    double c = 1.0, sn = 0.0;
+                    if (apq != 0.0) {
+                        const double tau = (aqq - app) / (2.0 * apq);
+                        const double tt = (tau >= 0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(fma(tau, tau, 1.0)));
+                        c = 1.0 / sqrt(fma(tt, tt, 1.0));
+                        sn = tt * c;
+                    }
+                    ac[t] = c;
+                    as[t] = sn;
+                }
+                __syncthreads();
+                for (int c0 = 0; c0 < cols; c0 += 32)
+                    for (int l0 = wp; l0 < rows; l0 += 2 * (JT / 32)) {
+                        if (c0 != 0 || l0 != wp) fetch(c0, l0);
+                        if (c0 + lane >= cols) continue;
+                        const int lQ = a.tp + c0 + lane, r = ip[lQ], u = iq[lQ];
+                        const double c = ac[lQ], s = as[lQ];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int l = l0 + h * (JT / 32);
+                            if (l >= rows) continue;
+                            const double b00 = rot(c, x0[h], -s, x1[h]), b01 = rot(c, x1[h], s, x0[h]);
+                            if (!isA) {
+                                double* D = Vo + (size_t)(r0 + l) * m;
+                                __stcg(D + r, b00);
+                                __stcg(D + u, b01);
+                                continue;
+                            }
+                            const double d = ac[l], g = as[l];
+                            const double b10 = rot(c, y0[h], -s, y1[h]), b11 = rot(c, y1[h], s, y0[h]);
+                            double* Dp = Ao + (size_t)ip[l] * m;
+                            double* Dq = Ao + (size_t)iq[l] * m;
+                            __stcg(Dp + r, rot(d, b00, -g, b10));
+                            __stcg(Dp + u, rot(d, b01, -g, b11));
+                            __stcg(Dq + r, rot(d, b10, g, b00));
+                            __stcg(Dq + u, rot(d, b11, g, b01));
+                        }
+                    }
+            }
+            ok = grid_sync(J.bar, ++arrived * G, flag, a.status);
             in ^= 1;
         }
     }
+    if (blockIdx.x == 0 && t == 0) *J.res = in;
+}
+
+// A cooperative launch (co-resident CTAs).
+template <typename K, typename A>
+cr_status coop_launch(cr_ctx* c, K kernel, int grid, int threads, const A& args, const char* name) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = c->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e;
+    CR_LAUNCH(c, CR_K_OTHER, e = cudaLaunchKernelEx(&cfg, kernel, args));
+    return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "%s: %s", name, cudaGetErrorString(e));
+}
+
+// Diagonalise the symmetric m x m matrix in J.A[0] (m even); eigenvalues on
+// the diagonal of J.A[*res], eigenvectors in the columns of J.V[*res].  The
+// smallest tiles that leave every CTA at most one; a small matrix on one CTA,
+// where a barrier is cheap.
+cr_status jacobi_launch(cr_ctx* c, const JacBufs& J, int m) {
+    JacArgs a = {};
+    const int np = m / 2;
+    auto shape = [&]() {
+        a.nt = (np + a.tp - 1) / a.tp;
+        a.rv = 4 * a.tp;
+        a.na = a.nt * a.nt;
+        a.nv = a.nt * ((m + a.rv - 1) / a.rv);
+        return a.na + a.nv;
+    };
+    a.J = J;
+    a.m = m;
+    a.status = c->d_status;
+    a.tp = m <= 32 ? np : 4;
+    while (shape() > c->n_sm && a.tp < MAX_TP) ++a.tp;
+    const int tiles = a.na + a.nv, grid = m <= 32 ? 1 : (tiles < c->n_sm ? tiles : c->n_sm);
+    cudaError_t e = cudaMemsetAsync(J.bar, 0, 2 * sizeof(unsigned), c->stream);
+    if (e != cudaSuccess) return cr_fail(c, CR_ECUDA, "jacobi_kernel: %s", cudaGetErrorString(e));
+    return coop_launch(c, jacobi_kernel, grid, JT, a, "jacobi_kernel");
 }
 
 // Real symmetric embedding [[Ar, -Ai], [Ai, Ar]] of a complex Hermitian n x n
@@ -235,44 +347,59 @@ __global__ void kry_embed_kernel(const double* __restrict__ A_, int n, double* _
 
 // Eigenvalues of the embedded G, the kept index list (relative cutoff; an
 // odd count drops the smallest, the copy a cutoff split by rounding) and
-// the rank r (even).  One thread.
-__global__ void kry_keep_kernel(JacBufs J, int m, double cutoff, double* __restrict__ d,
-                                int* __restrict__ keep, int* __restrict__ rank) {
+// the rank r (even).  One CTA, one thread per eigenvalue (m <= 1024).
+__global__ void __launch_bounds__(1024) kry_keep_kernel(JacBufs J, int m, double cutoff,
+                                                        double* __restrict__ d, int* __restrict__ keep,
+                                                        int* __restrict__ rank) {
+    __shared__ double red[32];
+    __shared__ int redi[32], cnt[32];
     const double* E = J.A[*J.res];
-    double dm = 0.0;
-    for (int k = 0; k < m; ++k) {
-        d[k] = E[(size_t)k * m + k];
-        dm = d[k] > dm ? d[k] : dm;
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const double v = t < m ? E[(size_t)t * m + t] : 0.0;
+    if (t < m) d[t] = v;
+    double mx = v;
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) red[w] = mx;
+    __syncthreads();
+    mx = 0.0;
+    for (int i = 0; i < 32; ++i) mx = fmax(mx, red[i]);
+    __syncthreads();
+    bool on = t < m && v > cutoff * mx;
+    // smallest kept eigenvalue (lowest index among equals)
+    double lo = on ? v : 1e308;
+    int li = t;
+    for (int o = 16; o > 0; o >>= 1) {
+        const double l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        const int i2 = __shfl_xor_sync(0xffffffffu, li, o);
+        if (l2 < lo || (l2 == lo && i2 < li)) {
+            lo = l2;
+            li = i2;
+        }
     }
-    int r = 0;
-    for (int k = 0; k < m; ++k)
-        if (d[k] > cutoff * dm) keep[r++] = k;
-    if (r & 1) {
-        int lo = 0;
-        for (int q = 1; q < r; ++q)
-            if (d[keep[q]] < d[keep[lo]]) lo = q;
-        for (int q = lo; q < r - 1; ++q) keep[q] = keep[q + 1];
-        --r;
+    const unsigned b0 = __ballot_sync(0xffffffffu, on);
+    if (lane == 0) {
+        red[w] = lo;
+        redi[w] = li;
+        cnt[w] = __popc(b0);
     }
-    *rank = r;
-}
-
-// Y[i][j] = sum_kept V[i][k] V[j][k] / d[k], i < m, j < n: the pseudo-inverse
-// of the embedded G, first n columns (G^+ = Y[0:n] + i Y[n:2n]).
-__global__ void kry_pinv_kernel(JacBufs J, int m, const double* __restrict__ d,
-                                const int* __restrict__ keep, const int* __restrict__ rank,
-                                double* __restrict__ Y) {
-    const int n = m / 2;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= m * n) return;
-    const double* V = J.V[*J.res];
-    const int i = e / n, j = e % n, r = *rank;
-    double s = 0.0;
-    for (int q = 0; q < r; ++q) {
-        const int k = keep[q];
-        s += V[(size_t)i * m + k] * V[(size_t)j * m + k] / d[k];
+    __syncthreads();
+    int tot = 0;
+    for (int i = 0; i < 32; ++i) {
+        tot += cnt[i];
+        if (red[i] < lo || (red[i] == lo && redi[i] < li)) {
+            lo = red[i];
+            li = redi[i];
+        }
     }
-    Y[e] = s;
+    if ((tot & 1) && t == li) on = false;
+    __syncthreads();
+    const unsigned b1 = __ballot_sync(0xffffffffu, on);
+    if (lane == 0) cnt[w] = __popc(b1);
+    __syncthreads();
+    int at = 0;
+    for (int i = 0; i < w; ++i) at += cnt[i];
+    if (on) keep[at + __popc(b1 & ((1u << lane) - 1u))] = t;
+    if (t == 0) *rank = tot & ~1;
 }
 
 // X[i][q] = V[i][keep q] / sqrt(d) for q < r, 0 for r <= q < m (padding).
@@ -286,25 +413,48 @@ __global__ void kry_x_kernel(JacBufs J, int m, const double* __restrict__ d,
     X[e] = q < r ? V[(size_t)i * m + keep[q]] / sqrt(d[keep[q]]) : 0.0;
 }
 
-// C = A^T B or A B (m x m, row-major), one output per thread (float64).
-template <bool TRANS_A>
+// C = A^T B, A B or A B^T (m x m, row-major), one output per thread (float64).
+template <bool TRANS_A, bool TRANS_B>
 __global__ void kry_gemm_kernel(const double* __restrict__ A, const double* __restrict__ B, int m,
                                 double* __restrict__ C) {
     __shared__ double as[16][17], bs[16][17];
     const int i = blockIdx.y * 16 + threadIdx.y, j = blockIdx.x * 16 + threadIdx.x;
+    const int ty = threadIdx.y, tx = threadIdx.x;
     double s = 0.0;
     for (int l0 = 0; l0 < m; l0 += 16) {
-        const int la = l0 + threadIdx.x, lb = l0 + threadIdx.y;
-        const int ia = blockIdx.y * 16 + threadIdx.y;
-        as[threadIdx.y][threadIdx.x] =
-            (ia < m && la < m) ? (TRANS_A ? A[(size_t)la * m + ia] : A[(size_t)ia * m + la]) : 0.0;
-        bs[threadIdx.y][threadIdx.x] = (lb < m && j < m) ? B[(size_t)lb * m + j] : 0.0;
+        const int ia = blockIdx.y * 16, jb = blockIdx.x * 16;
+        if (TRANS_A) as[tx][ty] = (ia + tx < m && l0 + ty < m) ? A[(size_t)(l0 + ty) * m + ia + tx] : 0.0;
+        else as[ty][tx] = (i < m && l0 + tx < m) ? A[(size_t)i * m + l0 + tx] : 0.0;
+        if (TRANS_B) bs[tx][ty] = (jb + ty < m && l0 + tx < m) ? B[(size_t)(jb + ty) * m + l0 + tx] : 0.0;
+        else bs[ty][tx] = (l0 + ty < m && j < m) ? B[(size_t)(l0 + ty) * m + j] : 0.0;
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 16; ++q) s += as[threadIdx.y][q] * bs[q][threadIdx.x];
+        for (int q = 0; q < 16; ++q) s += as[ty][q] * bs[q][tx];
         __syncthreads();
     }
     if (i < m && j < m) C[(size_t)i * m + j] = s;
+}
+
+// C = Y S with Y = G^+ = Yr + i Yi from the first n columns of the embedded
+// pseudo-inverse [[Yr, .], [Yi, .]] and S = H or G (n x n complex).
+__global__ void __launch_bounds__(256) kry_pgemm_kernel(const double* __restrict__ Y,
+                                                        const double* __restrict__ S_, int n,
+                                                        zd* __restrict__ C) {
+    __shared__ zd as[16][17], bs[16][17];
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4, m = 2 * n;
+    const int i = blockIdx.y * 16 + ty, j = blockIdx.x * 16 + tx;
+    const zd* S = (const zd*)S_;
+    const zd zero = {0.0, 0.0};
+    zd s = zero;
+    for (int l0 = 0; l0 < n; l0 += 16) {
+        as[ty][tx] = i < n && l0 + tx < n ? zd{Y[(size_t)i * m + l0 + tx], Y[(size_t)(i + n) * m + l0 + tx]} : zero;
+        bs[ty][tx] = l0 + ty < n && j < n ? S[(size_t)(l0 + ty) * n + j] : zero;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 16; ++q) s = s + as[ty][q] * bs[q][tx];
+        __syncthreads();
+    }
+    if (i < n && j < n) C[(size_t)i * n + j] = s;
 }
 
 // out = (C + C^T) / 2 into the Jacobi input buffer; g0 = X^T [Re G e0; Im G e0].
@@ -315,117 +465,137 @@ __global__ void kry_sym_kernel(const double* __restrict__ C, int m, double* __re
     out[e] = 0.5 * (C[e] + C[(size_t)b * m + a]);
 }
 
-__global__ void kry_g0_kernel(const double* __restrict__ G_, const double* __restrict__ X, int m,
-                              double* __restrict__ g0) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= m) return;
-    const int n = m / 2;
-    const cpx<double>* G = (const cpx<double>*)G_;
+__global__ void __launch_bounds__(256) kry_g0_kernel(const double* __restrict__ G_,
+                                                     const double* __restrict__ X, int m,
+                                                     double* __restrict__ g0) {
+    const int q = blockIdx.x * 32 + (threadIdx.x & 31), part = threadIdx.x >> 5, n = m / 2;
+    __shared__ double red[8][32];
+    const zd* G = (const zd*)G_;
     double s = 0.0;
-    for (int l = 0; l < n; ++l) {
-        const cpx<double> gl = G[(size_t)l * n];
-        s += X[(size_t)l * m + q] * gl.x + X[(size_t)(l + n) * m + q] * gl.y;
-    }
-    g0[q] = s;
-}
-
-// Moment correction (one CTA): c_0 = e_0, c_1 = G^+ H c_0,
-// c_{k+1} = G^+ (2 H c_k - G c_{k-1}); mu'_k = (G c_k)_0.
-__global__ void __launch_bounds__(1024) kry_moments_kernel(const double* __restrict__ G_,
-                                                           const double* __restrict__ H_, int n,
-                                                           const double* __restrict__ Y, int n_out,
-                                                           double* __restrict__ vec,
-                                                           double* __restrict__ mu_out) {
-    const cpx<double>* G = (const cpx<double>*)G_;
-    const cpx<double>* H = (const cpx<double>*)H_;
-    cpx<double>* c0 = (cpx<double>*)vec;
-    cpx<double>* c1 = c0 + n;
-    cpx<double>* t1 = c1 + n;
-    cpx<double>* t2 = t1 + n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        c0[i] = {i == 0 ? 1.0 : 0.0, 0.0};
-        c1[i] = {0.0, 0.0};
-    }
+    if (q < m)
+        for (int l = part; l < n; l += 8) {
+            const zd gl = G[(size_t)l * n];
+            s += X[(size_t)l * m + q] * gl.x + X[(size_t)(l + n) * m + q] * gl.y;
+        }
+    red[part][threadIdx.x & 31] = s;
     __syncthreads();
-    for (int k = 0; k < n_out; ++k) {
-        if (threadIdx.x == 0) {
-            cpx<double> s = {0.0, 0.0};
-            for (int l = 0; l < n; ++l) s = s + G[l] * c0[l];
-            mu_out[2 * k] = s.x;
-            mu_out[2 * k + 1] = s.y;
-        }
-        if (k == n_out - 1) break;
-        // t1 = (k == 0 ? H c0 : 2 H c0 - G c1)   (c1 holds c_{k-1})
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            cpx<double> s = {0.0, 0.0}, gsum = {0.0, 0.0};
-            for (int l = 0; l < n; ++l) {
-                s = s + H[(size_t)i * n + l] * c0[l];
-                gsum = gsum + G[(size_t)i * n + l] * c1[l];
-            }
-            t1[i] = k == 0 ? s : (2.0 * s - gsum);
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            cpx<double> s = {0.0, 0.0};
-            for (int l = 0; l < n; ++l) {
-                const cpx<double> gp = {Y[(size_t)i * n + l], Y[(size_t)(i + n) * n + l]};
-                s = s + gp * t1[l];
-            }
-            t2[i] = s;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            c1[i] = c0[i];
-            c0[i] = t2[i];
-        }
-        __syncthreads();
+    if (part == 0 && q < m) {
+        for (int w = 1; w < 8; ++w) s += red[w][threadIdx.x & 31];
+        g0[q] = s;
     }
 }
 
-// Poles and weights from the diagonalised projection (one CTA): eigenvalue
-// k = E[k][k] for k < r, weight (V[:, k] . g0)^2; sorted, and the doubled
-// eigenvalues of the embedding merged in pairs.
-__global__ void __launch_bounds__(1024) kry_final_kernel(JacBufs J, int m,
-                                                         const double* __restrict__ g0,
+// Moment correction: c_0 = e_0, c_1 = K c_0, c_{k+1} = 2 K c_k - Q c_{k-1}
+// with K = G^+ H and Q = G^+ G formed once; mu'_k = (G c_k)_0.  One cooperative
+// launch, a warp per row, one grid barrier per k; the moments of a block of
+// vectors follow it.
+constexpr int MOM_CHUNK = 512;
+
+struct MomArgs {
+    const zd* K;
+    const zd* Q;
+    zd* c;       // [MOM_CHUNK + 2][n]: c_{first-2}, c_{first-1}, then the chunk's vectors
+    int n, first, count;
+    unsigned* bar;
+    int* status;
+};
+
+constexpr int REC_WARPS = 2;  // rows per CTA: few, since a row's 8 n operations wait for the float64 pipe
+__global__ void __launch_bounds__(32 * REC_WARPS) kry_recur_kernel(const MomArgs a) {
+    __shared__ int flag_;
+    volatile int* flag = &flag_;
+    const int n = a.n, lane = threadIdx.x & 31, warp = blockIdx.x * REC_WARPS + (threadIdx.x >> 5);
+    const int nw = gridDim.x * REC_WARPS;
+    if (threadIdx.x == 0) *flag = 0;
+    __syncthreads();
+    for (int k = 0; k < a.count; ++k) {
+        const int step = a.first + k;
+        const zd* c0 = a.c + (size_t)(k + 1) * n;  // c_{step-1}
+        const zd* c1 = a.c + (size_t)k * n;        // c_{step-2}
+        zd* out = a.c + (size_t)(k + 2) * n;
+        for (int i = warp; i < n; i += nw) {
+            zd s = {0.0, 0.0}, q = {0.0, 0.0};
+            if (step == 0) {
+                s = {i == 0 ? 1.0 : 0.0, 0.0};
+            } else {
+                for (int l = lane; l < n; l += 32) {
+                    const double2 x = __ldcg((const double2*)(c0 + l));
+                    s = s + ldg(a.K + (size_t)i * n + l) * zd{x.x, x.y};
+                    if (step >= 2) {
+                        const double2 y = __ldcg((const double2*)(c1 + l));
+                        q = q + ldg(a.Q + (size_t)i * n + l) * zd{y.x, y.y};
+                    }
+                }
+                if (step >= 2) s = 2.0 * s - q;
+                s = warp_sum(s);
+            }
+            if (lane == 0) __stcg((double2*)(out + i), make_double2(s.x, s.y));
+        }
+        if (!grid_sync(a.bar, (unsigned)(k + 1) * gridDim.x, flag, a.status)) return;
+    }
+}
+
+__global__ void __launch_bounds__(128) kry_mu_kernel(const zd* __restrict__ G, const zd* __restrict__ c, int n,
+                                                     int first, double* __restrict__ mu) {
+    __shared__ zd red[4];
+    const int t = threadIdx.x;
+    const zd* v = c + (size_t)(blockIdx.x + 2) * n;
+    zd s = {0.0, 0.0};
+    for (int l = t; l < n; l += 128) s = s + G[l] * v[l];
+    s = warp_sum(s);
+    if ((t & 31) == 0) red[t >> 5] = s;
+    __syncthreads();
+    if (t == 0) ((zd*)mu)[first + blockIdx.x] = (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+// Eigenvalue k = E[k][k] and weight (V[:, k] . g0)^2 of the diagonalised
+// projection, k < r; one warp each.
+__global__ void __launch_bounds__(256) kry_weight_kernel(JacBufs J, int m, const double* __restrict__ g0,
                                                          const int* __restrict__ rank,
-                                                         double* __restrict__ d,
-                                                         double* __restrict__ wk,
-                                                         double* __restrict__ poles,
-                                                         double* __restrict__ weights,
-                                                         int32_t* __restrict__ rank_out) {
+                                                         double* __restrict__ d, double* __restrict__ wk) {
+    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, r = *rank;
+    if (k >= r) return;
     const double* E = J.A[*J.res];
     const double* V = J.V[*J.res];
-    const int r = *rank, n = m / 2;
-    for (int k = threadIdx.x; k < r; k += blockDim.x) {
-        double s = 0.0;
-        for (int q = 0; q < r; ++q) s += V[(size_t)q * m + k] * g0[q];
+    double s = 0.0;
+    for (int q = lane; q < r; q += 32) s += V[(size_t)q * m + k] * g0[q];
+    s = warp_sum(s);
+    if (lane == 0) {
         wk[k] = s * s;
         d[k] = E[(size_t)k * m + k];
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < r; ++i) {
-            const double dv = d[i], wv = wk[i];
-            int j = i - 1;
-            while (j >= 0 && d[j] > dv) {
-                d[j + 1] = d[j];
-                wk[j + 1] = wk[j];
-                --j;
-            }
-            d[j + 1] = dv;
-            wk[j + 1] = wv;
-        }
-        for (int k = 0; k < n; ++k) {
-            if (2 * k + 1 < r) {
-                poles[k] = 0.5 * (d[2 * k] + d[2 * k + 1]);
-                weights[k] = wk[2 * k] + wk[2 * k + 1];
-            } else {
-                poles[k] = 0.0;
-                weights[k] = 0.0;
-            }
-        }
-        if (rank_out) *rank_out = r / 2;
+}
+
+// Poles in ascending order (by rank counting, one thread per eigenvalue) and
+// the doubled eigenvalues of the embedding merged in pairs.
+__global__ void __launch_bounds__(1024) kry_final_kernel(int m, const int* __restrict__ rank,
+                                                         const double* __restrict__ d,
+                                                         const double* __restrict__ wk,
+                                                         double* __restrict__ poles,
+                                                         double* __restrict__ weights,
+                                                         int32_t* __restrict__ rank_out) {
+    __shared__ long long key[1024];  // order-preserving integers (the float64 pipe is narrow)
+    __shared__ double se[1024], sw[1024];
+    const int t = threadIdx.x, r = *rank, n = m / 2;
+    if (t < r) {
+        const long long b = __double_as_longlong(d[t]);
+        key[t] = b < 0 ? b ^ 0x7fffffffffffffffll : b;
     }
+    __syncthreads();
+    if (t < r) {
+        const long long mine = key[t];
+        int at = 0;
+        for (int k = 0; k < r; ++k) at += key[k] < mine || (key[k] == mine && k < t);
+        se[at] = d[t];
+        sw[at] = wk[t];
+    }
+    __syncthreads();
+    if (t < n) {
+        const bool on = 2 * t + 1 < r;
+        poles[t] = on ? 0.5 * (se[2 * t] + se[2 * t + 1]) : 0.0;
+        weights[t] = on ? sw[2 * t] + sw[2 * t + 1] : 0.0;
+    }
+    if (t == 0 && rank_out) *rank_out = r / 2;
 }
 
 }  // namespace
@@ -438,11 +608,12 @@ extern "C" cr_status cheb_krylov(cr_ctx* ctx, const double* G, const double* H, 
     CR_CHECK_ARG(n_out >= 1, "cheb_krylov: n_out < 1");
     CR_CHECK_ARG(G && H && mu_corr_out && poles_out && weights_out, "cheb_krylov: null array");
     const int n = Nm, m = 2 * Nm;
-    const size_t mm = (size_t)m * m;
-    // workspace (doubles): A0, A1, V0, V1, X, C [m*m]; Y [m*n]; d, wk, g0 [m];
-    // 4 complex vectors [n]; norm shares [2 NORM_GRID]; ints: keep [m], rank, res, flag
-    const size_t need = 6 * mm + (size_t)m * n + 3 * (size_t)m + 8 * (size_t)n +
-                        2 * NORM_GRID + ((size_t)m + 3 + 1) / 2 + 1;
+    const size_t mm = (size_t)m * m, nn = (size_t)n * n;
+    // workspace (doubles): A0, A1, V0, V1, X, C, Y [m*m]; K, Q [n*n] and the
+    // recursion's vectors, complex; d, wk, g0 [m]; norm shares; ints: keep [m],
+    // rank, res, barriers
+    const size_t need = 7 * mm + 4 * nn + 2 * (size_t)(MOM_CHUNK + 2) * n + 3 * (size_t)m +
+                        2 * (size_t)ctx->n_sm + ((size_t)m + 6 + 1) / 2 + 1;
     if (ctx->kry_len < need) {
         // first use at this size: the only allocation outside cr_create
         if (ctx->kry) cudaFree(ctx->kry);
@@ -453,49 +624,78 @@ extern "C" cr_status cheb_krylov(cr_ctx* ctx, const double* G, const double* H, 
         ctx->kry_len = need;
     }
     double* w = ctx->kry;
+    auto take = [&](size_t k) {
+        double* p = w;
+        w += k;
+        return p;
+    };
     JacBufs J;
-    J.A[0] = w;
-    J.A[1] = w + mm;
-    J.V[0] = w + 2 * mm;
-    J.V[1] = w + 3 * mm;
-    double* X = w + 4 * mm;
-    double* C = w + 5 * mm;
-    double* Y = w + 6 * mm;
-    double* d = Y + (size_t)m * n;
-    double* wk = d + m;
-    double* g0 = wk + m;
-    double* vec = g0 + m;
-    double* part = vec + 8 * (size_t)n;
-    int* keep = (int*)(part + 2 * NORM_GRID);
+    J.A[0] = take(mm);
+    J.A[1] = take(mm);
+    J.V[0] = take(mm);
+    J.V[1] = take(mm);
+    double* X = take(mm);
+    double* C = take(mm);
+    double* Y = take(mm);
+    zd* K = (zd*)take(2 * nn);
+    zd* Q = (zd*)take(2 * nn);
+    zd* cv = (zd*)take(2 * (size_t)(MOM_CHUNK + 2) * n);
+    double* d = take(m);
+    double* wk = take(m);
+    double* g0 = take(m);
+    J.part = take(2 * (size_t)ctx->n_sm);
+    int* keep = (int*)w;
     int* rank = keep + m;
     J.res = rank + 1;
-    J.flag = rank + 2;
+    J.bar = (unsigned*)(rank + 2);
     const unsigned gm = (unsigned)((mm + 255) / 256);
-    const unsigned gn = (unsigned)(((size_t)n * n + 255) / 256);
-    const dim3 g16((m + 15) / 16, (m + 15) / 16);
+    const unsigned gn = (unsigned)((nn + 255) / 256);
+    const dim3 g16((m + 15) / 16, (m + 15) / 16), b16(16, 16), n16((n + 15) / 16, (n + 15) / 16);
     cudaStream_t st = ctx->stream;
-    // 1. G through its embedding: eigenvalues, kept rank, pseudo-inverse
+    cr_status s;
+    // 1. G through its embedding: eigenvalues, kept rank, X = V_kept d^-1/2
+    //    (zero-padded to m columns), pseudo-inverse Y = X X^T
     cudaError_t e = cudaMemsetAsync(J.A[0], 0, mm * sizeof(double), st);
     if (e != cudaSuccess) return cr_fail(ctx, CR_ECUDA, "cheb_krylov: %s", cudaGetErrorString(e));
     CR_LAUNCH(ctx, CR_K_OTHER, kry_embed_kernel<<<gn, 256, 0, st>>>(G, n, J.A[0]));
-    jacobi_launch(ctx, J, m, part);
-    CR_LAUNCH(ctx, CR_K_OTHER, kry_keep_kernel<<<1, 1, 0, st>>>(J, m, cutoff, d, keep, rank));
-    CR_LAUNCH(ctx, CR_K_OTHER,
-              kry_pinv_kernel<<<(unsigned)(((size_t)m * n + 255) / 256), 256, 0, st>>>(J, m, d, keep, rank, Y));
-    // 2. corrected moments
-    CR_LAUNCH(ctx, CR_K_OTHER, kry_moments_kernel<<<1, 1024, 0, st>>>(G, H, n, Y, n_out, vec, mu_corr_out));
-    // 3. projected eigenproblem: X = V_kept d^-1/2 (zero-padded to m columns),
-    //    Hx = X^T Hemb X, diagonalised by the same Jacobi (padding stays zero)
+    if ((s = jacobi_launch(ctx, J, m)) != CR_OK) return s;
+    CR_LAUNCH(ctx, CR_K_OTHER, kry_keep_kernel<<<1, 1024, 0, st>>>(J, m, cutoff, d, keep, rank));
     CR_LAUNCH(ctx, CR_K_OTHER, kry_x_kernel<<<gm, 256, 0, st>>>(J, m, d, keep, rank, X));
-    CR_LAUNCH(ctx, CR_K_OTHER, kry_g0_kernel<<<(m + 255) / 256, 256, 0, st>>>(G, X, m, g0));
+    CR_LAUNCH(ctx, CR_K_OTHER, (kry_gemm_kernel<false, true><<<g16, b16, 0, st>>>(X, X, m, Y)));
+    // 2. corrected moments
+    CR_LAUNCH(ctx, CR_K_OTHER, kry_pgemm_kernel<<<n16, 256, 0, st>>>(Y, H, n, K));
+    CR_LAUNCH(ctx, CR_K_OTHER, kry_pgemm_kernel<<<n16, 256, 0, st>>>(Y, G, n, Q));
+    for (int first = 0; first < n_out; first += MOM_CHUNK) {
+        MomArgs a;
+        a.K = K;
+        a.Q = Q;
+        a.c = cv;
+        a.n = n;
+        a.first = first;
+        a.count = n_out - first < MOM_CHUNK ? n_out - first : MOM_CHUNK;
+        a.bar = J.bar;
+        a.status = ctx->d_status;
+        e = cudaMemsetAsync(J.bar, 0, 2 * sizeof(unsigned), st);
+        if (e == cudaSuccess && first > 0)  // the last two vectors of the previous chunk
+            e = cudaMemcpyAsync(cv, cv + (size_t)MOM_CHUNK * n, 2 * (size_t)n * sizeof(zd),
+                                cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return cr_fail(ctx, CR_ECUDA, "cheb_krylov: %s", cudaGetErrorString(e));
+        const int want = (n + REC_WARPS - 1) / REC_WARPS, grid = want < ctx->n_sm ? want : ctx->n_sm;
+        if ((s = coop_launch(ctx, kry_recur_kernel, grid, 32 * REC_WARPS, a, "kry_recur_kernel")) != CR_OK) return s;
+        CR_LAUNCH(ctx, CR_K_OTHER, kry_mu_kernel<<<a.count, 128, 0, st>>>((const zd*)G, cv, n, first, mu_corr_out));
+    }
+    // 3. projected eigenproblem: Hx = X^T Hemb X, diagonalised by the same
+    //    Jacobi (padding stays zero)
+    CR_LAUNCH(ctx, CR_K_OTHER, kry_g0_kernel<<<(m + 31) / 32, 256, 0, st>>>(G, X, m, g0));
     e = cudaMemsetAsync(C, 0, mm * sizeof(double), st);
     if (e != cudaSuccess) return cr_fail(ctx, CR_ECUDA, "cheb_krylov: %s", cudaGetErrorString(e));
     CR_LAUNCH(ctx, CR_K_OTHER, kry_embed_kernel<<<gn, 256, 0, st>>>(H, n, C));
-    CR_LAUNCH(ctx, CR_K_OTHER, kry_gemm_kernel<false><<<g16, dim3(16, 16), 0, st>>>(C, X, m, J.A[1]));
-    CR_LAUNCH(ctx, CR_K_OTHER, kry_gemm_kernel<true><<<g16, dim3(16, 16), 0, st>>>(X, J.A[1], m, C));
+    CR_LAUNCH(ctx, CR_K_OTHER, (kry_gemm_kernel<false, false><<<g16, b16, 0, st>>>(C, X, m, J.A[1])));
+    CR_LAUNCH(ctx, CR_K_OTHER, (kry_gemm_kernel<true, false><<<g16, b16, 0, st>>>(X, J.A[1], m, C)));
     CR_LAUNCH(ctx, CR_K_OTHER, kry_sym_kernel<<<gm, 256, 0, st>>>(C, m, J.A[0]));
-    jacobi_launch(ctx, J, m, part);
+    if ((s = jacobi_launch(ctx, J, m)) != CR_OK) return s;
+    CR_LAUNCH(ctx, CR_K_OTHER, kry_weight_kernel<<<(m + 7) / 8, 256, 0, st>>>(J, m, g0, rank, d, wk));
     CR_LAUNCH(ctx, CR_K_OTHER,
-              kry_final_kernel<<<1, 1024, 0, st>>>(J, m, g0, rank, d, wk, poles_out, weights_out, rank_out));
+              kry_final_kernel<<<1, 1024, 0, st>>>(m, rank, d, wk, poles_out, weights_out, rank_out));
     return cr_check_launch(ctx, "cheb_krylov");
 }
