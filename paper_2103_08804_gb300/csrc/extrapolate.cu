@@ -275,22 +275,39 @@ __global__ void __launch_bounds__(LP_THREADS) lp_kernel(const LpArgs A) {
     }
     __syncthreads();
     for (int n = tid; n < N; n += nt) out[n] = mu[n];
-    for (int t = tid; t < A.n_out - N; t += nt) {
-        zd acc = {0.0, 0.0};
-        if (flag) {
-            acc = {nan, nan};
-        } else {
-            const double m = (double)(p + t);
-            for (int k = 0; k < p; ++k) {
-                const zd w = sz2[k];
-                const double lw = 0.5 * log(abs2(w)), ph = atan2(w.y, w.x);
-                double sn, cs;
-                sincos(m * ph, &sn, &cs);
-                const double mag = exp(m * lw);
-                acc = acc + sa[k] * zd{mag * cs, mag * sn};
+    // mu_{N+t} = sum_k c_k w_k^{p+t}.  With t = t0 + BK a + b the power is
+    // (c_k w_k^{p+t0+BK a}) w_k^b: the two factors are tabulated (R and V are
+    // free here), so a predicted value costs one complex multiply-add per root
+    // where its logarithm, angle, exponential and sine per root were 13 of the
+    // 15 ms of 36 sequences of order 100 continued from 300 to 3000.
+    const int T = A.n_out - N, BK = min(p, 64), NA = min(p, (T + BK - 1) / BK);
+    zd* wa = R;  // [NA][p] c_k w_k^{p + t0 + BK a}
+    zd* wb = V;  // [BK][p] w_k^b
+    auto power = [&](zd w, double m) {
+        const double lw = 0.5 * log(abs2(w)), ph = atan2(w.y, w.x);
+        double sn, cs;
+        sincos(m * ph, &sn, &cs);
+        const double mag = exp(m * lw);
+        return zd{mag * cs, mag * sn};
+    };
+    if (flag) {
+        for (int t = tid; t < T; t += nt) out[N + t] = {nan, nan};
+    } else {
+        for (int e = tid; e < BK * p; e += nt) wb[e] = e < p ? zd{1.0, 0.0} : power(sz2[e % p], (double)(e / p));
+        for (int t0 = 0; t0 < T; t0 += BK * NA) {
+            __syncthreads();
+            for (int e = tid; e < NA * p; e += nt)
+                wa[e] = sa[e % p] * power(sz2[e % p], (double)(p + t0 + BK * (e / p)));
+            __syncthreads();
+            const int t1 = min(T, t0 + BK * NA);
+            for (int t = t0 + tid; t < t1; t += nt) {
+                const zd* x = wa + (size_t)((t - t0) / BK) * p;
+                const zd* y = wb + (size_t)((t - t0) % BK) * p;
+                zd acc = {0.0, 0.0};
+                for (int k = 0; k < p; ++k) acc = acc + x[k] * y[k];
+                out[N + t] = acc;
             }
         }
-        out[N + t] = acc;
     }
     if (tid == 0) {
         if (A.info) A.info[s] = flag ? -2 : iters;
