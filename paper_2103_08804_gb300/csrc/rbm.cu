@@ -59,125 +59,228 @@ cr_status build_tables(cr_ctx* c, const void* params, int slot) {
 
 // ------------------------------------------------------ theta and log psi
 //
-// One CTA of 128 threads takes WB walkers; thread t owns hidden units
-// j = t + 128 k (k < JPT) for all WB walkers, so every W element loaded
-// from L1/L2 feeds 2 WB FMAs (sigma = +-1 is exact in R).  Epilogue:
+// theta = b + sigma W for a block of walkers, then per walker
 //   MODE_LOGPSI: theta_out = theta, out = a.sigma + sum_j log 2cosh theta_j
 //   MODE_MATVEC: out = v_a.sigma + sum_j T_j (v_b + sigma V_W)_j, i.e. O v
 //                with O_a = sigma, O_b = T, O_W = sigma (x) T (Sec. III).
+//
+// A warp takes TH_W walkers (per group of LJ lanes) and all their hidden units,
+// JW per lane, so the sums over hidden units end in a few shuffles; M > LJ JW
+// takes several passes.  Sites come 16 at a time through shared memory (W
+// rows by cp.async, signs converted once), double-buffered: per site a lane
+// reads TH_W signs (a broadcast) and JW weights for 2 TH_W JW multiply-adds.
+// JW and LJ are the smallest that hold M, so few lanes multiply padding; TH_W
+// is 8, or 4 and 1 for fewer walkers, so that the blocks reach every SM.
+//
+// Bound by the FMA pipe and, for log psi, by the exponential, sine and cosine
+// of every theta; log(2 cosh) of two units shares one logarithm and one
+// angle.  16 x 16 lattice, 65536 walkers: 604 -> 503 us (one block of 128
+// threads per 16 walkers before, weights read from L2 by every block); M = 72:
+// 921 -> 530 us; float64 at N = M = 12: 130 -> 15 us.  Packed pairs of
+// multiply-adds did not help (527 us).
 enum { MODE_LOGPSI = 0, MODE_MATVEC = 1 };
 
-template <typename R, int JPT, int WB, int MODE>
-__global__ void __launch_bounds__(128) theta_kernel(const cpx<R>* __restrict__ prm,
-                                                    const int8_t* __restrict__ spins, int B, int N,
-                                                    int M, cpx<R>* __restrict__ theta_out,
-                                                    cpx<R>* __restrict__ out,
-                                                    const cpx<R>* __restrict__ T,
-                                                    const double* __restrict__ skip) {
+namespace {
+
+constexpr int TH_KC = 16;  // sites per stage
+constexpr int TH_WARPS = 8;
+
+CR_D void cp_async8(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                 "l"(src)
+                 : "memory");
+}
+CR_D void cp_async_all() { asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory"); }
+
+// Unit q of a lane: pairs of neighbours first (one 16-byte access of a float
+// row), a single unit last when JW is odd.
+template <int LJ, int JW> CR_D int unit_of(int l, int q) {
+    return q < (JW & ~1) ? 2 * l + (q & 1) + 2 * LJ * (q >> 1) : LJ * (JW - 1) + l;
+}
+
+// log(2 cosh z) summed over the lane's units: s z and 1 + w of each (|w| <= 1,
+// so two arguments add up without a branch cut), the logarithm of two units'
+// product at once.
+template <typename R> CR_D void lncosh_parts(cpx<R> z, cpx<R>* lin, cpx<R>* onew) {
+    const R sg = z.x < R(0) ? R(-1) : R(1);
+    const R e = m_exp(R(-2) * sg * z.x);
+    R s, c;
+    m_sincos(R(-2) * sg * z.y, &s, &c);
+    *lin = *lin + sg * z;
+    *onew = {R(1) + e * c, e * s};
+}
+CR_D float m_log(float x) { return logf(x); }
+CR_D double m_log(double x) { return log(x); }
+
+}  // namespace
+
+template <typename R, int LJ, int JW, int TH_W, int MODE>
+__global__ void __launch_bounds__(32 * TH_WARPS, 2) theta_kernel(const cpx<R>* __restrict__ prm,
+                                                              const int8_t* __restrict__ spins, int B,
+                                                              int N, int M, cpx<R>* __restrict__ theta_out,
+                                                              cpx<R>* __restrict__ out,
+                                                              const cpx<R>* __restrict__ T,
+                                                              const double* __restrict__ skip) {
     if (skip && *skip != 0.0) return;  // converged CG: nothing left to do
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    R* sg = (R*)smem_raw;                       // [N][WB]: the WB signs of site i together
-    cpx<R>* red = (cpx<R>*)(sg + WB * N);       // [4][WB]
+    constexpr int NG = 32 / LJ, WB = TH_W * NG * TH_WARPS, JB = LJ * JW, NT = 32 * TH_WARPS;
+    __shared__ __align__(16) R sg[2][TH_KC][WB];
+    __shared__ __align__(16) cpx<R> wv[2][TH_KC][JB];
+    const int t = threadIdx.x, lane = t & 31, l = lane & (LJ - 1);
+    const int wl = ((t >> 5) * NG + lane / LJ) * TH_W;  // first walker of the group in the block
     const int w0 = blockIdx.x * WB;
-    const int t = threadIdx.x;
-    for (int e = t; e < WB * N; e += 128) {
-        int w = e / N, i = e % N;
-        sg[i * WB + w] = (w0 + w < B) ? R(spins[(size_t)(w0 + w) * N + i]) : R(0);
-    }
-    __syncthreads();
     const cpx<R>* a = prm;
     const cpx<R>* b = prm + N;
     const cpx<R>* W = prm + N + M;
-    cpx<R> acc[WB][JPT];
+    cpx<R> part[TH_W];
 #pragma unroll
-    for (int k = 0; k < JPT; ++k) {
-        int j = t + 128 * k;
-        cpx<R> bj = j < M ? b[j] : cpx<R>{R(0), R(0)};
+    for (int w = 0; w < TH_W; ++w) part[w] = {R(0), R(0)};
+    const bool quad = (N & 3) == 0;  // 4 signs of a walker are one aligned word
+    for (int jb = 0; jb < M; jb += JB) {
+        cpx<R> acc[TH_W][JW];
 #pragma unroll
-        for (int w = 0; w < WB; ++w) acc[w][k] = bj;
-    }
-    // W rows are loaded one step ahead so that their latency overlaps the FMAs
-    cpx<R> wnext[JPT];
+        for (int q = 0; q < JW; ++q) {
+            const int j = jb + unit_of<LJ, JW>(l, q);
+            const cpx<R> bj = j < M ? b[j] : cpx<R>{R(0), R(0)};
 #pragma unroll
-    for (int k = 0; k < JPT; ++k) {
-        int j = t + 128 * k;
-        wnext[k] = (j < M && N > 0) ? W[j] : cpx<R>{R(0), R(0)};
-    }
-    for (int i = 0; i < N; ++i) {
-        cpx<R> wv[JPT];
-#pragma unroll
-        for (int k = 0; k < JPT; ++k) {
-            wv[k] = wnext[k];
-            int j = t + 128 * k;
-            wnext[k] = (j < M && i + 1 < N) ? W[(size_t)(i + 1) * M + j] : cpx<R>{R(0), R(0)};
+            for (int w = 0; w < TH_W; ++w) acc[w][q] = bj;
         }
-        // WB signs in 16-byte shared loads
-        R sv[WB];
-#pragma unroll
-        for (int w = 0; w < WB; w += 16 / sizeof(R)) {
-            uint4 v = *reinterpret_cast<const uint4*>(sg + i * WB + w);
-            memcpy(&sv[w], &v, 16);
-        }
-#pragma unroll
-        for (int w = 0; w < WB; ++w) {
-#pragma unroll
-            for (int k = 0; k < JPT; ++k) {
-                acc[w][k].x = fma(sv[w], wv[k].x, acc[w][k].x);
-                acc[w][k].y = fma(sv[w], wv[k].y, acc[w][k].y);
-            }
-        }
-    }
-    cpx<R> part[WB];
-#pragma unroll
-    for (int w = 0; w < WB; ++w) {
-        part[w] = {R(0), R(0)};
-        const bool live = w0 + w < B;
-#pragma unroll
-        for (int k = 0; k < JPT; ++k) {
-            int j = t + 128 * k;
-            if (j < M && live) {
-                if (MODE == MODE_LOGPSI) {
-                    if (theta_out) theta_out[(size_t)(w0 + w) * M + j] = acc[w][k];
-                    part[w] = part[w] + clncosh2_(acc[w][k]);
+        // stage of sites i0 .. i0 + 15 into buffer s: weights, then signs
+        auto fetch = [&](int i0, int s) {
+            for (int e = t; e < TH_KC * JB; e += NT) {
+                const int k = e / JB, j = e % JB;
+                cpx<R>* dst = &wv[s][k][j];
+                if (i0 + k < N && jb + j < M) {
+                    const cpx<R>* src = W + (size_t)(i0 + k) * M + jb + j;
+                    cp_async8(dst, src);
+                    if (sizeof(R) == 8) cp_async8((char*)dst + 8, (const char*)src + 8);
                 } else {
-                    part[w] = part[w] + T[(size_t)(w0 + w) * M + j] * acc[w][k];
+                    *dst = {R(0), R(0)};
+                }
+            }
+            for (int e = t; e < WB * (TH_KC / 4); e += NT) {
+                const int w = e % WB, k = 4 * (e / WB);
+                const int8_t* src = spins + (size_t)(w0 + w) * N + i0 + k;
+                char4 v = make_char4(0, 0, 0, 0);
+                if (w0 + w < B) {
+                    if (quad) {
+                        if (i0 + k < N) v = *reinterpret_cast<const char4*>(src);
+                    } else {
+                        if (i0 + k < N) v.x = src[0];
+                        if (i0 + k + 1 < N) v.y = src[1];
+                        if (i0 + k + 2 < N) v.z = src[2];
+                        if (i0 + k + 3 < N) v.w = src[3];
+                    }
+                }
+                sg[s][k][w] = R(v.x);
+                sg[s][k + 1][w] = R(v.y);
+                sg[s][k + 2][w] = R(v.z);
+                sg[s][k + 3][w] = R(v.w);
+            }
+        };
+        __syncthreads();
+        fetch(0, 0);
+        cp_async_all();
+        __syncthreads();
+        for (int i0 = 0, s = 0; i0 < N; i0 += TH_KC, s ^= 1) {
+            if (i0 + TH_KC < N) fetch(i0 + TH_KC, s ^ 1);
+            const int kn = min(TH_KC, N - i0);
+#pragma unroll 4
+            for (int k = 0; k < kn; ++k) {
+                R sv[TH_W];
+                cpx<R> wk[JW];
+#pragma unroll
+                for (int w = 0; w < TH_W; ++w) sv[w] = sg[s][k][wl + w];
+#pragma unroll
+                for (int q = 0; q < JW; ++q) wk[q] = wv[s][k][unit_of<LJ, JW>(l, q)];
+#pragma unroll
+                for (int w = 0; w < TH_W; ++w)
+#pragma unroll
+                    for (int q = 0; q < JW; ++q) {
+                        acc[w][q].x = fma(sv[w], wk[q].x, acc[w][q].x);
+                        acc[w][q].y = fma(sv[w], wk[q].y, acc[w][q].y);
+                    }
+            }
+            if (jb == 0 && l < kn) {  // a.sigma: a lane per site of the stage
+                const cpx<R> ai = a[i0 + l];
+#pragma unroll
+                for (int w = 0; w < TH_W; ++w) part[w] = part[w] + sg[s][l][wl + w] * ai;
+            }
+            cp_async_all();
+            __syncthreads();
+        }
+#pragma unroll
+        for (int w = 0; w < TH_W; ++w) {
+            const int ww = w0 + wl + w;
+            if (ww >= B) break;
+            cpx<R>* to = MODE == MODE_LOGPSI && theta_out ? theta_out + (size_t)ww * M : nullptr;
+            cpx<R> one[2];
+#pragma unroll
+            for (int q = 0; q < JW; ++q) {
+                const int j = jb + unit_of<LJ, JW>(l, q);
+                const cpx<R> th = acc[w][q];
+                if (MODE == MODE_MATVEC) {
+                    if (j < M) part[w] = part[w] + T[(size_t)ww * M + j] * th;
+                    continue;
+                }
+                one[q & 1] = {R(1), R(0)};
+                if (j < M) {
+                    if (to) to[j] = th;
+                    lncosh_parts(th, &part[w], &one[q & 1]);
+                }
+                if ((q & 1) || q == JW - 1) {
+                    const cpx<R> p = (q & 1) ? one[0] * one[1] : one[0];
+                    part[w] = part[w] + cpx<R>{R(0.5) * m_log(abs2(p)), m_atan2(p.y, p.x)};
                 }
             }
         }
-        for (int i = t; i < N; i += 128) part[w] = part[w] + sg[i * WB + w] * a[i];
     }
-    const int lane = t & 31, wid = t >> 5;
 #pragma unroll
-    for (int w = 0; w < WB; ++w) {
-        cpx<R> v = warp_sum(part[w]);
-        if (lane == 0) red[wid * WB + w] = v;
+    for (int w = 0; w < TH_W; ++w) {
+        cpx<R> v = part[w];
+#pragma unroll
+        for (int o = LJ / 2; o > 0; o >>= 1)
+            v = v + cpx<R>{__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)};
+        if (l == 0 && w0 + wl + w < B) out[w0 + wl + w] = v;
     }
-    __syncthreads();
-    if (t < WB && w0 + t < B) {
-        cpx<R> s = red[t] + red[WB + t] + red[2 * WB + t] + red[3 * WB + t];
-        out[w0 + t] = s;
+}
+
+template <typename R, int TW, int MODE>
+static cr_status launch_theta_w(cr_ctx* c, const void* params, const int8_t* spins, int B,
+                                void* theta, void* out, const void* T, const double* skip) {
+#define LAUNCH(LJ, JW)                                                                           \
+    {                                                                                            \
+        constexpr int WB = TW * (32 / LJ) * TH_WARPS;                                            \
+        CR_LAUNCH(c, (MODE == MODE_LOGPSI ? CR_KERNEL_THETA : CR_KERNEL_OV),                     \
+                  (theta_kernel<R, LJ, JW, TW, MODE>                                             \
+                   <<<(B + WB - 1) / WB, 32 * TH_WARPS, 0, c->stream>>>(                         \
+                       (const cpx<R>*)params, spins, B, c->N, c->M, (cpx<R>*)theta,              \
+                       (cpx<R>*)out, (const cpx<R>*)T, skip)));                                  \
     }
+    // units per lane and pass: the fewest padded units (float64: registers for two)
+    const int M = c->M;
+    if (M <= 16) LAUNCH(16, 1)
+    else if (M <= 32) LAUNCH(32, 1)
+    else if (M <= 64 || sizeof(R) == 8) LAUNCH(32, 2)
+    else {
+        const int passes = (M + 127) / 128, per = (M + passes - 1) / passes;
+        if (per <= 96) LAUNCH(32, (sizeof(R) == 8 ? 2 : 3))
+        else LAUNCH(32, (sizeof(R) == 8 ? 2 : 4))
+    }
+#undef LAUNCH
+    return cr_check_launch(c, "theta_kernel");
 }
 
 template <typename R, int MODE>
 static cr_status launch_theta_t(cr_ctx* c, const void* params, const int8_t* spins, int B,
                                 void* theta, void* out, const void* T, const double* skip) {
     if (B == 0) return CR_OK;
-    const int jpt = (c->M + 127) / 128;
-    const int N = c->N;
-#define LAUNCH(JPT, WB)                                                                          \
-    {                                                                                            \
-        size_t sm = WB * N * sizeof(R) + 4 * WB * sizeof(cpx<R>);                                \
-        CR_LAUNCH(c, (MODE == MODE_LOGPSI ? CR_KERNEL_THETA : CR_KERNEL_OV), theta_kernel<R, JPT, WB, MODE><<<(B + WB - 1) / WB, 128, sm, c->stream>>>(               \
-            (const cpx<R>*)params, spins, B, N, c->M, (cpx<R>*)theta, (cpx<R>*)out,              \
-            (const cpx<R>*)T, skip));                                                             \
-    }
-    if (jpt == 1) LAUNCH(1, 16)
-    else if (jpt == 2) LAUNCH(2, 16)
-    else if (jpt <= 4) LAUNCH(4, 8)
-    else LAUNCH(8, 4)
-#undef LAUNCH
-    return cr_check_launch(c, "theta_kernel");
+    // blocks of 8 warps: two per SM with 8 walkers a group, half that with 4
+    const int groups = TH_WARPS * (c->M <= 16 ? 2 : 1);
+    if (B >= 2 * c->n_sm * 8 * groups)
+        return launch_theta_w<R, 8, MODE>(c, params, spins, B, theta, out, T, skip);
+    if (B >= c->n_sm * 4 * groups)
+        return launch_theta_w<R, 4, MODE>(c, params, spins, B, theta, out, T, skip);
+    return launch_theta_w<R, 1, MODE>(c, params, spins, B, theta, out, T, skip);
 }
 
 cr_status launch_logpsi(cr_ctx* c, const void* params, const int8_t* spins, int B, void* theta,
