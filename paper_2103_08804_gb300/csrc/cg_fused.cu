@@ -33,9 +33,10 @@
 // Per CG iteration:
 //   W   walker phase (each CTA its walker range), the product A u:
 //       W1: D1 = sigma V on the tensor cores (A = sigma tile [128 walkers x
-//           32 sites] exact in bf16, B = three bf16 planes of V [256 columns
-//           (Re/Im of 128 hidden units) x 32 sites], streamed by bulk copies
-//           through a 3-stage ring), then u_s from D1 (TMEM) and T (global);
+//           32 sites] exact in bf16, B = three bf16 planes of V [128 columns
+//           (Re/Im of 64 hidden units) x 32 sites], streamed by bulk copies
+//           through a 4-stage ring; two walker tiles share a stage of V where
+//           a CTA has them), then u_s from D1 (TMEM) and T (global);
 //       W2: D2^T = Y^T sigma on the tensor cores (A = three bf16 planes of
 //           Y_sn = (conj(T_sj) w_s).{re,im} [128 columns x 32 walkers],
 //           formed by the compute warps, B = sigma^T [sites x 32 walkers]),
@@ -49,10 +50,26 @@
 // The convergence test |r| <= tol |F| opens each walker phase; the operand
 // copies of that phase start before it, the MMAs after it.
 //
-// Warp 0 (one thread) issues the bulk copies and the MMAs; warps 1-8
-// ("compute warps") do everything else.  Every wait is bounded: a wait that
-// gives up sets CR_ETIMEOUT and a global abort flag, after which all CTAs
-// leave the solve at their next grid barrier.
+// Warp 0 (one thread) issues the MMAs, warp 17 (one thread) the bulk copies,
+// warps 1-16 ("compute warps") do everything else.  Every wait is bounded: a
+// wait that gives up sets CR_ETIMEOUT and a global abort flag, after which
+// all CTAs leave the solve at their next grid barrier.
+//
+// What bounds it (16 x 16 lattice, alpha = 1, 65536 walkers; us per CG
+// iteration from %globaltimer): W1 73 and W2 72 wait on latency -- the ring
+// of V and the read of T in W1, the read of T and the stores of Y to shared
+// memory in W2 --, the slice phase 22 moves the partial rows (2 x 80 MB)
+// through L2, a- and b-sums 10, barriers 11.  With one thread for copies and
+// MMAs, which divided for its ring positions and built every descriptor
+// anew, W1 took 133 whatever was taken out of it (T, copies, MMAs): the
+// issuing thread was the bound, so copies and MMAs have a thread each and
+// advance by constants.  A float64 warp instruction takes the SM 16 cycles
+// however many lanes need it, so the slice phase packs its float64 work into
+// full warps, the scalars of an iteration are one thread's work, and sums of
+// several scalars split their slots over the lanes.  With 8 compute warps,
+// one walker tile per stage of V, one issuing thread and float64 scalars in
+// every warp an iteration took 248 (W1 105, W2 84, slice 35), now 188; a
+// chain of 64 sites (alpha = 2, 16384 walkers) 46 (slice 12), now 37 (8).
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -60,12 +77,14 @@
 
 namespace {
 
-constexpr int FC_THREADS = 288;                 // warp 0 + 8 compute warps
-constexpr int NCT = 256;                        // compute threads
-constexpr int NS1 = 3;                          // W1 operand stages
+constexpr int NCW = 16;                         // compute warps
+constexpr int NCT = 32 * NCW;                   // compute threads
+constexpr int FC_THREADS = NCT + 64;            // warp 0 issues MMAs, the last warp copies
+constexpr int NS1 = 4;                          // W1 operand stages
 constexpr int W1_A = 128 * 32 * 2;              // sigma tile of one K-chunk
-constexpr int W1_B_PLANE = 256 * 32 * 2;        // one bf16 plane of V, 256 columns
-constexpr int W1_STAGE = W1_A + 3 * W1_B_PLANE; // 56 KB
+constexpr int W1_W = 128;                       // columns of a W1 pass
+constexpr int W1_B_PLANE = W1_W * 32 * 2;       // one bf16 plane of V
+constexpr int W1_STAGE = 2 * W1_A + 3 * W1_B_PLANE; // 40 KB
 constexpr int Y_BLK = 128 * 32 * 2;             // one plane of one 128-column n-block
 constexpr uint32_t WAIT_LIMIT = 1u << 26;       // mbarrier polls
 constexpr unsigned BAR_LIMIT = 1u << 23;        // grid-barrier polls (~1 s with the sleeps)
@@ -76,11 +95,12 @@ struct Geo {
     int N, M, P, B;
     int G;       // CTAs
     int wpc;     // walkers per CTA (the last CTA may have fewer)
-    int ntpc;    // W1 walker tiles per CTA
+    int tpu;     // W1 walker tiles per unit (a pair shares the stages of V): 1 or 2
+    int ntpc;    // W1 walker tiles per CTA (a multiple of tpu)
     int trows;   // rows per W1 tile (<= 128)
     int Kp;      // sites padded to a multiple of 32 (W1 contraction length)
     int nkc1;    // W1 K-chunks of 32 sites
-    int npass1;  // W1 column passes of 256 (the last one wlast1 wide)
+    int npass1;  // W1 column passes of 128 (the last one wlast1 wide)
     int wlast1;
     int Np;      // sites padded to a multiple of 16 (W2 MMA N)
     int nb2;     // W2 n-blocks of 128 columns of Y
@@ -141,6 +161,13 @@ CR_D uint4 pack8(const __nv_bfloat16* v) {
     return r;
 }
 
+// 32 aligned bytes
+CR_D void ldg32(const void* p, float4* a, float4* b) {
+    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a->x), "=f"(a->y), "=f"(a->z), "=f"(a->w), "=f"(b->x), "=f"(b->y), "=f"(b->z), "=f"(b->w)
+                 : "l"(p));
+}
+
 CR_D void kadd(float& s, float& c, float v) {
     const float y = v - c;
     const float t = s + y;
@@ -151,8 +178,8 @@ CR_D void kadd(float& s, float& c, float v) {
 // generic-proxy global writes -> visible to later bulk copies (async proxy)
 CR_D void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;\n" ::: "memory"); }
 
-// barrier among the 256 compute threads (warps 1-8)
-CR_D void compute_sync() { asm volatile("bar.sync 1, 256;\n" ::: "memory"); }
+// barrier among the compute threads (warps 1-16)
+CR_D void compute_sync() { asm volatile("bar.sync 1, %0;\n" ::"n"(NCT) : "memory"); }
 
 CR_D void mbar_arrive(uint64_t* mbar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(mbar)) : "memory");
@@ -162,11 +189,11 @@ CR_D void mbar_arrive(uint64_t* mbar) {
 CR_D uint32_t koff(int row, int k) { return tc::kmajor_offset(row, k, 32); }
 
 // offset (bytes, within one plane) of element (column n, site i) of the W1
-// operand of V: blocks [pass of 256 columns][K-chunk of 32 sites]
+// operand of V: blocks [pass of 128 columns][K-chunk of 32 sites]
 CR_HD size_t v2_offset(const Geo& g, int n, int i) {
-    const int ps = n >> 8, nl = n & 255, kc = i >> 5, il = i & 31;
-    const int width = ps < g.npass1 - 1 ? 256 : g.wlast1;
-    return ((size_t)256 * ps * g.Kp + (size_t)width * 32 * kc) * 2 +
+    const int ps = n / W1_W, nl = n % W1_W, kc = i >> 5, il = i & 31;
+    const int width = ps < g.npass1 - 1 ? W1_W : g.wlast1;
+    return ((size_t)W1_W * ps * g.Kp + (size_t)width * 32 * kc) * 2 +
            tc::kmajor_offset(nl, il, 32);
 }
 
@@ -178,21 +205,22 @@ struct Smem {
     cpx<double>* p;
     cpx<double>* sv;    // s = A p
     cpx<double>* ob;    // Obar_k = (sum_s O_sk) / B
-    double* d;          // Jacobi diagonal (1 without preconditioning)
+    double* d;          // inverse of the Jacobi diagonal (1 without preconditioning)
+    cpx<double>* tot;   // [NCT] row sums of the row groups
     cpx<float>* wbuf;   // [wpc] centred u of the CTA's walkers
     cpx<float>* va;     // [N]
     cpx<float>* vb;     // [M]
-    cpx<float>* xch;    // [256] exchange
-    double* red;        // [64]
+    cpx<float>* xch;    // [NCT] exchange
+    double* red;        // [8 NCW]
     uint64_t* mb;       // mbarriers
     uint32_t* slot;     // TMEM address
     int* flag;          // [0] CTA abort, [1] done
-    double* bc;         // [8] broadcast scalars
+    double* bc;         // [10] broadcast scalars
 };
 
 // mbarrier indices
-enum { FULL1 = 0, EMPTY1 = 3, D1FULL = 6, D1EMPTY = 8, FULL2 = 10, EMPTY2 = 12, D2FULL = 14, GO = 15,
-       NMB = 16 };
+enum { FULL1 = 0, EMPTY1 = NS1, D1FULL = 2 * NS1, D1EMPTY = D1FULL + 2, FULL2 = D1EMPTY + 2,
+       EMPTY2 = FULL2 + 2, D2FULL = EMPTY2 + 2, GO, NMB };
 
 CR_D Smem carve(unsigned char* sm, const Geo& g) {
     Smem s;
@@ -210,6 +238,8 @@ CR_D Smem carve(unsigned char* sm, const Geo& g) {
     p += KS_MAX * 16;
     s.d = (double*)p;
     p += KS_MAX * 8;
+    s.tot = (cpx<double>*)p;
+    p += NCT * 16;
     s.wbuf = (cpx<float>*)p;
     p += (size_t)MAX_WPC * 8;
     s.va = (cpx<float>*)p;
@@ -217,11 +247,11 @@ CR_D Smem carve(unsigned char* sm, const Geo& g) {
     s.vb = (cpx<float>*)p;
     p += 256 * 8;
     s.xch = (cpx<float>*)p;
-    p += 256 * 8;
+    p += NCT * 8;
     s.red = (double*)p;
-    p += 64 * 8;
+    p += 8 * NCW * 8;
     s.bc = (double*)p;
-    p += 8 * 8;
+    p += 10 * 8;
     s.mb = (uint64_t*)p;
     p += NMB * 8;
     s.slot = (uint32_t*)p;
@@ -276,22 +306,51 @@ CR_D bool grid_sync(unsigned* bar, unsigned target, volatile int* flag, int* sta
     return flag[0] == 0;
 }
 
-// The CTA's partials of NV scalar slots (compute threads only): warp sums,
-// then one barrier, then the eight warp values of each slot added in a
-// fixed tree order and written to psc[cta * 8 + slot].
+// Warp sums of NV <= 8 values in 9 float64 additions, not 5 NV: the lanes split
+// the slots among them.  Lane l ends with the sum of slot l / 4.
 template <int NV>
-CR_D void put_psc(double* psc, int cta, const double (&v)[NV], const int (&sl)[NV], double* red) {
-    const int cw = (threadIdx.x >> 5) - 1, lane = threadIdx.x & 31;
+CR_D double warp_sums(const double (&v)[NV]) {
+    const int lane = threadIdx.x & 31;
+    double x[8];
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        const double w = warp_sum(v[q]);
-        if (lane == 0) red[cw * 8 + q] = w;
+    for (int q = 0; q < 8; ++q) x[q] = q < NV ? v[q < NV ? q : 0] : 0.0;
+#pragma unroll
+    for (int h = 4; h >= 1; h >>= 1) {
+        const bool up = lane & (4 * h);
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const double give = up ? x[q] : x[q + h], keep = up ? x[q + h] : x[q];
+            x[q] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+        }
+    }
+    x[0] += __shfl_xor_sync(0xffffffffu, x[0], 2);
+    return x[0] + __shfl_xor_sync(0xffffffffu, x[0], 1);
+}
+
+// The CTA's partials of NV scalar slots (compute threads only): warp sums,
+// then one barrier, then the warp values of each slot added in a fixed tree
+// order and written to psc[cta * 8 + slot].
+template <int NV>
+CR_D void put_psc(double* psc, int cta, const double (&v)[NV], const int (&sl)[NV], double* red,
+                  bool live = true) {
+    const int cw = (threadIdx.x >> 5) - 1, lane = threadIdx.x & 31;
+    if (!live) {  // a warp of zeros
+        if (lane < 8) red[cw * 8 + lane] = 0.0;
+    } else if (NV == 1) {
+        const double w = warp_sum(v[0]);
+        if (lane == 0) red[cw * 8] = w;
+    } else {
+        const double x = warp_sums<NV>(v);
+        if ((lane & 3) == 0) red[cw * 8 + (lane >> 2)] = x;
     }
     compute_sync();
     const int ct = threadIdx.x - 32;
     if (ct < NV) {
         const double* r = red + ct;
-        const double tot = ((r[0] + r[8]) + (r[16] + r[24])) + ((r[32] + r[40]) + (r[48] + r[56]));
+        double tot = 0.0;
+#pragma unroll
+        for (int w = 0; w < NCW; w += 4)
+            tot += (r[8 * w] + r[8 * w + 8]) + (r[8 * w + 16] + r[8 * w + 24]);
         psc[(size_t)cta * 8 + sl[ct]] = tot;
     }
 }
@@ -301,7 +360,7 @@ CR_D void put_psc(double* psc, int cta, const double (&v)[NV], const int (&sl)[N
 template <int NV>
 CR_D void sum_psc(const double* psc, int G, const int (&sl)[NV], double (&out)[NV]) {
     const int lane = threadIdx.x & 31;
-    double v[NV][5];
+    double v[NV][5], s[NV];
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
         const int cc = lane + 32 * m;
@@ -312,7 +371,14 @@ CR_D void sum_psc(const double* psc, int G, const int (&sl)[NV], double (&out)[N
     for (int q = 0; q < NV; ++q) {
         double x = (v[q][0] + v[q][1]) + (v[q][2] + v[q][3]);
         for (int cc = lane + 160; cc < G; cc += 32) x += psc[(size_t)cc * 8 + sl[q]];
-        out[q] = warp_sum(x + v[q][4]);
+        s[q] = x + v[q][4];
+    }
+    if (NV == 1) {
+        out[0] = warp_sum(s[0]);
+    } else {
+        const double tot = warp_sums<NV>(s);
+#pragma unroll
+        for (int q = 0; q < NV; ++q) out[q] = __shfl_sync(0xffffffffu, tot, 4 * q);
     }
 }
 
@@ -342,7 +408,8 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
     const Geo& g = a.g;
     const int N = g.N, M = g.M, P = g.P, B = g.B, G = g.G;
     const int c = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
-    const int ct = t - 32;  // compute-thread index (warps 1-8)
+    const int ct = t >= 32 && t < 32 + NCT ? t - 32 : -1;  // compute-thread index (warps 1-16)
+    const bool copier = t == 32 + NCT;
     Smem s = carve(sm_raw, g);
     volatile int* flag = s.flag;  // [0] CTA abort, [1] solve finished
     const int s0 = c * g.wpc, s1 = min(B, s0 + g.wpc), nw = max(0, s1 - s0);
@@ -422,7 +489,7 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                 uk = (1.0 / d) * f;
                 s.x[kl] = {0.0, 0.0};
                 s.r[kl] = f;
-                s.d[kl] = d;
+                s.d[kl] = 1.0 / d;
                 ff += abs2(f);
                 gam += cmulc(f, uk).x;
             }
@@ -447,36 +514,45 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
     double ff = 0.0, rr = 0.0, gam = 0.0, gam_prev = 1.0, alpha_prev = 1.0;
     // pipeline counters (identical in every role of the CTA)
     uint32_t g1 = 0, u1 = 0, g2 = 0, u2 = 0;
-    // producer only: last copy issued into each stage and last MMA commit, so
-    // that an abort can wait (bounded) for what is still in flight
-    int last1[NS1] = {-1, -1, -1}, last2[2] = {-1, -1}, lastm1 = -1, lastm2 = -1;
-    const int units = g.ntpc * g.npass1;
+    // last copy issued into each stage (copy thread) and last MMA commit (MMA
+    // thread), so that an abort can wait (bounded) for what is still in flight
+    int last1[NS1] = {-1, -1, -1, -1}, last2[2] = {-1, -1}, lastm1 = -1, lastm2 = -1;
+    // a unit: tpu walker tiles x one column pass, D1 in TMEM columns [256 h, +128 tpu)
+    const int units = g.ntpc / g.tpu * g.npass1;
     const int total1 = units * g.nkc1;
-    auto width_of = [&](int ps) { return ps < g.npass1 - 1 ? 256 : g.wlast1; };
+    auto width_of = [&](int ps) { return ps < g.npass1 - 1 ? W1_W : g.wlast1; };
 
     while (ok) {
         // ======================================================= walker phase
         // producer: W1 operand copies start at once (their data was released
         // before the barrier); the MMAs wait for the convergence decision
-        auto load1 = [&](int q) {
-            const uint32_t gq = g1 + q, b = gq % NS1;
+        int cq = 0, ckc = 0, cps = 0, ct0 = 0;  // copy cursor: stage, K-chunk, column pass, first tile
+        auto load1 = [&]() {
+            const uint32_t gq = g1 + cq, b = gq & (NS1 - 1);
             if (gq >= NS1 && !wait_mb(&s.mb[EMPTY1 + b], ((gq / NS1) - 1) & 1, flag, a.bar, a.status))
                 return;
-            const int unit = q / g.nkc1, kc = q % g.nkc1;
-            const int tt = unit / g.npass1, ps = unit % g.npass1, w = width_of(ps);
+            const int w = width_of(cps);
             unsigned char* st = s.ring + (size_t)b * W1_STAGE;
-            tc::mbar_expect_tx(&s.mb[FULL1 + b], (uint32_t)(W1_A + 3 * w * 64));
-            tc::bulk_g2s(st, a.a1 + ((size_t)(c * g.ntpc + tt) * g.nkc1 + kc) * W1_A, W1_A,
-                         &s.mb[FULL1 + b]);
-            const size_t boff = ((size_t)256 * ps * g.Kp + (size_t)w * 32 * kc) * 2;
-            for (int pl = 0; pl < 3; ++pl)
-                tc::bulk_g2s(st + W1_A + pl * W1_B_PLANE, a.v2 + pl * a.v2_plane + boff,
-                             (uint32_t)(w * 64), &s.mb[FULL1 + b]);
+            tc::mbar_expect_tx(&s.mb[FULL1 + b], (uint32_t)(g.tpu * W1_A + 3 * w * 64));
+            const unsigned char* va = a.v2 + ((size_t)W1_W * cps * g.Kp + (size_t)w * 32 * ckc) * 2;
+            for (int pl = 0; pl < 3; ++pl, va += a.v2_plane)
+                tc::bulk_g2s(st + 2 * W1_A + pl * W1_B_PLANE, va, (uint32_t)(w * 64), &s.mb[FULL1 + b]);
+            const unsigned char* sa = a.a1 + ((size_t)(c * g.ntpc + ct0) * g.nkc1 + ckc) * W1_A;
+            tc::bulk_g2s(st, sa, W1_A, &s.mb[FULL1 + b]);
+            if (g.tpu == 2) tc::bulk_g2s(st + W1_A, sa + (size_t)g.nkc1 * W1_A, W1_A, &s.mb[FULL1 + b]);
             last1[b] = (int)gq;
+            ++cq;
+            if (++ckc == g.nkc1) {
+                ckc = 0;
+                if (++cps == g.npass1) {
+                    cps = 0;
+                    ct0 += g.tpu;
+                }
+            }
         };
         const int npre = NS1 - 1 < total1 ? NS1 - 1 : total1;
-        if (t == 0)
-            for (int q = 0; q < npre; ++q) load1(q);
+        if (copier)
+            for (int q = 0; q < npre; ++q) load1();
         if (warp == 1) {
             // the inner products of the current r and u, and the decision
             const int sl6[6] = {S_RR, S_GAM, S_OUR, S_OUI, S_UU, S_FF};
@@ -503,16 +579,16 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
             for (int i = ct; i < N; i += NCT) s.va[i] = a.vab[i];
             for (int j = ct; j < M; j += NCT) s.vb[j] = a.vab[N + j];
         }
-        // the decision reaches warp 0 through GO, the compute warps through
-        // their barrier; flag[1], written once before either, is uniform
-        if (warp == 0) wait_mb(&s.mb[GO], (uint32_t)its & 1, flag, a.bar, a.status);
+        // the decision reaches warps 0 and 17 through GO, the compute warps
+        // through their barrier; flag[1], written once before either, is uniform
+        if (ct < 0) wait_mb(&s.mb[GO], (uint32_t)its & 1, flag, a.bar, a.status);
         if (ct >= 0) compute_sync();
         ff = s.bc[0];
         rr = s.bc[1];
         gam = s.bc[6];
         if (flag[1]) {
             // finished: let the copies issued above land, then leave
-            if (t == 0)
+            if (copier)
                 for (int q = 0; q < npre; ++q) {
                     const uint32_t gq = g1 + q;
                     tc::mbar_wait(&s.mb[FULL1 + gq % NS1], (gq / NS1) & 1, WAIT_LIMIT);
@@ -527,58 +603,69 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
         double ww = 0.0;  // sum |w_s|^2 of this thread's walkers
         if (warp == 0) {
             if (lane == 0) {
-                // ----------------------------------------- W1 producer / MMA
-                for (int q = 0; q < total1; ++q) {
-                    if (q + NS1 - 1 < total1 && q + NS1 - 1 >= npre) load1(q + NS1 - 1);
-                    const uint32_t gq = g1 + q, b = gq % NS1;
-                    const int unit = q / g.nkc1, kc = q % g.nkc1, ps = unit % g.npass1;
-                    const uint32_t uu1 = u1 + unit, h = uu1 & 1;
-                    if (kc == 0 && uu1 >= 2)
-                        wait_mb(&s.mb[D1EMPTY + h], ((uu1 >> 1) - 1) & 1, flag, a.bar, a.status);
-                    wait_mb(&s.mb[FULL1 + b], (gq / NS1) & 1, flag, a.bar, a.status);
-                    tc::fence_after_sync();
-                    const int w = width_of(ps);
-                    const uint32_t idesc = tc::make_idesc_bf16(128, w);
-                    const uint32_t sa = tc::smem_u32(s.ring + (size_t)b * W1_STAGE);
+                // ------------------------------------------------- W1 MMAs
+                const uint64_t d0 = tc::make_desc(tc::smem_u32(s.ring), 128, 512);
+                uint32_t gq = g1, uu1 = u1;
+                for (int un = 0; un < units; un += g.npass1)
+                    for (int ps = 0; ps < g.npass1; ++ps, ++uu1) {
+                        const uint32_t h = uu1 & 1, idesc = tc::make_idesc_bf16(128, width_of(ps));
+                        if (uu1 >= 2)
+                            wait_mb(&s.mb[D1EMPTY + h], ((uu1 >> 1) - 1) & 1, flag, a.bar, a.status);
+                        for (int kc = 0; kc < g.nkc1; ++kc, ++gq) {
+                            const uint32_t b = gq & (NS1 - 1);
+                            wait_mb(&s.mb[FULL1 + b], (gq / NS1) & 1, flag, a.bar, a.status);
+                            tc::fence_after_sync();
+                            uint64_t ad = d0 + b * (W1_STAGE >> 4);
+                            const uint64_t bd = ad + (2 * W1_A >> 4);
+                            uint32_t dt = taddr + 256 * h;
+                            for (int i = 0; i < g.tpu; ++i, ad += W1_A >> 4, dt += W1_W) {
+                                // small terms first: they are added to a small accumulator
 #pragma unroll
-                    for (int ks = 0; ks < 2; ++ks)
+                                for (int pl = 2; pl >= 0; --pl)
 #pragma unroll
-                        for (int pl = 0; pl < 3; ++pl) {
-                            const uint64_t ad = tc::make_desc(sa + ks * 256, 128, 512);
-                            const uint64_t bd =
-                                tc::make_desc(sa + W1_A + pl * W1_B_PLANE + ks * 256, 128, 512);
-                            tc::mma_bf16(taddr + 256 * h, ad, bd, idesc, (kc | ks | pl) != 0);
+                                    for (int ks = 0; ks < 2; ++ks)
+                                        tc::mma_bf16(dt, ad + ks * 16, bd + ((pl * W1_B_PLANE + ks * 256) >> 4),
+                                                     idesc, kc != 0 || pl != 2 || ks != 0);
+                            }
+                            tc::commit(&s.mb[EMPTY1 + b]);
                         }
-                    tc::commit(&s.mb[EMPTY1 + b]);
-                    lastm1 = (int)gq;
-                    if (kc == g.nkc1 - 1) tc::commit(&s.mb[D1FULL + h]);
-                }
+                        tc::commit(&s.mb[D1FULL + h]);
+                    }
+                lastm1 = (int)gq - 1;
             }
+            __syncwarp();
+        } else if (ct < 0) {
+            if (copier)
+                while (cq < total1 && !flag[0]) load1();
             __syncwarp();
         } else {
             // --------------------------------------------- W1 compute warps
-            const int lb = warp & 3, hf = (warp - 1) >> 2, row = 32 * lb + lane;
-            const bool vecT = (M & 1) == 0;
+            // a TMEM lane block is read by four warps: two tiles x two column
+            // splits, or four splits of one tile; each thread sums its walker's
+            // u over its 16-column groups (8 hidden units)
+            const int lb = warp & 3, qd = (warp - 1) >> 2, row = 32 * lb + lane;
+            const int nsp = 4 / g.tpu, ti = qd / nsp, sp = qd % nsp;
+            // whole 32-byte sectors per lane: rows are M apart, and next to the
+            // operand ring there is no L1 to keep the other half of one
+            const bool vecT = (M & 3) == 0 && ((uintptr_t)a.T & 31) == 0;
             cpx<float> uacc = {0.f, 0.f};
             for (int unit = 0; unit < units; ++unit) {
-                const int tt = unit / g.npass1, ps = unit % g.npass1;
+                const int tt = unit / g.npass1 * g.tpu + ti, ps = unit % g.npass1;
                 const uint32_t uu1 = u1 + unit, h = uu1 & 1;
                 const int sl = tt * g.trows + row;
                 const bool valid = row < g.trows && sl < nw;
                 const int sw = s0 + sl;
                 const cpx<float>* Tr = a.T + (size_t)sw * M;
                 const int w = width_of(ps), ngr = w / 16;
-                // T of a 16-column group (8 hidden units) as four 16-byte
-                // loads, fetched two groups ahead of its use
+                // T of a group as four 16-byte loads, fetched a group ahead of its use
                 auto fetchT = [&](int grp, float4* tv) {
-                    const int j0 = 128 * ps + 8 * grp;
+                    const int j0 = W1_W / 2 * ps + 8 * grp;
                     if (grp >= ngr || !valid) {
 #pragma unroll
                         for (int q = 0; q < 4; ++q) tv[q] = make_float4(0.f, 0.f, 0.f, 0.f);
                     } else if (vecT && j0 + 8 <= M) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            tv[q] = __ldg(reinterpret_cast<const float4*>(Tr + j0) + q);
+                        ldg32(Tr + j0, &tv[0], &tv[1]);
+                        ldg32(Tr + j0 + 4, &tv[2], &tv[3]);
                     } else {
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
@@ -589,17 +676,16 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                         }
                     }
                 };
-                float4 tc0[4], tc1[4], tc2[4];
-                fetchT(hf, tc0);
-                fetchT(hf + 2, tc1);
+                float4 tc0[4], tc1[4];
+                fetchT(sp, tc0);
                 if (ps == 0) {
-                    // sigma . va: the two threads of a row take alternate
-                    // 16-site blocks of the row (16-byte loads when N % 16 == 0)
+                    // sigma . va: the threads of a row take 16-site blocks in turn
+                    // (16-byte loads when N % 16 == 0)
                     uacc = {0.f, 0.f};
                     if (valid) {
                         const int8_t* sr = a.spins + (size_t)sw * N;
                         if ((N & 15) == 0) {
-                            for (int b16 = hf; b16 < N / 16; b16 += 2) {
+                            for (int b16 = sp; b16 < N / 16; b16 += nsp) {
                                 const int4 raw = __ldg(reinterpret_cast<const int4*>(sr) + b16);
                                 const int8_t* sv = reinterpret_cast<const int8_t*>(&raw);
 #pragma unroll
@@ -607,17 +693,17 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                                     uacc = uacc + (float)sv[q] * s.va[16 * b16 + q];
                             }
                         } else {
-                            for (int i = hf; i < N; i += 2) uacc = uacc + (float)sr[i] * s.va[i];
+                            for (int i = sp; i < N; i += nsp) uacc = uacc + (float)sr[i] * s.va[i];
                         }
                     }
                 }
                 wait_mb(&s.mb[D1FULL + h], (uu1 >> 1) & 1, flag, a.bar, a.status);
                 tc::fence_after_sync();
-                for (int grp = hf; grp < ngr; grp += 2) {
-                    fetchT(grp + 4, tc2);
+                for (int grp = sp; grp < ngr; grp += nsp) {
+                    fetchT(grp + nsp, tc1);
                     float d[16];
-                    tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + 256 * h + 16 * grp, d);
-                    const int j0 = 128 * ps + 8 * grp;
+                    tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + 256 * h + W1_W * ti + 16 * grp, d);
+                    const int j0 = W1_W / 2 * ps + 8 * grp;
 #pragma unroll
                     for (int q = 0; q < 8; ++q) {
                         const int j = j0 + q;
@@ -628,21 +714,19 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                         uacc = uacc + tj * x;  // tj = 0 past M and on invalid rows
                     }
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        tc0[q] = tc1[q];
-                        tc1[q] = tc2[q];
-                    }
+                    for (int q = 0; q < 4; ++q) tc0[q] = tc1[q];
                 }
                 tc::fence_before_sync();
                 mbar_arrive(&s.mb[D1EMPTY + h]);
                 if (ps == g.npass1 - 1) {
-                    // u of the tile's rows: the two column halves meet
-                    if (hf == 1) s.xch[row] = uacc;
+                    // u of the tile's rows: the splits meet
+                    if (sp > 0) s.xch[(ti * nsp + sp) * 128 + row] = uacc;
                     compute_sync();
-                    if (hf == 0 && row < g.trows && sl < g.wpc) {
+                    if (sp == 0 && row < g.trows && sl < g.wpc) {
                         cpx<float> wv = {0.f, 0.f};
                         if (valid) {
-                            const cpx<float> u = uacc + s.xch[row];
+                            cpx<float> u = uacc;
+                            for (int r = 1; r < nsp; ++r) u = u + s.xch[(ti * nsp + r) * 128 + row];
                             if (a.u_out) a.u_out[sw] = u;
                             wv = u - ubar32;
                             ww += (double)abs2(wv);
@@ -665,7 +749,7 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
         // walkers' loads in flight; each site's nsub partial sums are then
         // added in a fixed order, through the operand ring (idle here).
         if (ct >= 0) {
-            const int NG = (N + 15) / 16, nsub = NCT / NG;
+            const int NG = (N + 15) / 16, nsub = min(NCT / NG, 32);
             const int b16 = ct % NG, sub = ct / NG;
             cpx<float>* xa = (cpx<float>*)s.ring;  // [nsub][NG * 16]
             if (sub < nsub) {
@@ -726,60 +810,57 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
             const size_t stage2 = (size_t)g.nbp * 3 * Y_BLK + (size_t)g.Np * 64;
             if (warp == 0) {
                 if (lane == 0) {
-                    // ------------------------------------ W2 producer / MMA
-                    auto load = [&](int wc) {
-                        const uint32_t gq = g2 + wc, b = gq & 1;
-                        if (gq >= 2 && !wait_mb(&s.mb[EMPTY2 + b], ((gq >> 1) - 1) & 1, flag, a.bar,
-                                                a.status))
-                            return;
-                        unsigned char* st = s.ring + b * stage2 + (size_t)g.nbp * 3 * Y_BLK;
-                        tc::mbar_expect_tx(&s.mb[FULL2 + b], (uint32_t)(g.Np * 64));
-                        tc::bulk_g2s(st, a.b2 + ((size_t)c * g.nwc + wc) * g.Np * 64,
-                                     (uint32_t)(g.Np * 64), &s.mb[FULL2 + b]);
-                        last2[b] = (int)gq;
-                    };
+                    // --------------------------------------------- W2 MMAs
                     const uint32_t idesc = tc::make_idesc_bf16(128, g.Np);
-                    load(0);
+                    const uint64_t d0 = tc::make_desc(tc::smem_u32(s.ring), 128, 512);
+                    const uint64_t so = (uint64_t)(g.nbp * 3 * Y_BLK) >> 4, po = (uint64_t)(g.nbp * Y_BLK) >> 4;
                     for (int wc = 0; wc < g.nwc; ++wc) {
-                        if (wc + 1 < g.nwc) load(wc + 1);
                         const uint32_t gq = g2 + wc, b = gq & 1;
                         wait_mb(&s.mb[FULL2 + b], (gq >> 1) & 1, flag, a.bar, a.status);
                         tc::fence_after_sync();
-                        const uint32_t sy = tc::smem_u32(s.ring + b * stage2);
-                        const uint32_t ss = sy + (uint32_t)(g.nbp * 3 * Y_BLK);
+                        const uint64_t yd = d0 + b * (stage2 >> 4), sd = yd + so;
                         for (int nb = 0; nb < nbq; ++nb)
 #pragma unroll
-                            for (int pl = 0; pl < 3; ++pl)
+                            for (int pl = 2; pl >= 0; --pl)
 #pragma unroll
-                                for (int ks = 0; ks < 2; ++ks) {
-                                    const uint64_t ad =
-                                        tc::make_desc(sy + (pl * g.nbp + nb) * Y_BLK + ks * 256, 128, 512);
-                                    const uint64_t bd = tc::make_desc(ss + ks * 256, 128, 512);
-                                    tc::mma_bf16(taddr + nb * g.Np, ad, bd, idesc, (wc | pl | ks) != 0);
-                                }
+                                for (int ks = 0; ks < 2; ++ks)
+                                    tc::mma_bf16(taddr + nb * g.Np, yd + pl * po + nb * (Y_BLK >> 4) + ks * 16,
+                                                 sd + ks * 16, idesc, wc != 0 || pl != 2 || ks != 0);
                         tc::commit(&s.mb[EMPTY2 + b]);
                         lastm2 = (int)gq;
                     }
                     tc::commit(&s.mb[D2FULL]);
                 }
                 __syncwarp();
+            } else if (ct < 0) {
+                if (copier) {
+                    const unsigned char* src = a.b2 + (size_t)c * g.nwc * g.Np * 64;
+                    for (int wc = 0; wc < g.nwc && !flag[0]; ++wc, src += (size_t)g.Np * 64) {
+                        const uint32_t gq = g2 + wc, b = gq & 1;
+                        if (gq >= 2 && !wait_mb(&s.mb[EMPTY2 + b], ((gq >> 1) - 1) & 1, flag, a.bar, a.status))
+                            break;
+                        tc::mbar_expect_tx(&s.mb[FULL2 + b], (uint32_t)(g.Np * 64));
+                        tc::bulk_g2s(s.ring + b * stage2 + (size_t)g.nbp * 3 * Y_BLK, src,
+                                     (uint32_t)(g.Np * 64), &s.mb[FULL2 + b]);
+                        last2[b] = (int)gq;
+                    }
+                }
+                __syncwarp();
             } else {
                 // ---------------------------------------- W2 compute warps
-                const int tpj = NCT / Jp;  // threads per hidden unit: 2 or 4
-                const int j = jp0 + ct % Jp;
-                const int ng = 4 / tpj;    // walker groups of 8 per thread and chunk (1 or 2)
+                const int tpj = NCT / Jp;  // threads per hidden unit: 4 or 8
+                const int j = jp0 + ct % Jp, grp = ct / Jp;
+                const bool live = grp < 4;  // a chunk has four groups of 8 walkers
                 float bsx = 0.f, bsy = 0.f, bcx = 0.f, bcy = 0.f;
                 // T of this thread's walkers of a chunk, fetched one chunk ahead
                 // (compile-time indices throughout, so the buffers stay in registers)
-                cpx<float> tcur[2][8], tnxt[2][8];
+                cpx<float> tcur[8], tnxt[8];
+                const bool mine = live && j < M;
+                const cpx<float>* Tj = a.T + (size_t)(s0 + grp * 8) * M + j;
 #define FCG_FETCH_T(WC, TV)                                                                       \
-    _Pragma("unroll") for (int gi = 0; gi < 2; ++gi) {                                            \
-        const int grp = ct / Jp + gi * tpj;                                                       \
-        _Pragma("unroll") for (int q = 0; q < 8; ++q) {                                           \
-            const int sl = (WC) * 32 + grp * 8 + q;                                               \
-            TV[gi][q] = (gi < ng && sl < nw && j < M) ? ldg(a.T + (size_t)(s0 + sl) * M + j)       \
-                                                      : cpx<float>{0.f, 0.f};                     \
-        }                                                                                         \
+    _Pragma("unroll") for (int q = 0; q < 8; ++q) {                                               \
+        const int sl = (WC) * 32 + grp * 8 + q;                                                   \
+        TV[q] = (mine && sl < nw) ? ldg(Tj + (size_t)((WC) * 32 + q) * M) : cpx<float>{0.f, 0.f}; \
     }
                 FCG_FETCH_T(0, tcur)
                 for (int wc = 0; wc < g.nwc; ++wc) {
@@ -790,17 +871,14 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                     if (gq >= 2) wait_mb(&s.mb[EMPTY2 + b], ((gq >> 1) - 1) & 1, flag, a.bar, a.status);
                     tc::fence_after_sync();
                     unsigned char* sy = s.ring + b * stage2;
-#pragma unroll
-                    for (int gi = 0; gi < 2; ++gi) {
-                        if (gi >= ng) break;
-                        const int grp = ct / Jp + gi * tpj;
+                    if (live) {
                         __nv_bfloat16 h[2][8], m[2][8], l[2][8];
 #pragma unroll
                         for (int q = 0; q < 8; ++q) {
                             const int sl = wc * 32 + grp * 8 + q;
                             // walkers past the CTA's range contribute exact zeros (their
                             // slots of wbuf are never written)
-                            const cpx<float> y = sl < nw ? conj(tcur[gi][q]) * s.wbuf[sl] : cpx<float>{0.f, 0.f};
+                            const cpx<float> y = sl < nw ? conj(tcur[q]) * s.wbuf[sl] : cpx<float>{0.f, 0.f};
                             kadd(bsx, bcx, y.x);
                             kadd(bsy, bcy, y.y);
                             split3(y.x, &h[0][q], &m[0][q], &l[0][q]);
@@ -818,18 +896,16 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                     tc::fence_proxy_async();
                     mbar_arrive(&s.mb[FULL2 + b]);
 #pragma unroll
-                    for (int gi = 0; gi < 2; ++gi)
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) tcur[gi][q] = tnxt[gi][q];
+                    for (int q = 0; q < 8; ++q) tcur[q] = tnxt[q];
                 }
 #undef FCG_FETCH_T
                 // the pass's D2^T rows -> partial row (W part); b-sums
                 wait_mb(&s.mb[D2FULL], u2 & 1, flag, a.bar, a.status);
                 tc::fence_after_sync();
-                const int lb = warp & 3, hf = (warp - 1) >> 2, row = 32 * lb + lane;
+                const int lb = warp & 3, qd = (warp - 1) >> 2, row = 32 * lb + lane;
                 for (int nb = 0; nb < nbq; ++nb) {
                     const int nl = 128 * nb + row, jj = jp0 + (nl >> 1), cmp = nl & 1;
-                    for (int grp = hf; grp < g.Np / 16; grp += 2) {
+                    for (int grp = qd; grp < g.Np / 16; grp += 4) {
                         float d[16];
                         tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + nb * g.Np + 16 * grp, d);
                         if (jj < M)
@@ -869,89 +945,96 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
             const int sl1[1] = {S_WW};
             double v1[1];
             sum_psc<1>(a.psc, G, sl1, v1);
-            if (lane == 0) s.bc[5] = v1[0];
+            // delta = (u, A u) = (1/B) sum_s |w_s|^2 + lambda |u|^2; one thread
+            // does the scalars (float64 divisions of all warps queue up)
+            const double delta = v1[0] * invB + a.shift * uu;
+            // (p, A p) by the recurrence, delta - beta^2 (p_prev, A p_prev); it holds
+            // while the directions stay A-conjugate.  When rounding has eroded that
+            // (float32-accurate products at a large condition number) it can come
+            // out tiny or negative: then the recurrence restarts with beta = 0
+            // (p = u, s = A u, a steepest-descent step, whose denominator delta
+            // is a sum of squares).
+            if (lane == 0) {
+                const double beta0 = its == 0 ? 0.0 : gam / gam_prev;
+                const double den = its == 0 ? delta : delta - beta0 * gam / alpha_prev;
+                const bool restart = its == 0 || !(den > 1e-6 * delta);
+                s.bc[5] = restart ? 0.0 : beta0;
+                s.bc[8] = gam / (restart ? delta : den);
+            }
         }
         __syncthreads();
-        // delta = (u, A u) = (1/B) sum_s |w_s|^2 + lambda |u|^2
-        const double delta = s.bc[5] * invB + a.shift * uu;
-        // (p, A p) by the recurrence, delta - beta^2 (p_prev, A p_prev); it holds
-        // while the directions stay A-conjugate.  When rounding has eroded that
-        // (float32-accurate products at a large condition number) it can come
-        // out tiny or negative: then the recurrence restarts with beta = 0
-        // (p = u, s = A u, a steepest-descent step, whose denominator delta
-        // is a sum of squares).
-        const double beta0 = its == 0 ? 0.0 : gam / gam_prev;
-        const double den = its == 0 ? delta : delta - beta0 * gam / alpha_prev;
-        const bool restart = its == 0 || !(den > 1e-6 * delta);
-        const double beta = restart ? 0.0 : beta0;
-        const double alpha = gam / (restart ? delta : den);
+        const double beta = s.bc[5], alpha = s.bc[8];
         if (ct >= 0) {
             double r2 = 0.0, gm = 0.0, our = 0.0, oui = 0.0, u2s = 0.0;
-            const int L = k1 - k0;
-            const int tpk = L <= 64 ? 4 : (L <= 128 ? 2 : 1);
-            const int cg = ct % tpk, per = NCT / tpk;
+            // Row sums: a warp takes 32 neighbouring parameters and every
+            // ng-th partial row, as many row groups as there are warps for.
+            // Float64 work (a warp instruction takes the SM 16 cycles,
+            // however many lanes are live) is then left to full warps.
+            const int L = k1 - k0, cw = ct >> 5, nlw = (L + 31) >> 5, ng = nlw ? NCW / nlw : 1;
+            const int rg = nlw ? cw / nlw : 0, kk = nlw ? 32 * (cw % nlw) + lane : 0, k = k0 + kk;
             const cpx<double> du = ubar - ccast<double>(ubar32);
-            constexpr int BATCH = 40;
-            for (int base = 0; base < L; base += per) {
-                const int kk = base + ct / tpk, k = k0 + kk;
-                double tx = 0.0, ty = 0.0;
-                if (kk < L) {
-                    float sx = 0.f, sy = 0.f, cx = 0.f, cy = 0.f;
-                    // rows cg, cg + tpk, ... with BATCH loads in flight
-                    for (int cb = cg; cb < G; cb += BATCH * tpk) {
-                        float2 v[BATCH];
+            constexpr int BATCH = 19;
+            double tx = 0.0, ty = 0.0;
+            if (rg < ng && kk < L) {
+                float sx = 0.f, sy = 0.f, cx = 0.f, cy = 0.f;
+                // rows rg, rg + ng, ... with BATCH loads in flight
+                for (int cb = rg; cb < G; cb += BATCH * ng) {
+                    float2 v[BATCH];
 #pragma unroll
-                        for (int q = 0; q < BATCH; ++q) {
-                            const int cc = cb + q * tpk;
-                            v[q] = cc < G ? *reinterpret_cast<const float2*>(a.part + 2 * ((size_t)cc * P + k))
-                                          : make_float2(0.f, 0.f);
-                        }
+                    for (int q = 0; q < BATCH; ++q) {
+                        const int cc = cb + q * ng;
+                        v[q] = cc < G ? *reinterpret_cast<const float2*>(a.part + 2 * ((size_t)cc * P + k))
+                                      : make_float2(0.f, 0.f);
+                    }
 #pragma unroll
-                        for (int q = 0; q < BATCH; ++q) {
-                            kadd(sx, cx, v[q].x);
-                            kadd(sy, cy, v[q].y);
-                        }
+                    for (int q = 0; q < BATCH; ++q) {
+                        kadd(sx, cx, v[q].x);
+                        kadd(sy, cy, v[q].y);
                     }
-                    tx = (double)sx - (double)cx;
-                    ty = (double)sy - (double)cy;
                 }
-                // fixed-order combination of the tpk lanes (bitwise identical in each)
-                for (int o = 1; o < tpk; o <<= 1) {
-                    tx += __shfl_xor_sync(0xffffffffu, tx, o);
-                    ty += __shfl_xor_sync(0xffffffffu, ty, o);
+                tx = (double)sx - (double)cx;
+                ty = (double)sy - (double)cy;
+            }
+            if (ng > 1) {
+                s.tot[ct] = {tx, ty};
+                compute_sync();
+            }
+            if (rg == 0 && kk < L) {
+                // the row groups in a fixed order
+                for (int r = 1; r < ng; ++r) {
+                    tx += s.tot[ct + 32 * nlw * r].x;
+                    ty += s.tot[ct + 32 * nlw * r].y;
                 }
-                if (kk < L && cg == 0) {
-                    const cpx<double> uk = (1.0 / s.d[kk]) * s.r[kk];
-                    // (A u)_k = (S + lambda) u: the centred O^dag w with the
-                    // rounding of ubar put back
-                    const cpx<double> auk =
-                        invB * cpx<double>{tx, ty} - conj(s.ob[kk]) * du + a.shift * uk;
-                    if (a.apply_only) {
-                        Ap[k] = auk;
-                    } else {
-                        const cpx<double> pk = uk + beta * s.p[kk];
-                        const cpx<double> sk = auk + beta * s.sv[kk];
-                        s.p[kk] = pk;
-                        s.sv[kk] = sk;
-                        s.x[kk] = s.x[kk] + alpha * pk;
-                        const cpx<double> rk = s.r[kk] - alpha * sk;
-                        s.r[kk] = rk;
-                        const cpx<double> un = (1.0 / s.d[kk]) * rk;
-                        emit_p(a, k, un);
-                        r2 += abs2(rk);
-                        gm += cmulc(rk, un).x;
-                        const cpx<double> ou = s.ob[kk] * un;
-                        our += ou.x;
-                        oui += ou.y;
-                        u2s += abs2(un);
-                    }
+                const cpx<double> uk = s.d[kk] * s.r[kk];
+                // (A u)_k = (S + lambda) u: the centred O^dag w with the
+                // rounding of ubar put back
+                const cpx<double> auk =
+                    invB * cpx<double>{tx, ty} - conj(s.ob[kk]) * du + a.shift * uk;
+                if (a.apply_only) {
+                    Ap[k] = auk;
+                } else {
+                    const cpx<double> pk = uk + beta * s.p[kk];
+                    const cpx<double> sk = auk + beta * s.sv[kk];
+                    s.p[kk] = pk;
+                    s.sv[kk] = sk;
+                    s.x[kk] = s.x[kk] + alpha * pk;
+                    const cpx<double> rk = s.r[kk] - alpha * sk;
+                    s.r[kk] = rk;
+                    const cpx<double> un = s.d[kk] * rk;
+                    emit_p(a, k, un);
+                    r2 += abs2(rk);
+                    gm += cmulc(rk, un).x;
+                    const cpx<double> ou = s.ob[kk] * un;
+                    our += ou.x;
+                    oui += ou.y;
+                    u2s += abs2(un);
                 }
             }
             if (!a.apply_only) {
                 fence_proxy_async_global();
                 const double pv[5] = {r2, gm, our, oui, u2s};
                 const int ps[5] = {S_RR, S_GAM, S_OUR, S_OUI, S_UU};
-                put_psc<5>(a.psc, c, pv, ps, s.red);
+                put_psc<5>(a.psc, c, pv, ps, s.red, rg == 0);
             }
         }
         gam_prev = gam;
@@ -972,11 +1055,13 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
     // nothing of this CTA is in flight past here on the normal path; after an
     // abort, wait (bounded) for the copies it issued to land and for its last
     // MMA commits, before the shared memory and TMEM are released
-    if (flag[0] && t == 0) {
+    if (flag[0] && copier) {
         for (int b = 0; b < NS1; ++b)
             if (last1[b] >= 0) tc::mbar_wait(&s.mb[FULL1 + b], (last1[b] / NS1) & 1, WAIT_LIMIT);
         for (int b = 0; b < 2; ++b)
             if (last2[b] >= 0) tc::mbar_wait(&s.mb[FULL2 + b], (last2[b] >> 1) & 1, WAIT_LIMIT);
+    }
+    if (flag[0] && t == 0) {
         if (lastm1 >= 0)
             tc::mbar_wait(&s.mb[EMPTY1 + lastm1 % NS1], (lastm1 / NS1) & 1, WAIT_LIMIT);
         if (lastm2 >= 0) tc::mbar_wait(&s.mb[EMPTY2 + (lastm2 & 1)], (lastm2 >> 1) & 1, WAIT_LIMIT);
@@ -987,6 +1072,9 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
 }
 
 // ------------------------------------------------------------------ host
+
+// W1 walker tiles of a CTA with wpc walkers: one, or pairs.
+static int w1_tiles(int wpc) { return wpc > 128 ? 2 * ((wpc + 255) / 256) : 1; }
 
 static bool fcg_geometry(const cr_ctx* c, int B, Geo* g) {
     const int N = c->N, M = c->M;
@@ -1005,13 +1093,14 @@ static bool fcg_geometry(const cr_ctx* c, int B, Geo* g) {
     g->G = G;
     g->wpc = (B + G - 1) / G;
     if (g->wpc > MAX_WPC) return false;
-    g->ntpc = (g->wpc + 127) / 128;
+    g->tpu = g->wpc > 128 ? 2 : 1;
+    g->ntpc = w1_tiles(g->wpc);
     g->trows = (g->wpc + g->ntpc - 1) / g->ntpc;
     g->Kp = ((N + 31) / 32) * 32;
     g->nkc1 = g->Kp / 32;
     const int nc1 = ((2 * M + 15) / 16) * 16;
-    g->npass1 = (nc1 + 255) / 256;
-    g->wlast1 = nc1 - 256 * (g->npass1 - 1);
+    g->npass1 = (nc1 + W1_W - 1) / W1_W;
+    g->wlast1 = nc1 - W1_W * (g->npass1 - 1);
     g->Np = ((N + 15) / 16) * 16;
     g->nb2 = (2 * M + 127) / 128;
     g->nbp = g->nb2 < 2 ? g->nb2 : 2;
@@ -1022,8 +1111,8 @@ static bool fcg_geometry(const cr_ctx* c, int B, Geo* g) {
     const size_t r1 = (size_t)NS1 * W1_STAGE;
     const size_t r2 = 2 * ((size_t)g->nbp * 3 * Y_BLK + (size_t)g->Np * 64);
     g->ring = r1 > r2 ? r1 : r2;
-    g->smem = g->ring + (size_t)KS_MAX * 88 + (size_t)MAX_WPC * 8 + 3 * 256 * 8 + 64 * 8 + 8 * 8 +
-              NMB * 8 + 16 + 16;
+    g->smem = g->ring + (size_t)KS_MAX * 88 + (size_t)MAX_WPC * 8 + 2 * 256 * 8 + NCT * 24 +
+              8 * NCW * 8 + 10 * 8 + NMB * 8 + 16 + 16;
     return g->smem <= 227 * 1024;
 }
 
@@ -1039,19 +1128,17 @@ void fcg_sizes(const cr_ctx* c, size_t* a1, size_t* b2, size_t* v2plane, size_t*
     fcg_geometry(c, c->max_walkers, &g);
     // the largest tile / chunk counts over walker counts up to max_walkers:
     // every CTA count G <= n_sm with wpc = ceil(B / G) <= ceil(max_walkers / G)
-    const int ntpc = (((c->max_walkers + c->n_sm - 1) / c->n_sm) + 127) / 128;
     size_t nt = 0, nc = 0;
     for (int G = 1; G <= c->n_sm; ++G) {
         const int wpc = (c->max_walkers + G - 1) / G;
         if (wpc > MAX_WPC) continue;
-        const size_t t1 = (size_t)G * ((wpc + 127) / 128), t2 = (size_t)G * ((wpc + 31) / 32);
+        const size_t t1 = (size_t)G * w1_tiles(wpc), t2 = (size_t)G * ((wpc + 31) / 32);
         if (t1 > nt) nt = t1;
         if (t2 > nc) nc = t2;
     }
-    (void)ntpc;
     *a1 = nt * g.nkc1 * W1_A;
     *b2 = nc * (size_t)g.Np * 64;
-    *v2plane = (size_t)256 * g.npass1 * g.Kp * 2;
+    *v2plane = (size_t)W1_W * g.npass1 * g.Kp * 2;
     *part = (size_t)c->n_sm * c->P * 8;
 }
 
