@@ -10,6 +10,8 @@
 //   trsm_kernel       L_IJ = A_IJ X_JJ^dag, I > J             (64 x 64 tiles)
 //   syrk_tc_kernel    A_IK -= L_IJ L_KJ^dag, J < K <= I       (mixed: tcgen05)
 //   syrk_kernel       the same on the FMA pipes               (float32)
+// (mixed: the first panel of a pair updates the second's columns only, and
+// the rest of A is read and written once per pair)
 // The inverses X_JJ turn the panel's triangular solve into a product, and,
 // merged pairwise into the inverses of 512 x 512 diagonal blocks, the
 // triangular solves of the refinement into two products per 512 rows.
@@ -174,12 +176,13 @@ CR_D void tile_step(const cf (*As)[NB + 1], const cf (*Bs)[BP], int tx, int ty, 
 // explicit S takes.
 constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded mbarrier polls
 constexpr int TC_ROWS = 256, TC_COLS = 64;  // tile of A
-constexpr int TC_KC = 32, TC_NKC = 2 * NB / TC_KC;
+constexpr int TC_KC = 32, TC_NKC = 2 * NB / TC_KC;  // K tiles of a panel; operands hold two panels
 constexpr int N_TILE = TC_ROWS * TC_KC * 2, M_TILE = 2 * TC_COLS * TC_KC * 2;  // bytes, one plane
 constexpr int TC_STAGE = 3 * (N_TILE + M_TILE);
 constexpr int TC_NSTG = 3;
 constexpr size_t TC_SMEM = (size_t)TC_NSTG * TC_STAGE + 256;
-constexpr int TC_THREADS = 288;
+constexpr int TC_DRAIN = 512;                 // 16 drain warps
+constexpr int TC_THREADS = TC_DRAIN + 64;
 
 CR_D void split3(float x, __nv_bfloat16* hi, __nv_bfloat16* mid, __nv_bfloat16* lo) {
     *hi = __float2bfloat16_rn(x);
@@ -211,10 +214,13 @@ CR_D void put_row(unsigned char* tile, int plane, int row, int kk, const float* 
 
 // L_IJ = A_IJ X_JJ^dag for one 64-row block below block J (full here: it is
 // not the last block).  planes: also the bf16 operands of the trailing
-// update (rows past P are zero there); a thread's outputs are 4 adjacent
-// columns, so it forms 16-byte operand groups from its own registers.
+// update (rows past P are zero there; rows count from the first row below
+// the pair's first panel, second: the pair's second panel); a thread's
+// outputs are 4 adjacent columns, so it forms 16-byte operand groups from its
+// own registers.
 __global__ void __launch_bounds__(256) trsm_kernel(cf* __restrict__ L, int P, int J, cf* __restrict__ X,
-                                                   unsigned char* __restrict__ planes, size_t m_off) {
+                                                   unsigned char* __restrict__ planes, size_t m_off,
+                                                   int second) {
     __shared__ __align__(16) cf As[KT][NB + 1];
     __shared__ __align__(16) cf Bs[KT][BP];
     const int base = J * NB, r0 = base + NB, i0 = r0 + blockIdx.x * NB, ld = lcols(P);
@@ -253,35 +259,45 @@ __global__ void __launch_bounds__(256) trsm_kernel(cf* __restrict__ L, int P, in
             out[1] = make_float4(re[4], re[5], re[6], re[7]);
         }
         if (!planes) continue;
-        const int row = i0 - r0 + r, k = 8 * tx, kc = k / TC_KC, kk = k % TC_KC;
-        put_row(planes + ((size_t)(row / TC_ROWS) * TC_NKC + kc) * 3 * N_TILE, N_TILE, row % TC_ROWS, kk, re);
-        unsigned char* mt = planes + m_off + ((size_t)(row / TC_COLS) * TC_NKC + kc) * 3 * M_TILE;
+        const int row = i0 - r0 + second * NB + r, k = 8 * tx, kc = second * TC_NKC + k / TC_KC, kk = k % TC_KC;
+        put_row(planes + ((size_t)(row / TC_ROWS) * 2 * TC_NKC + kc) * 3 * N_TILE, N_TILE, row % TC_ROWS, kk, re);
+        unsigned char* mt = planes + m_off + ((size_t)(row / TC_COLS) * 2 * TC_NKC + kc) * 3 * M_TILE;
         put_row(mt, M_TILE, 2 * (row % TC_COLS), kk, re);
         put_row(mt, M_TILE, 2 * (row % TC_COLS) + 1, kk, im);
     }
 }
 
-// Tiles of the trailing matrix (from row r0): row block rb takes the column
-// blocks cb <= 4 rb + 3 that exist; tile index 2 rb (rb + 1) + cb.
-// Persistent, 288 threads: warp 0 (one thread) copies operand stages and
-// issues the MMAs, tile t into TMEM columns [256 (t % 2), +256); warps 1-8
-// fetch their part of the tile of A while the MMAs run, subtract and store.
+// Tiles of the matrix below the pair's first panel (from row r0), 256 rows x
+// 64 columns.  npan = 1, after the first panel: the tiles of column block 0,
+// the second panel's.  npan = 2, after the second: row block rb takes the
+// column blocks 1 <= cb <= 4 rb + 3 that exist (tile index 2 rb^2 + rb + cb -
+// 1), one subtraction per panel, but not the first 64 rows, which are done.
+//
+// Bound: 16 bytes of A per entry and update against 1.5 KB of MMA operands,
+// which L2 serves.  A panel at a time (10 x 10 lattice, alpha = 1: P = 10200)
+// the kernel moved A at 3.9 TB/s, waiting for the loads of 8 drain warps: 159
+// launches, 11.4 ms.  In pairs, with 16 drain warps that have a whole tile of
+// A in flight while its MMAs run: SYRK_NOW.
+//
+// Persistent: warp 0 (one thread) issues the MMAs, panel by panel into TMEM
+// columns [256 h, +256), warps 1-16 drain (warp w: lanes 32 (w % 4), rows 64
+// ((w - 1) / 4)), warp 17 (one thread) copies operand stages.
 __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restrict__ Lf, int P, int r0,
-                                                                int ntiles,
+                                                                int npan, int ntiles,
                                                                 const unsigned char* __restrict__ planes,
                                                                 size_t m_off, int* __restrict__ status) {
     extern __shared__ __align__(1024) unsigned char sm[];
     uint64_t* full = (uint64_t*)(sm + TC_NSTG * TC_STAGE);
     uint64_t* empty = full + TC_NSTG;
     uint64_t* dfull = empty + TC_NSTG;  // [2] MMAs of a tile done
-    uint64_t* dempty = dfull + 2;       // [2] TMEM half read by the 256 drain threads
+    uint64_t* dempty = dfull + 2;       // [2] TMEM half read by the drain threads
     uint32_t* slot = (uint32_t*)(dempty + 2);
     volatile int* abort = (volatile int*)(slot + 1);
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     if (t == 0) {
         for (int i = 0; i < 2 * TC_NSTG + 2; ++i) tc::mbar_init(&full[i], 1);
-        tc::mbar_init(&dempty[0], 256);
-        tc::mbar_init(&dempty[1], 256);
+        tc::mbar_init(&dempty[0], TC_DRAIN);
+        tc::mbar_init(&dempty[1], TC_DRAIN);
         tc::fence_mbar_init();
         *abort = 0;
     }
@@ -302,109 +318,133 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
         return false;
     };
     auto tile_of = [&](int idx, int* rb, int* cb) {
-        int r = (int)((sqrtf(1.0f + 2.0f * (float)idx) - 1.0f) * 0.5f);
-        while (2 * r * (r + 1) > idx) --r;
-        while (2 * (r + 1) * (r + 2) <= idx) ++r;
+        if (npan == 1) {
+            *rb = idx;
+            *cb = 0;
+            return;
+        }
+        int r = (int)((sqrtf(1.0f + 8.0f * (float)idx) - 1.0f) * 0.25f);
+        while (2 * r * r + r > idx) --r;
+        while (2 * (r + 1) * (r + 1) + r + 1 <= idx) ++r;
         *rb = r;
-        *cb = idx - 2 * r * (r + 1);
+        *cb = idx - (2 * r * r + r) + 1;
     };
     const int nmine = ntiles > (int)blockIdx.x ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
     if (warp == 0) {
         if (lane == 0) {
             constexpr int PA[6] = {0, 0, 1, 0, 1, 2}, PB[6] = {0, 1, 0, 2, 1, 0};
             const uint32_t idesc = tc::make_idesc_bf16(2 * TC_COLS, TC_ROWS);
-            const int total = nmine * TC_NKC;
-            uint32_t pend = 0, pend_par = 0;
-            int last_g = -1;
+            const uint64_t d0 = tc::make_desc(tc::smem_u32(sm), 128, 16 * TC_KC);
+            uint32_t b = 0, ph = 0;
+            int last = -1, lastph = 0;  // stage of the last commit
             bool ok = true;
-            auto load = [&](int g) {
-                const uint32_t b = g % TC_NSTG;
-                if (g >= TC_NSTG && !wait(&empty[b], ((g - TC_NSTG) / TC_NSTG) & 1)) return false;
-                int rb, cb;
-                tile_of(blockIdx.x + (g / TC_NKC) * gridDim.x, &rb, &cb);
-                const int kc = g % TC_NKC;
-                pend |= 1u << b;
-                pend_par = (pend_par & ~(1u << b)) | (((uint32_t)(g / TC_NSTG) & 1u) << b);
-                unsigned char* st = sm + (size_t)b * TC_STAGE;
-                tc::mbar_expect_tx(&full[b], (uint32_t)TC_STAGE);
-                tc::bulk_g2s(st, planes + ((size_t)rb * TC_NKC + kc) * 3 * N_TILE, 3 * N_TILE, &full[b]);
-                tc::bulk_g2s(st + 3 * N_TILE, planes + m_off + ((size_t)cb * TC_NKC + kc) * 3 * M_TILE,
-                             3 * M_TILE, &full[b]);
-                return true;
-            };
-            for (int g = 0; g < TC_NSTG - 1 && g < total && ok; ++g) ok = load(g);
-            for (int g = 0; g < total && ok; ++g) {
-                const int ti = g / TC_NKC, kc = g % TC_NKC, b = g % TC_NSTG;
-                const uint32_t h = ti & 1;
-                if (kc == 0 && ti >= 2 && !wait(&dempty[h], ((ti - 2) >> 1) & 1)) {
+            for (int gc = 0; gc < nmine * npan && ok; ++gc) {
+                const uint32_t h = gc & 1, dt = taddr + h * 256;
+                if (gc >= 2 && !wait(&dempty[h], ((gc >> 1) - 1) & 1)) {
                     ok = false;
                     break;
                 }
-                if (!wait(&full[b], (g / TC_NSTG) & 1)) {
-                    ok = false;
-                    break;
+                for (int kc = 0; kc < TC_NKC; ++kc) {
+                    if (!wait(&full[b], ph)) {
+                        ok = false;
+                        break;
+                    }
+                    tc::fence_after_sync();
+                    const uint64_t nd = d0 + b * (uint32_t)(TC_STAGE >> 4);
+                    const uint64_t md = nd + (3 * N_TILE >> 4);
+#pragma unroll
+                    for (int ks = 0; ks < TC_KC / 16; ++ks)
+#pragma unroll
+                        for (int pr = 0; pr < 6; ++pr)
+                            tc::mma_bf16(dt, md + (PA[pr] * (M_TILE >> 4) + ks * 16),
+                                         nd + (PB[pr] * (N_TILE >> 4) + ks * 16), idesc,
+                                         kc != 0 || ks != 0 || pr != 0);
+                    tc::commit(&empty[b]);
+                    last = (int)b;
+                    lastph = (int)ph;
+                    if (++b == TC_NSTG) {
+                        b = 0;
+                        ph ^= 1;
+                    }
                 }
-                pend &= ~(1u << b);
-                tc::fence_after_sync();
-                const uint32_t ns = tc::smem_u32(sm + (size_t)b * TC_STAGE), ms = ns + 3 * N_TILE;
-#pragma unroll
-                for (int ks = 0; ks < TC_KC / 16; ++ks)
-#pragma unroll
-                    for (int pr = 0; pr < 6; ++pr)
-                        tc::mma_bf16(taddr + h * 256,
-                                     tc::make_desc(ms + PA[pr] * M_TILE + ks * 256, 128, 16 * TC_KC),
-                                     tc::make_desc(ns + PB[pr] * N_TILE + ks * 256, 128, 16 * TC_KC),
-                                     idesc, !(kc == 0 && ks == 0 && pr == 0));
-                tc::commit(&empty[b]);
-                last_g = g;
-                if (kc == TC_NKC - 1) tc::commit(&dfull[h]);
-                if (g + TC_NSTG - 1 < total && !load(g + TC_NSTG - 1)) ok = false;
+                if (ok) tc::commit(&dfull[h]);
             }
             if (!ok) {
                 *abort = 1;
                 set_status(status, CR_ETIMEOUT);
-                // let copies in flight land and issued MMAs finish (bounded)
-                for (int b = 0; b < TC_NSTG; ++b)
-                    if (pend & (1u << b)) tc::mbar_wait(&full[b], (pend_par >> b) & 1u, WAIT_LIMIT);
-                if (last_g >= 0)
-                    tc::mbar_wait(&empty[last_g % TC_NSTG], (uint32_t)(last_g / TC_NSTG) & 1u, WAIT_LIMIT);
+                // let issued MMAs finish (bounded)
+                if (last >= 0) tc::mbar_wait(&empty[last], (uint32_t)lastph, WAIT_LIMIT);
+            }
+        }
+        __syncwarp();
+    } else if (warp == TC_THREADS / 32 - 1) {
+        if (lane == 0) {
+            uint32_t b = 0, ph = 0, g = 0;
+            bool ok = true;
+            for (int ti = 0; ti < nmine && ok; ++ti) {
+                int rb, cb;
+                tile_of(blockIdx.x + ti * gridDim.x, &rb, &cb);
+                const unsigned char* ns = planes + (size_t)rb * 2 * TC_NKC * 3 * N_TILE;
+                const unsigned char* ms = planes + m_off + (size_t)cb * 2 * TC_NKC * 3 * M_TILE;
+                for (int kc = 0; kc < npan * TC_NKC; ++kc, ++g, ns += 3 * N_TILE, ms += 3 * M_TILE) {
+                    if (g >= TC_NSTG && !wait(&empty[b], ph ^ 1)) {
+                        ok = false;
+                        break;
+                    }
+                    unsigned char* st = sm + (size_t)b * TC_STAGE;
+                    tc::mbar_expect_tx(&full[b], (uint32_t)TC_STAGE);
+                    tc::bulk_g2s(st, ns, 3 * N_TILE, &full[b]);
+                    tc::bulk_g2s(st + 3 * N_TILE, ms, 3 * M_TILE, &full[b]);
+                    if (++b == TC_NSTG) {
+                        b = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+            // every copy lands before the CTA leaves (bounded): the last
+            // stages; where MMAs consumed them all this does not wait
+            for (uint32_t q = 0; q < TC_NSTG && q < g; ++q) {
+                if (b == 0) ph ^= 1;
+                b = b == 0 ? TC_NSTG - 1 : b - 1;
+                tc::mbar_wait(&full[b], ph, WAIT_LIMIT);
             }
         }
         __syncwarp();
     } else {
-        const int lb = warp & 3, c2 = (warp - 1) >> 2;
+        const int lb = warp & 3, c4 = (warp - 1) >> 2;
+        const size_t ld = 2 * (size_t)lcols(P);
         bool ok = true;
+        int gc = 0;
         for (int ti = 0; ti < nmine && ok; ++ti) {
             int rb, cb;
             tile_of(blockIdx.x + ti * gridDim.x, &rb, &cb);
-            const size_t ld = 2 * (size_t)lcols(P);
-            float* Af = Lf + ((size_t)r0 + rb * TC_ROWS + 128 * c2) * ld + 2 * (r0 + cb * TC_COLS) +
+            float* Af = Lf + ((size_t)r0 + rb * TC_ROWS + 64 * c4) * ld + 2 * (r0 + cb * TC_COLS) +
                         32 * lb + lane;
-            // 16 rows at a time, fetched two groups ahead of their use
-            float c[3][16];
-            auto fetch = [&](int ch, float (&v)[16]) {
+            const bool live = npan == 1 || rb > 0 || c4 > 0;  // warp-uniform
+            float c[64];
 #pragma unroll
-                for (int q = 0; q < 16; ++q) v[q] = Af[(16 * ch + q) * ld];
-            };
-            fetch(0, c[0]);
-            fetch(1, c[1]);
-            const uint32_t h = ti & 1;
-            if (!__all_sync(0xffffffffu, wait(&dfull[h], (ti >> 1) & 1))) {
-                ok = false;
-                break;
+            for (int q = 0; q < 64; ++q) c[q] = live ? Af[q * ld] : 0.f;
+            for (int pn = 0; pn < npan; ++pn, ++gc) {
+                const uint32_t h = gc & 1;
+                if (!__all_sync(0xffffffffu, wait(&dfull[h], (gc >> 1) & 1))) {
+                    ok = false;
+                    break;
+                }
+                tc::fence_after_sync();
+#pragma unroll
+                for (int ch = 0; ch < 4; ++ch) {
+                    float v[16];
+                    tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + h * 256 + 64 * c4 + 16 * ch, v);
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) c[16 * ch + q] = __fsub_rn(c[16 * ch + q], v[q]);
+                }
+                tc::fence_before_sync();
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(&dempty[h]))
+                             : "memory");
             }
-            tc::fence_after_sync();
+            if (ok && live)
 #pragma unroll
-            for (int ch = 0; ch < 8; ++ch) {
-                if (ch + 2 < 8) fetch(ch + 2, c[(ch + 2) % 3]);
-                float v[16];
-                tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + h * 256 + 128 * c2 + 16 * ch, v);
-#pragma unroll
-                for (int q = 0; q < 16; ++q) Af[(16 * ch + q) * ld] = __fsub_rn(c[ch % 3][q], v[q]);
-            }
-            tc::fence_before_sync();
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(&dempty[h]))
-                         : "memory");
+                for (int q = 0; q < 64; ++q) Af[q * ld] = c[q];
         }
         if (!ok && t == 32) set_status(status, CR_ETIMEOUT);
     }
@@ -686,9 +726,9 @@ __global__ void __launch_bounds__(1024) refine_check_kernel(int P, double* __res
 
 // Bytes of the trailing update's operands: the N side (rows in blocks of
 // 256), then the M side (two real rows per column).
-size_t n_plane_bytes(int P) { return (size_t)((P + TC_ROWS - 1) / TC_ROWS) * TC_NKC * 3 * N_TILE; }
+size_t n_plane_bytes(int P) { return (size_t)((P + TC_ROWS - 1) / TC_ROWS) * 2 * TC_NKC * 3 * N_TILE; }
 size_t m_plane_bytes(int P) {
-    return (size_t)((P + TC_ROWS - 1) / TC_ROWS) * (TC_ROWS / TC_COLS) * TC_NKC * 3 * M_TILE;
+    return (size_t)((P + TC_ROWS - 1) / TC_ROWS) * (TC_ROWS / TC_COLS) * 2 * TC_NKC * 3 * M_TILE;
 }
 
 cr_status factor32(cr_ctx* c) {
@@ -703,16 +743,18 @@ cr_status factor32(cr_ctx* c) {
         CR_LAUNCH(c, CR_KERNEL_CHOL, potrf_inv_kernel<<<1, 256, 0, c->stream>>>(L, P, J, X, c->d_status));
         const int rows = P - (J + 1) * NB;
         if (rows <= 0) break;
-        const int nrb = (rows + TC_ROWS - 1) / TC_ROWS, ncb = (rows + NB - 1) / NB;
-        // the tensor-core update takes rows in blocks of 256, zero past P
+        // mixed: rows below the first panel of the pair (J - second, + 1), in
+        // blocks of 256, zero past P
+        const int second = tcu ? J & 1 : 0, r0 = (J + 1 - second) * NB;
+        const int nrb = (P - r0 + TC_ROWS - 1) / TC_ROWS, ncb = (P - r0 + NB - 1) / NB;
         CR_LAUNCH(c, CR_KERNEL_CHOL,
-                  trsm_kernel<<<tcu ? 4 * nrb : ncb, 256, 0, c->stream>>>(
-                      L, P, J, X, tcu ? c->chol_pl : nullptr, m_off));
+                  trsm_kernel<<<tcu ? 4 * nrb - second : ncb, 256, 0, c->stream>>>(
+                      L, P, J, X, tcu ? c->chol_pl : nullptr, m_off, second));
         if (tcu) {
-            const int nt = 2 * (nrb - 1) * nrb + ncb;
+            const int nt = second ? 2 * (nrb - 1) * (nrb - 1) + (nrb - 1) + ncb - 1 : nrb;
             CR_LAUNCH(c, CR_KERNEL_CHOL,
                       syrk_tc_kernel<<<nt < c->n_sm ? nt : c->n_sm, TC_THREADS, TC_SMEM, c->stream>>>(
-                          (float*)c->Lf, P, (J + 1) * NB, nt, c->chol_pl, m_off, c->d_status));
+                          (float*)c->Lf, P, r0, 1 + second, nt, c->chol_pl, m_off, c->d_status));
         } else {
             const long long T = nb - J - 1;
             CR_LAUNCH(c, CR_KERNEL_CHOL,
