@@ -208,8 +208,8 @@ struct cr_ctx {
     size_t gram_tiles_cap;
     int gram_key;            // 2 Nm + (H wanted) of the tile list held, 0 if none
     // estimator sums on the tensor cores (mixed contexts; allocated at creation)
-    unsigned char* ored_x;   // bf16 planes of A = [sigma, 1], Y0, Y1
-    double* ored_part;       // per-segment sums
+    unsigned char* ored_x;   // bf16 planes of Y0, Y1 and A = sigma
+    double* ored_part;       // per-segment sums, border sums per 512 walkers
     int2* ored_tiles;
     int ored;                // 1 when the path is set up
     void* lp_work;           // linear-prediction scratch (sized on first use)

@@ -17,6 +17,7 @@
 // split both operands, or one (see there).
 #include <cuda_bf16.h>
 
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -414,12 +415,14 @@ __global__ void __launch_bounds__(RED_THREADS, 1) oreduce_tc_kernel(
 // The operands lie in memory as bf16 planes, each an array of tiles
 // [row block of 128 G rows][walker chunk of KC] in the K-major no-swizzle
 // core-matrix layout, so one bulk copy moves one tile.
-// sgram_tc_kernel: persistent, 288 threads.  Warp 0 (one thread) copies
-// operand tiles through NSTG stages (running ahead across tiles) and issues
-// the MMAs of chunk c into TMEM columns [256 (c % 2), +256); warps 1-8 wait
-// for the chunk, add it to their register tile of G (entries formed from
-// adjacent lanes = rows 2k, 2k + 1), release the TMEM half, and at the end
-// of a tile write its sums.
+// sgram_tc_kernel: persistent.  Warp 9 (one thread) copies operand tiles
+// through NSTG stages (running ahead across tiles), warp 0 (one thread)
+// issues the MMAs of chunk c into TMEM columns [256 (c % 2), +256) -- one
+// thread for both, dividing for its ring positions, took 1.1 us a stage whose
+// three MMAs run 0.2 --; warps 1-8 wait for the chunk, add it to their
+// register tile of G (entries formed from adjacent lanes = rows 2k, 2k + 1),
+// release the TMEM half, and at the end of a tile write its sums.  Then what
+// L2 delivers bounds it (28 or 36 KB a stage).
 struct SGram {
     static constexpr int NPL = 3;                     // bf16 planes of a split operand
     static constexpr int KC = 16;                     // walkers per operand tile
@@ -440,33 +443,33 @@ struct SGram {
         return v[pr];
     }
 };
-constexpr int GR_THREADS = 288;
+constexpr int GR_THREADS = 320;
 
 // Arguments of sgram_tc_kernel.  A work item is one tile (rt, ct) of G over
 // one K segment of kseg walker tiles; items run segment-major (item i:
 // segment i / ntiles, tile i % ntiles), so that CTAs running at the same
 // time share operand tiles in L2.  tiles[t] = (rt, ct + 65536 op): the
 // column operand of op-0 tiles is xb0, of op-1 tiles xb1 (two products with
-// one row operand in one launch).  a_exact: the row operand is exact in
-// bf16 (spins, ones) and has one plane, so three products (its plane times
-// each plane of the column operand) replace the split's six.
+// one row operand in one launch).  EXACT: the row operand is real (row n is
+// x_n itself) and exact in bf16 (spins) and has one plane, so three products
+// (its plane times each plane of the column operand) replace the split's six.
 struct GramArgs {
     const unsigned char* xa;   // planes of the row operand
     const unsigned char* xb0;  // planes of the column operand of op-0 tiles
     const unsigned char* xb1;  // planes of the column operand of op-1 tiles
-    int a_exact;
     size_t plane_bytes;
     int nkc_max;              // walker tiles per row block in the planes
     int kseg, nseg;           // walker tiles per item, K segments per tile
     const int2* tiles;
     int ntiles;
-    // the float32 sums of every item, complex128
+    // the float32 sums of every item, complex128 (EXACT: complex64)
     // part[((op * nseg + seg) * Na + n) * Nb + m], n < Na, m < Nb
     double* part;
     int Na, Nb;
     int* status;
 };
 
+template <bool EXACT>
 __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs a) {
     using G = SGram;
     constexpr int NPL = G::NPL, NSTG = G::NSTG, TILE = G::TILE, KPC = G::CH / G::KC;  // tiles per chunk
@@ -511,99 +514,96 @@ __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs 
     };
     if (warp == 0) {
         if (lane == 0) {
-            // ---------------------------------------------- producer / MMA issuer
-            // One flat sequence of stages over all tiles of this CTA, so the
-            // copies run NSTG - 1 stages ahead across tile boundaries too.
+            // -------------------------------------------------- MMA issuer
             const uint32_t idesc = tc::make_idesc_bf16(128, 256);
-            const int total = nmine * kseg;
-            uint32_t pend = 0, pend_par = 0;
-            int last_g = -1;  // last stage whose MMAs were committed
+            const uint64_t d0 = tc::make_desc(tc::smem_u32(sm), 128, 16 * G::KC);
+            uint32_t b = 0, ph = 0, gc = 0;
+            int last = -1, lastph = 0;  // stage of the last commit
             bool ok = true;
-            // copy the operands of stage g; its buffer was last read by the MMAs
-            // of stage g - NSTG
-            auto load = [&](int g) {
-                const uint32_t b = g % NSTG;
-                if (g >= NSTG && !wait(&empty[b], ((g - NSTG) / NSTG) & 1)) return false;
-                const int item = blockIdx.x + (g / kseg) * gridDim.x;
-                const int2 tl = tiles[item % ntiles];
-                const int kc = (item / ntiles) * kseg + g % kseg;
-                const int rt = tl.x, ct = tl.y & 0xffff;
-                const unsigned char* xb = (tl.y >> 16) ? a.xb1 : a.xb0;
-                pend |= 1u << b;
-                pend_par = (pend_par & ~(1u << b)) | (((uint32_t)(g / NSTG) & 1u) << b);
-                unsigned char* st = sm + (size_t)b * G::STAGE;
-                const int npa = a.a_exact ? 1 : NPL;  // planes of the row operand
-                tc::mbar_expect_tx(&full[b], (uint32_t)((npa + 2 * NPL) * TILE));
-                for (int pl = 0; pl < NPL; ++pl) {
-                    if (pl < npa)
-                        tc::bulk_g2s(st + pl * TILE,
-                                     a.xa + (size_t)pl * plane_bytes +
-                                         ((size_t)rt * nkc_max + kc) * TILE,
-                                     TILE, &full[b]);
-                    for (int q = 0; q < 2; ++q)
-                        tc::bulk_g2s(st + NPL * TILE + (pl * 2 + q) * TILE,
-                                     xb + (size_t)pl * plane_bytes +
-                                         ((size_t)(2 * ct + q) * nkc_max + kc) * TILE,
-                                     TILE, &full[b]);
-                }
-                return true;
-            };
-            for (int g = 0; g < NSTG - 1 && g < total && ok; ++g) ok = load(g);
-            for (int g = 0; g < total && ok; ++g) {
-                const int kc = g % kseg, b = g % NSTG;
-                const int gc = (g / kseg) * nchunk + kc / KPC, first = (kc % KPC) == 0;
-                const uint32_t h = gc & 1;
-                // the TMEM half of chunk gc was last used by chunk gc - 2
-                if (first && gc >= 2 && !wait(&drained[h], ((gc - 2) >> 1) & 1)) {
-                    ok = false;
-                    break;
-                }
-                if (!wait(&full[b], (g / NSTG) & 1)) {
-                    ok = false;
-                    break;
-                }
-                pend &= ~(1u << b);
-                tc::fence_after_sync();
-                const unsigned char* st = sm + (size_t)b * G::STAGE;
-                const uint32_t a0 = tc::smem_u32(st), b0 = tc::smem_u32(st + NPL * TILE);
-                if (a.a_exact) {
+            for (int ti = 0; ti < nmine && ok; ++ti)
+                for (int kc = 0; kc < kseg && ok; kc += KPC, ++gc) {
+                    const uint32_t h = gc & 1, dt = taddr + h * 256;
+                    // the TMEM half of chunk gc was last used by chunk gc - 2
+                    if (gc >= 2 && !wait(&drained[h], ((gc >> 1) - 1) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    const int n = min(KPC, kseg - kc);
+                    for (int k = 0; k < n; ++k) {
+                        if (!wait(&full[b], ph)) {
+                            ok = false;
+                            break;
+                        }
+                        tc::fence_after_sync();
+                        const uint64_t ad = d0 + b * (uint32_t)(G::STAGE >> 4);
+                        const uint64_t bd = ad + (NPL * TILE >> 4);
 #pragma unroll
-                    for (int ks = 0; ks < G::KC / 16; ++ks) {
-                        const uint64_t ad = tc::make_desc(a0 + ks * 256, 128, 16 * G::KC);
+                        for (int ks = 0; ks < G::KC / 16; ++ks)
 #pragma unroll
-                        for (int pl = 0; pl < NPL; ++pl) {
-                            const uint64_t bd =
-                                tc::make_desc(b0 + pl * 2 * TILE + ks * 256, 128, 16 * G::KC);
-                            tc::mma_bf16(taddr + h * 256, ad, bd, idesc, !(first && ks == 0 && pl == 0));
+                            for (int pr = 0; pr < (EXACT ? NPL : G::NPROD); ++pr)
+                                tc::mma_bf16(dt, ad + ((EXACT ? 0 : G::pa(pr)) * (TILE >> 4) + ks * 16),
+                                             bd + ((EXACT ? pr : G::pb(pr)) * (2 * TILE >> 4) + ks * 16),
+                                             idesc, k != 0 || ks != 0 || pr != 0);
+                        tc::commit(&empty[b]);
+                        last = (int)b;
+                        lastph = (int)ph;
+                        if (++b == NSTG) {
+                            b = 0;
+                            ph ^= 1;
                         }
                     }
-                } else {
-#pragma unroll
-                    for (int ks = 0; ks < G::KC / 16; ++ks) {
-#pragma unroll
-                        for (int pr = 0; pr < G::NPROD; ++pr) {
-                            const uint64_t ad =
-                                tc::make_desc(a0 + G::pa(pr) * TILE + ks * 256, 128, 16 * G::KC);
-                            const uint64_t bd =
-                                tc::make_desc(b0 + G::pb(pr) * 2 * TILE + ks * 256, 128, 16 * G::KC);
-                            tc::mma_bf16(taddr + h * 256, ad, bd, idesc,
-                                         !(first && ks == 0 && pr == 0));
-                        }
-                    }
+                    if (ok) tc::commit(&cdone[h]);
                 }
-                tc::commit(&empty[b]);
-                last_g = g;
-                if ((kc + 1) % KPC == 0 || kc + 1 == kseg) tc::commit(&cdone[h]);
-                if (g + NSTG - 1 < total && !load(g + NSTG - 1)) ok = false;
-            }
             if (!ok) {
                 *abort = 1;
                 set_status(status, CR_ETIMEOUT);
-                // let copies in flight land and issued MMAs finish (bounded)
-                for (int b = 0; b < NSTG; ++b)
-                    if (pend & (1u << b)) tc::mbar_wait(&full[b], (pend_par >> b) & 1u, WAIT_LIMIT);
-                if (last_g >= 0)
-                    tc::mbar_wait(&empty[last_g % NSTG], (uint32_t)(last_g / NSTG) & 1u, WAIT_LIMIT);
+                // let issued MMAs finish (bounded)
+                if (last >= 0) tc::mbar_wait(&empty[last], (uint32_t)lastph, WAIT_LIMIT);
+            }
+        }
+        __syncwarp();
+    } else if (warp == GR_THREADS / 32 - 1) {
+        if (lane == 0) {
+            // One flat sequence of stages over all tiles of this CTA, so the
+            // copies run ahead across tile boundaries too.
+            constexpr int npa = EXACT ? 1 : NPL;  // planes of the row operand
+            uint32_t b = 0, ph = 0, g = 0;
+            bool ok = true;
+            for (int ti = 0; ti < nmine && ok; ++ti) {
+                const int item = blockIdx.x + ti * gridDim.x;
+                const int2 tl = tiles[item % ntiles];
+                const int kc0 = (item / ntiles) * kseg, rt = tl.x, ct = tl.y & 0xffff;
+                const unsigned char* xa = a.xa + ((size_t)rt * nkc_max + kc0) * TILE;
+                const unsigned char* xb = ((tl.y >> 16) ? a.xb1 : a.xb0) + ((size_t)2 * ct * nkc_max + kc0) * TILE;
+                const size_t rbs = (size_t)nkc_max * TILE;  // one row block
+                for (int kc = 0; kc < kseg; ++kc, ++g, xa += TILE, xb += TILE) {
+                    // the buffer was last read by the MMAs of NSTG stages before
+                    if (g >= NSTG && !wait(&empty[b], ph ^ 1)) {
+                        ok = false;
+                        break;
+                    }
+                    unsigned char* st = sm + (size_t)b * G::STAGE;
+                    tc::mbar_expect_tx(&full[b], (uint32_t)((npa + 2 * NPL) * TILE));
+#pragma unroll
+                    for (int pl = 0; pl < NPL; ++pl) {
+                        if (pl < npa) tc::bulk_g2s(st + pl * TILE, xa + pl * plane_bytes, TILE, &full[b]);
+#pragma unroll
+                        for (int q = 0; q < 2; ++q)
+                            tc::bulk_g2s(st + NPL * TILE + (pl * 2 + q) * TILE, xb + pl * plane_bytes + q * rbs,
+                                         TILE, &full[b]);
+                    }
+                    if (++b == NSTG) {
+                        b = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+            // every copy lands before the CTA leaves (bounded): the last
+            // stages; where MMAs consumed them all this does not wait
+            for (uint32_t q = 0; q < NSTG && q < g; ++q) {
+                if (b == 0) ph ^= 1;
+                b = b == 0 ? NSTG - 1 : b - 1;
+                tc::mbar_wait(&full[b], ph, WAIT_LIMIT);
             }
         }
         __syncwarp();
@@ -621,11 +621,14 @@ __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs 
             const int item = blockIdx.x + ti * gridDim.x;
             const int2 tl = tiles[item % ntiles];
             const int rt = tl.x, ct = tl.y & 0xffff;
-            float acc[8][4][2];  // [16-column chunk][entry][Re, Im]
+            // [16-column chunk][entry][Re, Im]; EXACT: a lane has 8 entries of
+            // its row, else 4 of its pair of rows
+            constexpr int NE = EXACT ? 8 : 4;
+            float acc[8][NE][2];
 #pragma unroll
             for (int ch = 0; ch < 8; ++ch)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[ch][q][0] = acc[ch][q][1] = 0.f;
+                for (int q = 0; q < NE; ++q) acc[ch][q][0] = acc[ch][q][1] = 0.f;
             for (int ck = 0; ck < nchunk; ++ck) {
                 const int gc = ti * nchunk + ck;
                 const uint32_t h = gc & 1;
@@ -640,17 +643,25 @@ __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs 
                     float v[16], p[16];
                     tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + h * 256 + 128 * c2 + 16 * ch,
                                   v);
+                    if constexpr (EXACT) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) p[i] = __shfl_xor_sync(0xffffffffu, v[i], 1);
+                        for (int q = 0; q < NE; ++q) {
+                            acc[ch][q][0] = __fadd_rn(acc[ch][q][0], v[2 * q]);
+                            acc[ch][q][1] = __fadd_rn(acc[ch][q][1], v[2 * q + 1]);
+                        }
+                    } else {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        // even lane: row 2k is its own (v), row 2k+1 the partner's (p); odd: swapped
-                        const float e0 = odd ? p[8 + 2 * q] : v[2 * q];
-                        const float e1 = odd ? p[9 + 2 * q] : v[2 * q + 1];
-                        const float o0 = odd ? v[8 + 2 * q] : p[2 * q];
-                        const float o1 = odd ? v[9 + 2 * q] : p[2 * q + 1];
-                        acc[ch][q][0] = __fadd_rn(acc[ch][q][0], __fadd_rn(e0, o1));
-                        acc[ch][q][1] = __fadd_rn(acc[ch][q][1], __fsub_rn(e1, o0));
+                        for (int i = 0; i < 16; ++i) p[i] = __shfl_xor_sync(0xffffffffu, v[i], 1);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            // even lane: row 2k is its own (v), row 2k+1 the partner's (p); odd: swapped
+                            const float e0 = odd ? p[8 + 2 * q] : v[2 * q];
+                            const float e1 = odd ? p[9 + 2 * q] : v[2 * q + 1];
+                            const float o0 = odd ? v[8 + 2 * q] : p[2 * q];
+                            const float o1 = odd ? v[9 + 2 * q] : p[2 * q + 1];
+                            acc[ch][q][0] = __fadd_rn(acc[ch][q][0], __fadd_rn(e0, o1));
+                            acc[ch][q][1] = __fadd_rn(acc[ch][q][1], __fsub_rn(e1, o0));
+                        }
                     }
                 }
                 tc::fence_before_sync();
@@ -659,18 +670,18 @@ __global__ void __launch_bounds__(GR_THREADS, 1) sgram_tc_kernel(const GramArgs 
                              : "memory");
             }
             if (!ok) break;
-            // the item's sums: n = row pair, m = column
-            const int n = 64 * rt + (row >> 1), Na = a.Na, Nb = a.Nb;
-            cpx<double>* out = (cpx<double>*)a.part +
-                               (size_t)((tl.y >> 16) * a.nseg + item / ntiles) * Na * Nb;
+            // the item's sums: n = row (pair), m = column
+            const int n = EXACT ? 128 * rt + row : 64 * rt + (row >> 1), Na = a.Na, Nb = a.Nb;
+            using Out = cpx<std::conditional_t<EXACT, float, double>>;
+            Out* out = (Out*)a.part + (size_t)((tl.y >> 16) * a.nseg + item / ntiles) * Na * Nb;
             if (n < Na) {
 #pragma unroll
                 for (int ch = 0; ch < 8; ++ch)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int m = 128 * ct + 64 * c2 + 8 * ch + 4 * odd + q;
+                    for (int q = 0; q < NE; ++q) {
+                        const int m = 128 * ct + 64 * c2 + 8 * ch + (EXACT ? 0 : 4 * odd) + q;
                         if (m < Nb)
-                            out[(size_t)n * Nb + m] = {(double)acc[ch][q][0], (double)acc[ch][q][1]};
+                            out[(size_t)n * Nb + m] = ccast<decltype(out->x)>(cpx<float>{acc[ch][q][0], acc[ch][q][1]});
                     }
             }
         }
@@ -898,7 +909,7 @@ cr_status launch_gram_tc(cr_ctx* c, const void* Bm, const void* HBm, int Nm, int
     const int items = a.ntiles * a.nseg;
     const int grid = items < c->n_sm ? items : c->n_sm;
     CR_LAUNCH(c, CR_KERNEL_GRAM,
-              sgram_tc_kernel<<<grid, GR_THREADS, SGram::SMEM, c->stream>>>(a));
+              sgram_tc_kernel<false><<<grid, GR_THREADS, SGram::SMEM, c->stream>>>(a));
     CR_LAUNCH(c, CR_K_OTHER, gram_reduce_kernel<<<(Nm * Nm + 255) / 256, 256, 0, c->stream>>>(
                                  c->gram_part, g.nseg, Nm, B, G, H));
     return cr_check_launch(c, "cheb_gram (tensor cores)");
@@ -909,15 +920,22 @@ cr_status launch_gram_tc(cr_ctx* c, const void* Bm, const void* HBm, int Nm, int
 // The two walker sums of a natural-gradient step (Sec. III),
 //   redR = [sum sigma_i g | sum conj(T_j) g | sum sigma_i conj(T_j) g | sum g | sum |g|^2]
 //   redO = [sum sigma_i   | sum T_j         | sum sigma_i T_j         | B     | B      ]
-// (g = R; the layout of oreduce's rows), as one launch of sgram_tc_kernel:
-// row operand A = [sigma_0 .. sigma_{N-1}, 1] (exact in bf16: one plane),
-// column operands Y0 = [conj(T_j) g, g, |g|^2] (op 0) and Y1 = [T_j, 1]
-// (op 1), split into three bf16 planes; out = sum_s A_k(s) Y_l(s) over K
-// segments, added in float64 by ored_reduce_kernel.  The sums of |T_j|^2
-// (the Jacobi diagonal) are not formed here.
+// (g = R; the layout of oreduce's rows).  The N x M blocks are one launch of
+// sgram_tc_kernel: row operand A = sigma (exact in bf16: one plane), column
+// operands Y0 = conj(T_j) g (op 0) and Y1 = T_j (op 1), split into three bf16
+// planes, summed over K segments that ored_reduce_kernel adds in float64.
+// The border (the sums without a product of sigma and T) comes out of the
+// pass over T and sigma that writes the planes, in compensated float32: as a
+// row and columns of the product it filled further tiles of 128 x 256.
+// 16 x 16 lattice, alpha = 1, 65536 walkers: 1.30 ms (product 0.93), now
+// 0.30 (planes 0.157, product 0.114, reduction 0.029).
+// The sums of |T_j|^2 (the Jacobi diagonal) are not formed here.
+constexpr int ORP_CHUNK = 512;  // walkers of a block of ored_prep_kernel
+
 struct OredGeo {
-    int R2, nrb, nseg, nkc_cap, Na, Nb;
-    size_t plane_bytes, x_bytes, part_bytes;
+    int nrt, nct;  // tiles of 128 sites, of 128 hidden units
+    int nseg, nkc_cap;
+    size_t plane_bytes, x_bytes, part_bytes, border_off;
     std::vector<int2> tiles;
 };
 
@@ -925,25 +943,21 @@ static OredGeo ored_geometry(const cr_ctx* c) {
     using G = SGram;
     constexpr int KPC = G::CH / G::KC;
     OredGeo g;
-    g.Na = c->N + 1;
-    g.Nb = c->M + 2;
-    const int ra = 2 * g.Na, rb0 = 2 * (c->M + 2), rb1 = 2 * (c->M + 1);
-    const int rmax = ra > rb0 ? ra : rb0;
-    g.R2 = ((rmax + 255) / 256) * 256;
-    g.nrb = g.R2 / 128;
-    const int nrt = (ra + 127) / 128;
-    for (int op = 0; op < 2; ++op) {
-        const int nct = ((op ? rb1 : rb0) + 255) / 256;
-        for (int ct = 0; ct < nct; ++ct)
-            for (int rt = 0; rt < nrt; ++rt) g.tiles.push_back(make_int2(rt, ct + 65536 * op));
-    }
+    g.nrt = (c->N + 127) / 128;
+    g.nct = (c->M + 127) / 128;
+    for (int op = 0; op < 2; ++op)
+        for (int ct = 0; ct < g.nct; ++ct)
+            for (int rt = 0; rt < g.nrt; ++rt) g.tiles.push_back(make_int2(rt, ct + 65536 * op));
     const int nt = (int)g.tiles.size();
     g.nseg = c->n_sm / nt > 1 ? c->n_sm / nt : 1;
     const int nch = (c->max_walkers + G::CH - 1) / G::CH;
     g.nkc_cap = g.nseg * ((nch + g.nseg - 1) / g.nseg) * KPC;
-    g.plane_bytes = (size_t)g.nrb * g.nkc_cap * G::TILE;
-    g.x_bytes = 7 * g.plane_bytes;  // A: one plane; Y0, Y1: three each
-    g.part_bytes = (size_t)2 * g.nseg * g.Na * g.Nb * 16;
+    g.plane_bytes = (size_t)2 * g.nct * g.nkc_cap * G::TILE;
+    // Y0, Y1: three planes each; A: one
+    g.x_bytes = 6 * g.plane_bytes + (size_t)g.nrt * g.nkc_cap * G::TILE;
+    g.border_off = (size_t)2 * g.nseg * c->N * c->M * 8;
+    g.part_bytes = g.border_off +
+                   (size_t)((g.nkc_cap * G::KC + ORP_CHUNK - 1) / ORP_CHUNK) * 2 * (c->M + c->N + 2) * 16;
     return g;
 }
 
@@ -954,104 +968,159 @@ void ored_sizes(const cr_ctx* c, size_t* x_bytes, size_t* part_bytes, std::vecto
     *tiles = g.tiles;
 }
 
-// Planes of A (plane 0 only) and of Y0, Y1 for walker tiles kc < nkc (zero
-// past B): one thread per (row, 8 walkers); T is read once for both Y.
-__global__ void ored_prep_kernel(const int8_t* __restrict__ spins, const cpx<float>* __restrict__ T,
-                                 const cpx<float>* __restrict__ g, int B, int N, int M, int nrb,
-                                 int nkc, int nkc_cap, size_t plane_bytes,
-                                 unsigned char* __restrict__ X) {
+CR_D void kadd(float& s, float& c, float v) {
+    const float y = v - c;
+    const float t = s + y;
+    c = (t - s) - y;
+    s = t;
+}
+
+// Planes of A, Y0 and Y1 for walker tiles kc < nkc (zero past B, N and M) and
+// the border sums of each chunk of 512 walkers, complex128 border[chunk]:
+// [sum T_j | sum conj(T_j) g | sum sigma_i, B | 0 | sum sigma_i g | sum g | sum |g|^2].
+// Blocks of 8 warps: 32 hidden units (blockIdx.y < nyt) or sites, a warp takes
+// every eighth group of 8 walkers, so that T is read in whole rows of 256
+// bytes and a thread forms the 16-byte operand groups of its two rows.
+// Bound by the writes of the planes.
+__global__ void __launch_bounds__(256) ored_prep_kernel(const int8_t* __restrict__ spins,
+                                                        const cpx<float>* __restrict__ T,
+                                                        const cpx<float>* __restrict__ g, int B, int N,
+                                                        int M, int nkc, int nkc_cap, int nyt,
+                                                        size_t plane_bytes, unsigned char* __restrict__ X,
+                                                        double* __restrict__ border_) {
     using G = SGram;
-    constexpr int NG = G::KC / 8;
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)nrb * nkc * NG * 128) return;
-    const int r = (int)(idx % 128), grp = (int)((idx / 128) % NG);
-    const size_t rest = idx / (128 * NG);
-    const int kc = (int)(rest % nkc), rb = (int)(rest / nkc);
-    const int row = rb * 128 + r, k = row >> 1, im = row & 1;
-    __nv_bfloat16 a[8], y0[3][8], y1[3][8];
+    __shared__ float rs[4][8][32], rc[4][8][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool hid = (int)blockIdx.y < nyt;
+    const int e = 32 * (hid ? blockIdx.y : blockIdx.y - nyt) + lane;  // hidden unit or site
+    const int Nr = ((N + 127) / 128) * 128;
+    float s[4] = {0.f, 0.f, 0.f, 0.f}, c[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int grp = warp; grp < ORP_CHUNK / 8; grp += 8) {
+        const int s0 = blockIdx.x * ORP_CHUNK + 8 * grp, kc = s0 / G::KC;
+        if (kc >= nkc) break;
+        const uint32_t half = (uint32_t)(s0 % G::KC);
+        cpx<float> gs[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-        const int s = kc * G::KC + grp * 8 + q;
-        float xa = 0.f, x0 = 0.f, x1 = 0.f;
-        if (s < B) {
-            if (!im) xa = k < N ? (float)spins[(size_t)s * N + k] : (k == N ? 1.f : 0.f);
-            const cpx<float> gs = g[s];
-            cpx<float> v0 = {0.f, 0.f}, v1 = {0.f, 0.f};
-            if (k < M) {
-                const cpx<float> t = T[(size_t)s * M + k];
-                v0 = conj(t) * gs;
-                v1 = t;
-            } else if (k == M) {
-                v0 = gs;
-                v1 = {1.f, 0.f};
-            } else if (k == M + 1) {
-                v0 = {abs2(gs), 0.f};
+        for (int q = 0; q < 8; ++q) gs[q] = s0 + q < B ? ldg(g + s0 + q) : cpx<float>{0.f, 0.f};
+        if (hid) {
+            cpx<float> tv[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                tv[q] = e < M && s0 + q < B ? ldg(T + (size_t)(s0 + q) * M + e) : cpx<float>{0.f, 0.f};
+#pragma unroll
+            for (int im = 0; im < 2; ++im) {
+                __nv_bfloat16 y0[3][8], y1[3][8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const cpx<float> v = conj(tv[q]) * gs[q];
+                    const float x1 = im ? tv[q].y : tv[q].x, x0 = im ? v.y : v.x;
+                    kadd(s[im], c[im], x1);
+                    kadd(s[2 + im], c[2 + im], x0);
+                    split3(x0, &y0[0][q], &y0[1][q], &y0[2][q]);
+                    split3(x1, &y1[0][q], &y1[1][q], &y1[2][q]);
+                }
+                const int row = 2 * e + im;
+                const size_t off = ((size_t)(row >> 7) * nkc_cap + kc) * G::TILE +
+                                   tc::kmajor_offset(row & 127, half, G::KC);
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) {
+                    *reinterpret_cast<uint4*>(X + pl * plane_bytes + off) = pack8(y0[pl]);
+                    *reinterpret_cast<uint4*>(X + (3 + pl) * plane_bytes + off) = pack8(y1[pl]);
+                }
             }
-            x0 = im ? v0.y : v0.x;
-            x1 = im ? v1.y : v1.x;
-        }
-        a[q] = __float2bfloat16_rn(xa);  // exact: +-1, 1 or 0
-        split3(x0, &y0[0][q], &y0[1][q], &y0[2][q]);
-        split3(x1, &y1[0][q], &y1[1][q], &y1[2][q]);
-    }
-    const size_t off = ((size_t)rb * nkc_cap + kc) * G::TILE + tc::kmajor_offset(r, grp * 8, G::KC);
-    *reinterpret_cast<uint4*>(X + off) = pack8(a);
+        } else {
+            __nv_bfloat16 x[8];
 #pragma unroll
-    for (int pl = 0; pl < 3; ++pl) {
-        *reinterpret_cast<uint4*>(X + (1 + pl) * plane_bytes + off) = pack8(y0[pl]);
-        *reinterpret_cast<uint4*>(X + (4 + pl) * plane_bytes + off) = pack8(y1[pl]);
+            for (int q = 0; q < 8; ++q) {
+                const bool in = s0 + q < B;
+                const float v = in && e < N ? (float)spins[(size_t)(s0 + q) * N + e] : 0.f;
+                x[q] = __float2bfloat16_rn(v);  // exact: +-1 or 0
+                const float w = e == N && in ? 1.f : v;
+                kadd(s[0], c[0], w);
+                kadd(s[2], c[2], e == N + 1 ? abs2(gs[q]) : w * gs[q].x);
+                kadd(s[3], c[3], w * gs[q].y);
+            }
+            if (e < Nr)
+                *reinterpret_cast<uint4*>(X + 6 * plane_bytes + ((size_t)(e >> 7) * nkc_cap + kc) * G::TILE +
+                                          tc::kmajor_offset(e & 127, half, G::KC)) = pack8(x);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        rs[q][warp][lane] = s[q];
+        rc[q][warp][lane] = c[q];
+    }
+    __syncthreads();
+    if (warp < 4) {
+        // one warp per sum, the eight warps' in a fixed order
+        float t = 0.f, tc = 0.f;
+        for (int w = 0; w < 8; ++w) kadd(t, tc, rs[warp][w][lane]);
+        for (int w = 0; w < 8; ++w) kadd(t, tc, -rc[warp][w][lane]);
+        double* out = border_ + (size_t)blockIdx.x * 4 * (M + N + 2);
+        const double v = (double)t - (double)tc;
+        const int len = hid ? M : N + 2, first = hid ? 0 : 2 * M;
+        if (e < len) out[2 * (first + (warp >> 1) * len + e) + (warp & 1)] = v;
     }
 }
 
-__global__ void ored_reduce_kernel(const double* __restrict__ part_, int nseg, int N, int M, int P,
-                                   int Na, int Nb, double* __restrict__ redR_,
-                                   double* __restrict__ redO_) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= P + 2 + M) return;
-    cpx<double>* redR = (cpx<double>*)redR_;
-    cpx<double>* redO = (cpx<double>*)redO_;
-    if (k >= P + 2) {
-        redO[k] = {0.0, 0.0};  // sums of |T_j|^2: not formed on this path
-        return;
-    }
-    int n, m;  // (row of A, column of Y)
-    if (k < N) { n = k; m = M; }
-    else if (k < N + M) { n = N; m = k - N; }
-    else if (k < P) { n = (k - N - M) / M; m = (k - N - M) % M; }
-    else { n = N; m = M + (k - P); }
-    const cpx<double>* part = (const cpx<double>*)part_;
-    const size_t NN = (size_t)Na * Nb, e = (size_t)n * Nb + m;
+// Blocks of 32 entries x 8 groups of segments (or chunks), the groups added
+// in a fixed order: the loads of an entry are spread over eight threads.
+__global__ void __launch_bounds__(256) ored_reduce_kernel(const double* __restrict__ part_,
+                                                          const double* __restrict__ border_, int nseg,
+                                                          int nchunk, int N, int M, int P,
+                                                          double* __restrict__ redR_,
+                                                          double* __restrict__ redO_) {
+    __shared__ cpx<double> sr[8][32], so[8][32];
+    const int lane = threadIdx.x & 31, gr = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
     cpx<double> r = {0.0, 0.0}, o = {0.0, 0.0};
-    for (int sg = 0; sg < nseg; ++sg) {
-        r = r + part[sg * NN + e];
-        if (k <= P) o = o + part[(nseg + sg) * NN + e];
+    if (k >= N + M && k < P) {
+        const cpx<float>* part = (const cpx<float>*)part_;
+        const size_t NN = (size_t)N * M, e = (size_t)(k - N - M);
+#pragma unroll 4
+        for (int sg = gr; sg < nseg; sg += 8) {
+            r = r + ccast<double>(part[sg * NN + e]);
+            o = o + ccast<double>(part[(nseg + sg) * NN + e]);
+        }
+    } else if (k < P + 2) {
+        // entries of the border: sums without g at o0, with g at r0
+        const int o0 = k < N ? 2 * M + k : (k < N + M ? k - N : 2 * M + N);
+        const int r0 = k < N ? o0 + N + 2 : (k < N + M ? o0 + M : 2 * M + N + 2 + N + (k - P));
+        const cpx<double>* b = (const cpx<double>*)border_;
+#pragma unroll 4
+        for (int ch = gr; ch < nchunk; ch += 8) {
+            o = o + b[(size_t)ch * 2 * (M + N + 2) + o0];
+            r = r + b[(size_t)ch * 2 * (M + N + 2) + r0];
+        }
     }
-    if (k == P + 1) {
-        // sum |1|^2 = sum 1, the B of entry P
-        for (int sg = 0; sg < nseg; ++sg) o = o + part[(nseg + sg) * NN + (size_t)N * Nb + M];
-        r.y = 0.0;
-    }
-    redR[k] = r;
-    redO[k] = o;
+    sr[gr][lane] = r;
+    so[gr][lane] = o;
+    __syncthreads();
+    if (gr > 1 || k >= P + 2 + M) return;
+    cpx<double> t = gr ? so[0][lane] : sr[0][lane];
+    for (int q = 1; q < 8; ++q) t = t + (gr ? so[q][lane] : sr[q][lane]);
+    // redO past P + 2, the sums of |T_j|^2, is not formed on this path: zero
+    if (gr) ((cpx<double>*)redO_)[k] = t;
+    else if (k < P + 2) ((cpx<double>*)redR_)[k] = t;
 }
 
 cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const void* g, int B,
                             double* redR, double* redO) {
     using G = SGram;
-    constexpr int KPC = G::CH / G::KC, NG = G::KC / 8;
+    constexpr int KPC = G::CH / G::KC;
     OredGeo geo = ored_geometry(c);
     const int nch = (B + G::CH - 1) / G::CH;
     const int cps = (nch + geo.nseg - 1) / geo.nseg;
     const int nseg = (nch + cps - 1) / cps, kseg = cps * KPC, nkc = nseg * kseg;
-    const size_t n = (size_t)geo.nrb * nkc * NG * 128;
-    CR_LAUNCH(c, CR_K_OTHER, ored_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(
+    const int nchunk = (nkc * G::KC + ORP_CHUNK - 1) / ORP_CHUNK;
+    const int nyt = 4 * geo.nct, sites = geo.nrt * 128 > c->N + 2 ? geo.nrt * 128 : c->N + 2;
+    double* border = c->ored_part + geo.border_off / 8;
+    CR_LAUNCH(c, CR_K_OTHER, ored_prep_kernel<<<dim3(nchunk, nyt + (sites + 31) / 32), 256, 0, c->stream>>>(
                                  spins, (const cpx<float>*)T, (const cpx<float>*)g, B, c->N, c->M,
-                                 geo.nrb, nkc, geo.nkc_cap, geo.plane_bytes, c->ored_x));
+                                 nkc, geo.nkc_cap, nyt, geo.plane_bytes, c->ored_x, border));
     GramArgs a{};
-    a.xa = c->ored_x;
-    a.xb0 = c->ored_x + geo.plane_bytes;
-    a.xb1 = c->ored_x + 4 * geo.plane_bytes;
-    a.a_exact = 1;
+    a.xa = c->ored_x + 6 * geo.plane_bytes;
+    a.xb0 = c->ored_x;
+    a.xb1 = c->ored_x + 3 * geo.plane_bytes;
     a.plane_bytes = geo.plane_bytes;
     a.nkc_max = geo.nkc_cap;
     a.kseg = kseg;
@@ -1059,16 +1128,16 @@ cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const
     a.tiles = c->ored_tiles;
     a.ntiles = (int)geo.tiles.size();
     a.part = c->ored_part;
-    a.Na = geo.Na;
-    a.Nb = geo.Nb;
+    a.Na = c->N;
+    a.Nb = c->M;
     a.status = c->d_status;
     const int items = a.ntiles * nseg;
     const int grid = items < c->n_sm ? items : c->n_sm;
     CR_LAUNCH(c, CR_KERNEL_REDUCE,
-              sgram_tc_kernel<<<grid, GR_THREADS, SGram::SMEM, c->stream>>>(a));
+              sgram_tc_kernel<true><<<grid, GR_THREADS, SGram::SMEM, c->stream>>>(a));
     const int len = c->P + 2 + c->M;
-    CR_LAUNCH(c, CR_K_OTHER, ored_reduce_kernel<<<(len + 255) / 256, 256, 0, c->stream>>>(
-                                 c->ored_part, nseg, c->N, c->M, c->P, geo.Na, geo.Nb, redR, redO));
+    CR_LAUNCH(c, CR_K_OTHER, ored_reduce_kernel<<<(len + 31) / 32, 256, 0, c->stream>>>(
+                                 c->ored_part, border, nseg, nchunk, c->N, c->M, c->P, redR, redO));
     return cr_check_launch(c, "estimator sums (tensor cores)");
 }
 
@@ -1076,9 +1145,12 @@ cr_status launch_oreduce_tc(cr_ctx* c, const int8_t* spins, const void* T, const
 // per context (not from a hot call, so that hot calls stay capturable).
 cr_status tc_prepare(cr_ctx* c) {
     if (c->prec == CR_MIXED) {
-        cudaError_t e = cudaFuncSetAttribute(sgram_tc_kernel,
+        cudaError_t e = cudaFuncSetAttribute(sgram_tc_kernel<true>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)SGram::SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(sgram_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)SGram::SMEM);
         if (e != cudaSuccess) return cr_fail(c, CR_ECUDA, "tc_prepare: %s", cudaGetErrorString(e));
     }
     if (!tc_supported(c)) return CR_OK;
