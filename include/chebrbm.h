@@ -191,7 +191,9 @@ cr_status cr_set_stream(cr_ctx* ctx, void* stream);
 /* Walker chunks of the split-K reductions (the sums over walkers in F, the
    O averages and O^dag u are formed per chunk, then combined in float64 in
    chunk order).  cr_create picks ceil(max_walkers / 128), at most 128, which
-   is also the largest value cr_set_chunks accepts (cr_max_chunks).  Fewer
+   is also the largest value cr_set_chunks accepts (cr_max_chunks); until a
+   value is set, few walkers are split further, down to 32 per chunk, to
+   occupy the GPU.  Fewer
    chunks launch fewer CTAs, which pays when several contexts run
    concurrently on one GPU; the results change only by the summation order.
    Returns CR_EINVAL outside [1, cr_max_chunks]. */

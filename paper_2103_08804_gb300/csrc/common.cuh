@@ -168,6 +168,8 @@ struct cr_ctx {
     cr_prec prec;
     int max_walkers, flags;
     int n_chunks;            // walker chunks of the reductions (<= max_chunks)
+    int red_rows;            // chunk rows allocated (>= max_chunks), used while !chunks_set
+    bool chunks_set;         // n_chunks was asked for
     int max_chunks;          // chunks the partial-row workspace holds
     int n_sm;                // multiprocessors of the device
     cudaStream_t stream;
@@ -183,13 +185,13 @@ struct cr_ctx {
     void* theta_tmp;         // [maxB][M]
     void* lp_tmp;            // [2][maxB]
     void* u_tmp;             // [maxB]
-    double* partial;         // [n_chunks][P + 2 + M] complex, context precision
+    double* partial;         // [red_rows][P + 2 + M] complex, context precision
     double* red;             // [3][P + 2 + M] complex128 reduced sums
     double* F;               // [P] complex128
-    double* cg;              // x, r, p, Ap, diag: [5][P] complex128
+    double* cg;              // x, r, p, Ap, 1 / diag: [5][P] complex128
     void* p_lo;              // [P] context precision
     double* cgpart;          // per-CTA dot products of a CG step: p.Ap [ceil(P/32)],
-                             // r.r and r.z [2][ceil(P/256)]
+                             // r.r and r.z [2][ceil(P/64)]
     double* scal;            // scalars [64]
     double* S;               // [P][P] complex128 (explicit S only)
     double* kry;             // Krylov workspace

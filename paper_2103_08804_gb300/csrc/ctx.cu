@@ -132,6 +132,14 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     c->n_chunks = (max_walkers + 127) / 128;
     if (c->n_chunks > 128) c->n_chunks = 128;
     c->max_chunks = c->n_chunks;
+    // rows of partial sums the reductions use unless told otherwise: up to
+    // four CTAs on each of 152 SMs, of 32 walkers or more (red_chunks)
+    const int red_tiles = ((M + 31) / 32) * ((c->N + 63) / 64);
+    int rows = (608 + red_tiles - 1) / red_tiles;
+    if (rows > (max_walkers + 31) / 32) rows = (max_walkers + 31) / 32;
+    if (rows > 128) rows = 128;
+    c->red_rows = rows > c->n_chunks ? rows : c->n_chunks;
+    c->chunks_set = false;
     if (c->N > 1024 || c->N % 2) {
         free(c);
         return CR_EINVAL;
@@ -160,12 +168,12 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     ALLOC(c->theta_tmp, B * M * cs);
     ALLOC(c->lp_tmp, 2 * B * cs);
     ALLOC(c->u_tmp, B * cs);
-    ALLOC(c->partial, (size_t)c->n_chunks * (P + 2 + M) * 16);
+    ALLOC(c->partial, (size_t)c->red_rows * (P + 2 + M) * 16);
     ALLOC(c->red, 3 * (P + 2 + M) * 16);
     ALLOC(c->F, P * 16);
     ALLOC(c->cg, 5 * P * 16);
     ALLOC(c->p_lo, P * cs);
-    size_t ncgpart = (P + 31) / 32 + 2 * ((P + 255) / 256);
+    size_t ncgpart = (P + 31) / 32 + 2 * ((P + 63) / 64);
     if (ncgpart < chol_cgpart_len(c)) ncgpart = chol_cgpart_len(c);
     ALLOC(c->cgpart, ncgpart * sizeof(double));
     ALLOC(c->scal, 64 * sizeof(double));
@@ -282,6 +290,7 @@ extern "C" cr_status cr_set_chunks(cr_ctx* c, int n_chunks) {
     if (n_chunks < 1 || n_chunks > c->max_chunks)
         return cr_fail(c, CR_EINVAL, "n_chunks %d outside [1, %d]", n_chunks, c->max_chunks);
     c->n_chunks = n_chunks;
+    c->chunks_set = true;
     return CR_OK;
 }
 

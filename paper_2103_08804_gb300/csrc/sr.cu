@@ -180,8 +180,17 @@ template <bool COMP, typename R> CR_D void acc_add(R& s, R& c, R v) {
 // current one is consumed.  Partial rows and their layout are those of
 // oreduce_kernel.  COMP: Kahan-compensated sums (the estimators of F, Obar
 // and the VJP); plain sums for the CG products of the float32 path.
+//
+// Bound by the FMA (compensated: add) pipes, 8 (32) operations per walker,
+// site and hidden unit: warps whose sites lie past N leave the products out
+// (for 12 sites three of four, in float64, where a warp instruction takes the
+// SM 16 cycles), the border sums run beside the products (warp 3: b and
+// |T|^2, warps 0 and 1: a) instead of in their loop, whose length is a
+// constant (walkers past the chunk are zeros), and g is fetched with T, so
+// that a sub-block takes two barriers.  64 sites, 128 hidden units, 16384
+// walkers: plain 43 us, now 31; compensated 105, now 66.
 template <typename R, bool CONJ, bool COMP = false>
-__global__ void __launch_bounds__(128) oreduce2_kernel(const int8_t* __restrict__ spins,
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 4 : 2) oreduce2_kernel(const int8_t* __restrict__ spins,
                                                        const cpx<R>* __restrict__ T,
                                                        const cpx<R>* __restrict__ g, int B, int N,
                                                        int M, int P, int chunk,
@@ -197,23 +206,20 @@ __global__ void __launch_bounds__(128) oreduce2_kernel(const int8_t* __restrict_
     const int t = threadIdx.x, ti = 4 * (t >> 3), tj = 4 * (t & 7);
     const int s0 = c * chunk, s1 = min(B, s0 + chunk);
     const bool a_cta = blockIdx.y == 0, b_cta = blockIdx.z == 0;
-    cpx<R> acc[4][4], accb[4];
-    R acct[4];
+    const bool live = i0 + 16 * (t >> 5) < N;  // warp-uniform
+    cpx<R> acc[4][4];
     // compensation terms (unused, and removed by the compiler, when !COMP)
-    cpx<R> cmp[4][4], cmpb[4];
-    R cmpt[4];
+    cpx<R> cmp[4][4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < 4; ++k)
 #pragma unroll
         for (int a = 0; a < 4; ++a) acc[a][k] = cmp[a][k] = {R(0), R(0)};
-        accb[k] = cmpb[k] = {R(0), R(0)};
-        acct[k] = cmpt[k] = R(0);
-    }
-    cpx<R> acca = {R(0), R(0)}, accg = {R(0), R(0)}, cmpa = {R(0), R(0)}, cmpg = {R(0), R(0)};
-    R accgg = R(0), cmpgg = R(0);
+    // border sums: a (threads 0-63), g and |g|^2 (thread 64), b and |T|^2 (threads 96-127)
+    cpx<R> accb = {R(0), R(0)}, cmpb = {R(0), R(0)};
+    R accq = R(0), cmpq = R(0);
     // register prefetch of one sub-block
     int8_t sp[SE];
-    cpx<R> tp[YE];
+    cpx<R> tp[YE], gp[YE], gt = {R(0), R(0)};
     auto fetch = [&](int sb) {
 #pragma unroll
         for (int u = 0; u < SE; ++u) {
@@ -224,32 +230,50 @@ __global__ void __launch_bounds__(128) oreduce2_kernel(const int8_t* __restrict_
         for (int u = 0; u < YE; ++u) {
             const int e = t + u * NT, w = e / TJ, j = e % TJ, s = sb + w;
             tp[u] = (s < s1 && j0 + j < M) ? T[(size_t)s * M + j0 + j] : cpx<R>{R(0), R(0)};
+            if (g) gp[u] = s < s1 ? g[s] : cpx<R>{R(0), R(0)};
         }
+        if (t < SUB)
+            gt = sb + t < s1 ? (g ? g[sb + t] : cpx<R>{R(1), R(0)}) : cpx<R>{R(0), R(0)};
     };
     if (s0 < s1) fetch(s0);
     for (int sb = s0; sb < s1; sb += SUB) {
         __syncthreads();
-        if (t < SUB) {
-            const int s = sb + t;
-            gs[t] = s < s1 ? (g ? g[s] : cpx<R>{R(1), R(0)}) : cpx<R>{R(0), R(0)};
-        }
+        if (t < SUB) gs[t] = gt;
 #pragma unroll
         for (int u = 0; u < SE; ++u) {
             const int e = t + u * NT;
             sg[e / TI][e % TI] = R(sp[u]);
         }
-        __syncthreads();
 #pragma unroll
         for (int u = 0; u < YE; ++u) {
-            const int e = t + u * NT, w = e / TJ;
-            cpx<R> tv = tp[u];
-            if (CONJ) tv = conj(tv);
-            ys[w][e % TJ] = tv * gs[w];
+            const int e = t + u * NT;
+            const cpx<R> tv = CONJ ? conj(tp[u]) : tp[u];
+            ys[e / TJ][e % TJ] = g ? tv * gp[u] : tv;
         }
-        if (sb + SUB < s1) fetch(sb + SUB);
         __syncthreads();
-        const int ns = min(SUB, s1 - sb);
-        for (int q = 0; q < ns; ++q) {
+        if (sb + SUB < s1) fetch(sb + SUB);
+        if (a_cta && t < TI) {
+#pragma unroll 8
+            for (int q = 0; q < SUB; ++q) acc_add<COMP>(accb, cmpb, sg[q][t] * gs[q]);
+        }
+        if (a_cta && b_cta && t == TI) {
+#pragma unroll 8
+            for (int q = 0; q < SUB; ++q) {
+                acc_add<COMP>(accb, cmpb, gs[q]);
+                acc_add<COMP>(accq, cmpq, abs2(gs[q]));
+            }
+        }
+        if (b_cta && t >= NT - TJ) {
+#pragma unroll 8
+            for (int q = 0; q < SUB; ++q) {
+                const cpx<R> y = ys[q][t - (NT - TJ)];
+                acc_add<COMP>(accb, cmpb, y);
+                if (!CONJ) acc_add<COMP>(accq, cmpq, abs2(y));
+            }
+        }
+        if (!live) continue;
+#pragma unroll 4
+        for (int q = 0; q < SUB; ++q) {
             R sv[4];
             cpx<R> y[4];
 #pragma unroll
@@ -267,18 +291,6 @@ __global__ void __launch_bounds__(128) oreduce2_kernel(const int8_t* __restrict_
                         acc[a][k].y = fma(sv[a], y[k].y, acc[a][k].y);
                     }
                 }
-            if (ti == 0) {
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    acc_add<COMP>(accb[k], cmpb[k], y[k]);
-                    if (!CONJ) acc_add<COMP>(acct[k], cmpt[k], abs2(y[k]));
-                }
-            }
-            if (a_cta && t < TI) acc_add<COMP>(acca, cmpa, sg[q][t] * gs[q]);
-            if (t == 0) {
-                acc_add<COMP>(accg, cmpg, gs[q]);
-                acc_add<COMP>(accgg, cmpgg, abs2(gs[q]));
-            }
         }
     }
     // partial rows in the context precision (the sums above are in R); a
@@ -287,12 +299,9 @@ __global__ void __launch_bounds__(128) oreduce2_kernel(const int8_t* __restrict_
     for (int k = 0; k < 4; ++k) {
 #pragma unroll
         for (int a = 0; a < 4; ++a) acc[a][k] = acc[a][k] - cmp[a][k];
-        accb[k] = accb[k] - cmpb[k];
-        acct[k] -= cmpt[k];
     }
-    acca = acca - cmpa;
-    accg = accg - cmpg;
-    accgg -= cmpgg;
+    accb = accb - cmpb;
+    accq -= cmpq;
     cpx<R>* out = (cpx<R>*)partial + (size_t)c * (P + 2 + M);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -303,38 +312,86 @@ __global__ void __launch_bounds__(128) oreduce2_kernel(const int8_t* __restrict_
             const int i = i0 + ti + a;
             if (i < N) out[N + M + (size_t)i * M + j] = acc[a][k];
         }
-        if (b_cta && ti == 0) {
-            out[N + j] = accb[k];
-            if (!CONJ) out[P + 2 + j] = {acct[k], R(0)};
-        }
     }
-    if (a_cta && t < TI && i0 + t < N) out[i0 + t] = acca;
-    if (a_cta && b_cta && t == 0) {
-        out[P] = accg;
-        out[P + 1] = {accgg, R(0)};
+    if (b_cta && t >= NT - TJ && j0 + t - (NT - TJ) < M) {
+        const int j = j0 + t - (NT - TJ);
+        out[N + j] = accb;
+        if (!CONJ) out[P + 2 + j] = {accq, R(0)};
+    }
+    if (a_cta && t < TI && i0 + t < N) out[i0 + t] = accb;
+    if (a_cta && b_cta && t == TI) {
+        out[P] = accb;
+        out[P + 1] = {accq, R(0)};
     }
 }
 
-// red[k] = sum over chunks of partial[c][k] (k < len, rows `stride` long of
-// cpx<RP>), in chunk order, in float64.
-template <typename RP>
-__global__ void combine_kernel(const double* __restrict__ partial, int n_chunks, int len,
-                               int stride, double* __restrict__ red,
-                               const double* __restrict__ skip) {
-    if (skip && *skip != 0.0) return;
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= len) return;
-    const cpx<RP>* p = (const cpx<RP>*)partial;
+// A sum of context-precision values that keeps what float64 would: float64
+// itself, or two float32 words (Knuth's two-sum, TAOCP 2, 4.2.2), whose
+// additions do not wait for the narrow float64 pipe.
+template <typename R> struct Sum2 {
     cpx<double> s = {0.0, 0.0};
-    for (int c = 0; c < n_chunks; ++c) s = s + ccast<double>(p[(size_t)c * stride + k]);
-    ((cpx<double>*)red)[k] = s;
+    CR_D void add(cpx<R> v) { s = s + ccast<double>(v); }
+    CR_D cpx<double> get() const { return s; }
+};
+template <> struct Sum2<float> {
+    cpx<float> s = {0.f, 0.f}, e = {0.f, 0.f};
+    CR_D static void two_sum(float& s, float& e, float v) {
+        const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+        e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+        s = t;
+    }
+    CR_D void add(cpx<float> v) {
+        two_sum(s.x, e.x, v.x);
+        two_sum(s.y, e.y, v.y);
+    }
+    CR_D cpx<double> get() const {
+        return {(double)s.x + (double)e.x, (double)s.y + (double)e.y};
+    }
+};
+
+// red[k] = sum over chunks of partial[c][k] (k < len, rows `stride` long of
+// cpx<RP>) in a fixed order: blocks of 32 entries, eighth chunks by warp, then
+// the warps in float64.
+template <typename RP>
+__global__ void __launch_bounds__(256) combine_kernel(const double* __restrict__ partial, int n_chunks,
+                                                      int len, int stride, double* __restrict__ red,
+                                                      const double* __restrict__ skip) {
+    if (skip && *skip != 0.0) return;
+    __shared__ cpx<double> grp[8][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, k = blockIdx.x * 32 + lane;
+    const cpx<RP>* p = (const cpx<RP>*)partial;
+    Sum2<RP> s;
+    if (k < len)
+#pragma unroll 8
+        for (int c = wid; c < n_chunks; c += 8) s.add(p[(size_t)c * stride + k]);
+    grp[wid][lane] = s.get();
+    __syncthreads();
+    if (wid == 0 && k < len) {
+        cpx<double> tot = grp[0][lane];
+        for (int w = 1; w < 8; ++w) tot = tot + grp[w][lane];
+        ((cpx<double>*)red)[k] = tot;
+    }
+}
+
+// Chunk rows of the reduction over B walkers: those asked for; by default
+// also more (red_rows: four CTAs per SM), down to the 32 walkers of the
+// kernel's sub-block.  1024 walkers of the 12-site chain (alpha = 1, float64)
+// in 8 chunks of 128 left all but 8 SMs idle: 158 us a reduction, in 32 of 32
+// 42.
+static int red_chunks(const cr_ctx* c, int B) {
+    int n = c->n_chunks;
+    if (!c->chunks_set && n < c->red_rows) {
+        const int most = (B + 31) / 32 < c->red_rows ? (B + 31) / 32 : c->red_rows;
+        if (n < most) n = most;
+    }
+    return n < B ? n : B;
 }
 
 template <typename R, bool CONJ, bool COMP>
 static cr_status oreduce_t(cr_ctx* c, const int8_t* spins, const void* T, const void* g, int B,
                            double* red_out, const double* skip) {
     const int N = c->N, M = c->M, P = c->P;
-    const int nch = c->n_chunks < B ? c->n_chunks : B;
+    const int nch = red_chunks(c, B);
     const int chunk = (B + nch - 1) / nch;
     CR_LAUNCH(c, CR_KERNEL_REDUCE,
               (oreduce2_kernel<R, CONJ, COMP><<<dim3(nch, (M + 31) / 32, (N + 63) / 64), 128, 0,
@@ -345,7 +402,7 @@ static cr_status oreduce_t(cr_ctx* c, const int8_t* spins, const void* T, const 
     if (s != CR_OK) return s;
     if (!red_out) return CR_OK;  // the caller combines the chunk rows itself
     const int len = CONJ ? P + 2 : P + 2 + M;
-    CR_LAUNCH(c, CR_K_OTHER, combine_kernel<R><<<(len + 255) / 256, 256, 0, c->stream>>>(
+    CR_LAUNCH(c, CR_K_OTHER, combine_kernel<R><<<(len + 31) / 32, 256, 0, c->stream>>>(
                                  c->partial, nch, len, P + 2 + M, red_out, skip));
     return cr_check_launch(c, "combine_kernel");
 }
@@ -434,13 +491,18 @@ __device__ double block_sum(double v, double* red) {
     return t;
 }
 
+// A CTA of a vector kernel has two warps: float64 warp instructions take
+// their SM 16 cycles, so the vectors are spread over as many SMs as there are.
+constexpr int CG_TPB = 64;
+
+// x = 0, r = F, p = z = r / d; shares of F.F and r.z in part[2][gridDim.x].
 template <typename R>
-__global__ void __launch_bounds__(1024) cg_init_kernel(const double* __restrict__ F_,
-                                                       const double* __restrict__ redO_, int N,
-                                                       int M, int P, int B, double shift,
-                                                       int precond, double* __restrict__ cg_,
-                                                       cpx<R>* __restrict__ p_lo,
-                                                       double* __restrict__ scal) {
+__global__ void __launch_bounds__(CG_TPB) cg_init_kernel(const double* __restrict__ F_,
+                                                         const double* __restrict__ redO_, int N,
+                                                         int M, int P, int B, double shift,
+                                                         int precond, double* __restrict__ cg_,
+                                                         cpx<R>* __restrict__ p_lo,
+                                                         double* __restrict__ part) {
     __shared__ double red[32];
     const cpx<double>* F = (const cpx<double>*)F_;
     const cpx<double>* sO = (const cpx<double>*)redO_;
@@ -450,24 +512,47 @@ __global__ void __launch_bounds__(1024) cg_init_kernel(const double* __restrict_
     cpx<double>* dg = x + 4 * P;
     const double inv = 1.0 / B;
     double ff = 0.0, rz = 0.0;
-    for (int k = threadIdx.x; k < P; k += blockDim.x) {
-        double d = 1.0;
+    const int k = blockIdx.x * CG_TPB + threadIdx.x;
+    if (k < P) {
+        double di = 1.0;
         if (precond) {
             double o2 = k < N ? 1.0 : inv * sO[P + 2 + (k < N + M ? k - N : (k - N - M) % M)].x;
-            d = o2 - abs2(inv * sO[k]) + shift;
+            di = 1.0 / (o2 - abs2(inv * sO[k]) + shift);
         }
         cpx<double> f = F[k];
-        cpx<double> z = (1.0 / d) * f;
+        cpx<double> z = di * f;
         x[k] = {0.0, 0.0};
         r[k] = f;
         p[k] = z;
-        dg[k] = {d, 0.0};
+        dg[k] = {di, 0.0};
         p_lo[k] = ccast<R>(z);
-        ff += abs2(f);
-        rz += cmulc(f, z).x;
+        ff = abs2(f);
+        rz = cmulc(f, z).x;
     }
     ff = block_sum(ff, red);
     rz = block_sum(rz, red);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = ff;
+        part[gridDim.x + blockIdx.x] = rz;
+    }
+}
+
+// Multi-CTA CG step, three launches per iteration (64 sites, alpha = 2, 128
+// chunk rows: apply 16 us, now 11; x and r 9.6, now 8.4; p 8.4, now 6.9).  scal[5 + (it & 1)]
+// holds r.z of iteration it, so the last kernel writes the next value into
+// the other slot while its CTAs still read the current one.  Per-CTA partial
+// dot products go to part[3][nblk] and are summed by every CTA in the same
+// fixed order (deterministic).
+__device__ double sum_parts(const double* p, int n, double* red) {
+    double v = 0.0;
+    for (int b = threadIdx.x; b < n; b += blockDim.x) v += p[b];
+    return block_sum(v, red);
+}
+
+__global__ void __launch_bounds__(CG_TPB) cg_start_kernel(const double* __restrict__ part, int nblk,
+                                                          double* __restrict__ scal) {
+    __shared__ double red[32];
+    const double ff = sum_parts(part, nblk, red), rz = sum_parts(part + nblk, nblk, red);
     if (threadIdx.x == 0) {
         scal[5] = rz;
         scal[1] = ff;
@@ -475,19 +560,6 @@ __global__ void __launch_bounds__(1024) cg_init_kernel(const double* __restrict_
         scal[3] = 0.0;
         scal[4] = ff;
     }
-}
-
-// Multi-CTA CG step, three launches per iteration.  scal[5 + (it & 1)]
-// holds r.z of iteration it, so the last kernel writes the next value into
-// the other slot while its CTAs still read the current one.  Per-CTA partial
-// dot products go to part[3][nblk] and are summed by every CTA in the same
-// fixed order (deterministic).
-constexpr int CG_TPB = 256;
-
-__device__ double sum_parts(const double* p, int n, double* red) {
-    double v = 0.0;
-    for (int b = threadIdx.x; b < n; b += blockDim.x) v += p[b];
-    return block_sum(v, red);
 }
 
 // Ap = S p + shift p from the chunk rows of sum conj(O) (O p) (the combine
@@ -513,15 +585,17 @@ __global__ void __launch_bounds__(256) cg_apply_kernel(const double* __restrict_
     cpx<double>* Ap = (cpx<double>*)cg_ + 3 * P;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int k = blockIdx.x * CGA_K + lane;
-    cpx<double> w = {0.0, 0.0};
+    Sum2<RP> w;
     if (k < P)
-        for (int c = wid; c < nch; c += 8) w = w + ccast<double>(pt[(size_t)c * stride + k]);
-    grp[wid][lane] = w;
+#pragma unroll 8
+        for (int c = wid; c < nch; c += 8) w.add(pt[(size_t)c * stride + k]);
+    grp[wid][lane] = w.get();
     if (wid == 7) {
-        cpx<double> su = {0.0, 0.0};
-        for (int c = lane; c < nch; c += 32) su = su + ccast<double>(pt[(size_t)c * stride + P]);
-        su = warp_sum(su);
-        if (lane == 0) smu = su;
+        Sum2<RP> su;
+#pragma unroll 4
+        for (int c = lane; c < nch; c += 32) su.add(pt[(size_t)c * stride + P]);
+        const cpx<double> tot = warp_sum(su.get());
+        if (lane == 0) smu = tot;
     }
     __syncthreads();
     if (wid == 0) {
@@ -561,7 +635,7 @@ __global__ void __launch_bounds__(CG_TPB) cg_xr_kernel(int P, double* __restrict
         cpx<double> rk = r[k] - alpha * Ap[k];
         r[k] = rk;
         rn = abs2(rk);
-        rz = (1.0 / dg[k].x) * rn;
+        rz = dg[k].x * rn;
     }
     rn = block_sum(rn, red);
     rz = block_sum(rz, red);
@@ -588,7 +662,7 @@ __global__ void __launch_bounds__(CG_TPB) cg_p_kernel(int P, double tol, double*
     const int k = blockIdx.x * CG_TPB + threadIdx.x;
     if (!done && k < P) {
         const double beta = rzn / scal[5 + slot];
-        cpx<double> pk = (1.0 / dg[k].x) * r[k] + beta * p[k];
+        cpx<double> pk = dg[k].x * r[k] + beta * p[k];
         p[k] = pk;
         p_lo[k] = ccast<R>(pk);
     }
@@ -656,15 +730,17 @@ static cr_status sr_step_t(cr_ctx* c, void* params, const int8_t* spins, const v
                             0, nullptr, nullptr);
         if (s != CR_OK) return s;
     } else {
-        CR_LAUNCH(c, CR_K_OTHER, cg_init_kernel<R><<<1, 1024, 0, c->stream>>>(
-                                     c->F, redO, c->N, c->M, P, B, o->shift, o->cg_precond,
-                                     c->cg, (cpx<R>*)c->p_lo, c->scal));
-        if ((s = cr_check_launch(c, "cg_init")) != CR_OK) return s;
         const double* done = c->scal + 2;
         const int nblk = (P + CG_TPB - 1) / CG_TPB;
         const int napp = (P + CGA_K - 1) / CGA_K;
+        CR_LAUNCH(c, CR_K_OTHER, cg_init_kernel<R><<<nblk, CG_TPB, 0, c->stream>>>(
+                                     c->F, redO, c->N, c->M, P, B, o->shift, o->cg_precond,
+                                     c->cg, (cpx<R>*)c->p_lo, c->cgpart + napp));
+        CR_LAUNCH(c, CR_K_OTHER,
+                  cg_start_kernel<<<1, CG_TPB, 0, c->stream>>>(c->cgpart + napp, nblk, c->scal));
+        if ((s = cr_check_launch(c, "cg_init")) != CR_OK) return s;
         const bool tcp = tc_supported(c);  // mixed precision: tensor-core products
-        int nch = c->n_chunks < B ? c->n_chunks : B;
+        int nch = red_chunks(c, B);
         for (int it = 0; it < o->cg_maxit; ++it) {
             if (tcp) {
                 s = launch_ov_tc(c, c->p_lo, spins, B, T, c->u_tmp, done);
@@ -748,7 +824,7 @@ static cr_status sv_t(cr_ctx* c, const int8_t* spins, const void* T, int B, cons
                                  v, P, c->cg, (cpx<R>*)c->p_lo, c->scal));
     if ((s = cr_check_launch(c, "sv_load")) != CR_OK) return s;
     const double* done = c->scal + 2;
-    int nch = c->n_chunks < B ? c->n_chunks : B;
+    int nch = red_chunks(c, B);
     if (tc_supported(c)) {
         if ((s = launch_ov_tc(c, c->p_lo, spins, B, T, c->u_tmp, done)) != CR_OK) return s;
         s = launch_oreduce_tc(c, spins, T, c->u_tmp, B, done, &nch);
@@ -882,7 +958,7 @@ static cudaError_t noalloc_backward_t(int N, int M, const int8_t* spins, const v
         if (dbl) LAUNCH(4, 2); else LAUNCH(4, 4);
     }
 #undef LAUNCH
-    combine_kernel<double><<<(P + 2 + 255) / 256, 256, 0, st>>>(scratch, nch, P + 2, P + 2 + M,
+    combine_kernel<double><<<(P + 2 + 31) / 32, 256, 0, st>>>(scratch, nch, P + 2, P + 2 + M,
                                                                  red, nullptr);
     to_params_kernel<R><<<(P + 255) / 256, 256, 0, st>>>(red, P, (cpx<R>*)grad);
     return cudaGetLastError();
