@@ -297,6 +297,21 @@ cr_status logpsi_backward(cr_ctx* ctx, const cr_state* state, const int8_t* spin
                           const void* tanh_theta, int B, const void* grad_logpsi,
                           void* grad_params);
 
+/* The overlap loss of the fit on fixed samples of |psi_0|^2 (Sec. III),
+   L = -log(|sum w R'|^2 / (sum w |R'|^2 sum w)), w = |psi / psi_0|^2,
+   R' = R psi_0 / psi, from log psi, log psi_0 and R (complex [B], context
+   precision), and its gradient with respect to log psi (dL/dRe + i dL/dIm)
+   times the scalar grad_loss.  sums: 4 + 4 * 128 float64 of the caller's,
+   written by the first call and read by the second; loss and grad_loss: one
+   real of the context precision on the device.  overlap_loss overwrites logpsi
+   with d = log psi - log psi_0, the backward's input.  Both run on `stream`.
+   B >= 1. */
+cr_status overlap_loss(cr_ctx* ctx, void* logpsi, const void* logpsi0, const void* R, int B,
+                       double* sums, void* loss, void* stream);
+cr_status overlap_loss_backward(cr_ctx* ctx, const void* d, const void* R, int B,
+                                const double* sums, const void* grad_loss, void* grad_logpsi,
+                                void* stream);
+
 /* logpsi_backward without any allocation.  The paper has no counterpart:
    this entry point exists for callers that cannot allocate device memory
    themselves -- code inside a framework whose caching allocator owns the

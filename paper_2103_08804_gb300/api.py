@@ -32,7 +32,7 @@ SYMBOLS = ("cr_create", "cr_destroy", "cr_set_stream", "cr_last_error", "cr_sync
            "logpsi_backward_noalloc", "cr_set_chunks", "cr_max_chunks", "sr_smatrix",
            "cheb_spectrum", "cheb_lorentzian", "cheb_extrapolate", "sym_workspace_bytes", "sym_btilde",
            "sym_h_workspace_bytes", "sym_hbtilde", "cheb_init_params", "sr_sv", "cr_fused_cg",
-           "cr_set_fcg_ctas", "cr_batch_run")
+           "cr_set_fcg_ctas", "cr_batch_run", "overlap_loss", "overlap_loss_backward")
 KERNEL = {"sweep": 0, "target": 1, "theta": 2, "ov": 3, "reduce": 4, "cg": 5, "sbuild": 6,
           "chol": 7, "trsv": 8, "fcg": 9, "gram": 10}
 
@@ -100,6 +100,8 @@ def load(path=None):
     lib.cheb_local_target.argtypes = [vp, ctypes.POINTER(Target), vp, vp, i, vp, vp]
     lib.logderiv.argtypes = [vp, ctypes.POINTER(State), vp, vp, i, vp, vp]
     lib.logpsi_backward.argtypes = [vp, ctypes.POINTER(State), vp, vp, i, vp, vp]
+    lib.overlap_loss.argtypes = [vp, vp, vp, vp, i, vp, vp, vp]
+    lib.overlap_loss_backward.argtypes = [vp, vp, vp, i, vp, vp, vp, vp]
     lib.sr_step.argtypes = [vp, vp, vp, vp, vp, i, ctypes.POINTER(SROpts), vp]
     lib.cheb_moment.argtypes = [vp, ctypes.POINTER(State), vp, d, d, vp, vp, i,
                                 ctypes.POINTER(d), vp, vp, vp]
@@ -325,6 +327,32 @@ class Context:
                                              _ptr(tanh_theta), B, _ptr(grad_logpsi),
                                              _ptr(grad_params)), "logpsi_backward")
         return grad_params
+
+    def overlap_loss(self, logpsi, logpsi0, R):
+        """The overlap loss of log psi against the targets R on samples of psi_0
+        (a real scalar) and the sums its backward needs, on torch's current
+        stream; logpsi becomes logpsi - logpsi0."""
+        B = logpsi.shape[0]
+        for t, name in ((logpsi, "logpsi"), (logpsi0, "logpsi0"), (R, "R")):
+            self._c(t, (B,), name)
+        sums = torch.empty(4 + 4 * 128, dtype=torch.float64, device=logpsi.device)
+        loss = torch.empty((), dtype=logpsi.real.dtype, device=logpsi.device)
+        st = torch.cuda.current_stream(logpsi.device).cuda_stream
+        self._check(self.lib.overlap_loss(self.h, _ptr(logpsi), _ptr(logpsi0), _ptr(R), B, _ptr(sums),
+                                          _ptr(loss), ctypes.c_void_p(st)), "overlap_loss")
+        return loss, sums
+
+    def overlap_loss_backward(self, d, R, sums, grad_loss):
+        """The gradient of overlap_loss with respect to logpsi, times grad_loss;
+        d is what overlap_loss left in its logpsi."""
+        B = d.shape[0]
+        self._c(d, (B,), "d")
+        self._c(R, (B,), "R")
+        g = torch.empty_like(d)
+        st = torch.cuda.current_stream(d.device).cuda_stream
+        self._check(self.lib.overlap_loss_backward(self.h, _ptr(d), _ptr(R), B, _ptr(sums), _ptr(grad_loss),
+                                                   _ptr(g), ctypes.c_void_p(st)), "overlap_loss_backward")
+        return g
 
     def cheb_init_params(self, n, psi, prev, out):
         """Starting parameters of projection step n into out (n == 1: psi with

@@ -913,6 +913,141 @@ extern "C" cr_status logpsi_backward(cr_ctx* ctx, const cr_state* st, const int8
     return cr_check_launch(ctx, "to_params");
 }
 
+// ------------------------------------------------------ overlap loss
+//
+// L = -log(|S1|^2 / (S2 S3)), with d = log psi - log psi_0, w = exp(2 Re d),
+// Ra = R exp(-d), S1 = sum w Ra, S2 = sum w |Ra|^2, S3 = sum w; and its
+// gradient dL/dRe + i dL/dIm of each log psi_s, 2 (w / S3 - w Ra / S1) (S2 does
+// not depend on psi).  Terms in the context precision, sums in float64 in a
+// fixed order.  As separate tensor operations the loss and its gradient were
+// some sixty launches, whose host time, 1.1 ms, was that of a whole gradient
+// of the 10 x 10 lattice (32768 walkers, float32); as three the gradient takes
+// 0.35 ms.
+constexpr int OVL_BLOCKS = 128;
+
+template <typename R> struct ovl_term {
+    R w;
+    cpx<R> wra;
+    R w2;
+    CR_D ovl_term(cpx<R> d, cpx<R> r) {
+        R sn, cs;
+        if constexpr (sizeof(R) == 8) sincos(-d.y, &sn, &cs);
+        else sincosf(-d.y, &sn, &cs);
+        const R m = exp(-d.x);
+        w = exp(R(2) * d.x);
+        const cpx<R> ra = r * cpx<R>{m * cs, m * sn};
+        wra = w * ra;
+        w2 = w * abs2(ra);
+    }
+};
+
+template <typename R>
+__global__ void __launch_bounds__(256) overlap_sums_kernel(cpx<R>* __restrict__ lp,
+                                                           const cpx<R>* __restrict__ lp0,
+                                                           const cpx<R>* __restrict__ Rt, int B,
+                                                           double* __restrict__ part) {
+    __shared__ double red[4][8];
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int s = blockIdx.x * 256 + threadIdx.x; s < B; s += gridDim.x * 256) {
+        const cpx<R> d = lp[s] - lp0[s];
+        lp[s] = d;
+        const ovl_term<R> t(d, Rt[s]);
+        v[0] += (double)t.wra.x;
+        v[1] += (double)t.wra.y;
+        v[2] += (double)t.w2;
+        v[3] += (double)t.w;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        v[q] = warp_sum(v[q]);
+        if ((threadIdx.x & 31) == 0) red[q][threadIdx.x >> 5] = v[q];
+    }
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[threadIdx.x][w];
+        part[4 * blockIdx.x + threadIdx.x] = t;
+    }
+}
+
+// sums[0..3] = S1 (re, im), S2, S3 from the block sums behind them; the loss.
+template <typename R>
+__global__ void __launch_bounds__(32) overlap_loss_kernel(double* __restrict__ sums, int nblk,
+                                                          R* __restrict__ loss) {
+    const int lane = threadIdx.x;
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        v[q] = 0.0;
+        for (int b = lane; b < nblk; b += 32) v[q] += sums[4 + 4 * b + q];
+        v[q] = warp_sum(v[q]);
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sums[q] = v[q];
+        *loss = (R)(-log((v[0] * v[0] + v[1] * v[1]) / (v[2] * v[3])));
+    }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) overlap_grad_kernel(const cpx<R>* __restrict__ d,
+                                                           const cpx<R>* __restrict__ Rt, int B,
+                                                           const double* __restrict__ sums,
+                                                           const R* __restrict__ up,
+                                                           cpx<R>* __restrict__ g) {
+    // the two factors once per block
+    __shared__ cpx<double> f1;
+    __shared__ double f3;
+    if (threadIdx.x == 0) {
+        const double u = 2.0 * (double)*up;
+        f1 = cdiv(cpx<double>{u, 0.0}, cpx<double>{sums[0], sums[1]});
+        f3 = u / sums[3];
+    }
+    __syncthreads();
+    const int s = blockIdx.x * 256 + threadIdx.x;
+    if (s >= B) return;
+    const ovl_term<R> t(d[s], Rt[s]);
+    const cpx<double> v = cpx<double>{f3 * (double)t.w, 0.0} - f1 * ccast<double>(t.wra);
+    g[s] = ccast<R>(v);
+}
+
+extern "C" cr_status overlap_loss(cr_ctx* ctx, void* logpsi, const void* logpsi0, const void* R,
+                                  int B, double* sums, void* loss, void* stream) {
+    if (!ctx) return CR_EINVAL;
+    CR_CHECK_ARG(B >= 1, "overlap_loss: B=%d < 1", B);
+    CR_CHECK_ARG(logpsi && logpsi0 && R && sums && loss, "overlap_loss: null array");
+    cudaStream_t st = (cudaStream_t)stream;
+    const int nblk = (B + 255) / 256 < OVL_BLOCKS ? (B + 255) / 256 : OVL_BLOCKS;
+    if (ctx->prec == CR_FP64) {
+        overlap_sums_kernel<double><<<nblk, 256, 0, st>>>((cpx<double>*)logpsi, (const cpx<double>*)logpsi0,
+                                                          (const cpx<double>*)R, B, sums + 4);
+        overlap_loss_kernel<double><<<1, 32, 0, st>>>(sums, nblk, (double*)loss);
+    } else {
+        overlap_sums_kernel<float><<<nblk, 256, 0, st>>>((cpx<float>*)logpsi, (const cpx<float>*)logpsi0,
+                                                         (const cpx<float>*)R, B, sums + 4);
+        overlap_loss_kernel<float><<<1, 32, 0, st>>>(sums, nblk, (float*)loss);
+    }
+    ctx->n_launches += 2;
+    return cr_check_launch(ctx, "overlap_loss");
+}
+
+extern "C" cr_status overlap_loss_backward(cr_ctx* ctx, const void* d, const void* R, int B,
+                                           const double* sums, const void* grad_loss, void* grad_logpsi, void* stream) {
+    if (!ctx) return CR_EINVAL;
+    CR_CHECK_ARG(B >= 1, "overlap_loss_backward: B=%d < 1", B);
+    CR_CHECK_ARG(d && R && sums && grad_loss && grad_logpsi,
+                 "overlap_loss_backward: null array");
+    cudaStream_t st = (cudaStream_t)stream;
+    if (ctx->prec == CR_FP64)
+        overlap_grad_kernel<double><<<(B + 255) / 256, 256, 0, st>>>(
+            (const cpx<double>*)d, (const cpx<double>*)R, B, sums, (const double*)grad_loss, (cpx<double>*)grad_logpsi);
+    else
+        overlap_grad_kernel<float><<<(B + 255) / 256, 256, 0, st>>>(
+            (const cpx<float>*)d, (const cpx<float>*)R, B, sums, (const float*)grad_loss, (cpx<float>*)grad_logpsi);
+    ++ctx->n_launches;
+    return cr_check_launch(ctx, "overlap_loss_backward");
+}
+
 // ------------------------------------- VJP of log psi without allocation
 //
 // For callers that cannot allocate device memory themselves: code running
