@@ -17,9 +17,10 @@
 // therefore copied into the warp's shared memory (cp.async, every lane its own
 // 16 bytes) while the present one is computed, and theta, which only the
 // output needs, is left out of the chain: accepted moves go to a list, and
-// replay_*_kernel applies them in order afterwards (the same subtractions in
-// the same order, independent loads, the table of a slice of 32 units held in
-// L1).  16 x 16 lattice, 65536 walkers: 8.0 -> 6.1 ms, of which the sweep
+// replay_slice_kernel or finish_kernel applies them in order afterwards (the
+// same subtractions in the same order, independent loads, a table too large
+// for L1 taken in slices of its units that fit in shared memory).  16 x 16
+// lattice, 65536 walkers: 8.0 -> 5.5 ms, of which the sweep
 // kernel 4.8; it issues on 65% of its cycles, 480 instructions per evaluated
 // proposal, at 27% of the L2 rate.
 #include "common.cuh"
@@ -241,19 +242,79 @@ CR_D void replay_list(const uint16_t* __restrict__ lst, int n, const cpx<R>* __r
     }
 }
 
-// One warp per (walker, slice of 32 hidden units); slices are the slow grid
-// dimension, so the CTAs running together share one slice of the table in L1.
-template <typename R>
-__global__ void __launch_bounds__(256) replay_slice_kernel(cpx<R>* __restrict__ theta, int B, int M,
-                                                           int Mp, const cpx<R>* __restrict__ Dt,
-                                                           const uint16_t* __restrict__ list, int cap,
-                                                           const int* __restrict__ count) {
-    const int lane = threadIdx.x & 31, w = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (w >= B) return;
-    const int j = 32 * blockIdx.y + lane;
-    cpx<R> th[1] = {j < M ? theta[(size_t)w * M + j] : cpx<R>{R(0), R(0)}};
-    replay_list<R, 1>(list + (size_t)w * cap, count[w], Dt + j, Mp, lane, th);
-    if (j < M) theta[(size_t)w * M + j] = th[0];
+// 16 aligned bytes: two units in float32, one in float64
+CR_D void lds16(const unsigned char* p, cpx<float> (&d)[2]) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    d[0] = {v.x, v.y};
+    d[1] = {v.z, v.w};
+}
+CR_D void lds16(const unsigned char* p, cpx<double> (&d)[1]) {
+    const double2 v = *reinterpret_cast<const double2*>(p);
+    d[0] = {v.x, v.y};
+}
+
+// The same for a table that does not fit in L1: a CTA holds a slice of the
+// units of all bonds in shared memory (LPW pieces of 16 bytes per bond) and
+// takes every ncta-th group of walkers, LPW lanes to a walker.  Bound by
+// shared memory, 8 bytes per move and unit (16 x 16 lattice, alpha = 1, 65536
+// walkers: 0.60 ms; through L1, a warp to a walker and one unit to a lane,
+// 1.17).
+template <typename R, int LPW>
+__global__ void __launch_bounds__(1024, 1) replay_slice_kernel(cpx<R>* __restrict__ theta, int B, int M,
+                                                               int Mp, int Nb, int ncta,
+                                                               const cpx<R>* __restrict__ Dt,
+                                                               const uint16_t* __restrict__ list, int cap,
+                                                               const int* __restrict__ count) {
+    constexpr int U = 16 / sizeof(cpx<R>), JW = LPW * U, GPW = 32 / LPW;
+    extern __shared__ __align__(16) unsigned char sm_rp[];
+    const int slice = blockIdx.x / ncta, part = blockIdx.x % ncta;
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31, grp = lane / LPW, li = lane % LPW;
+    for (int e = t; e < Nb * LPW; e += 1024)
+        cp16(sm_rp + (size_t)e * 16, Dt + (size_t)(e / LPW) * Mp + slice * JW + (e % LPW) * U);
+    cp_commit();
+    cp_wait<0>();
+    __syncthreads();
+    const unsigned char* Ds = sm_rp + li * 16;
+    const int j = slice * JW + li * U;
+    for (int wb = (part * 32 + warp) * GPW; wb < B; wb += ncta * 32 * GPW) {
+        const int w = wb + grp;
+        const int n = w < B ? count[w] : 0;
+        const int nmax = __reduce_max_sync(0xffffffffu, n);
+        const uint16_t* lst = list + (size_t)(w < B ? w : 0) * cap;
+        cpx<R> th[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            th[u] = w < B && j + u < M ? theta[(size_t)w * M + j + u] : cpx<R>{R(0), R(0)};
+        for (int e0 = 0; e0 < nmax; e0 += 4 * LPW) {
+            // four entries a lane (lists start on 8 bytes)
+            uint2 mine = make_uint2(0u, 0u);
+            if (e0 + 4 * li < n) mine = *reinterpret_cast<const uint2*>(lst + e0 + 4 * li);
+            const int m = min(4 * LPW, nmax - e0);
+            for (int c = 0; c < m; c += 4) {
+                const uint32_t x = __shfl_sync(0xffffffffu, mine.x, c >> 2, LPW);
+                const uint32_t y = __shfl_sync(0xffffffffu, mine.y, c >> 2, LPW);
+                cpx<R> d[4][U];
+                R s[4];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    const uint32_t q = v < 2 ? x : y, ent = (v & 1) ? q >> 16 : q & 0xffffu;
+                    const bool in = e0 + c + v < n;
+                    s[v] = ent & LIST_NEG ? R(-1) : R(1);
+                    const unsigned char* row = Ds + (in ? ent & (LIST_NEG - 1) : 0u) * (LPW * 16);
+                    lds16(row, d[v]);
+                }
+#pragma unroll
+                for (int v = 0; v < 4; ++v)
+                    if (e0 + c + v < n)
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            th[u] = {th[u].x - s[v] * d[v][u].x, th[u].y - s[v] * d[v][u].y};
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (w < B && j + u < M) theta[(size_t)w * M + j + u] = th[u];
+    }
 }
 
 // One warp per walker: the listed moves (list may be null: none left), then
@@ -310,6 +371,35 @@ static size_t sweep_smem(const cr_ctx* c) {
     return (size_t)8 * 2 * 32 * KPL * sizeof(cpx<R>) + (size_t)c->Nb * 4 + 4 * (size_t)c->N;
 }
 
+// Lanes per walker of the sliced replay: the widest slice whose table of all
+// bonds fits in shared memory.
+constexpr int REPLAY_SMEM = 224 * 1024;
+static int replay_lanes(const cr_ctx* c, int lanes) {
+    while ((size_t)c->Nb * lanes * 16 > REPLAY_SMEM) lanes /= 2;
+    return lanes;
+}
+
+template <typename R, int LPW>
+static void launch_replay(cr_ctx* c, cpx<R>* th, int B, const cpx<R>* D, int cap) {
+    constexpr int JW = LPW * 16 / (int)sizeof(cpx<R>), walkers = 32 * (32 / LPW);
+    const int ns = (c->M + JW - 1) / JW, most = (B + walkers - 1) / walkers;
+    int ncta = c->n_sm / ns > 1 ? c->n_sm / ns : 1;
+    if (ncta > most) ncta = most;
+    CR_LAUNCH(c, CR_K_OTHER,
+              (replay_slice_kernel<R, LPW><<<ns * ncta, 1024, (size_t)c->Nb * LPW * 16, c->stream>>>(
+                  th, B, c->M, c->Mp, c->Nb, ncta, D, c->sw_list, cap, c->sw_count)));
+}
+
+template <typename R>
+static void launch_replay_slices(cr_ctx* c, cpx<R>* th, int B, const cpx<R>* D, int cap) {
+    switch (replay_lanes(c, sizeof(R) == 4 ? 16 : 32)) {
+        case 32: launch_replay<R, 32>(c, th, B, D, cap); break;
+        case 16: launch_replay<R, 16>(c, th, B, D, cap); break;
+        case 8: launch_replay<R, 8>(c, th, B, D, cap); break;
+        default: launch_replay<R, 4>(c, th, B, D, cap); break;
+    }
+}
+
 template <typename R, int KPL>
 static cr_status sweep_k(cr_ctx* c, const void* params, int8_t* spins, void* theta, int B, int n_prop,
                          uint64_t seed, uint64_t counter, const uint64_t* dcounter, void* logpsi_out,
@@ -319,7 +409,7 @@ static cr_status sweep_k(cr_ctx* c, const void* params, int8_t* spins, void* the
     const cpx<R>* D = (const cpx<R>*)t.D;
     const int cap = sweep_list_cap(c), grid = (B + 3) / 4;
     // a table that fits in L1 beside the loads in flight is replayed whole, by the finishing warps;
-    // a larger one in slices of 32 units, each of which does
+    // a larger one in slices of units that fit in shared memory
     const bool slices = (size_t)c->Nb * c->Mp * sizeof(cpx<R>) > 128 * 1024 && KPL > 1;
     int p = 0;
     do {
@@ -332,10 +422,7 @@ static cr_status sweep_k(cr_ctx* c, const void* params, int8_t* spins, void* the
                           (const cpx<R>*)t.CS, (const cpx<R>*)t.ea, p, np, !last, (uint32_t)seed,
                           (uint32_t)(seed >> 32), (unsigned long long)counter,
                           (const unsigned long long*)dcounter, c->sw_list, cap, c->sw_count)));
-        if (np > 0 && slices)
-            CR_LAUNCH(c, CR_K_OTHER,
-                      (replay_slice_kernel<R><<<dim3((B + 7) / 8, KPL), 256, 0, c->stream>>>(
-                          th, B, c->M, c->Mp, D, c->sw_list, cap, c->sw_count)));
+        if (np > 0 && slices) launch_replay_slices<R>(c, th, B, D, cap);
         CR_LAUNCH(c, CR_K_OTHER,
                   (finish_kernel<R, KPL><<<grid, 128, 0, c->stream>>>(
                       (const cpx<R>*)params, spins, th, B, c->N, c->M, D,
@@ -376,6 +463,13 @@ static cr_status sweep_prepare_t(cr_ctx* c) {
         OPT(1) OPT(2) OPT(4) OPT(8) OPT(16)
     }
 #undef OPT
+    const auto opt = [&](const void* f) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, REPLAY_SMEM);
+    };
+    opt((const void*)replay_slice_kernel<R, 32>);
+    opt((const void*)replay_slice_kernel<R, 16>);
+    opt((const void*)replay_slice_kernel<R, 8>);
+    opt((const void*)replay_slice_kernel<R, 4>);
     return e == cudaSuccess ? CR_OK : cr_fail(c, CR_ECUDA, "sweep_prepare: %s", cudaGetErrorString(e));
 }
 

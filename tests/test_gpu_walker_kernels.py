@@ -101,3 +101,27 @@ def test_exchange_sums_at_tile_edges(Lx, Ly, M, n, sigma, tol):
     lp_ref = rbm.logpsi(psin, N, M, spins)
     ref = target.local_target(n, prev, prev2, bp, bp2, N, M, Lx, Ly, J, E0, a, Wp, q, spins, lp_ref)
     assert relerr(host(R) * np.exp(host(lpn) - lp_ref), ref) < tol
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("Lx,Ly,M,B", [(10, 10, 130, 41), (28, 28, 40, 5), (32, 32, 33, 3)])
+def test_sweep_replays_large_tables_in_slices(prec, Lx, Ly, M, B):
+    """Tables over 128 KB: slices of the widest to the narrowest kind, walker
+    counts that fill no group, hidden units that end inside a slice."""
+    from paper_2103_08804_gb300 import api
+    N = Lx * Ly
+    p, cd, _ = PRECS[prec]
+    params = synth.rbm_params(7 + M, N, M, 0.02)
+    spins0 = synth.sz0_spins(8, B, N)
+    ctx = api.Context(Lx, Ly, M, B, prec=p)
+    sp, pr = dev(spins0, torch.int8), dev(params, cd)
+    th = torch.empty(B, M, dtype=cd, device="cuda")
+    ctx.rbm_logpsi(pr, sp, theta_out=th)
+    rng = api.Philox(4321, 7)
+    ctx.mc_sweep(pr, sp, th, 1, rng)
+    s_ref, _, _ = sampler.mc_sweep(params, N, M, lattice.bonds(Lx, Ly), spins0, 1, 4321, 7,
+                                   walker_ids=np.arange(B))
+    s = host(sp)
+    same = np.all(s == s_ref, axis=1)
+    assert np.all(same) if p == 0 else same.sum() >= B - 2
+    assert relerr(host(th), rbm.theta(params, N, M, s)) < (1e-10 if p == 0 else 1e-4)
