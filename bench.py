@@ -856,10 +856,10 @@ def run_reference_sym6(args, ws, cores, n_samples=24):
 
 
 SYM6 = {"L": 6, "M": 72, "walkers": 4096, "states": 150, "sigma": 0.02, "Wp": 0.9875}
-# sym_hprime_kernel work per (antiparallel bond, hidden unit): cosh(theta - s D)
-# = cosh(theta) cosh(D) - s sinh(theta) sinh(D), two complex multiplies and
-# one complex subtract, then one complex multiply into the running product
-SYM6_FLOP_PER_BOND_UNIT = 20
+# xsum_kernel work per (antiparallel bond, hidden unit): the factor a + z q of
+# cosh(theta - s D), one complex multiply-add with a real addend (7 flop), and
+# one complex multiply into the running product (6)
+SYM6_FLOP_PER_BOND_UNIT = 13
 
 
 def sym6_oracle_seconds(n_samples=48):
@@ -967,7 +967,7 @@ def run_sym6(args):
     Bi = sum(t.numel() * t.element_size() for t in pin.values())
     Bo = 2 * G_h.numel() * G_h.element_size()
 
-    # live timing of the dominant kernel (sym_hprime_kernel, (H' t_n)(s') /
+    # live timing of the dominant kernel (xsum_kernel, (H' t_n)(s') /
     # psi(s) at every transformed configuration), as an FP32 ALU roofline
     ctx.time_kernel("target", 4096)
     step(params, spins, lref)
@@ -982,8 +982,8 @@ def run_sym6(args):
     f_sm = clocks.get("sm_mhz") or 2070.0
     peak = fp32_peak(f_sm)
     achieved = flop / (k_ms * 1e-3) / 1e12 if k_ms else None
-    roof = {"kernel": "sym_hprime_kernel ((H' t_n)(s') / psi(s) of one state at 4 N B "
-                      "transformed configurations, FP32 FMA over cosh/sinh bond tables)",
+    roof = {"kernel": "xsum_kernel (the exchange sums of (H' t_n)(s') / psi(s) of one state at "
+                      "4 N B transformed configurations, FP32 FMA over a bond table)",
             "bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": (achieved / peak) if achieved else None, "traffic": None,
             "work_per_launch": flop,
@@ -1129,18 +1129,19 @@ def run_explicit(args):
     ref.sync_status()
     s_err_x3 = float(torch.linalg.norm(S32 - S64) / nrm)
     del S64, S32, ref, x3
-    P, B = wl.P, wl.walkers
-    flops = 8.0 * P * (P + 1) / 2 * B          # Hermitian half of O^dag O, complex MACs x 8
+    B = wl.walkers
+    # sums of (spin pair) x (tanh pair) over the walkers, real MACs x 2
+    flops = 2.0 * (1 + wl.N * (wl.N + 1) / 2) * (wl.M + 1) ** 2 * B
     peaks, peak_src = measured_peaks()
     peak = float(peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]))
     achieved = flops / (gram_ms * 1e-3) / 1e12
-    roof = {"kernel": "sgram_tc_kernel<3> (tcgen05, three-term bf16 splits: six bf16 "
-                      "products per float32 product, float32 accumulation in TMEM)",
+    roof = {"kernel": "spair_tc_kernel (tcgen05: sums of spin pairs, exact in bf16, times tanh "
+                      "pairs in three bf16 terms, float32 accumulation in TMEM)",
             "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": None, "work_per_launch": flops,
             "avg_launch_ms": gram_ms,
-            "peak_source": f"MEASURED_PEAKS.json bf16_tflops_sustained ({peak_src}); six bf16 "
-                           f"products per product, so frac <= 1/6"}
+            "peak_source": f"MEASURED_PEAKS.json bf16_tflops_sustained ({peak_src}); three bf16 "
+                           f"products per product, so frac <= 1/3"}
     sweeps_per_moment = cfg.n_therm + cfg.n_iter * cfg.sweeps_per_iter + cfg.sweeps_per_iter
     e2e_ms, Bi, Bo = e2e(seq, ctx, K, stream)
     e2e_ms = max_over_ranks(ws, e2e_ms)
@@ -1148,7 +1149,7 @@ def run_explicit(args):
         "metric": "Chebyshev moments/hour", "value": ws * 3600.0 * 1000.0 / ms,
         "unit": "moments/hour", "n_gpus": ws, "steps": K, "warmup": W, "ms_per_step": ms,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "mixed: S on tensor cores from three-term bf16 splits (six products, f32 "
+        "dtype": "mixed: S on tensor cores from spin pairs (exact) and three-term bf16 splits (f32 "
                  "accumulation), f32 Cholesky factor, f64 refinement, f32 elsewhere",
         "data": "synthetic (random complex RBM, sigma=0.01; seeded S^z=0 walkers)",
         "config": {"workload": "square10: periodic 10x10 Heisenberg lattice, RBM alpha=1 (M=100, "
@@ -1166,7 +1167,7 @@ def run_explicit(args):
         "s_error_sample": f"{Bs} walkers of the fit set, RBM of the last fitted moment",
         "iteration_ms": iter_ms, "sbuild_ms": gram_ms,
         "factor_ms": chol_ms, "trsv_ms": trsv_ms,
-        "factor_note": "factor_ms: blocked factor (potrf, trsm, syrk kernels) of one iteration; "
+        "factor_note": "factor_ms: blocked factor (potrf_inv, trsm, syrk_tc kernels) of one iteration; "
                        "trsv_ms: the triangular solves of all its refinement steps",
         "refine_steps_mean": float(st[..., 5].mean()),
         "refine_residual_max": float(st[..., 6].max()),

@@ -417,7 +417,9 @@ cr_status sym_btilde(cr_ctx* ctx, const cr_state* states, int Nm, const int8_t* 
    then gives G^(k) and H^(k) for cheb_krylov.  workspace: caller-owned
    device memory of sym_h_workspace_bytes(ctx, B) bytes (sym_workspace_bytes
    plus theta at the 4 N B transformed configurations, 4 N B M complex
-   values, and two more complex arrays); the call allocates nothing.
+   values, two more complex arrays and, in CR_FP32 and CR_MIXED contexts, the
+   sums over exchanged amplitudes of each configuration); the call allocates
+   nothing.
    Errors as sym_btilde; a == 0 or a NULL hprime / HBt_out is CR_EINVAL. */
 size_t sym_h_workspace_bytes(const cr_ctx* ctx, int B);
 cr_status sym_hbtilde(cr_ctx* ctx, const cr_state* states, int Nm, const int8_t* spins,

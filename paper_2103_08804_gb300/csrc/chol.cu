@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(256) trsm_kernel(cf* __restrict__ L, int P, in
 // which L2 serves.  A panel at a time (10 x 10 lattice, alpha = 1: P = 10200)
 // the kernel moved A at 3.9 TB/s, waiting for the loads of 8 drain warps: 159
 // launches, 11.4 ms.  In pairs, with 16 drain warps that have a whole tile of
-// A in flight while its MMAs run: SYRK_NOW.
+// A in flight while its MMAs run: 7.5 ms.
 //
 // Persistent: warp 0 (one thread) issues the MMAs, panel by panel into TMEM
 // columns [256 h, +256), warps 1-16 drain (warp w: lanes 32 (w % 4), rows 64
