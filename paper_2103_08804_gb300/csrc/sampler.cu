@@ -189,10 +189,13 @@ __global__ void __launch_bounds__(128) sweep_kernel(
                 if ((nacc & 31) == 0) lst[nacc - 32 + lane] = (uint16_t)ent;
             }
             if (nxt < 64 && !((((nxt & 1) ? A1 : A0) >> (nxt >> 1)) & 1u)) {
-                // the prefetched proposal turned parallel: take the one after it
+                // the prefetched proposal turned parallel: take the one after it.  Its
+                // copy lands first, also where none follows in this block: copies have no
+                // order among themselves, and the next block's first rows go to the
+                // same buffer
                 nxt = next_after(A0, A1, nxt);
+                cp_wait<0>();
                 if (nxt < 64) {
-                    cp_wait<0>();
                     fetch(__shfl_sync(0xffffffffu, (nxt & 1) ? b1 : b0, nxt >> 1), q ^ 1);
                     cp_commit();
                 }
