@@ -707,7 +707,11 @@ __global__ void __launch_bounds__(1024) refine_check_kernel(int P, double* __res
                                                             const double* __restrict__ part,
                                                             int npart, double tol,
                                                             double* __restrict__ scal) {
-    if (scal[2] != 0.0) return;
+    // every thread has read the flag before thread 0 sets it below: a warp that
+    // saw it set would leave its part of the last correction out
+    const bool done = scal[2] != 0.0;
+    __syncthreads();
+    if (done) return;
     cpx<double>* x = (cpx<double>*)x_;
     const cpx<double>* d = (const cpx<double>*)d_;
     for (int k = threadIdx.x; k < P; k += blockDim.x) x[k] = x[k] + d[k];
