@@ -417,6 +417,7 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
     cpx<double>* X = (cpx<double>*)a.cg;
     cpx<double>* Ap = X + 3 * P;
     const double invB = 1.0 / B;
+    const bool vecS = (N & 15) == 0 && ((uintptr_t)a.spins & 15) == 0;  // 16-byte loads of spins
 
     if (t == 0) {
         for (int i = 0; i < NMB; ++i) {
@@ -680,13 +681,15 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                 fetchT(sp, tc0);
                 if (ps == 0) {
                     // sigma . va: the threads of a row take 16-site blocks in turn
-                    // (16-byte loads when N % 16 == 0)
+                    // (16-byte loads when N % 16 == 0 and the spins are aligned)
                     uacc = {0.f, 0.f};
                     if (valid) {
                         const int8_t* sr = a.spins + (size_t)sw * N;
                         if ((N & 15) == 0) {
                             for (int b16 = sp; b16 < N / 16; b16 += nsp) {
-                                const int4 raw = __ldg(reinterpret_cast<const int4*>(sr) + b16);
+                                int4 raw;
+                                if (vecS) raw = __ldg(reinterpret_cast<const int4*>(sr) + b16);
+                                else memcpy(&raw, sr + 16 * b16, 16);
                                 const int8_t* sv = reinterpret_cast<const int8_t*>(&raw);
 #pragma unroll
                                 for (int q = 0; q < 16; ++q)
@@ -764,7 +767,7 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                         const int8_t* sr = a.spins + (size_t)(s0 + (sl < nw ? sl : 0)) * N;
                         if (sl >= nw) {
                             raw[m] = make_int4(0, 0, 0, 0);
-                        } else if ((N & 15) == 0) {
+                        } else if (vecS) {
                             raw[m] = __ldg(reinterpret_cast<const int4*>(sr) + b16);
                         } else {
                             int8_t sv[16];

@@ -134,7 +134,8 @@ __global__ void __launch_bounds__(32 * TH_WARPS, 2) theta_kernel(const cpx<R>* _
     cpx<R> part[TH_W];
 #pragma unroll
     for (int w = 0; w < TH_W; ++w) part[w] = {R(0), R(0)};
-    const bool quad = (N & 3) == 0;  // 4 signs of a walker are one aligned word
+    // 4 signs of a walker are one aligned word (spins may start at any byte)
+    const bool quad = (N & 3) == 0 && ((uintptr_t)spins & 3) == 0;
     for (int jb = 0; jb < M; jb += JB) {
         cpx<R> acc[TH_W][JW];
 #pragma unroll

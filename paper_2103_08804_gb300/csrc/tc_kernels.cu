@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(OV_THREADS, 1) ov_tc_kernel(
     const uint32_t idesc = tc::make_idesc_bf16(128, NCp);
     const int ntiles = (B + 127) / 128;
     const int nchunk = (M + TJC - 1) / TJC;
-    const bool vec16 = (N % 16) == 0;
+    const bool vec16 = (N % 16) == 0 && ((uintptr_t)spins & 7) == 0;  // spins may start at any byte
     const int lb = warp & 3, half = warp >> 2;   // TMEM lane block, column half
     const int row = 32 * lb + lane;
     bool ok = true;
