@@ -47,7 +47,8 @@ CR_HD int lrows(int P) { return lcols(P) + 256; }  // a 256-row tile may start a
 
 // L <- S in float32 (only the lower triangle is used).
 __global__ void chol_copy_kernel(const double* __restrict__ S_, int P, cf* __restrict__ L) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y, ld = lcols(P);
+    // (rows on the grid's x axis: there may be more than its y axis holds)
+    const int k = blockIdx.y * blockDim.x + threadIdx.x, i = blockIdx.x, ld = lcols(P);
     if (k >= ld) return;
     L[(size_t)i * ld + k] = i < P && k < P ? ccast<float>(((const cpx<double>*)S_)[(size_t)i * P + k])
                                            : cf{0.f, 0.f};
@@ -742,7 +743,7 @@ cr_status factor32(cr_ctx* c) {
     const bool tcu = c->prec == CR_MIXED;
     const size_t m_off = n_plane_bytes(P);
     CR_LAUNCH(c, CR_K_OTHER,
-              chol_copy_kernel<<<dim3((lcols(P) + 255) / 256, lrows(P)), 256, 0, c->stream>>>(c->S, P, L));
+              chol_copy_kernel<<<dim3(lrows(P), (lcols(P) + 255) / 256), 256, 0, c->stream>>>(c->S, P, L));
     for (int J = 0; J < nb; ++J) {
         CR_LAUNCH(c, CR_KERNEL_CHOL, potrf_inv_kernel<<<1, 256, 0, c->stream>>>(L, P, J, X, c->d_status));
         const int rows = P - (J + 1) * NB;
