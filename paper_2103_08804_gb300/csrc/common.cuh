@@ -54,6 +54,10 @@ CR_D cpx<double> ldg(const cpx<double>* p) {
 // Math wrappers (CUDA's own functions for each precision).
 CR_D float m_exp(float x) { return expf(x); }
 CR_D double m_exp(double x) { return exp(x); }
+CR_D float m_log(float x) { return logf(x); }
+CR_D double m_log(double x) { return log(x); }
+CR_D float m_expm1(float x) { return expm1f(x); }
+CR_D double m_expm1(double x) { return expm1(x); }
 CR_D float m_log1p(float x) { return log1pf(x); }
 CR_D double m_log1p(double x) { return log1p(x); }
 CR_D float m_atan2(float y, float x) { return atan2f(y, x); }
@@ -75,6 +79,27 @@ template <typename R> CR_D cpx<R> cexp_(cpx<R> z) {
     return {e * c, e * s};
 }
 
+// With e = exp(-2|x|) and w = exp(-2 sign(x) z), z = x + iy,
+//   |1 + w|^2 = 1 + e^2 + 2 e cos 2y = (1 - e)^2 + 4 e cos^2 y,
+// the denominator of tanh z and, under a logarithm, |2 cosh z|^2 e^{-2|x|}.  The
+// first sum cancels next to a zero of cosh z: within 3e-4 of one, float32 can
+// leave nothing or less than nothing, and an infinite or NaN tanh stops its
+// walker and every sum it enters.  The second sum does not cancel (1 - e from
+// expm1, cos y itself); it is taken where the first has lost six bits, so that
+// values away from a zero keep the bits they had, and as a call, so that the
+// rare branch costs the kernels no registers.
+template <typename R> struct NearNode {
+    R d, om, s, c;  // |1 + w|^2, 1 - e, sin y, cos y
+};
+template <typename R> __device__ __noinline__ NearNode<R> near_node_terms(R ax, R y, R e) {
+    NearNode<R> n;
+    n.om = -m_expm1(R(-2) * ax);
+    m_sincos(y, &n.s, &n.c);
+    n.d = n.om * n.om + R(4) * e * n.c * n.c;
+    return n;
+}
+template <typename R> CR_D bool near_node(R d) { return d < R(0.015625); }
+
 // tanh(x + iy) = (sign(x)(1 - e^2) + 2 i e sin 2y) / (1 + e^2 + 2 e cos 2y),
 // e = exp(-2|x|): the identity tanh z = sinh 2z-ish form rescaled by e so
 // that nothing overflows for large |x|.
@@ -83,9 +108,19 @@ template <typename R> CR_D cpx<R> ctanh_(cpx<R> z) {
     R e = m_exp(R(-2) * ax);
     R e2 = e * e, s, c;
     m_sincos(R(2) * z.y, &s, &c);
-    R inv = R(1) / (R(1) + e2 + R(2) * e * c);
-    R re = (R(1) - e2) * inv;
-    return {z.x < R(0) ? -re : re, R(2) * e * s * inv};
+    const R d = R(1) + e2 + R(2) * e * c;
+    R re, im;
+    if (near_node(d)) {
+        const NearNode<R> n = near_node_terms(ax, z.y, e);
+        const R inv = R(1) / n.d;
+        re = n.om * (R(1) + e) * inv;
+        im = R(4) * e * n.s * n.c * inv;
+    } else {
+        const R inv = R(1) / d;
+        re = (R(1) - e2) * inv;
+        im = R(2) * e * s * inv;
+    }
+    return {z.x < R(0) ? -re : re, im};
 }
 
 // log(2 cosh z) = s z + log(1 + w), s = sign(Re z), w = exp(-2 s z), |w| <= 1.
@@ -94,7 +129,13 @@ template <typename R> CR_D cpx<R> clncosh2_(cpx<R> z) {
     R e = m_exp(R(-2) * sg * z.x), s, c;
     m_sincos(R(-2) * sg * z.y, &s, &c);
     R wr = e * c, wi = e * s;
-    return {sg * z.x + R(0.5) * m_log1p(R(2) * wr + e * e), sg * z.y + m_atan2(wi, R(1) + wr)};
+    const R q = R(2) * wr + e * e;  // |1 + w|^2 - 1
+    if (near_node(R(1) + q)) {
+        const NearNode<R> n = near_node_terms(sg * z.x, z.y, e);
+        return {sg * z.x + R(0.5) * m_log(n.d),
+                sg * z.y + m_atan2(R(-2) * sg * e * n.s * n.c, n.om + R(2) * e * n.c * n.c)};
+    }
+    return {sg * z.x + R(0.5) * m_log1p(q), sg * z.y + m_atan2(wi, R(1) + wr)};
 }
 
 // cosh and sinh of a complex number.

@@ -108,9 +108,11 @@ template <typename R> CR_D void lncosh_parts(cpx<R> z, cpx<R>* lin, cpx<R>* onew
     m_sincos(R(-2) * sg * z.y, &s, &c);
     *lin = *lin + sg * z;
     *onew = {R(1) + e * c, e * s};
+    if (near_node(abs2(*onew))) {
+        const NearNode<R> n = near_node_terms(sg * z.x, z.y, e);
+        *onew = {n.om + R(2) * e * n.c * n.c, R(-2) * sg * e * n.s * n.c};
+    }
 }
-CR_D float m_log(float x) { return logf(x); }
-CR_D double m_log(double x) { return log(x); }
 
 }  // namespace
 
