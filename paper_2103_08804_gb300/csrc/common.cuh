@@ -86,12 +86,11 @@ template <typename R> CR_D cpx<R> cexp_(cpx<R> z) {
 // leave nothing or less than nothing, and an infinite or NaN tanh stops its
 // walker and every sum it enters.  The second sum does not cancel (1 - e from
 // expm1, cos y itself); it is taken where the first has lost six bits, so that
-// values away from a zero keep the bits they had, and as a call, so that the
-// rare branch costs the kernels no registers.
+// values away from a zero keep the bits they had.
 template <typename R> struct NearNode {
     R d, om, s, c;  // |1 + w|^2, 1 - e, sin y, cos y
 };
-template <typename R> __device__ __noinline__ NearNode<R> near_node_terms(R ax, R y, R e) {
+template <typename R> CR_D NearNode<R> near_node_terms(R ax, R y, R e) {
     NearNode<R> n;
     n.om = -m_expm1(R(-2) * ax);
     m_sincos(y, &n.s, &n.c);
@@ -102,40 +101,45 @@ template <typename R> CR_D bool near_node(R d) { return d < R(0.015625); }
 
 // tanh(x + iy) = (sign(x)(1 - e^2) + 2 i e sin 2y) / (1 + e^2 + 2 e cos 2y),
 // e = exp(-2|x|): the identity tanh z = sinh 2z-ish form rescaled by e so
-// that nothing overflows for large |x|.
-template <typename R> CR_D cpx<R> ctanh_(cpx<R> z) {
+// that nothing overflows for large |x|.  *d: the denominator.
+template <typename R> CR_D cpx<R> ctanh_far(cpx<R> z, R* d) {
     R ax = z.x < R(0) ? -z.x : z.x;
     R e = m_exp(R(-2) * ax);
     R e2 = e * e, s, c;
     m_sincos(R(2) * z.y, &s, &c);
-    const R d = R(1) + e2 + R(2) * e * c;
-    R re, im;
-    if (near_node(d)) {
-        const NearNode<R> n = near_node_terms(ax, z.y, e);
-        const R inv = R(1) / n.d;
-        re = n.om * (R(1) + e) * inv;
-        im = R(4) * e * n.s * n.c * inv;
-    } else {
-        const R inv = R(1) / d;
-        re = (R(1) - e2) * inv;
-        im = R(2) * e * s * inv;
-    }
-    return {z.x < R(0) ? -re : re, im};
+    *d = R(1) + e2 + R(2) * e * c;
+    R inv = R(1) / *d;
+    R re = (R(1) - e2) * inv;
+    return {z.x < R(0) ? -re : re, R(2) * e * s * inv};
+}
+template <typename R> CR_D cpx<R> ctanh_near(cpx<R> z) {
+    const R ax = z.x < R(0) ? -z.x : z.x, e = m_exp(R(-2) * ax);
+    const NearNode<R> n = near_node_terms(ax, z.y, e);
+    const R inv = R(1) / n.d, re = n.om * (R(1) + e) * inv;
+    return {z.x < R(0) ? -re : re, R(4) * e * n.s * n.c * inv};
+}
+template <typename R> CR_D cpx<R> ctanh_(cpx<R> z) {
+    R d;
+    const cpx<R> t = ctanh_far(z, &d);
+    return near_node(d) ? ctanh_near(z) : t;
 }
 
 // log(2 cosh z) = s z + log(1 + w), s = sign(Re z), w = exp(-2 s z), |w| <= 1.
-template <typename R> CR_D cpx<R> clncosh2_(cpx<R> z) {
+// *d: |1 + w|^2.
+template <typename R> CR_D cpx<R> clncosh2_far(cpx<R> z, R* d) {
     R sg = z.x < R(0) ? R(-1) : R(1);
     R e = m_exp(R(-2) * sg * z.x), s, c;
     m_sincos(R(-2) * sg * z.y, &s, &c);
     R wr = e * c, wi = e * s;
-    const R q = R(2) * wr + e * e;  // |1 + w|^2 - 1
-    if (near_node(R(1) + q)) {
-        const NearNode<R> n = near_node_terms(sg * z.x, z.y, e);
-        return {sg * z.x + R(0.5) * m_log(n.d),
-                sg * z.y + m_atan2(R(-2) * sg * e * n.s * n.c, n.om + R(2) * e * n.c * n.c)};
-    }
+    const R q = R(2) * wr + e * e;
+    *d = R(1) + q;
     return {sg * z.x + R(0.5) * m_log1p(q), sg * z.y + m_atan2(wi, R(1) + wr)};
+}
+template <typename R> CR_D cpx<R> clncosh2_near(cpx<R> z) {
+    const R sg = z.x < R(0) ? R(-1) : R(1), e = m_exp(R(-2) * sg * z.x);
+    const NearNode<R> n = near_node_terms(sg * z.x, z.y, e);
+    return {sg * z.x + R(0.5) * m_log(n.d),
+            sg * z.y + m_atan2(R(-2) * sg * e * n.s * n.c, n.om + R(2) * e * n.c * n.c)};
 }
 
 // cosh and sinh of a complex number.
@@ -345,8 +349,8 @@ cr_status xsum_prepare(cr_ctx* c);
 cr_status launch_xsum(cr_ctx* c, const void* params, const int8_t* spins, const void* theta, int n,
                       int probe, double qx, double qy, xsum_out* out);
 
-// Tables for a state (rbm.cu).
-cr_status build_tables(cr_ctx* c, const void* params, int slot);
+// Tables for a state (rbm.cu); planar: CS as [b][cosh row, sinh row].
+cr_status build_tables(cr_ctx* c, const void* params, int slot, int planar = 0);
 // theta / log psi of an RBM at a walker batch (rbm.cu).
 cr_status launch_logpsi(cr_ctx* c, const void* params, const int8_t* spins, int B, void* theta,
                         void* logpsi);

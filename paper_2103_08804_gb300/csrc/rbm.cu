@@ -10,12 +10,12 @@
 // and the visible factor by exp(-s 2 (a_i - a_i')).  The tables hold D, cosh D,
 // sinh D per (bond, hidden unit), padded to Mp columns with the neutral
 // values (0, 1, 0), and exp(-/+ 2 (a_i - a_i')) per bond: cosh and sinh
-// interleaved for the sampler (slot 0), transposed for the float64 local
-// target (slot 1).
+// interleaved, or in a row each (planar), for the sampler (slot 0), transposed
+// for the float64 local target (slot 1).
 template <typename R>
 __global__ void tables_kernel(const cpx<R>* __restrict__ prm, const int2* __restrict__ bonds, int N,
                               int M, int Mp, int Nb, cpx<R>* D, cpx<R>* CS, cpx<R>* ChT, cpx<R>* ShT,
-                              cpx<R>* ea) {
+                              cpx<R>* ea, int planar) {
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= Nb * Mp) return;
     int b = idx / Mp, m = idx % Mp;
@@ -29,8 +29,9 @@ __global__ void tables_kernel(const cpx<R>* __restrict__ prm, const int2* __rest
     }
     if (CS) {
         D[idx] = d;
-        CS[2 * (size_t)idx] = ch;
-        CS[2 * (size_t)idx + 1] = sh;
+        const size_t at = planar ? (size_t)2 * Mp * b + m : 2 * (size_t)idx;
+        CS[at] = ch;
+        CS[at + (planar ? Mp : 1)] = sh;
     } else {
         ChT[(size_t)m * Nb + b] = ch;
         ShT[(size_t)m * Nb + b] = sh;
@@ -43,18 +44,18 @@ __global__ void tables_kernel(const cpx<R>* __restrict__ prm, const int2* __rest
 }
 
 template <typename R>
-static cr_status build_tables_t(cr_ctx* c, const void* params, int slot) {
+static cr_status build_tables_t(cr_ctx* c, const void* params, int slot, int planar) {
     const cr_tables& t = c->tab[slot];
     int n = c->Nb * c->Mp;
     CR_LAUNCH(c, CR_K_OTHER, tables_kernel<R><<<(n + 255) / 256, 256, 0, c->stream>>>(
         (const cpx<R>*)params, c->d_bonds, c->N, c->M, c->Mp, c->Nb, (cpx<R>*)t.D, (cpx<R>*)t.CS,
-        (cpx<R>*)t.ChT, (cpx<R>*)t.ShT, (cpx<R>*)t.ea));
+        (cpx<R>*)t.ChT, (cpx<R>*)t.ShT, (cpx<R>*)t.ea, planar));
     return cr_check_launch(c, "tables_kernel");
 }
 
-cr_status build_tables(cr_ctx* c, const void* params, int slot) {
-    return c->prec == CR_FP64 ? build_tables_t<double>(c, params, slot)
-                              : build_tables_t<float>(c, params, slot);
+cr_status build_tables(cr_ctx* c, const void* params, int slot, int planar) {
+    return c->prec == CR_FP64 ? build_tables_t<double>(c, params, slot, planar)
+                              : build_tables_t<float>(c, params, slot, planar);
 }
 
 // ------------------------------------------------------ theta and log psi
@@ -98,6 +99,11 @@ template <int LJ, int JW> CR_D int unit_of(int l, int q) {
     return q < (JW & ~1) ? 2 * l + (q & 1) + 2 * LJ * (q >> 1) : LJ * (JW - 1) + l;
 }
 
+// near_node_terms as a call: inlined, its rare branch makes theta_kernel spill.
+template <typename R> __device__ __noinline__ NearNode<R> near_node_call(R ax, R y, R e) {
+    return near_node_terms(ax, y, e);
+}
+
 // log(2 cosh z) summed over the lane's units: s z and 1 + w of each (|w| <= 1,
 // so two arguments add up without a branch cut), the logarithm of two units'
 // product at once.
@@ -109,7 +115,7 @@ template <typename R> CR_D void lncosh_parts(cpx<R> z, cpx<R>* lin, cpx<R>* onew
     *lin = *lin + sg * z;
     *onew = {R(1) + e * c, e * s};
     if (near_node(abs2(*onew))) {
-        const NearNode<R> n = near_node_terms(sg * z.x, z.y, e);
+        const NearNode<R> n = near_node_call(sg * z.x, z.y, e);
         *onew = {n.om + R(2) * e * n.c * n.c, R(-2) * sg * e * n.s * n.c};
     }
 }

@@ -11,6 +11,9 @@
 // after an accepted move only the bonds that share one site with it change
 // sides.
 //
+// sweep_l1_kernel takes smaller tables, which stay in L1 (sweep_in_l1 has the
+// rule and both sides' times); what follows is the form for large ones.
+//
 // What bounds it: a proposal is a chain of a table read (4 KB from L2 at 256
 // hidden units), the product across the warp, the accept test and, mostly,
 // the update.  The rows of the next proposal that can be evaluated are
@@ -67,6 +70,71 @@ template <bool YY> CR_D cpx<float> cdiv_rn(cpx<float> a, cpx<float> b) {
 }
 template <bool YY> CR_D cpx<double> cdiv_rn(cpx<double> a, cpx<double> b) { return cdiv(a, b); }
 
+// the same product in every lane (one value for the whole warp)
+template <typename R> CR_D cpx<R> warp_prod_rn(cpx<R> v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        v = cmul_rn<true>(v, cpx<R>{__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)});
+    return {__shfl_sync(0xffffffffu, v.x, 0), __shfl_sync(0xffffffffu, v.y, 0)};
+}
+
+// tanh of a lane's units 32 k + lane < M (0 past M).  The values next to a node,
+// which are rare, are formed again behind one branch: a branch per unit would
+// keep the units' chains of exponentials and sines from running side by side.
+template <typename R, int KPL>
+CR_D void tanh_units(const cpx<R> (&th)[KPL], int M, int lane, cpx<R> (&T)[KPL]) {
+    R d[KPL];
+    bool near = false;
+#pragma unroll
+    for (int k = 0; k < KPL; ++k) {
+        T[k] = {R(0), R(0)};
+        d[k] = R(1);
+        if (32 * k + lane < M) T[k] = ctanh_far(th[k], &d[k]);
+        near = near || near_node(d[k]);
+    }
+    if (near)
+#pragma unroll
+        for (int k = 0; k < KPL; ++k)
+            if (near_node(d[k])) T[k] = ctanh_near(th[k]);
+}
+
+// theta (theta_out may be null: in place already), tanh theta and log psi of
+// walker w, whose units 32 k + lane are th[k].
+template <typename R, int KPL>
+CR_D void walker_outputs(const cpx<R> (&th)[KPL], int lane, int w, int M, int N, const cpx<R>* prm,
+                         const int8_t* sg, cpx<R>* theta_out, cpx<R>* logpsi_out, cpx<R>* tanh_out) {
+    cpx<R> lp = {R(0), R(0)}, v[KPL];
+    R d[KPL];
+    bool near = false;
+#pragma unroll
+    for (int k = 0; k < KPL; ++k) {
+        v[k] = {R(0), R(0)};
+        d[k] = R(1);
+        if (32 * k + lane < M) {
+            if (theta_out) theta_out[(size_t)w * M + 32 * k + lane] = th[k];
+            v[k] = clncosh2_far(th[k], &d[k]);
+        }
+        near = near || near_node(d[k]);
+    }
+    if (near)
+#pragma unroll
+        for (int k = 0; k < KPL; ++k)
+            if (near_node(d[k])) v[k] = clncosh2_near(th[k]);
+#pragma unroll
+    for (int k = 0; k < KPL; ++k)
+        if (32 * k + lane < M) lp = lp + v[k];
+    if (tanh_out) {
+        tanh_units(th, M, lane, v);
+#pragma unroll
+        for (int k = 0; k < KPL; ++k)
+            if (32 * k + lane < M) tanh_out[(size_t)w * M + 32 * k + lane] = v[k];
+    }
+    if (!logpsi_out) return;
+    for (int i = lane; i < N; i += 32) lp = lp + R(sg[i]) * prm[i];
+    lp = warp_sum(lp);
+    if (lane == 0) logpsi_out[w] = lp;
+}
+
 constexpr int LIST_NEG = 0x8000;  // list entry: bond, this bit for s = -1
 
 }  // namespace
@@ -99,8 +167,13 @@ __global__ void __launch_bounds__(128) sweep_kernel(
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
         const int j = 32 * k + lane;
-        const cpx<R> v = j < M ? (p_base ? Tws : theta)[(size_t)w * M + j] : cpx<R>{R(0), R(0)};
-        T[k] = p_base ? v : ctanh_(v);
+        T[k] = j < M ? (p_base ? Tws : theta)[(size_t)w * M + j] : cpx<R>{R(0), R(0)};
+    }
+    if (!p_base) {
+        cpx<R> t[KPL];
+        tanh_units(T, M, lane, t);
+#pragma unroll
+        for (int k = 0; k < KPL; ++k) T[k] = t[k];
     }
     // copy the rows of bond b into buffer q: every lane the pairs it will read
     auto fetch = [&](int b, int q) {
@@ -160,13 +233,7 @@ __global__ void __launch_bounds__(128) sweep_kernel(
                 f[k] = {ch.x - s * ts.x, ch.y - s * ts.y};
                 pl = cmul_rn<false>(pl, f[k]);
             }
-            cpx<R> pw = pl;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                pw = cmul_rn<true>(pw, cpx<R>{__shfl_xor_sync(0xffffffffu, pw.x, o),
-                                              __shfl_xor_sync(0xffffffffu, pw.y, o)});
-            pw.x = __shfl_sync(0xffffffffu, pw.x, 0);  // one value for the whole warp
-            pw.y = __shfl_sync(0xffffffffu, pw.y, 0);
+            const cpx<R> pw = warp_prod_rn(pl);
             const R ratio2 = abs2_rn<false>(e) * abs2_rn<false>(pw);
             const R u = (R(ua >> 9) + R(0.5)) * R(1.1920928955078125e-07);
             if (u < ratio2) {
@@ -213,6 +280,92 @@ __global__ void __launch_bounds__(128) sweep_kernel(
         for (int k = 0; k < KPL; ++k)
             if (32 * k + lane < M) Tws[(size_t)w * M + 32 * k + lane] = T[k];
     if (lane == 0) count[w] = nacc;
+}
+
+// The same sweep where the tables stay in L1: the rows are read as they are
+// needed (cosh and sinh in rows of their own) and theta is carried along, so
+// that neither a list nor a second pass over it is needed.  The same operations
+// in the same order on every value.
+template <typename R, int KPL>
+__global__ void __launch_bounds__(128) sweep_l1_kernel(
+    const cpx<R>* __restrict__ prm, int8_t* __restrict__ spins, cpx<R>* __restrict__ theta, int B, int N,
+    int M, int Nb, const int2* __restrict__ bonds_g, const cpx<R>* __restrict__ Dt,
+    const cpx<R>* __restrict__ CS, const cpx<R>* __restrict__ ea, int n_prop, uint32_t k0, uint32_t k1,
+    unsigned long long counter, const unsigned long long* __restrict__ dcounter,
+    cpx<R>* __restrict__ logpsi_out, cpx<R>* __restrict__ tanh_out, int32_t* __restrict__ n_acc) {
+    if (dcounter) counter = *dcounter;  // stream position kept on the device
+    constexpr int Mp = 32 * KPL;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int2* bonds = (int2*)smem_raw;                       // [Nb]
+    int8_t* sg_all = (int8_t*)(bonds + Nb);              // [4][N]
+    for (int e = threadIdx.x; e < Nb; e += blockDim.x) bonds[e] = bonds_g[e];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int w = blockIdx.x * 4 + wid;
+    int8_t* sg = sg_all + wid * N;
+    if (w < B)
+        for (int i = lane; i < N; i += 32) sg[i] = spins[(size_t)w * N + i];
+    __syncthreads();
+    if (w >= B) return;
+
+    cpx<R> th[KPL], T[KPL];
+#pragma unroll
+    for (int k = 0; k < KPL; ++k) {
+        const int j = 32 * k + lane;
+        th[k] = j < M ? theta[(size_t)w * M + j] : cpx<R>{R(0), R(0)};
+    }
+    tanh_units(th, M, lane, T);
+    int nacc = 0;
+    uint4 rnd = make_uint4(0, 0, 0, 0);
+    for (int p = 0; p < n_prop; ++p) {
+        if ((p & 63) == 0) {
+            const unsigned long long step = counter + (unsigned long long)(p >> 1) + lane;
+            rnd = philox4x32_10(make_uint4((uint32_t)w, (uint32_t)step, (uint32_t)(step >> 32), 0u), k0, k1);
+        }
+        const int src = (p >> 1) & 31;
+        const uint32_t ub = __shfl_sync(0xffffffffu, (p & 1) ? rnd.z : rnd.x, src);
+        const uint32_t ua = __shfl_sync(0xffffffffu, (p & 1) ? rnd.w : rnd.y, src);
+        const int b = (int)__umulhi(ub, (uint32_t)Nb);
+        const int2 bd = bonds[b];
+        const int si = sg[bd.x];
+        if (si == sg[bd.y]) continue;  // parallel: no-op, counts as rejected
+        const R s = R(si);
+        const cpx<R>* row = CS + 2 * (size_t)b * Mp + lane;
+        cpx<R> ch[KPL], sh[KPL], f[KPL];
+        cpx<R> pl = {R(1), R(0)};
+#pragma unroll
+        for (int k = 0; k < KPL; ++k) {
+            ch[k] = ldg(row + 32 * k);
+            sh[k] = ldg(row + Mp + 32 * k);
+            const cpx<R> ts = cmul_rn<false>(T[k], sh[k]);
+            f[k] = {ch[k].x - s * ts.x, ch[k].y - s * ts.y};
+            pl = cmul_rn<false>(pl, f[k]);
+        }
+        const cpx<R> pw = warp_prod_rn(pl);
+        const cpx<R> e = ea[2 * b + (si > 0 ? 0 : 1)];
+        const R ratio2 = abs2_rn<false>(e) * abs2_rn<false>(pw);
+        const R u = (R(ua >> 9) + R(0.5)) * R(1.1920928955078125e-07);
+        if (u < ratio2) {
+            const cpx<R>* dr = Dt + (size_t)b * Mp + lane;
+#pragma unroll
+            for (int k = 0; k < KPL; ++k) {
+                const cpx<R> d = ldg(dr + 32 * k);
+                th[k] = {th[k].x - s * d.x, th[k].y - s * d.y};
+                const cpx<R> tc = cmul_rn<(KPL > 1)>(T[k], ch[k]);
+                T[k] = cdiv_rn<KPL == 1>(cpx<R>{tc.x - s * sh[k].x, tc.y - s * sh[k].y}, f[k]);
+            }
+            __syncwarp();
+            if (lane == 0) {
+                sg[bd.x] = (int8_t)(-si);
+                sg[bd.y] = (int8_t)si;
+            }
+            __syncwarp();
+            ++nacc;
+        }
+    }
+    __syncwarp();
+    for (int i = lane; i < N; i += 32) spins[(size_t)w * N + i] = sg[i];
+    if (lane == 0 && n_acc) n_acc[w] = nacc;
+    walker_outputs<R, KPL>(th, lane, w, M, N, prm, sg, theta, logpsi_out, tanh_out);
 }
 
 // theta -> theta - sum of the listed moves' s D, in the list's order, for one
@@ -345,25 +498,35 @@ __global__ void __launch_bounds__(128) finish_kernel(
     }
     if (lane == 0 && n_acc) n_acc[w] = (first ? 0 : n_acc[w]) + n;
     if (!last) return;
-    cpx<R> lp = {R(0), R(0)};
-#pragma unroll
-    for (int k = 0; k < KPL; ++k) {
-        int j = 32 * k + lane;
-        if (j < M) {
-            lp = lp + clncosh2_(th[k]);
-            if (tanh_out) tanh_out[(size_t)w * M + j] = ctanh_(th[k]);
-        }
-    }
-    if (!logpsi_out) return;
-    const int8_t* sg = spins + (size_t)w * N;
-    for (int i = lane; i < N; i += 32) lp = lp + R(sg[i]) * prm[i];
-    lp = warp_sum(lp);
-    if (lane == 0) logpsi_out[w] = lp;
+    walker_outputs<R, KPL>(th, lane, w, M, N, prm, spins + (size_t)w * N, (cpx<R>*)nullptr, logpsi_out,
+                           tanh_out);
 }
 
 // Advance a device-resident stream position (after the sweep that used it).
 __global__ void advance_counter_kernel(unsigned long long* ctr, unsigned long long calls) {
     *ctr += calls;
+}
+
+// Whether a sweep reads its tables through L1 (sweep_l1_kernel) or prefetches
+// rows and replays lists (sweep_kernel).  The first has no second pass and no
+// list, but every evaluated proposal waits for its rows; warps hide that where
+// there are many of them with few units each, or where the tables (cosh, sinh
+// and D, 24 or 48 bytes a bond and unit) stay in L1.  Times of four sweeps, us,
+// lists / L1: 8 x 8 lattice with 33 units (192 KB), 16384 walkers 662 / 492, 200
+// walkers 110 / 100; 64 sites with 128 units (192 KB), 926 / 711 and 136 / 121;
+// 10 x 10 with 60 units (300 KB), 1002 / 808 and 157 / 168; 8 x 8 with 128
+// units (384 KB), 915 / 845 and 133 / 158; 10 x 10 with 100 units (600 KB), 4096
+// walkers 458 / 545; 96 sites with 192 units, 8 units a lane (576 KB), 2145 /
+// 2706.  With 8 units a lane the few warps an SM holds hide little, and L1 pays
+// from some 48 proposals on small tables only.  Float64: the pipe is the bound,
+// L1 is 1 to 10% ahead up to 4 units a lane and 5 to 15% behind above.
+static bool sweep_in_l1(const cr_ctx* c, int B, int n_prop) {
+    const int kpl = c->Mp / 32;
+    if (c->prec == CR_FP64) return kpl <= 4;
+    const size_t tab = (size_t)c->Nb * c->Mp * 24;
+    if (kpl <= 2) return tab <= 256 * 1024 || B >= 24 * c->n_sm;
+    if (kpl == 4) return tab <= 256 * 1024 || (tab <= 512 * 1024 && B >= 64 * c->n_sm);
+    return kpl == 8 && tab <= 160 * 1024 && n_prop >= 48;
 }
 
 // Proposals per sweep launch: its list of accepted moves per walker.
@@ -409,6 +572,15 @@ static cr_status sweep_k(cr_ctx* c, const void* params, int8_t* spins, void* the
                          void* tanh_out, int32_t* n_acc) {
     const cr_tables& t = c->tab[0];
     cpx<R>* th = (cpx<R>*)theta;
+    if (sweep_in_l1(c, B, n_prop)) {
+        CR_LAUNCH(c, CR_KERNEL_SWEEP,
+                  (sweep_l1_kernel<R, KPL><<<(B + 3) / 4, 128, c->Nb * sizeof(int2) + 4 * c->N, c->stream>>>(
+                      (const cpx<R>*)params, spins, th, B, c->N, c->M, c->Nb, c->d_bonds, (const cpx<R>*)t.D,
+                      (const cpx<R>*)t.CS, (const cpx<R>*)t.ea, n_prop, (uint32_t)seed,
+                      (uint32_t)(seed >> 32), (unsigned long long)counter,
+                      (const unsigned long long*)dcounter, (cpx<R>*)logpsi_out, (cpx<R>*)tanh_out, n_acc)));
+        return cr_check_launch(c, "mc_sweep");
+    }
     const cpx<R>* D = (const cpx<R>*)t.D;
     const int cap = sweep_list_cap(c), grid = (B + 3) / 4;
     // a table that fits in L1 beside the loads in flight is replayed whole, by the finishing warps;
@@ -495,7 +667,7 @@ extern "C" cr_status mc_sweep(cr_ctx* ctx, const cr_state* st, int8_t* spins, vo
     const uint64_t calls = (uint64_t)(n_prop + 1) / 2;
     if (B > 0) {
         CR_CHECK_ARG(spins && theta, "mc_sweep: null spins or theta");
-        cr_status s = build_tables(ctx, st->params, 0);
+        cr_status s = build_tables(ctx, st->params, 0, sweep_in_l1(ctx, B, n_prop));
         if (s != CR_OK) return s;
         s = ctx->prec == CR_FP64
                 ? sweep_t<double>(ctx, st->params, spins, theta, B, n_prop, rng->seed,
