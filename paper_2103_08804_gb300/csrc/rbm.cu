@@ -71,7 +71,7 @@ cr_status build_tables(cr_ctx* c, const void* params, int slot, int planar) {
 // rows by cp.async, signs converted once), double-buffered: per site a lane
 // reads TH_W signs (a broadcast) and JW weights for 2 TH_W JW multiply-adds.
 // JW and LJ are the smallest that hold M, so few lanes multiply padding; TH_W
-// is 8, or 4 and 1 for fewer walkers, so that the blocks reach every SM.
+// is 1 to 8 by the number of walkers (launch_theta_t).
 //
 // Bound by the FMA pipe and, for log psi, by the exponential, sine and cosine
 // of every theta; log(2 cosh) of two units shares one logarithm and one
@@ -279,17 +279,45 @@ static cr_status launch_theta_w(cr_ctx* c, const void* params, const int8_t* spi
     return cr_check_launch(c, "theta_kernel");
 }
 
+// Walkers per group (TH_W) of a launch over B walkers.  A block is one unit of
+// time on its SM, two share one: with nb blocks for the fullest SM the launch
+// takes nb / 2 pairs and perhaps a single, and the TH_W with the least total is
+// taken.  The two tables are a block's time alone and a pair's, us at N = M =
+// 256; they keep their order at other sizes (N = 64 with 33 and 128 units, N =
+// 100 with 100, N = 36 with 72).  B = 3000 at N = M = 256: 97 us with the
+// smallest count that gave every SM a block, now 56; 10000: 133, now 107; the
+// values do not depend on the choice.  Float64 is bound by its pipe: one walker
+// a group is the best or equal up to 8192 walkers (64 sites, 33 units: 224 us,
+// four 254), and the weights it reads again are hidden.
 template <typename R, int MODE>
 static cr_status launch_theta_t(cr_ctx* c, const void* params, const int8_t* spins, int B,
                                 void* theta, void* out, const void* T, const double* skip) {
     if (B == 0) return CR_OK;
-    // blocks of 8 warps: two per SM with 8 walkers a group, half that with 4
+    if constexpr (sizeof(R) == 8) return launch_theta_w<R, 1, MODE>(c, params, spins, B, theta, out, T, skip);
+    static const struct { int tw, single, pair; } shapes[] = {{1, 42, 64},  {2, 43, 66},  {4, 56, 84},
+                                                              {5, 63, 107}, {6, 70, 110}, {8, 90, 144}};
     const int groups = TH_WARPS * (c->M <= 16 ? 2 : 1);
-    if (B >= 2 * c->n_sm * 8 * groups)
-        return launch_theta_w<R, 8, MODE>(c, params, spins, B, theta, out, T, skip);
-    if (B >= c->n_sm * 4 * groups)
-        return launch_theta_w<R, 4, MODE>(c, params, spins, B, theta, out, T, skip);
-    return launch_theta_w<R, 1, MODE>(c, params, spins, B, theta, out, T, skip);
+    int tw = 1;
+    long long best = -1;
+    for (const auto& q : shapes) {
+        const long long blocks = ((long long)B + q.tw * groups - 1) / (q.tw * groups);
+        const long long nb = (blocks + c->n_sm - 1) / c->n_sm;
+        const long long cost = nb / 2 * q.pair + (nb & 1) * q.single;
+        if (best < 0 || cost < best) {
+            best = cost;
+            tw = q.tw;
+        }
+    }
+#define TW(K) return launch_theta_w<R, K, MODE>(c, params, spins, B, theta, out, T, skip)
+    switch (tw) {
+        case 1: TW(1);
+        case 2: TW(2);
+        case 4: TW(4);
+        case 5: TW(5);
+        case 6: TW(6);
+        default: TW(8);
+    }
+#undef TW
 }
 
 cr_status launch_logpsi(cr_ctx* c, const void* params, const int8_t* spins, int B, void* theta,
