@@ -172,9 +172,10 @@ CR_D void tile_step(const cf (*As)[NB + 1], const cf (*Bs)[BP], int tx, int ty, 
 //   cols   M side, row 2k: [Re, Im] of L_kc; row 2k + 1: [-Im, Re]
 // so that D[2k + part][i] = (Re, Im)(L_i . conj(L_k)): lanes (D rows) hold
 // consecutive floats of a row of A, and a tile's 256 rows x 64 columns are
-// read and written coalesced.  A panel is 128 real deep: 48 MMAs into one
-// float32 accumulator, then one float32 subtraction, as long a run as the
-// explicit S takes.
+// read and written coalesced.  A panel is 128 real deep.  An MMA's addition
+// truncates, so its error grows with the number of them: the eight MMAs of
+// the leading products have an accumulator of their own, and the forty others,
+// 2^-8 of it, another; then one float32 addition and subtraction.
 constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded mbarrier polls
 constexpr int TC_ROWS = 256, TC_COLS = 64;  // tile of A
 constexpr int TC_KC = 32, TC_NKC = 2 * NB / TC_KC;  // K tiles of a panel; operands hold two panels
@@ -278,11 +279,17 @@ __global__ void __launch_bounds__(256) trsm_kernel(cf* __restrict__ L, int P, in
 // which L2 serves.  A panel at a time (10 x 10 lattice, alpha = 1: P = 10200)
 // the kernel moved A at 3.9 TB/s, waiting for the loads of 8 drain warps: 159
 // launches, 11.4 ms.  In pairs, with 16 drain warps that have a whole tile of
-// A in flight while its MMAs run: 7.5 ms.
+// A in flight while its MMAs run: 8.0 ms; 10.2 with an accumulator for the leading
+// products, since both fill TMEM and the MMAs of a panel wait for the drain
+// of the last.  That buys the factor's accuracy: the residual left by one
+// correction, over P = 168 ... 10200, went from 2.15 times that of a factor by
+// float32 multiply-adds and substitution to 1.15 (1.12 on the FMA pipes here,
+// the inverses' share), the corrections needed from 3.03 to 2.69 on average.
 //
 // Persistent: warp 0 (one thread) issues the MMAs, panel by panel into TMEM
-// columns [256 h, +256), warps 1-16 drain (warp w: lanes 32 (w % 4), rows 64
-// ((w - 1) / 4)), warp 17 (one thread) copies operand stages.
+// columns [0, 256) (leading products) and [256, 512), warps 1-16 drain (warp w:
+// lanes 32 (w % 4), rows 64 ((w - 1) / 4)), warp 17 (one thread) copies operand
+// stages.
 __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restrict__ Lf, int P, int r0,
                                                                 int npan, int ntiles,
                                                                 const unsigned char* __restrict__ planes,
@@ -290,15 +297,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
     extern __shared__ __align__(1024) unsigned char sm[];
     uint64_t* full = (uint64_t*)(sm + TC_NSTG * TC_STAGE);
     uint64_t* empty = full + TC_NSTG;
-    uint64_t* dfull = empty + TC_NSTG;  // [2] MMAs of a tile done
-    uint64_t* dempty = dfull + 2;       // [2] TMEM half read by the drain threads
-    uint32_t* slot = (uint32_t*)(dempty + 2);
+    uint64_t* dfull = empty + TC_NSTG;  // MMAs of a tile's panel done
+    uint64_t* dempty = dfull + 1;       // both accumulators read by the drain threads
+    uint32_t* slot = (uint32_t*)(dempty + 1);
     volatile int* abort = (volatile int*)(slot + 1);
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     if (t == 0) {
-        for (int i = 0; i < 2 * TC_NSTG + 2; ++i) tc::mbar_init(&full[i], 1);
-        tc::mbar_init(&dempty[0], TC_DRAIN);
-        tc::mbar_init(&dempty[1], TC_DRAIN);
+        for (int i = 0; i < 2 * TC_NSTG + 1; ++i) tc::mbar_init(&full[i], 1);
+        tc::mbar_init(dempty, TC_DRAIN);
         tc::fence_mbar_init();
         *abort = 0;
     }
@@ -340,8 +346,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
             int last = -1, lastph = 0;  // stage of the last commit
             bool ok = true;
             for (int gc = 0; gc < nmine * npan && ok; ++gc) {
-                const uint32_t h = gc & 1, dt = taddr + h * 256;
-                if (gc >= 2 && !wait(&dempty[h], ((gc >> 1) - 1) & 1)) {
+                if (gc >= 1 && !wait(dempty, (gc - 1) & 1)) {
                     ok = false;
                     break;
                 }
@@ -357,9 +362,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
                     for (int ks = 0; ks < TC_KC / 16; ++ks)
 #pragma unroll
                         for (int pr = 0; pr < 6; ++pr)
-                            tc::mma_bf16(dt, md + (PA[pr] * (M_TILE >> 4) + ks * 16),
+                            tc::mma_bf16(taddr + (pr ? 256 : 0), md + (PA[pr] * (M_TILE >> 4) + ks * 16),
                                          nd + (PB[pr] * (N_TILE >> 4) + ks * 16), idesc,
-                                         kc != 0 || ks != 0 || pr != 0);
+                                         kc != 0 || ks != 0 || pr > 1);
                     tc::commit(&empty[b]);
                     last = (int)b;
                     lastph = (int)ph;
@@ -368,7 +373,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
                         ph ^= 1;
                     }
                 }
-                if (ok) tc::commit(&dfull[h]);
+                if (ok) tc::commit(dfull);
             }
             if (!ok) {
                 *abort = 1;
@@ -426,21 +431,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
 #pragma unroll
             for (int q = 0; q < 64; ++q) c[q] = live ? Af[q * ld] : 0.f;
             for (int pn = 0; pn < npan; ++pn, ++gc) {
-                const uint32_t h = gc & 1;
-                if (!__all_sync(0xffffffffu, wait(&dfull[h], (gc >> 1) & 1))) {
+                if (!__all_sync(0xffffffffu, wait(dfull, gc & 1))) {
                     ok = false;
                     break;
                 }
                 tc::fence_after_sync();
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {
-                    float v[16];
-                    tc::tmem_ld16(taddr + ((uint32_t)(32 * lb) << 16) + h * 256 + 64 * c4 + 16 * ch, v);
+                for (int ch = 0; ch < 8; ++ch) {
+                    float v[8], w[8];
+                    const uint32_t at = taddr + ((uint32_t)(32 * lb) << 16) + 64 * c4 + 8 * ch;
+                    tc::tmem_ld8x2(at, at + 256, v, w);
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) c[16 * ch + q] = __fsub_rn(c[16 * ch + q], v[q]);
+                    for (int q = 0; q < 8; ++q)
+                        c[8 * ch + q] = __fsub_rn(c[8 * ch + q], __fadd_rn(v[q], w[q]));
                 }
                 tc::fence_before_sync();
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(&dempty[h]))
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(dempty))
                              : "memory");
             }
             if (ok && live)
