@@ -17,9 +17,12 @@
 // NPL = 2 (CR_CTX_S_BF16X3) is good to about 2^-17 per product.  That is the
 // form of CR_MIXED contexts; the others form the same sums on the FMA pipes
 // (spair_fma_kernel), an eighth of the additions of the P x P sums: float64
-// in CR_FP64, compensated float32 in CR_FP32 (products rounded to float32 as
-// before, the sum and its compensation together good to about 2^-46; the
-// float64 pipe does 1/64 of the float32 rate here).
+// in CR_FP64, two float32 words in CR_FP32 (products rounded to float32 as
+// before; error-free additions, so that the two words hold the sum to about
+// 2^-46; the float64 pipe does 1/64 of the float32 rate here).  Against 64 bits
+// the float32 form's S has the error of float64 sums of the same products,
+// 8.6e-9 of its norm (12 to 48 sites, 1024 to 32768 walkers); a Kahan sum,
+// which rounds each corrected term, had 1.16e-8.
 //
 // TMEM accumulates in float32 with an error that grows with the number of
 // MMAs added into one accumulator (measured: relative ~1e-8 each), so a
@@ -477,8 +480,9 @@ __global__ void __launch_bounds__(256) spair_expand_kernel(const T* __restrict__
 // The pair sums on the FMA pipes: a tile of 8 Q pairs x 16 Q columns of Y per
 // CTA and K segment, 8 x 16 threads with Q x Q sums each.  32 walkers at a
 // time, their spin products and tanh products formed in shared memory.
-// Float32: products rounded to float32, Kahan sums (s - c carries them);
-// float64: plain sums, Q = 2, so that small systems still spread over the SMs.
+// Float32: products rounded to float32, sums s + c by two-sum (Knuth, The Art
+// of Computer Programming vol. 2, 4.2.2); float64: plain sums, Q = 2, so that
+// small systems still spread over the SMs.
 template <typename R> struct FmaTile { static constexpr int Q = sizeof(R) == 4 ? 4 : 2; };
 constexpr int FMA_W = 32;
 
@@ -553,10 +557,11 @@ __global__ void __launch_bounds__(128) spair_fma_kernel(const int8_t* __restrict
                     if constexpr (sizeof(R) == 8) {
                         acc[p][q] = fma(av[p], yv[q], acc[p][q]);
                     } else {
-                        // Kahan: av = +-1, so the product is exact
-                        const R x = __fmaf_rn(av[p], yv[q], -cmp[p][q]);
-                        const R u = __fadd_rn(acc[p][q], x);
-                        cmp[p][q] = __fsub_rn(__fsub_rn(u, acc[p][q]), x);
+                        // (av = +-1: the product is exact)
+                        const R x = __fmul_rn(av[p], yv[q]), u = __fadd_rn(acc[p][q], x);
+                        const R z = __fsub_rn(u, acc[p][q]);
+                        cmp[p][q] = __fadd_rn(cmp[p][q], __fadd_rn(__fsub_rn(acc[p][q], __fsub_rn(u, z)),
+                                                                   __fsub_rn(x, z)));
                         acc[p][q] = u;
                     }
                 }
@@ -568,7 +573,7 @@ __global__ void __launch_bounds__(128) spair_fma_kernel(const int8_t* __restrict
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int r = a0 + ty + 8 * p, y = y0 + Q * tx + q;
-            if (r < nA && y < nY) out[(size_t)r * (nY + (nY & 1)) + y] = (double)acc[p][q] - (double)cmp[p][q];
+            if (r < nA && y < nY) out[(size_t)r * (nY + (nY & 1)) + y] = (double)acc[p][q] + (double)cmp[p][q];
         }
 }
 
