@@ -147,15 +147,17 @@ struct XArgs {
 };
 
 // e_b^s prod_m (a_m + z_m q_bm^s) of one bond by the whole warp, from cosh and
-// sinh with a running exponent; ysum = sum_m y_m, scaled by 2^-ex.
-__device__ __noinline__ zd slow_product(const XArgs& A, int w, int b, int s, double ysum, int ex0) {
+// sinh with a running exponent, scaled by 2^-ex0.
+__device__ __noinline__ zd slow_product(const XArgs& A, int w, int b, int s, int ex0) {
     const int lane = threadIdx.x & 31;
     const int2 bd = A.bonds[b];
     const cf* W = A.prm + A.N + A.M;
     cf pr = {1.f, 0.f};
     int ex = 0;
+    double ysum = 0.0;  // sum_m y_m, the phase that the common factor carries
     for (int m = lane; m < A.M; m += 32) {
         const cf th = A.th[(size_t)w * A.M + m];
+        ysum += (double)th.y;
         const cf d = 2.f * (W[(size_t)bd.x * A.M + m] - W[(size_t)bd.y * A.M + m]);
         cf ch, sh;
         ccoshsinh_(d, &ch, &sh);
@@ -182,7 +184,7 @@ __device__ __noinline__ zd slow_product(const XArgs& A, int w, int b, int s, dou
     pr = {__shfl_sync(0xffffffffu, pr.x, 0), __shfl_sync(0xffffffffu, pr.y, 0)};
     const zd da = 2.0 * (ccast<double>(A.prm[bd.x]) - ccast<double>(A.prm[bd.y]));
     const zd e = cexp_((s > 0 ? -1.0 : 1.0) * da);
-    const zd v = e * (cexp_(zd{0.0, -ysum}) * ccast<double>(pr));
+    const zd v = e * (cexp_(zd{0.0, -warp_sum(ysum)}) * ccast<double>(pr));
     return {ldexp(v.x, ex + A.M - ex0), ldexp(v.y, ex + A.M - ex0)};
 }
 
@@ -270,14 +272,12 @@ __global__ void __launch_bounds__(32 * XW, 1) xsum_kernel(const __grid_constant_
         u64 zr[WPW][KP], zi[WPW][KP], av[WPW][KP];
         ff sx[WPW], sy[WPW], dx[WPW], dy[WPW];
         int ex[WPW];
-        float ysum[WPW];
         // ------------------------------------------------ the warp's walkers
 #pragma unroll
         for (int u = 0; u < WPW; ++u) {
             const int w = w0 + u;
             sx[u] = sy[u] = dx[u] = dy[u] = ff{0.f, 0.f};
             ex[u] = 0;
-            ysum[u] = 0.f;
             const bool live = w < A.n;
             __syncwarp();
             if (live)
@@ -357,7 +357,6 @@ __global__ void __launch_bounds__(32 * XW, 1) xsum_kernel(const __grid_constant_
             bi = ff_warp_sum(bi);
             ff_add(bi, ys.hi);
             bi.lo += ys.lo;
-            ysum[u] = ys.hi;  // (slow_product's phase; its own terms are float32)
             if (live && lane == 0) {
                 A.out[w].base = make_float4(br.hi, br.lo, bi.hi, bi.lo);
                 A.out[w].nanti = nanti;
@@ -446,7 +445,7 @@ __global__ void __launch_bounds__(32 * XW, 1) xsum_kernel(const __grid_constant_
                         bm &= bm - 1;
                         const int e = lst[__shfl_sync(0xffffffffu, idx, src)];
                         const int s = e >> 15 ? -1 : 1, b = b0 + (e & 0x7fff);
-                        const zd term = slow_product(A, w0 + u, b, s, (double)ysum[u], ex[u]);
+                        const zd term = slow_product(A, w0 + u, b, s, ex[u]);
                         if (lane == 0) {
                             const float4 c = tile[(size_t)(2 * (e & 0x7fff) + (e >> 15)) * rowf4 + rowf4 - 1];
                             A.out[w0 + u].slow = A.out[w0 + u].slow + term;
