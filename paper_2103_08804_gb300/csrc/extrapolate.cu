@@ -23,6 +23,7 @@ namespace {
 constexpr int LP_THREADS = 256;
 constexpr int LP_MAX_ORDER = 512;
 constexpr int ABERTH_MAX_IT = 500;
+constexpr int LP_TABLE_ORDER = 8;  // roots from which the prediction uses tables
 
 using zd = cpx<double>;
 
@@ -280,7 +281,9 @@ __global__ void __launch_bounds__(LP_THREADS) lp_kernel(const LpArgs A) {
     // free here), so a predicted value costs one complex multiply-add per root
     // where its logarithm, angle, exponential and sine per root were 13 of the
     // 15 ms of 36 sequences of order 100 continued from 300 to 3000.
-    const int T = A.n_out - N, BK = min(p, 64), NA = min(p, (T + BK - 1) / BK);
+    // A table holds p x p values at most: few roots leave nothing to share, and
+    // their powers are formed value by value.
+    const int T = A.n_out - N, BK = min(min(p, 64), T), NA = BK ? min(p, (T + BK - 1) / BK) : 0;
     zd* wa = R;  // [NA][p] c_k w_k^{p + t0 + BK a}
     zd* wb = V;  // [BK][p] w_k^b
     auto power = [&](zd w, double m) {
@@ -292,7 +295,13 @@ __global__ void __launch_bounds__(LP_THREADS) lp_kernel(const LpArgs A) {
     };
     if (flag) {
         for (int t = tid; t < T; t += nt) out[N + t] = {nan, nan};
-    } else {
+    } else if (p < LP_TABLE_ORDER) {
+        for (int t = tid; t < T; t += nt) {
+            zd acc = {0.0, 0.0};
+            for (int k = 0; k < p; ++k) acc = acc + sa[k] * power(sz2[k], (double)(p + t));
+            out[N + t] = acc;
+        }
+    } else if (T > 0) {
         for (int e = tid; e < BK * p; e += nt) wb[e] = e < p ? zd{1.0, 0.0} : power(sz2[e % p], (double)(e / p));
         for (int t0 = 0; t0 < T; t0 += BK * NA) {
             __syncthreads();
