@@ -223,8 +223,8 @@ struct cr_ctx {
     int* d_status;           // device status word
     int2* d_bonds;           // [Nb]
     cr_tables tab[2];        // 0: sampler, 1: local target (float64 contexts)
-    uint16_t* sw_list;       // accepted moves of a sweep launch [maxB][sweep_list_cap]
-    int* sw_count;           // their number [maxB]
+    uint16_t* sw_list;       // accepted moves of a sweep launch [maxB][sweep_list_cap], or null
+    int* sw_count;           // their number [maxB], or null
     void* xtab;              // exchange table (float32 contexts)
     void* xout;              // xsum_out [maxB] (float32 contexts)
     void* theta_tmp;         // [maxB][M]
@@ -341,6 +341,7 @@ cr_status launch_cg_fused(cr_ctx* c, const int8_t* spins, const void* T, int B, 
                           const double* v_in, void* u_out);
 
 int sweep_list_cap(const cr_ctx* c);
+bool sweep_takes_lists(const cr_ctx* c);  // for any number of walkers and proposals
 cr_status sweep_prepare(cr_ctx* c);
 
 // Sums over exchanged amplitudes in float32 (exchange.cu).

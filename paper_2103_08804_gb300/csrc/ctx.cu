@@ -98,7 +98,7 @@ static std::vector<int2> make_bonds(int Lx, int Ly) {
 }
 
 static cudaError_t alloc(void** p, size_t bytes) {
-    if (bytes == 0) bytes = 16;
+    if (bytes == 0) return cudaSuccess;  // a buffer this context has no use for
     return cudaMalloc(p, bytes);
 }
 
@@ -158,8 +158,10 @@ extern "C" cr_status cr_create(cr_ctx** out, const cr_lattice* lat, int M, int m
     ALLOC(c->tab[0].D, Nb * Mp * cs);
     ALLOC(c->tab[0].CS, 2 * Nb * Mp * cs);
     ALLOC(c->tab[0].ea, Nb * 2 * cs);
-    ALLOC(c->sw_list, B * sweep_list_cap(c) * sizeof(uint16_t));
-    ALLOC(c->sw_count, B * sizeof(int));
+    if (sweep_takes_lists(c)) {
+        ALLOC(c->sw_list, B * sweep_list_cap(c) * sizeof(uint16_t));
+        ALLOC(c->sw_count, B * sizeof(int));
+    }
     if (prec == CR_FP64) {
         ALLOC(c->tab[1].ChT, Nb * Mp * cs);
         ALLOC(c->tab[1].ShT, Nb * Mp * cs);

@@ -520,12 +520,17 @@ __global__ void advance_counter_kernel(unsigned long long* ctr, unsigned long lo
 // 2706.  With 8 units a lane the few warps an SM holds hide little, and L1 pays
 // from some 48 proposals on small tables only.  Float64: the pipe is the bound,
 // L1 is 1 to 10% ahead up to 4 units a lane and 5 to 15% behind above.
+static size_t sweep_table_bytes(const cr_ctx* c) { return (size_t)c->Nb * c->Mp * 24; }  // float32
+bool sweep_takes_lists(const cr_ctx* c) {
+    return c->Mp > 128 || (c->prec != CR_FP64 && sweep_table_bytes(c) > 256 * 1024);
+}
 static bool sweep_in_l1(const cr_ctx* c, int B, int n_prop) {
+    if (!sweep_takes_lists(c)) return true;
+    if (c->prec == CR_FP64) return false;
     const int kpl = c->Mp / 32;
-    if (c->prec == CR_FP64) return kpl <= 4;
-    const size_t tab = (size_t)c->Nb * c->Mp * 24;
-    if (kpl <= 2) return tab <= 256 * 1024 || B >= 24 * c->n_sm;
-    if (kpl == 4) return tab <= 256 * 1024 || (tab <= 512 * 1024 && B >= 64 * c->n_sm);
+    const size_t tab = sweep_table_bytes(c);
+    if (kpl <= 2) return B >= 24 * c->n_sm;
+    if (kpl == 4) return tab <= 512 * 1024 && B >= 64 * c->n_sm;
     return kpl == 8 && tab <= 160 * 1024 && n_prop >= 48;
 }
 
