@@ -685,16 +685,20 @@ __global__ void __launch_bounds__(FC_THREADS, 1) cg_fused_kernel(const __grid_co
                     uacc = {0.f, 0.f};
                     if (valid) {
                         const int8_t* sr = a.spins + (size_t)sw * N;
-                        if ((N & 15) == 0) {
+                        if (vecS) {
                             for (int b16 = sp; b16 < N / 16; b16 += nsp) {
-                                int4 raw;
-                                if (vecS) raw = __ldg(reinterpret_cast<const int4*>(sr) + b16);
-                                else memcpy(&raw, sr + 16 * b16, 16);
+                                const int4 raw = __ldg(reinterpret_cast<const int4*>(sr) + b16);
                                 const int8_t* sv = reinterpret_cast<const int8_t*>(&raw);
 #pragma unroll
                                 for (int q = 0; q < 16; ++q)
                                     uacc = uacc + (float)sv[q] * s.va[16 * b16 + q];
                             }
+                        } else if ((N & 15) == 0) {  // unaligned: the same order, byte by byte
+#pragma unroll 1
+                            for (int b16 = sp; b16 < N / 16; b16 += nsp)
+#pragma unroll 1
+                                for (int i = 16 * b16; i < 16 * b16 + 16; ++i)
+                                    uacc = uacc + (float)sr[i] * s.va[i];
                         } else {
                             for (int i = sp; i < N; i += nsp) uacc = uacc + (float)sr[i] * s.va[i];
                         }
