@@ -78,24 +78,24 @@ template <typename R> CR_D cpx<R> warp_prod_rn(cpx<R> v) {
     return {__shfl_sync(0xffffffffu, v.x, 0), __shfl_sync(0xffffffffu, v.y, 0)};
 }
 
-// tanh of a lane's units 32 k + lane < M (0 past M).  The values next to a node,
-// which are rare, are formed again behind one branch: a branch per unit would
-// keep the units' chains of exponentials and sines from running side by side.
+// tanh of a lane's units 32 k + lane < M (0 past M).  Next to a node, which is
+// rare, the lane's values are formed again behind one branch: a branch per unit
+// would keep the units' chains of exponentials and sines from running side by
+// side.
 template <typename R, int KPL>
 CR_D void tanh_units(const cpx<R> (&th)[KPL], int M, int lane, cpx<R> (&T)[KPL]) {
-    R d[KPL];
     bool near = false;
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
+        R d = R(1);
         T[k] = {R(0), R(0)};
-        d[k] = R(1);
-        if (32 * k + lane < M) T[k] = ctanh_far(th[k], &d[k]);
-        near = near || near_node(d[k]);
+        if (32 * k + lane < M) T[k] = ctanh_far(th[k], &d);
+        near = near || near_node(d);
     }
     if (near)
 #pragma unroll
         for (int k = 0; k < KPL; ++k)
-            if (near_node(d[k])) T[k] = ctanh_near(th[k]);
+            if (32 * k + lane < M) T[k] = ctanh_(th[k]);
 }
 
 // theta (theta_out may be null: in place already), tanh theta and log psi of
@@ -103,31 +103,31 @@ CR_D void tanh_units(const cpx<R> (&th)[KPL], int M, int lane, cpx<R> (&T)[KPL])
 template <typename R, int KPL>
 CR_D void walker_outputs(const cpx<R> (&th)[KPL], int lane, int w, int M, int N, const cpx<R>* prm,
                          const int8_t* sg, cpx<R>* theta_out, cpx<R>* logpsi_out, cpx<R>* tanh_out) {
-    cpx<R> lp = {R(0), R(0)}, v[KPL];
-    R d[KPL];
+    cpx<R> lp = {R(0), R(0)};
     bool near = false;
 #pragma unroll
     for (int k = 0; k < KPL; ++k) {
-        v[k] = {R(0), R(0)};
-        d[k] = R(1);
-        if (32 * k + lane < M) {
-            if (theta_out) theta_out[(size_t)w * M + 32 * k + lane] = th[k];
-            v[k] = clncosh2_far(th[k], &d[k]);
+        const int j = 32 * k + lane;
+        if (j < M) {
+            R d, dt = R(1);
+            if (theta_out) theta_out[(size_t)w * M + j] = th[k];
+            lp = lp + clncosh2_far(th[k], &d);
+            if (tanh_out) tanh_out[(size_t)w * M + j] = ctanh_far(th[k], &dt);
+            near = near || near_node(d) || near_node(dt);
         }
-        near = near || near_node(d[k]);
     }
-    if (near)
+    if (near) {
+        lp = {R(0), R(0)};
 #pragma unroll
-        for (int k = 0; k < KPL; ++k)
-            if (near_node(d[k])) v[k] = clncosh2_near(th[k]);
-#pragma unroll
-    for (int k = 0; k < KPL; ++k)
-        if (32 * k + lane < M) lp = lp + v[k];
-    if (tanh_out) {
-        tanh_units(th, M, lane, v);
-#pragma unroll
-        for (int k = 0; k < KPL; ++k)
-            if (32 * k + lane < M) tanh_out[(size_t)w * M + 32 * k + lane] = v[k];
+        for (int k = 0; k < KPL; ++k) {
+            const int j = 32 * k + lane;
+            if (j < M) {
+                R d;
+                const cpx<R> v = clncosh2_far(th[k], &d);
+                lp = lp + (near_node(d) ? clncosh2_near(th[k]) : v);
+                if (tanh_out) tanh_out[(size_t)w * M + j] = ctanh_(th[k]);
+            }
+        }
     }
     if (!logpsi_out) return;
     for (int i = lane; i < N; i += 32) lp = lp + R(sg[i]) * prm[i];
