@@ -39,7 +39,7 @@
  *   Parameters. An RBM with N visible and M hidden units is one complex
  *     vector alpha = [a (N) | b (M) | W (N x M, row-major, W[i*M + j])];
  *     its index is the k of O_k, S_kk' and F_k. P = N + M + N*M.
- *   Spins. int8 [B][N], entries +1 / -1, site r = x + Lx*y.
+ *   Spins. int8 [B][N], entries +1 / -1, site r = x + Lx*y, at any address.
  *   Lattice. Periodic; bonds are all (r, r + x-hat) in increasing r and
  *     then, when Ly > 1, all (r, r + y-hat) in increasing r.
  *   Hamiltonian. H = J sum_b S_i . S_j with S^z = sigma/2 (Sec. V);
@@ -88,10 +88,10 @@ typedef enum {
 /* Context flags. */
 #define CR_CTX_EXPLICIT_S 1 /* allocate the explicit P x P complex128 S for
                                Cholesky solves */
-#define CR_CTX_S_BF16X3 2   /* mixed contexts: build the explicit S from two-term
-                               bf16 splits (three products, about 2^-16 relative
-                               per product) instead of the default three-term
-                               splits (six products, about float32 accuracy).
+#define CR_CTX_S_BF16X3 2   /* mixed contexts: build the explicit S with two bf16
+                               terms of each product of tanh theta (about 2^-17
+                               relative) instead of the default three (all 24
+                               bits); the spins are exact in one.
                                Cheaper, but its error can make S + shift I
                                indefinite at small shifts (CR_ESINGULAR). */
 
@@ -106,17 +106,18 @@ typedef enum {
 
 /* Solvers for sr_step. */
 #define CR_SOLVE_CHOLESKY 0 /* explicit S and a direct solve (needs CR_CTX_EXPLICIT_S):
-                               float64 contexts with P <= 2048 factor S in float64 in one
-                               CTA; every other context factors S blocked (64 x 64
-                               blocks, many CTAs) in the factor precision (float64 for
-                               float64 contexts, float32 otherwise) and refines the
-                               solution in float64 against S until |r| <= 1e-12 |F|,
-                               the residual stops halving, or min(cg_maxit, 10) steps
-                               (stats [5] steps, [6] relative residual).  Mixed
-                               contexts build S on the tensor cores (bf16 splits of
-                               both operands, float32 accumulation; see
-                               CR_CTX_S_BF16X3); the others accumulate it in
-                               float64. */
+                               float64 contexts with P <= 2048 factor S in float64 and
+                               solve once; every other context factors S blocked in the
+                               factor precision (float64 for float64 contexts, float32
+                               otherwise) and refines the solution in float64 against S
+                               until |r| <= 1e-12 |F|, the residual stops halving, or
+                               min(cg_maxit, 10) steps (stats [5] steps, [6] relative
+                               residual).  S comes from sums over walkers of spin pairs
+                               times tanh pairs: on the tensor cores in mixed contexts
+                               (spins exact in bf16, tanh products in bf16 terms,
+                               float32 accumulation; see CR_CTX_S_BF16X3), in float64
+                               in CR_FP64, in two float32 words in CR_FP32 (products
+                               rounded to float32; the sums keep what float64 would). */
 #define CR_SOLVE_CG 1       /* matrix-free S v = O^dag (O v) / Ns, float64 CG */
 
 /* Length of the stats array written by sr_step (complex128 / float64 slots). */

@@ -10,9 +10,10 @@
 //   q_bm^s = e^{2 s D_bm},
 // so that v(s^{ij}) = e^{a.s + sum_m (|x_m| + i y_m)} e_b^s prod_m (a_m + z_m q_bm^s)
 // with the bond constant e_b^s = exp(-s [2 (a_i - a_i') + sum_m D_bm]).  A factor
-// is one complex multiply-add and one complex multiply (8 flops against the
-// 14 of cosh theta cosh D - s sinh theta sinh D) and takes one table value;
-// no factor divides, so a sample may sit at a node of v.
+// is one complex multiply-add and one complex multiply (13 flops in 8 operations
+// of the FMA pipe, against 14 operations for cosh theta cosh D - s sinh theta
+// sinh D) and takes one table value; no factor divides, so a sample may sit at
+// a node of v.
 //
 // The products run over hidden units spread across lanes: G lanes hold the
 // whole hidden layer of a walker, 2 KP units each, in registers, so a warp
@@ -64,7 +65,10 @@ CR_D u64 mul2(u64 a, u64 b) {
 CR_D u64 neg2(u64 a) { return a ^ 0x8000000080000000ull; }
 
 // Sums carried as an unevaluated pair hi + lo (error-free two-term additions,
-// Knuth, The Art of Computer Programming vol. 2, 4.2.2).
+// Knuth, The Art of Computer Programming vol. 2, 4.2.2).  The terms are float32,
+// so a pair keeps what a float64 sum of them would to 2^-46: against 64 bits
+// the target has 0.85 to 0.89 (14 draws, 12 to 256 sites) and the symmetry
+// projection 0.97 (5 draws) of the error of the form with float64 sums.
 struct ff { float hi, lo; };
 CR_D void ff_add(ff& s, float v) {
     const float t = __fadd_rn(s.hi, v), z = __fsub_rn(t, s.hi);

@@ -75,7 +75,7 @@ cr_status build_tables(cr_ctx* c, const void* params, int slot, int planar) {
 //
 // Bound by the FMA pipe and, for log psi, by the exponential, sine and cosine
 // of every theta; log(2 cosh) of two units shares one logarithm and one
-// angle.  16 x 16 lattice, 65536 walkers: 604 -> 503 us (one block of 128
+// angle.  16 x 16 lattice, 65536 walkers: 547 -> 487 us (one block of 128
 // threads per 16 walkers before, weights read from L2 by every block); M = 72:
 // 921 -> 530 us; float64 at N = M = 12: 130 -> 15 us.  Packed pairs of
 // multiply-adds did not help (527 us).
