@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(128) hprime_kernel(hp_args<R> A) {
                 shc[u] = A.ShT + bb[u];
             }
             // the products of M factors are kept as pr * 2^ex, renormalised
-            // every 16 factors, so they cannot overflow or underflow float32
+            // every 16 factors, so they cannot overflow or underflow
             for (int m = 0; m < A.M; ++m) {
                 const cpx<R> cm = Cm[m], sm = Sm[m];
 #pragma unroll
