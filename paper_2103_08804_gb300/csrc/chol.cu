@@ -173,9 +173,12 @@ CR_D void tile_step(const cf (*As)[NB + 1], const cf (*Bs)[BP], int tx, int ty, 
 // so that D[2k + part][i] = (Re, Im)(L_i . conj(L_k)): lanes (D rows) hold
 // consecutive floats of a row of A, and a tile's 256 rows x 64 columns are
 // read and written coalesced.  A panel is 128 real deep.  An MMA's addition
-// truncates, so its error grows with the number of them: the eight MMAs of
-// the leading products have an accumulator of their own, and the forty others,
-// 2^-8 of it, another; then one float32 addition and subtraction.
+// truncates 2^-24 or so of its accumulator, so its error grows with the number
+// of them that meet a large one: the eight MMAs of the first panel's leading
+// products have an accumulator of their own; the small products of both
+// panels, 2^-8 of those, go into another, and the second panel's leading ones
+// into that after them, from a second copy of their operands.  Then one float32
+// addition and subtraction for the pair.
 constexpr uint32_t WAIT_LIMIT = 1u << 26;  // bounded mbarrier polls
 constexpr int TC_ROWS = 256, TC_COLS = 64;  // tile of A
 constexpr int TC_KC = 32, TC_NKC = 2 * NB / TC_KC;  // K tiles of a panel; operands hold two panels
@@ -273,23 +276,25 @@ __global__ void __launch_bounds__(256) trsm_kernel(cf* __restrict__ L, int P, in
 // 64 columns.  npan = 1, after the first panel: the tiles of column block 0,
 // the second panel's.  npan = 2, after the second: row block rb takes the
 // column blocks 1 <= cb <= 4 rb + 3 that exist (tile index 2 rb^2 + rb + cb -
-// 1), one subtraction per panel, but not the first 64 rows, which are done.
+// 1), one subtraction for both panels, but not the first 64 rows, which are
+// done.
 //
 // Bound: 16 bytes of A per entry and update against 1.5 KB of MMA operands,
 // which L2 serves.  A panel at a time (10 x 10 lattice, alpha = 1: P = 10200)
 // the kernel moved A at 3.9 TB/s, waiting for the loads of 8 drain warps: 159
 // launches, 11.4 ms.  In pairs, with 16 drain warps that have a whole tile of
-// A in flight while its MMAs run: 8.0 ms; 10.2 with an accumulator for the leading
-// products, since both fill TMEM and the MMAs of a panel wait for the drain
-// of the last.  That buys the factor's accuracy: the residual left by one
-// correction, over P = 168 ... 10200, went from 2.15 times that of a factor by
-// float32 multiply-adds and substitution to 1.15 (1.12 on the FMA pipes here,
-// the inverses' share), the corrections needed from 3.03 to 2.69 on average.
+// A in flight while its MMAs run: 8.0 ms, with 48 MMAs a panel into one
+// accumulator, two of which alternate; 8.7 now, with both held for a tile.  That
+// buys the factor's accuracy: the residual that one correction leaves, over P =
+// 168 ... 10200, went from 2.15 times that of a factor by float32 multiply-adds
+// and substitution to 1.11 (1.12 on the FMA pipes here, the inverses' share),
+// the corrections needed from 3.03 to 2.62 on average (2.71).  A drain after each
+// panel gave 1.15 and 10.2 ms, both panels' leading products in one accumulator
+// 1.27 and 8.2.
 //
-// Persistent: warp 0 (one thread) issues the MMAs, panel by panel into TMEM
-// columns [0, 256) (leading products) and [256, 512), warps 1-16 drain (warp w:
-// lanes 32 (w % 4), rows 64 ((w - 1) / 4)), warp 17 (one thread) copies operand
-// stages.
+// Persistent: warp 0 (one thread) issues a tile's MMAs into TMEM columns [0,
+// 256) and [256, 512), warps 1-16 drain (warp w: lanes 32 (w % 4), rows 64 ((w -
+// 1) / 4)), warp 17 (one thread) copies operand stages.
 __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restrict__ Lf, int P, int r0,
                                                                 int npan, int ntiles,
                                                                 const unsigned char* __restrict__ planes,
@@ -297,7 +302,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
     extern __shared__ __align__(1024) unsigned char sm[];
     uint64_t* full = (uint64_t*)(sm + TC_NSTG * TC_STAGE);
     uint64_t* empty = full + TC_NSTG;
-    uint64_t* dfull = empty + TC_NSTG;  // MMAs of a tile's panel done
+    uint64_t* dfull = empty + TC_NSTG;  // MMAs of a tile done
     uint64_t* dempty = dfull + 1;       // both accumulators read by the drain threads
     uint32_t* slot = (uint32_t*)(dempty + 1);
     volatile int* abort = (volatile int*)(slot + 1);
@@ -337,6 +342,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
         *cb = idx - (2 * r * r + r) + 1;
     };
     const int nmine = ntiles > (int)blockIdx.x ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int nst = npan == 1 ? TC_NKC : 3 * TC_NKC;  // operand stages of a tile
     if (warp == 0) {
         if (lane == 0) {
             constexpr int PA[6] = {0, 0, 1, 0, 1, 2}, PB[6] = {0, 1, 0, 2, 1, 0};
@@ -345,12 +351,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
             uint32_t b = 0, ph = 0;
             int last = -1, lastph = 0;  // stage of the last commit
             bool ok = true;
-            for (int gc = 0; gc < nmine * npan && ok; ++gc) {
-                if (gc >= 1 && !wait(dempty, (gc - 1) & 1)) {
+            for (int ti = 0; ti < nmine && ok; ++ti) {
+                if (ti >= 1 && !wait(dempty, (ti - 1) & 1)) {
                     ok = false;
                     break;
                 }
-                for (int kc = 0; kc < TC_NKC; ++kc) {
+                for (int kc = 0; kc < nst; ++kc) {
                     if (!wait(&full[b], ph)) {
                         ok = false;
                         break;
@@ -358,13 +364,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
                     tc::fence_after_sync();
                     const uint64_t nd = d0 + b * (uint32_t)(TC_STAGE >> 4);
                     const uint64_t md = nd + (3 * N_TILE >> 4);
+                    // first panel: leading products to [0, 256), small ones to [256, 512);
+                    // second: its small ones there too, its leading ones last
+                    const bool lead = kc < TC_NKC || kc >= 2 * TC_NKC, small = kc < 2 * TC_NKC;
 #pragma unroll
-                    for (int ks = 0; ks < TC_KC / 16; ++ks)
+                    for (int ks = 0; ks < TC_KC / 16; ++ks) {
+                        if (lead)
+                            tc::mma_bf16(taddr + (small ? 0 : 256), md + ks * 16, nd + ks * 16, idesc,
+                                         kc != 0 || ks != 0);
+                        if (small)
 #pragma unroll
-                        for (int pr = 0; pr < 6; ++pr)
-                            tc::mma_bf16(taddr + (pr ? 256 : 0), md + (PA[pr] * (M_TILE >> 4) + ks * 16),
-                                         nd + (PB[pr] * (N_TILE >> 4) + ks * 16), idesc,
-                                         kc != 0 || ks != 0 || pr > 1);
+                            for (int pr = 1; pr < 6; ++pr)
+                                tc::mma_bf16(taddr + 256, md + (PA[pr] * (M_TILE >> 4) + ks * 16),
+                                             nd + (PB[pr] * (N_TILE >> 4) + ks * 16), idesc,
+                                             kc != 0 || ks != 0 || pr > 1);
+                    }
                     tc::commit(&empty[b]);
                     last = (int)b;
                     lastph = (int)ph;
@@ -392,15 +406,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
                 tile_of(blockIdx.x + ti * gridDim.x, &rb, &cb);
                 const unsigned char* ns = planes + (size_t)rb * 2 * TC_NKC * 3 * N_TILE;
                 const unsigned char* ms = planes + m_off + (size_t)cb * 2 * TC_NKC * 3 * M_TILE;
-                for (int kc = 0; kc < npan * TC_NKC; ++kc, ++g, ns += 3 * N_TILE, ms += 3 * M_TILE) {
+                for (int kc = 0; kc < nst; ++kc, ++g) {
                     if (g >= TC_NSTG && !wait(&empty[b], ph ^ 1)) {
                         ok = false;
                         break;
                     }
                     unsigned char* st = sm + (size_t)b * TC_STAGE;
-                    tc::mbar_expect_tx(&full[b], (uint32_t)TC_STAGE);
-                    tc::bulk_g2s(st, ns, 3 * N_TILE, &full[b]);
-                    tc::bulk_g2s(st + 3 * N_TILE, ms, 3 * M_TILE, &full[b]);
+                    // the second panel's leading terms come a second time, alone
+                    const bool again = kc >= 2 * TC_NKC;
+                    const int k = again ? kc - TC_NKC : kc, np = again ? 1 : 3;
+                    tc::mbar_expect_tx(&full[b], (uint32_t)(np * (N_TILE + M_TILE)));
+                    tc::bulk_g2s(st, ns + (size_t)k * 3 * N_TILE, np * N_TILE, &full[b]);
+                    tc::bulk_g2s(st + 3 * N_TILE, ms + (size_t)k * 3 * M_TILE, np * M_TILE, &full[b]);
                     if (++b == TC_NSTG) {
                         b = 0;
                         ph ^= 1;
@@ -420,7 +437,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
         const int lb = warp & 3, c4 = (warp - 1) >> 2;
         const size_t ld = 2 * (size_t)lcols(P);
         bool ok = true;
-        int gc = 0;
         for (int ti = 0; ti < nmine && ok; ++ti) {
             int rb, cb;
             tile_of(blockIdx.x + ti * gridDim.x, &rb, &cb);
@@ -430,26 +446,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) syrk_tc_kernel(float* __restric
             float c[64];
 #pragma unroll
             for (int q = 0; q < 64; ++q) c[q] = live ? Af[q * ld] : 0.f;
-            for (int pn = 0; pn < npan; ++pn, ++gc) {
-                if (!__all_sync(0xffffffffu, wait(dfull, gc & 1))) {
-                    ok = false;
-                    break;
-                }
-                tc::fence_after_sync();
+            ok = __all_sync(0xffffffffu, wait(dfull, ti & 1));
+            if (!ok) break;
+            tc::fence_after_sync();
 #pragma unroll
-                for (int ch = 0; ch < 8; ++ch) {
-                    float v[8], w[8];
-                    const uint32_t at = taddr + ((uint32_t)(32 * lb) << 16) + 64 * c4 + 8 * ch;
-                    tc::tmem_ld8x2(at, at + 256, v, w);
+            for (int ch = 0; ch < 8; ++ch) {
+                float v[8], w[8];
+                const uint32_t at = taddr + ((uint32_t)(32 * lb) << 16) + 64 * c4 + 8 * ch;
+                tc::tmem_ld8x2(at, at + 256, v, w);
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        c[8 * ch + q] = __fsub_rn(c[8 * ch + q], __fadd_rn(v[q], w[q]));
-                }
-                tc::fence_before_sync();
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(dempty))
-                             : "memory");
+                for (int q = 0; q < 8; ++q)
+                    c[8 * ch + q] = __fsub_rn(c[8 * ch + q], __fadd_rn(v[q], w[q]));
             }
-            if (ok && live)
+            tc::fence_before_sync();
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(tc::smem_u32(dempty)) : "memory");
+            if (live)
 #pragma unroll
                 for (int q = 0; q < 64; ++q) Af[q * ld] = c[q];
         }

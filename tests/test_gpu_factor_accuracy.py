@@ -2,7 +2,7 @@
 as good as that of float32 contexts (FMA pipes): the residual that one
 correction leaves, |F - S x| / |F| after a solve with the factor alone, is the
 factor's error times the condition number.  Both factors take the same panels
-and one float32 subtraction per panel, so the two differ by the roundings of the
+and subtract in float32, so the two differ by the roundings of the
 products only: within a factor 1.5 (they agree to 10% over P = 168 ... 10200;
 48 MMAs into one truncating accumulator had left 1.9 on average)."""
 
