@@ -512,14 +512,23 @@ __global__ void advance_counter_kernel(unsigned long long* ctr, unsigned long lo
 // list, but every evaluated proposal waits for its rows; warps hide that where
 // there are many of them with few units each, or where the tables (cosh, sinh
 // and D, 24 or 48 bytes a bond and unit) stay in L1.  Times of four sweeps, us,
-// lists / L1: 8 x 8 lattice with 33 units (192 KB), 16384 walkers 662 / 492, 200
-// walkers 110 / 100; 64 sites with 128 units (192 KB), 926 / 711 and 136 / 121;
-// 10 x 10 with 60 units (300 KB), 1002 / 808 and 157 / 168; 8 x 8 with 128
-// units (384 KB), 915 / 845 and 133 / 158; 10 x 10 with 100 units (600 KB), 4096
-// walkers 458 / 545; 96 sites with 192 units, 8 units a lane (576 KB), 2145 /
-// 2706.  With 8 units a lane the few warps an SM holds hide little, and L1 pays
-// from some 48 proposals on small tables only.  Float64: the pipe is the bound,
-// L1 is 1 to 10% ahead up to 4 units a lane and 5 to 15% behind above.
+// lists / L1, one GB300 (152 SMs):
+//   units, table             walkers: 608      1400     3001     6001     20005
+//   15 x 6 lattice, 40, 270 KB     146/151  165/158  214/179  390/333 1087/890
+//   14 x 9, 48, 378 KB             195/221  220/230  288/258  529/487 1489/1291
+//   16 x 16, 64, 768 KB            418/489  470/507  598/552 1087/1055 3035/2764
+//   90 sites, 128, 270 KB          181/185  211/203  275/235  511/447 1529/1410
+//   8 x 8, 128, 384 KB             132/159  153/167  200/189  368/354 1102/1126
+//   10 x 8, 128, 480 KB            164/203  191/216  257/240  466/452 1395/1447
+//   10 x 10, 100, 600 KB           197/261  231/275  315/303  570/576 1721/1855
+//   12 x 12, 128, 864 KB           289/385     -     456/443  819/851 2462/2782
+//   24 sites, 250, 144 KB (a sweep) 40/41    44/41    69/65   101/97   267/279
+// With 128 units an SM holds five blocks of four walkers, and L1 is as fast as
+// the lists or faster where its last wave is full (3001 and 6001 walkers; 3648:
+// 8 x 8 282/317), the more so beside lists that have just begun another block
+// per SM (from 2433 walkers).  With 8 units a lane the few warps hide little.
+// Float64: the pipe is the bound, L1 is 1 to 10% ahead up to 4 units a lane and
+// 5 to 15% behind above.
 static size_t sweep_table_bytes(const cr_ctx* c) { return (size_t)c->Nb * c->Mp * 24; }  // float32
 bool sweep_takes_lists(const cr_ctx* c) {
     return c->Mp > 128 || (c->prec != CR_FP64 && sweep_table_bytes(c) > 256 * 1024);
@@ -528,10 +537,14 @@ static bool sweep_in_l1(const cr_ctx* c, int B, int n_prop) {
     if (!sweep_takes_lists(c)) return true;
     if (c->prec == CR_FP64) return false;
     const int kpl = c->Mp / 32;
-    const size_t tab = sweep_table_bytes(c);
-    if (kpl <= 2) return B >= 24 * c->n_sm;
-    if (kpl == 4) return tab <= 512 * 1024 && B >= 64 * c->n_sm;
-    return kpl == 8 && tab <= 160 * 1024 && n_prop >= 48;
+    const size_t kb = sweep_table_bytes(c) / 1024;
+    const int sm = (B - 1) / c->n_sm;  // walkers of the fullest SM, less one
+    if (kpl <= 2) return sm >= (int)(kb < 600 ? kb / 50 : 12);
+    if (kpl == 4) {
+        if (kb <= 300) return sm >= 6;
+        return kb <= 448 ? sm % 20 >= 12 : kb <= 640 && sm < 40 && sm % 20 >= 16;
+    }
+    return kpl == 8 && kb <= 160 && (n_prop >= 48 || (sm >= 8 && sm < 48));
 }
 
 // Proposals per sweep launch: its list of accepted moves per walker.

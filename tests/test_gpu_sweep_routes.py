@@ -46,6 +46,12 @@ def test_routes_agree_bit_for_bit(Lx, Ly, M, many, n_sweeps):
     assert all(np.array_equal(x, y[:few]) for x, y in zip(a, b))
 
 
+@pytest.mark.parametrize("Lx,Ly,M,many", [(90, 1, 128, 1100), (8, 8, 128, 3000), (10, 10, 100, 3000),
+                                          (24, 1, 250, 1400)])
+def test_routes_where_a_wave_of_l1_is_full(Lx, Ly, M, many):
+    test_routes_agree_bit_for_bit(Lx, Ly, M, many, 1)
+
+
 @pytest.mark.parametrize("Lx,Ly,M", [(12, 1, 30), (6, 6, 60), (6, 4, 100), (8, 1, 200), (6, 1, 300)])
 @pytest.mark.parametrize("n_sweeps", [1, 20])
 def test_float64_routes(Lx, Ly, M, n_sweeps):
