@@ -75,10 +75,19 @@ cr_status build_tables(cr_ctx* c, const void* params, int slot, int planar) {
 //
 // Bound by the FMA pipe and, for log psi, by the exponential, sine and cosine
 // of every theta; log(2 cosh) of two units shares one logarithm and one
-// angle.  16 x 16 lattice, 65536 walkers: 547 -> 487 us (one block of 128
+// angle.  16 x 16 lattice, 65536 walkers: 547 -> 490 us (one block of 128
 // threads per 16 walkers before, weights read from L2 by every block); M = 72:
 // 921 -> 530 us; float64 at N = M = 12: 130 -> 15 us.  Packed pairs of
 // multiply-adds did not help (527 us).
+//
+// The sum over units is of log cosh; M log 2, which would be most of it where
+// theta is small, comes in with the last level, whose rounding errors are kept.
+// With log 2cosh summed plainly the error depends on where the layout's partial
+// sums pass powers of two.  Error of float32 against 64 bits, |theta| < 0.1, 48
+// sites with 96 units: 3.2e-6 with a sum of 128 threads, 3.5e-6 with this layout
+// and plain sums, 2.3e-6 so (the rounding of the result alone 2.2e-6); 64 sites
+// with 128 units 4.2e-6, 3.6e-6, 2.3e-6.  16 x 16 lattice, 65536 walkers: 486 us
+// with plain sums, 490 so.
 enum { MODE_LOGPSI = 0, MODE_MATVEC = 1 };
 
 namespace {
@@ -104,20 +113,27 @@ template <typename R> __device__ __noinline__ NearNode<R> near_node_call(R ax, R
     return near_node_terms(ax, y, e);
 }
 
-// log(2 cosh z) summed over the lane's units: s z and 1 + w of each (|w| <= 1,
-// so two arguments add up without a branch cut), the logarithm of two units'
+// log(cosh z) summed over the lane's units: s z and (1 + w) / 2 of each (|w| <=
+// 1, so two arguments add up without a branch cut), the logarithm of two units'
 // product at once.
-template <typename R> CR_D void lncosh_parts(cpx<R> z, cpx<R>* lin, cpx<R>* onew) {
+template <typename R> CR_D void lncosh_parts(cpx<R> z, cpx<R>* lin, cpx<R>* half) {
     const R sg = z.x < R(0) ? R(-1) : R(1);
-    const R e = m_exp(R(-2) * sg * z.x);
+    const R e = m_exp(R(-2) * sg * z.x), h = R(0.5) * e;
     R s, c;
     m_sincos(R(-2) * sg * z.y, &s, &c);
     *lin = *lin + sg * z;
-    *onew = {R(1) + e * c, e * s};
-    if (near_node(abs2(*onew))) {
+    *half = {R(0.5) + h * c, h * s};
+    if (abs2(*half) < R(0.015625 / 4)) {  // near_node of twice that
         const NearNode<R> n = near_node_call(sg * z.x, z.y, e);
-        *onew = {n.om + R(2) * e * n.c * n.c, R(-2) * sg * e * n.s * n.c};
+        *half = {R(0.5) * n.om + e * n.c * n.c, -sg * e * n.s * n.c};
     }
+}
+
+// s + v, its rounding error added to *e (Knuth's two-sum, TAOCP 2, 4.2.2).
+template <typename R> CR_D R add_exact(R s, R v, R* e) {
+    const R t = s + v, b = t - s;
+    *e += (s - (t - b)) + (v - b);
+    return t;
 }
 
 }  // namespace
@@ -128,7 +144,8 @@ __global__ void __launch_bounds__(32 * TH_WARPS, 2) theta_kernel(const cpx<R>* _
                                                               int N, int M, cpx<R>* __restrict__ theta_out,
                                                               cpx<R>* __restrict__ out,
                                                               const cpx<R>* __restrict__ T,
-                                                              const double* __restrict__ skip) {
+                                                              const double* __restrict__ skip,
+                                                              R ln2_hi, R ln2_lo) {
     if (skip && *skip != 0.0) return;  // converged CG: nothing left to do
     constexpr int NG = 32 / LJ, WB = TH_W * NG * TH_WARPS, JB = LJ * JW, NT = 32 * TH_WARPS;
     __shared__ __align__(16) R sg[2][TH_KC][WB];
@@ -247,10 +264,19 @@ __global__ void __launch_bounds__(32 * TH_WARPS, 2) theta_kernel(const cpx<R>* _
     for (int w = 0; w < TH_W; ++w) {
         cpx<R> v = part[w];
 #pragma unroll
-        for (int o = LJ / 2; o > 0; o >>= 1)
+        for (int o = LJ / 2; o > 1; o >>= 1)
             v = v + cpx<R>{__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)};
-        if (l == 0 && w0 + wl + w < B) out[w0 + wl + w] = v;
+        const cpx<R> v2 = {__shfl_xor_sync(0xffffffffu, v.x, 1), __shfl_xor_sync(0xffffffffu, v.y, 1)};
+        part[w] = v + v2;
+        if (MODE == MODE_LOGPSI) {
+            R e = ln2_lo;
+            const R t = add_exact(add_exact(v.x, v2.x, &e), ln2_hi, &e);
+            part[w].x = isfinite(e) ? t + e : t;  // an infinite sum has no remainder
+        }
     }
+#pragma unroll
+    for (int w = 0; w < TH_W; ++w)
+        if (l == 0 && w0 + wl + w < B) out[w0 + wl + w] = part[w];
 }
 
 template <typename R, int TW, int MODE>
@@ -263,10 +289,13 @@ static cr_status launch_theta_w(cr_ctx* c, const void* params, const int8_t* spi
                   (theta_kernel<R, LJ, JW, TW, MODE>                                             \
                    <<<(B + WB - 1) / WB, 32 * TH_WARPS, 0, c->stream>>>(                         \
                        (const cpx<R>*)params, spins, B, c->N, c->M, (cpx<R>*)theta,              \
-                       (cpx<R>*)out, (const cpx<R>*)T, skip)));                                  \
+                       (cpx<R>*)out, (const cpx<R>*)T, skip, hi, lo)));                          \
     }
     // units per lane and pass: the fewest padded units (float64: registers for two)
     const int M = c->M;
+    // M log 2 as two words; log 2 in two doubles
+    const double L = 0.6931471805599453, ln2 = M * L, rest = std::fma((double)M, L, -ln2) + M * 2.3190468138462996e-17;
+    const R hi = (R)ln2, lo = (R)(ln2 - (double)hi + rest);
     if (M <= 16) LAUNCH(16, 1)
     else if (M <= 32) LAUNCH(32, 1)
     else if (M <= 64 || sizeof(R) == 8) LAUNCH(32, 2)
